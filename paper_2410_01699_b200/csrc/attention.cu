@@ -23,10 +23,10 @@ constexpr int MAXD = 4;       // head dims per lane: head_dim <= 128
 template <typename T>
 __global__ void __launch_bounds__(NWARPS * 32) attention_partial_kernel(
     const float *__restrict__ q, KvLayout kv, const int32_t *__restrict__ in_pos, float *__restrict__ partial,
-    int rows_per_seq, int n_heads, int splits) {
+    RowSegs segs, int n_heads, int splits) {
   extern __shared__ float smem[];
   const int hd = kv.head_dim;
-  const int W = rows_per_seq;
+  const int W = segs.rows;
   float *Qs = smem;                       // [W][hd]
   float *Ks = Qs + W * hd;                // [TK][hd + 1]
   float *Vs = Ks + TK * (hd + 1);         // [TK][hd]
@@ -34,10 +34,11 @@ __global__ void __launch_bounds__(NWARPS * 32) attention_partial_kernel(
   __shared__ int s_pos[64];
   __shared__ int s_len;
 
-  const int h = blockIdx.x, b = blockIdx.y, s = blockIdx.z;
+  const int h = blockIdx.x, seg = blockIdx.y, s = blockIdx.z;
+  const int b = seg_sequence(segs, seg);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kvh = h / (n_heads / kv.n_kv_heads);
-  const int m0 = b * W;
+  const int m0 = seg * W;
 
   if (tid < 64) s_pos[tid] = tid < W ? in_pos[m0 + tid] : -1;
   __syncthreads();
@@ -163,7 +164,14 @@ __global__ void attention_combine_kernel(const float *__restrict__ partial, cons
   const int m = blockIdx.x, h = blockIdx.y;
   const float *src = partial + ((size_t)m * n_heads + h) * splits * (hd + 2);
   const size_t base = ((size_t)m * n_heads + h) * hd;
-  float *dst = out + base;
+  auto put = [&](int d, float v) {
+    if (out) out[base + d] = v;
+    if (hilo.base) {
+      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+      hilo.base[base + d] = hi;
+      hilo.base[hilo.lo_offset + base + d] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    }
+  };
   constexpr int NS = 8;
   if (splits <= NS && hd <= (int)blockDim.x) {
     // Few key ranges (the usual case): every thread fetches the row's position, all record heads and its own
@@ -194,21 +202,12 @@ __global__ void attention_combine_kernel(const float *__restrict__ partial, cons
         if (s < splits) acc += vv[s] * (mm[s] > -INFINITY ? expf(mm[s] - gmax) : 0.0f);
       v = denom > 0.0f ? acc / denom : 0.0f;
     }
-    dst[d] = v;
-    if (hilo.base) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      hilo.base[base + d] = hi;
-      hilo.base[hilo.lo_offset + base + d] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
+    put(d, v);
     return;
   }
   if (in_pos[m] < 0) {
     for (int d = threadIdx.x; d < hd; d += blockDim.x) {
-      dst[d] = 0.0f;
-      if (hilo.base) {
-        hilo.base[base + d] = __float2bfloat16_rn(0.0f);
-        hilo.base[hilo.lo_offset + base + d] = __float2bfloat16_rn(0.0f);
-      }
+      put(d, 0.0f);
     }
     return;
   }
@@ -233,26 +232,21 @@ __global__ void attention_combine_kernel(const float *__restrict__ partial, cons
 #pragma unroll 4
     for (int s = 0; s < ns; ++s) acc += src[(size_t)s * (hd + 2) + 2 + d] * s_w[s];
     const float v = denom > 0.0f ? acc / denom : 0.0f;
-    dst[d] = v;
-    if (hilo.base) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      hilo.base[base + d] = hi;
-      hilo.base[hilo.lo_offset + base + d] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
+    put(d, v);
   }
 }
 
 template <typename T>
-int attention_t(const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial, int M, int rows_per_seq,
+int attention_t(const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial, int M, RowSegs segs,
                 int n_heads, int splits, cudaStream_t stream, HiLoOut hilo) {
-  const int hd = kv.head_dim, W = rows_per_seq;
+  const int hd = kv.head_dim, W = segs.rows;
   if (W > NWARPS * MAXQ || hd > 32 * MAXD || M % W != 0) return SJD_ERR_UNSUPPORTED;
   const size_t smem = sizeof(float) * ((size_t)W * hd + TK * (hd + 1) + TK * hd + (size_t)W * TK);
   if (smem > 48 * 1024)
     SJD_CUDA(cudaFuncSetAttribute(attention_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid(n_heads, M / W, splits);
   attention_partial_kernel<T><<<grid, NWARPS * 32, smem, stream>>>(q, kv, in_pos, partial,
-                                                                  W, n_heads, splits);
+                                                                  segs, n_heads, splits);
   SJD_CHECK_LAUNCH();
   attention_combine_kernel<<<dim3(M, n_heads), 128, 0, stream>>>(partial, in_pos, out, n_heads, hd, splits, hilo);
   SJD_CHECK_LAUNCH();
@@ -270,11 +264,11 @@ int launch_attention_combine(const float *partial, const int32_t *in_pos, float 
 }
 
 int launch_attention(int dtype, const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial, int M,
-                     int rows_per_seq, int n_heads, int splits, cudaStream_t stream, HiLoOut hilo) {
+                     RowSegs segs, int n_heads, int splits, cudaStream_t stream, HiLoOut hilo) {
   if (dtype == SJD_F32)
-    return attention_t<float>(q, kv, in_pos, out, partial, M, rows_per_seq, n_heads, splits, stream, hilo);
+    return attention_t<float>(q, kv, in_pos, out, partial, M, segs, n_heads, splits, stream, hilo);
   if (dtype == SJD_BF16)
-    return attention_t<__nv_bfloat16>(q, kv, in_pos, out, partial, M, rows_per_seq, n_heads, splits, stream, hilo);
+    return attention_t<__nv_bfloat16>(q, kv, in_pos, out, partial, M, segs, n_heads, splits, stream, hilo);
   return SJD_ERR_UNSUPPORTED;
 }
 

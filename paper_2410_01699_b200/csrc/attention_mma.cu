@@ -86,10 +86,11 @@ struct AttnParams {
   const float *q;        // [M][H*HD]
   const int32_t *in_pos; // [M]
   float *partial;        // [M][H][splits][HD + 2]
-  float *out;            // [M][H*HD]: written here when splits == 1 (no merge launch needed)
+  float *out;            // [M][H*HD] or null: written here when splits == 1 (no merge launch needed)
   HiLoOut hilo;          // optional bf16 hi/lo planes of out (same case)
   int *status;
-  int rows_per_seq, n_heads, n_kv_heads, splits;
+  RowSegs segs;
+  int n_heads, n_kv_heads, splits;
   int plane0;            // first cache plane of this layer: planes are [b][k|v][kv_head]
   // paged cache: planes are [page][layer][k|v][kv_head], one page (KT positions) per tile
   const int32_t *page_table;   // [B][pages_per_seq]; null: contiguous
@@ -110,11 +111,12 @@ __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constan
   SJD_TL(TL_ATTN, 0, threadIdx.x == 0);
   pdl_wait();   // keys/values of this step were written by the preceding kernel
   SJD_TL(TL_ATTN, 1, threadIdx.x == 0);
-  const int h = blockIdx.x, b = blockIdx.y, split = blockIdx.z;
+  const int h = blockIdx.x, seg = blockIdx.y, split = blockIdx.z;
+  const int b = seg_sequence(p.segs, seg);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int W = p.rows_per_seq;
+  const int W = p.segs.rows;
   const int kvh = h / (p.n_heads / p.n_kv_heads);
-  const int m0 = b * W;
+  const int m0 = seg * W;
   const int g = lane >> 2, tq = lane & 3;
   const int n_rw = blockDim.x / (32 * KG);   // warps along the query rows
   const int rw = warp % n_rw, kg = warp / n_rw;   // this warp's 16 rows and its key group inside a tile
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constan
       for (int i = 0; i < HD / 8; ++i) {
         const float v0 = o[i][rr * 2] * inv, v1 = o[i][rr * 2 + 1] * inv;
         const size_t idx = base + i * 8 + tq * 2;
-        *reinterpret_cast<float2 *>(p.out + idx) = make_float2(v0, v1);
+        if (p.out) *reinterpret_cast<float2 *>(p.out + idx) = make_float2(v0, v1);
         if (p.hilo.base) {
           uint32_t hi, lo;
           split_pair(v0, v1, hi, lo);
@@ -415,8 +417,9 @@ bool attention_mma_supported(int head_dim, int rows_per_seq) { return (head_dim 
 // attention.cu; with a single key range it writes `out` (and `hilo`) itself and no merge is needed.
 int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const float *q, const int32_t *in_pos,
                          float *partial,
-                         float *out, HiLoOut hilo, int *status, int M, int rows_per_seq, int n_heads, int n_kv_heads,
+                         float *out, HiLoOut hilo, int *status, int M, RowSegs segs, int n_heads, int n_kv_heads,
                          int head_dim, int splits, cudaStream_t stream) {
+  const int rows_per_seq = segs.rows;
   if (!attention_mma_supported(head_dim, rows_per_seq) || M % rows_per_seq != 0) return SJD_ERR_UNSUPPORTED;
   AttnParams p;
   p.q = q;
@@ -425,7 +428,7 @@ int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const
   p.out = out;
   p.hilo = hilo;
   p.status = status;
-  p.rows_per_seq = rows_per_seq;
+  p.segs = segs;
   p.n_heads = n_heads;
   p.n_kv_heads = n_kv_heads;
   p.splits = splits;

@@ -309,7 +309,6 @@ struct RowScale {
 int resid_gain_parts(int d);
 int launch_resid_gain(int dtype, float *x, PlaneSet ps, const void *gain, HiLoOut h, float *ss_part, int M, int d,
                       cudaStream_t stream);
-int launch_swiglu_finish(PlaneSet ps, RowScale rs, HiLoOut act, int M, int F, cudaStream_t stream);
 
 // x[m][:] = tok_emb[tok[m]][:]  (fp32 residual stream)
 int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, int M, int d, int vocab,
@@ -317,8 +316,16 @@ int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, i
 // h[m][:] = x[m][:] * gain[:] / sqrt(mean(x[m]^2) + eps)  (gain of `dtype`)
 int launch_rmsnorm(int dtype, const float *x, const void *gain, float *h, int M, int d, float eps, cudaStream_t stream,
                    HiLoOut hilo = HiLoOut{nullptr, 0});
+// How the M rows of a pass map to sequences: segment m / rows holds consecutive positions of sequence
+// seq[m / rows] (null: of sequence m / rows).  A step has one segment per sequence (its window); a pre-fill pass
+// packs as many segments of the prompts as fit, several of one sequence among them.
+struct RowSegs {
+  int rows;
+  const int32_t *seq;
+};
+__device__ __forceinline__ int seg_sequence(const RowSegs &s, int seg) { return s.seq ? __ldg(s.seq + seg) : seg; }
 // Rotate q and k by their absolute position (pairs i, i + hd/2), store q as fp32 [M][H*hd],
-// append k and v to the cache row in_pos[m] of sequence m / rows_per_seq.  Rows with in_pos < 0 are skipped.
+// append k and v to the cache row in_pos[m] of the row's sequence.  Rows with in_pos < 0 are skipped.
 // Cache of one layer.  Contiguous: base is this layer's [B][2][KVh][max_seq][hd].  Paged (page_table != null): base is
 // the pool [page][layer][2][KVh][KV_PAGE][hd] shared by all layers, and logical page i of sequence b (positions
 // i * KV_PAGE .. i * KV_PAGE + KV_PAGE - 1) lives in physical page page_table[b * pages_per_seq + i].
@@ -344,17 +351,17 @@ struct QkNorm {
   float eps;
 };
 int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const float2 *rope_table, float *q,
-                       KvLayout kv, int M, int rows_per_seq, int n_heads, QkNorm qkn, cudaStream_t stream);
+                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
 int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
-                      KvLayout kv, int M, int rows_per_seq, int n_heads, QkNorm qkn, cudaStream_t stream);
+                      KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
 // act[m][f] = silu(gu[m][f]) * gu[m][F + f]
 int launch_swiglu(const float *gu, float *act, int M, int F, cudaStream_t stream, HiLoOut hilo = HiLoOut{nullptr, 0});
-// Window-causal attention: query row m (sequence m / rows_per_seq, position in_pos[m]) attends cache rows
+// Window-causal attention: query row m (position in_pos[m] of its segment's sequence) attends cache rows
 // 0 .. in_pos[m].  q, out: fp32 [M][H*hd]; cache of `dtype`.  partial: fp32 scratch [M][H][splits][hd + 2].
 int launch_attention(int dtype, const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial,
-                     int M, int rows_per_seq, int n_heads, int splits, cudaStream_t stream,
+                     int M, RowSegs segs, int n_heads, int splits, cudaStream_t stream,
                      HiLoOut hilo = HiLoOut{nullptr, 0});
-// merge of the split-KV partials only (used after launch_attention_mma)
+// merge of the split-KV partials only (used after launch_attention_mma); out may be null when only the hi/lo planes are wanted
 int launch_attention_combine(const float *partial, const int32_t *in_pos, float *out, int M, int n_heads, int head_dim,
                              int splits, cudaStream_t stream, HiLoOut hilo);
 // tensor-core split-KV attention for bf16 caches (attention_mma.cu)
@@ -363,7 +370,7 @@ bool attention_mma_supported(int head_dim, int rows_per_seq);
 // plane0: first plane of this layer in the contiguous map [planes][max_seq][hd]; with kv.page_table set the map is
 // the pool's [planes][KV_PAGE][hd] and the plane of a tile comes from the page table.
 int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const float *q, const int32_t *in_pos, float *partial,
-                         float *out, HiLoOut hilo, int *status, int M, int rows_per_seq, int n_heads, int n_kv_heads,
+                         float *out, HiLoOut hilo, int *status, int M, RowSegs segs, int n_heads, int n_kv_heads,
                          int head_dim, int splits, cudaStream_t stream);
 
 }  // namespace sjd

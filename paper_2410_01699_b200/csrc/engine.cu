@@ -29,14 +29,25 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 inline size_t esize(int dtype) { return dtype == SJD_F32 ? 4 : 2; }
 
 constexpr int kMaxGemmCtas = 160;    // upper bound on the SM count used to size split-K scratch
+// gate|up launch with SwiGLU in the epilogue: 64 gate rows and the same 64 up rows per CTA, one K split.
+// (Measured on the 7B shapes: 40 rows per CTA, which fills one wave of two CTAs per SM exactly, is no faster
+// than 64: every CTA reads the whole activation operand, so smaller tiles raise that traffic.)
+constexpr int kGuRows = 64;
+// Rows of one pre-fill pass: enough that a pass is bound by the tensor pipe and not by streaming the weights
+// once more (13.5 GB of weights take 2.1 ms, 1152 rows of the 7B layers about 30 ms), few enough that the
+// activations of a pass (157 KB per row at the 7B shapes) stay below 200 MB.  (Passes of max_window rows streamed the
+// weights once per 32 prompt tokens: 1063 tokens and one step took 124.2 ms on the 7B shapes, 37.3 ms this way.)  The generic pipeline keeps four
+// more fp32 buffers per row and is not bound by the weights: 256 rows.
+constexpr int kPrefillRowsTc = 1152, kPrefillRowsGeneric = 256;
+constexpr int kMaxTcRows = 1152;     // largest pass of the tensor-core pipeline
 
 struct WMap {
   TensorMap map;
   bool valid = false;
 };
 struct LayerMaps {
-  WMap wq, wk, wv, wo, w_gate, w_up, w_down;
-  WMap gate_gu, up_gu;   // gate and up matrices in boxes of gu_rows rows: the gate|up launch that applies SwiGLU itself
+  WMap wq, wk, wv, wo, w_down;
+  WMap gate_gu, up_gu;   // gate and up matrices in boxes of kGuRows rows: the gate|up launch applies SwiGLU itself
 };
 struct XMaps {
   TensorMap h, attn, act;
@@ -50,6 +61,8 @@ struct Layout {
   size_t ring, ring_stats, n_prev, w_prev;   // Sec. 4.2 (d): retained logits rows (max_ring > 0)
   size_t prompt_lens;                        // [max_batch] prompt length of every sequence
   size_t page_table;                         // [max_batch][pages_per_seq] (paged cache, kv_pages > 0)
+  size_t seg_seq, seg_start;                 // [prefill_segments] pre-fill: sequence and first position of every segment
+  size_t pass_rows;                          // rows of the largest pass (a step or a pre-fill chunk)
   size_t total;
 };
 
@@ -64,10 +77,29 @@ bool cfg_valid(const sjd_model_cfg *c) {
   return true;
 }
 
+// the tensor-core pipeline covers every projection of this model (the device allowing)
+bool tc_shapes(const sjd_model_cfg &c) {
+  const long nq = (long)c.n_heads * c.head_dim, nk = (long)c.n_kv_heads * c.head_dim;
+  return c.dtype == SJD_BF16 && c.d_model % 128 == 0 && nq % 128 == 0 && nk % 128 == 0 && c.ffn_hidden % 128 == 0 &&
+         c.vocab % 128 == 0;
+}
+// rows of the largest pre-fill pass: no more than the longest prompts of a full batch could fill
+size_t prefill_rows(const sjd_model_cfg &c, bool tc) {
+  const size_t cap = tc ? kPrefillRowsTc : kPrefillRowsGeneric;
+  const size_t all = (size_t)c.max_batch * ((c.max_seq + 63) / 64 * 64);
+  return all < cap ? all : cap;
+}
+// segments (of at least 16 positions) the prompts of a full batch can make
+size_t prefill_segments(const sjd_model_cfg &c) { return (size_t)c.max_batch * ((c.max_seq + 15) / 16); }
+
 Layout make_layout(const sjd_model_cfg &c) {
   Layout L;
   const size_t es = esize(c.dtype);
-  const size_t Mx = (size_t)c.max_batch * c.max_window;
+  const bool tc = tc_shapes(c);
+  const size_t Mx = (size_t)c.max_batch * c.max_window;   // rows of a step
+  const size_t Rg = prefill_rows(c, false), Mg = Mx > Rg ? Mx : Rg;          // of the largest pass, generic pipeline
+  const size_t Rp = prefill_rows(c, tc), Mp = Mx > Rp ? Mx : Rp;             // and of either pipeline
+  L.pass_rows = Mp;
   const size_t nq = (size_t)c.n_heads * c.head_dim, nk = (size_t)c.n_kv_heads * c.head_dim;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -87,33 +119,44 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.counters = take(((size_t)c.max_batch + 1) * 4);
   L.step = take(4);
   L.status = take(4);
-  L.x = take(Mx * c.d_model * 4);
-  L.h = take(Mx * c.d_model * 4);
-  L.qkv = take(Mx * (nq + 2 * nk) * 4);
-  L.q = take(Mx * nq * 4);
-  L.attn = take(Mx * nq * 4);
-  L.gu = take(Mx * 2 * c.ffn_hidden * 4);
-  L.act = take(Mx * c.ffn_hidden * 4);
+  L.x = take(Mp * c.d_model * 4);
+  L.q = take(Mp * nq * 4);
+  {   // a context runs one of the two pipelines: the generic one's buffers share their memory with the other's planes
+    const size_t generic = align256(Mg * c.d_model * 4) + align256(Mg * (nq + 2 * nk) * 4) + align256(Mg * nq * 4) +
+                           align256(Mg * 2 * c.ffn_hidden * 4) + align256(Mg * c.ffn_hidden * 4);
+    const size_t Ma = (Mp + 15) / 16 * 16;
+    const size_t planes = tc ? align256(2 * Ma * c.d_model * 2) + align256(2 * Ma * nq * 2) + align256(2 * Ma * c.ffn_hidden * 2) : 0;
+    const size_t base = off;
+    L.h = take(Mg * c.d_model * 4);
+    L.qkv = take(Mg * (nq + 2 * nk) * 4);
+    L.attn = take(Mg * nq * 4);
+    L.gu = take(Mg * 2 * c.ffn_hidden * 4);
+    L.act = take(Mg * c.ffn_hidden * 4);
+    off = base;   // bf16 hi/lo planes of the GEMM inputs
+    L.xs_h = take(tc ? 2 * Ma * c.d_model * 2 : 0);
+    L.xs_attn = take(tc ? 2 * Ma * nq * 2 : 0);
+    L.xs_act = take(tc ? 2 * Ma * c.ffn_hidden * 2 : 0);
+    off = base + (generic > planes ? generic : planes);
+  }
   size_t part = 0;
-  for (int b = 1; b <= c.max_batch; ++b) {
-    const size_t need = (size_t)b * c.max_window * c.n_heads * attention_splits(c.n_heads, b) * (c.head_dim + 2);
+  for (size_t b = 1; b * 16 <= Mp + 64 || b <= (size_t)c.max_batch; ++b) {   // b segments of a step or of a pre-fill pass
+    const int splits = attention_splits(c.n_heads, (int)b);
+    // with one key range the tensor-core attention writes its output itself: only the generic kernel needs records then
+    const bool direct = splits == 1 && tc && attention_mma_supported(c.head_dim, 64);
+    const size_t cap = direct ? Mg : Mp, rows = b * 64 < cap ? b * 64 : cap;
+    const size_t need = rows * c.n_heads * splits * (c.head_dim + 2);
     part = need > part ? need : part;
   }
   L.partial = take(part * 4);
-  // bf16 hi/lo planes of the GEMM inputs, stream-K partials and tickets (tensor-core path)
-  const size_t Ma = (Mx + 15) / 16 * 16;
-  L.xs_h = take(2 * Ma * c.d_model * 2);
-  L.xs_attn = take(2 * Ma * nq * 2);
-  L.xs_act = take(2 * Ma * c.ffn_hidden * 2);
   {
     // fp32 partial planes of one GEMM launch: the largest splits * rows * columns over the launches
-    const int tiles[4] = {(int)((nq + 2 * nk) / 128), c.d_model / 128, 2 * c.ffn_hidden / 128, c.d_model / 128};
-    const int kbs[4] = {c.d_model / 64, (int)(nq / 64), c.d_model / 64, c.ffn_hidden / 64};
-    const size_t cols[4] = {nq + 2 * nk, (size_t)c.d_model, (size_t)2 * c.ffn_hidden, (size_t)c.d_model};
+    const int tiles[3] = {(int)((nq + 2 * nk) / 128), c.d_model / 128, c.d_model / 128};
+    const int kbs[3] = {c.d_model / 64, (int)(nq / 64), c.ffn_hidden / 64};
+    const size_t cols[3] = {nq + 2 * nk, (size_t)c.d_model, (size_t)c.d_model};
     size_t need = 0;
-    for (int i = 0; i < 4; ++i) {
-      for (size_t rows = 16; rows < Mx + 16 && rows <= 1024; rows += 16) {   // splits shrink as the token slabs grow
-        const size_t m = rows < Mx ? rows : Mx;
+    for (int i = 0; i < 3 && tc; ++i) {
+      for (size_t rows = 16; rows < Mp + 16 && rows <= kMaxTcRows; rows += 16) {   // splits shrink as the token slabs grow
+        const size_t m = rows < Mp ? rows : Mp;
         const size_t n = (size_t)gemm_tc_splits(gemm_tc_plan((int)m), tiles[i] > 0 ? tiles[i] : 1, kbs[i],
                                                  kMaxGemmCtas) * m * cols[i];
         need = n > need ? n : need;
@@ -121,7 +164,7 @@ Layout make_layout(const sjd_model_cfg &c) {
     }
     L.gemm_planes = take(need * 4);
   }
-  L.ss_part = take(Mx * (size_t)resid_gain_parts(c.d_model) * 4);
+  L.ss_part = take(Mp * (size_t)resid_gain_parts(c.d_model) * 4);
   L.rope = take((size_t)c.max_seq * (c.head_dim / 2) * sizeof(float2));
   L.committed = take((size_t)c.max_batch * c.max_seq * 4);
   L.n = take((size_t)c.max_batch * 4);
@@ -130,8 +173,8 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.q_kind = take(Mx * 4);
   L.q_row = take(Mx * 4);
   L.q_draft = take(Mx * 4);
-  L.in_tok = take(Mx * 4);
-  L.in_pos = take(Mx * 4);
+  L.in_tok = take(Mp * 4);
+  L.in_pos = take(Mp * 4);
   const size_t ring_rows = (size_t)c.max_batch * (c.max_ring > 0 ? c.max_ring : 0);
   L.ring = take(ring_rows * c.vocab * es);
   L.ring_stats = take(ring_rows * sizeof(RowStats));
@@ -139,6 +182,8 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.w_prev = take((size_t)c.max_batch * 4);
   L.prompt_lens = take((size_t)c.max_batch * 4);
   L.page_table = take(c.kv_pages > 0 ? (size_t)c.max_batch * ((c.max_seq + KV_PAGE - 1) / KV_PAGE) * 4 : 0);
+  L.seg_seq = take(prefill_segments(c) * 4);
+  L.seg_start = take(prefill_segments(c) * 4);
   L.total = off;
   return L;
 }
@@ -207,15 +252,16 @@ __global__ void prefill_setup_kernel(const int32_t *prompt, int ld, SeqState st,
   }
 }
 
-__global__ void prefill_inputs_kernel(const int32_t *prompt, int ld, const int32_t *prompt_lens, int c0, int rows,
-                                      int32_t *in_tok, int32_t *in_pos) {
-  const int b = blockIdx.x;
+// one block per segment of a pre-fill pass: its tokens and positions (the last prompt token is not among them)
+__global__ void prefill_inputs_kernel(const int32_t *prompt, int ld, const int32_t *prompt_lens, const int32_t *seg_seq,
+                                      const int32_t *seg_start, int rows, int32_t *in_tok, int32_t *in_pos) {
+  const int seg = blockIdx.x, b = seg_seq[seg];
   const int P = prompt_lens[b];
   for (int k = threadIdx.x; k < rows; k += blockDim.x) {
-    const int pos = c0 + k;
+    const int pos = seg_start[seg] + k;
     const bool act = pos < P - 1;
-    in_tok[b * rows + k] = act ? prompt[(size_t)b * ld + pos] : 0;
-    in_pos[b * rows + k] = act ? pos : -1;
+    in_tok[seg * rows + k] = act ? prompt[(size_t)b * ld + pos] : 0;
+    in_pos[seg * rows + k] = act ? pos : -1;
   }
 }
 
@@ -257,6 +303,7 @@ struct sjd_ctx {
   int batch, prompt_len, window;   // prompt_len: the longest prompt of the batch
   std::vector<int32_t> prompt_lens;  // per sequence (host copy; the device copy is in the workspace)
   std::vector<int32_t> page_table;   // paged cache: host copy of [max_batch][pages_per_seq]
+  std::vector<int32_t> seg_seq, seg_start;   // pre-fill: host copies of the segment tables
   bool prefilled;
   uint32_t host_step;  // number of sjd_step calls since prefill == device step index
   cudaStream_t last_stream;
@@ -283,17 +330,13 @@ struct sjd_ctx {
   Tracer tracer;
   bool use_tc = false;   // bf16 model on a device with tensor memory: tensor-core GEMM path
   bool all_tc = false;   // every projection of the model is covered by it
-  bool gu_fused = false; // gate|up projection with SwiGLU in its epilogue (every layer has the maps for it)
-  int gu_rows = 0;       // feature rows of the gate (and of the up) matrix per CTA of that launch
-  int head_rows = 0;     // weight rows per CTA of the logits projection (0: 128)
-  WMap wmap_head_r;      // lm_head in boxes of head_rows rows
   int n_ctas = 0;
   std::vector<LayerMaps> wmaps;
   WMap wmap_head;
   std::map<int, XMaps> xmaps;   // keyed by padded row count
   TensorMap kv_map;             // whole KV cache as [planes][max_seq][head_dim]
   bool kv_map_valid = false;
-  int rows_alloc() const { return ((cfg.max_batch * cfg.max_window) + 15) / 16 * 16; }
+  int rows_alloc() const { return ((int)lay.pass_rows + 15) / 16 * 16; }
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
   SeqState state() const {
@@ -339,16 +382,17 @@ struct sjd_ctx {
 namespace sjd {
 namespace {
 
-// One forward pass of M = batch * rows_per_seq rows whose tokens / positions are in st.in_tok / in_pos.
+// One forward pass over n_segs segments of segs.rows rows, whose tokens / positions are in st.in_tok / in_pos.
+// Without logits_out (pre-fill) the pass ends with the last layer's keys and values: nothing reads what follows.
 // Two pipelines: the tensor-core one (bf16 model, every projection covered by the weight-streaming
 // GEMM: partial planes + fused consumer kernels) and the generic one (any dtype and shape).
 #define SJD_TRY(call) do { rc = (call); if (rc != SJD_OK) return rc; } while (0)
 #define SJD_TR(klass, call) do { tr.begin(klass, stream); rc = (call); tr.end(stream); if (rc != SJD_OK) return rc; } while (0)
 
-int forward_generic(sjd_ctx *c, int rows_per_seq, void *logits_out, cudaStream_t stream) {
+int forward_generic(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const sjd_model_cfg &g = c->cfg;
   const int dt = g.dtype;
-  const int M = c->batch * rows_per_seq;
+  const int M = n_segs * segs.rows;
   const int d = g.d_model, F = g.ffn_hidden;
   const int nq = g.n_heads * g.head_dim, nk = g.n_kv_heads * g.head_dim, nqkv = nq + 2 * nk;
   const SeqState st = c->state();
@@ -361,7 +405,7 @@ int forward_generic(sjd_ctx *c, int rows_per_seq, void *logits_out, cudaStream_t
   float *act = c->at<float>(c->lay.act);
   float *partial = c->at<float>(c->lay.partial);
   const float2 *rope = c->at<float2>(c->lay.rope);
-  const int splits = attention_splits(g.n_heads, c->batch);
+  const int splits = attention_splits(g.n_heads, n_segs);
   int rc;
   Tracer &tr = c->tracer;
   const double es = (double)esize(dt);
@@ -379,8 +423,9 @@ int forward_generic(sjd_ctx *c, int rows_per_seq, void *logits_out, cudaStream_t
     SJD_TRY(gemm(c->wk[l], h, d, qkv + nq, nqkv, nk, d, EPI_STORE_F32));
     SJD_TRY(gemm(c->wv[l], h, d, qkv + nq + nk, nqkv, nk, d, EPI_STORE_F32));
     const KvLayout kv = c->kv_layer(l);
-    SJD_TR(TC_OTHER, launch_rope_append(dt, qkv, st.in_pos, rope, q, kv, M, rows_per_seq, g.n_heads, c->qk_norm(l), stream));
-    SJD_TR(TC_ATTENTION, launch_attention(dt, q, kv, st.in_pos, attn, partial, M, rows_per_seq, g.n_heads, splits, stream));
+    SJD_TR(TC_OTHER, launch_rope_append(dt, qkv, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
+    if (!logits_out && l == g.n_layers - 1) break;
+    SJD_TR(TC_ATTENTION, launch_attention(dt, q, kv, st.in_pos, attn, partial, M, segs, g.n_heads, splits, stream));
     SJD_TRY(gemm(c->wo[l], attn, nq, x, d, d, nq, EPI_ADD_F32));
     SJD_TR(TC_OTHER, launch_rmsnorm(dt, x, c->ffn_norm[l], h, M, d, g.rms_eps, stream));
     SJD_TRY(gemm(c->w_gate[l], h, d, gu, 2 * F, F, d, EPI_STORE_F32));
@@ -395,21 +440,20 @@ int forward_generic(sjd_ctx *c, int rows_per_seq, void *logits_out, cudaStream_t
   return SJD_OK;
 }
 
-int forward_tc(sjd_ctx *c, const XMaps &xm, int rows_per_seq, void *logits_out, cudaStream_t stream) {
+int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const sjd_model_cfg &g = c->cfg;
   const int dt = g.dtype;
-  const int M = c->batch * rows_per_seq;
+  const int M = n_segs * segs.rows;
   const int d = g.d_model, F = g.ffn_hidden;
   const int nq = g.n_heads * g.head_dim, nk = g.n_kv_heads * g.head_dim, nqkv = nq + 2 * nk;
   const SeqState st = c->state();
   float *x = c->at<float>(c->lay.x);
   float *q = c->at<float>(c->lay.q);
-  float *attn = c->at<float>(c->lay.attn);
   float *partial = c->at<float>(c->lay.partial);
   float *planes = c->at<float>(c->lay.gemm_planes);
   int *status = c->at<int>(c->lay.status);
   const float2 *rope = c->at<float2>(c->lay.rope);
-  const int att_splits = attention_splits(g.n_heads, c->batch);
+  const int att_splits = attention_splits(g.n_heads, n_segs);
   const int Ma = c->rows_alloc();
   const HiLoOut hl_h{c->at<__nv_bfloat16>(c->lay.xs_h), (size_t)Ma * d};
   const HiLoOut hl_attn{c->at<__nv_bfloat16>(c->lay.xs_attn), (size_t)Ma * nq};
@@ -476,17 +520,18 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int rows_per_seq, void *logits_out, 
       SJD_TRY(gemm(wm, 3, n_out, xm.h, d, nqkv, planes, false, &ps));
     }
     const KvLayout kv = c->kv_layer(l);
-    SJD_TR(TC_OTHER, launch_qkv_finish(dt, ps, rs, st.in_pos, rope, q, kv, M, rows_per_seq, g.n_heads, c->qk_norm(l), stream));
-    if (c->kv_map_valid && attention_mma_supported(g.head_dim, rows_per_seq)) {
-      SJD_TR(TC_ATTENTION, launch_attention_mma(c->kv_map, l * g.max_batch * 2 * g.n_kv_heads, kv, q, st.in_pos, partial, attn,
-                                                hl_attn, status, M, rows_per_seq, g.n_heads, g.n_kv_heads, g.head_dim,
+    SJD_TR(TC_OTHER, launch_qkv_finish(dt, ps, rs, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
+    if (!logits_out && l == g.n_layers - 1) break;
+    if (c->kv_map_valid && attention_mma_supported(g.head_dim, segs.rows)) {
+      SJD_TR(TC_ATTENTION, launch_attention_mma(c->kv_map, l * g.max_batch * 2 * g.n_kv_heads, kv, q, st.in_pos, partial, nullptr,
+                                                hl_attn, status, M, segs, g.n_heads, g.n_kv_heads, g.head_dim,
                                                 att_splits, stream));
       if (att_splits > 1)
         SJD_TR(TC_ATTENTION,
-               launch_attention_combine(partial, st.in_pos, attn, M, g.n_heads, g.head_dim, att_splits, stream, hl_attn));
+               launch_attention_combine(partial, st.in_pos, nullptr, M, g.n_heads, g.head_dim, att_splits, stream, hl_attn));
     } else {
       SJD_TR(TC_ATTENTION,
-             launch_attention(dt, q, kv, st.in_pos, attn, partial, M, rows_per_seq, g.n_heads, att_splits, stream, hl_attn));
+             launch_attention(dt, q, kv, st.in_pos, nullptr, partial, M, segs, g.n_heads, att_splits, stream, hl_attn));
     }
     {
       const WMap *wm[1] = {&lm.wo};
@@ -494,15 +539,10 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int rows_per_seq, void *logits_out, 
       SJD_TRY(gemm(wm, 1, n_out, xm.attn, nq, d, planes, false, &ps));
     }
     SJD_TR(TC_OTHER, launch_resid_gain(dt, x, ps, c->ffn_norm[l], hl_h, ss_part, M, d, stream));
-    if (c->gu_fused) {
+    {
       const WMap *wm[2] = {&lm.gate_gu, &lm.up_gu};
       const int n_out[2] = {F, F};
-      SJD_TRY(gemm(wm, 2, n_out, xm.h, d, F, nullptr, false, nullptr, c->gu_rows, &hl_act));
-    } else {
-      const WMap *wm[2] = {&lm.w_gate, &lm.w_up};
-      const int n_out[2] = {F, F};
-      SJD_TRY(gemm(wm, 2, n_out, xm.h, d, 2 * F, planes, false, &ps));
-      SJD_TR(TC_OTHER, launch_swiglu_finish(ps, rs, hl_act, M, F, stream));
+      SJD_TRY(gemm(wm, 2, n_out, xm.h, d, F, nullptr, false, nullptr, kGuRows, &hl_act));
     }
     {
       const WMap *wm[1] = {&lm.w_down};
@@ -512,29 +552,28 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int rows_per_seq, void *logits_out, 
   }
   if (logits_out) {
     SJD_TR(TC_OTHER, launch_resid_gain(dt, x, pending, c->final_norm, hl_h, ss_part, M, d, stream));
-    const int head_rows = M <= 128 ? c->head_rows : 0;   // several token slabs share 128-row tiles through L2
-    const WMap *wm[1] = {head_rows ? &c->wmap_head_r : &c->wmap_head};
+    const WMap *wm[1] = {&c->wmap_head};
     const int n_out[1] = {g.vocab};
-    SJD_TRY(gemm(wm, 1, n_out, xm.h, d, g.vocab, logits_out, true, nullptr, head_rows));
+    SJD_TRY(gemm(wm, 1, n_out, xm.h, d, g.vocab, logits_out, true, nullptr));
   }
   return SJD_OK;
 }
 #undef SJD_TR
 #undef SJD_TRY
 
-int forward(sjd_ctx *c, int rows_per_seq, void *logits_out, cudaStream_t stream) {
-  const int M = c->batch * rows_per_seq;
-  if (c->use_tc && c->all_tc && M <= 1024) {
+int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
+  const int M = n_segs * segs.rows;
+  if (c->use_tc && c->all_tc && M <= kMaxTcRows) {
     auto it = c->xmaps.find((M + 15) / 16 * 16);
     if (it != c->xmaps.end()) {
       // every kernel of this pipeline waits for its predecessor itself: launch them overlapped
       g_pdl = !c->tracer.on;
-      const int rc = forward_tc(c, it->second, rows_per_seq, logits_out, stream);
+      const int rc = forward_tc(c, it->second, n_segs, segs, logits_out, stream);
       g_pdl = false;
       return rc;
     }
   }
-  return forward_generic(c, rows_per_seq, logits_out, stream);
+  return forward_generic(c, n_segs, segs, logits_out, stream);
 }
 
 int run_verify(sjd_ctx *c, const sjd_step_out *out, cudaStream_t stream) {
@@ -679,37 +718,12 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
       mk(lm.wk, c->wk[l], nk, d);
       mk(lm.wv, c->wv[l], nk, d);
       mk(lm.wo, c->wo[l], d, nq);
-      mk(lm.w_gate, c->w_gate[l], F, d);
-      mk(lm.w_up, c->w_up[l], F, d);
+      lm.gate_gu.valid = F % 128 == 0 && d % 64 == 0 && make_tensor_map_bf16(&lm.gate_gu.map, c->w_gate[l], F, d, kGuRows) == SJD_OK;
+      lm.up_gu.valid = F % 128 == 0 && d % 64 == 0 && make_tensor_map_bf16(&lm.up_gu.map, c->w_up[l], F, d, kGuRows) == SJD_OK;
       mk(lm.w_down, c->w_down[l], d, F);
     }
     mk(c->wmap_head, c->lm_head, cfg->vocab, d);
     c->all_tc = c->wmap_head.valid;
-    // gate|up with SwiGLU in the epilogue: 64 gate rows and the same 64 up rows per CTA, one K split.
-    // (Measured on the 7B shapes: 40 rows per CTA, which fills one wave of two CTAs per SM exactly, is no
-    // faster than 64: every CTA reads the whole activation operand, so smaller tiles raise that traffic.)
-    {
-      int r = 64;
-      if (const char *e = getenv("SJD_GU_ROWS")) r = atoi(e);   // tuning: 0 switches the fused launch off, else 8..64
-      c->gu_rows = r;
-      c->gu_fused = r >= 8 && r <= 64 && d % 64 == 0;
-      for (int l = 0; l < L && c->gu_fused; ++l) {
-        LayerMaps &lm = c->wmaps[l];
-        lm.gate_gu.valid = make_tensor_map_bf16(&lm.gate_gu.map, c->w_gate[l], F, d, r) == SJD_OK;
-        lm.up_gu.valid = make_tensor_map_bf16(&lm.up_gu.map, c->w_up[l], F, d, r) == SJD_OK;
-        c->gu_fused = lm.gate_gu.valid && lm.up_gu.valid;
-      }
-    }
-    // logits projection: optional tile height below 128 rows (SJD_HEAD_ROWS; measured on the 7B shapes: 112
-    // rows = two full waves of CTAs is 4 % slower than 128 rows in 1.7 waves, so the default stays 128)
-    if (const char *e = getenv("SJD_HEAD_ROWS")) {
-      const int r = atoi(e);
-      if (r >= 8 && r < 128 && c->wmap_head.valid &&
-          make_tensor_map_bf16(&c->wmap_head_r.map, c->lm_head, cfg->vocab, d, r) == SJD_OK) {
-        c->wmap_head_r.valid = true;
-        c->head_rows = r;
-      }
-    }
     // the cache as one 3-D tensor map for the tensor-core attention; unwritten rows must read as finite
     // numbers (a masked probability of 0 times NaN would poison the output), so the cache starts at zero
     // (paged cache: the planes are the pool's [page][layer][k|v][kv_head], each KV_PAGE rows long)
@@ -723,13 +737,29 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
       c->kv_map_valid = true;
     for (int l = 0; l < L; ++l) {
       const LayerMaps &lm = c->wmaps[l];
-      c->all_tc = c->all_tc && lm.wq.valid && lm.wk.valid && lm.wv.valid && lm.wo.valid && lm.w_gate.valid &&
-                  lm.w_up.valid && lm.w_down.valid;
+      c->all_tc = c->all_tc && lm.wq.valid && lm.wk.valid && lm.wv.valid && lm.wo.valid && lm.gate_gu.valid &&
+                  lm.up_gu.valid && lm.w_down.valid;
     }
   }
   *out = c;
   return SJD_OK;
 }
+
+namespace {
+// activation descriptors for passes of `rows` rows (once per padded row count and context)
+void add_x_maps(sjd_ctx *c, int rows) {
+  const int Mp = (rows + 15) / 16 * 16;
+  if (rows > kMaxTcRows || c->xmaps.count(Mp)) return;
+  const int Ma = c->rows_alloc();
+  const int nq = c->cfg.n_heads * c->cfg.head_dim;
+  XMaps xm;
+  const int box = gemm_tc_plan(rows).slab_rows;
+  const bool ok = make_tensor_map_bf16(&xm.h, c->ws + c->lay.xs_h, 2L * Ma, c->cfg.d_model, box) == SJD_OK &&
+                  make_tensor_map_bf16(&xm.attn, c->ws + c->lay.xs_attn, 2L * Ma, nq, box) == SJD_OK &&
+                  make_tensor_map_bf16(&xm.act, c->ws + c->lay.xs_act, 2L * Ma, c->cfg.ffn_hidden, box) == SJD_OK;
+  if (ok) c->xmaps[Mp] = xm;
+}
+}  // namespace
 
 extern "C" int sjd_prefill(sjd_ctx *c, int batch, const int32_t *prompt, int prompt_len, const sjd_sample_cfg *sample,
                            void *cuda_stream) {
@@ -785,33 +815,49 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   c->last_stream = stream;
   c->prefilled = false;
   c->drop_graphs();
-  if (c->use_tc) {
-    // activation descriptors for the two row counts used: the step's window and the pre-fill chunk
-    const int Ma = c->rows_alloc();
-    const int nq = c->cfg.n_heads * c->cfg.head_dim;
-    const int row_counts[2] = {batch * sample->window, batch * c->cfg.max_window};
-    for (int i = 0; i < 2; ++i) {
-      const int Mp = (row_counts[i] + 15) / 16 * 16;
-      if (row_counts[i] > 1024 || c->xmaps.count(Mp)) continue;
-      XMaps xm;
-      const int box = gemm_tc_plan(row_counts[i]).slab_rows;
-      const bool ok = make_tensor_map_bf16(&xm.h, c->ws + c->lay.xs_h, 2L * Ma, c->cfg.d_model, box) == SJD_OK &&
-                      make_tensor_map_bf16(&xm.attn, c->ws + c->lay.xs_attn, 2L * Ma, nq, box) == SJD_OK &&
-                      make_tensor_map_bf16(&xm.act, c->ws + c->lay.xs_act, 2L * Ma, c->cfg.ffn_hidden, box) == SJD_OK;
-      if (ok) c->xmaps[Mp] = xm;
-    }
-  }
+  const bool tc = c->use_tc && c->all_tc;
+  if (tc) add_x_maps(c, batch * sample->window);
   const SeqState st = c->state();
   prefill_setup_kernel<<<batch, 128, 0, stream>>>(prompt, row_stride, st, c->at<uint32_t>(c->lay.step),
                                                   c->at<int32_t>(c->lay.counters), batch);
   SJD_CHECK_LAUNCH();
-  // cache keys/values of c[0..P-1) in chunks of max_window rows per sequence
-  const int rows = c->cfg.max_window;
-  for (int c0 = 0; c0 < prompt_len - 1; c0 += rows) {
-    prefill_inputs_kernel<<<batch, 64, 0, stream>>>(prompt, row_stride, st.prompt_lens, c0, rows, st.in_tok, st.in_pos);
-    SJD_CHECK_LAUNCH();
-    rc = forward(c, rows, nullptr, stream);
-    if (rc != SJD_OK) return rc;
+  // Cache keys/values of c[0..P-1): the prompts are cut into segments of `rows` positions, which are packed into as
+  // few passes as the activation buffers allow.  Short segments waste fewer padding rows, long ones re-read fewer
+  // cached keys per row: the padded rows decide, with a small charge per segment.
+  int rows = 64;
+  double best = 0.0;
+  for (int r = 64; r >= 16; r /= 2) {
+    long padded = 0;
+    for (int b = 0; b < batch; ++b) padded += (prompt_lens[b] - 1 + r - 1) / r * r;
+    const double cost = (double)padded * (1.0 + 4.0 / r);
+    if (r == 64 || cost < best) {
+      best = cost;
+      rows = r;
+    }
+  }
+  c->seg_seq.clear();
+  c->seg_start.clear();
+  for (int b = 0; b < batch; ++b)
+    for (int p0 = 0; p0 < prompt_lens[b] - 1; p0 += rows) {
+      c->seg_seq.push_back(b);
+      c->seg_start.push_back(p0);
+    }
+  const int n_segs = (int)c->seg_seq.size();
+  if (n_segs > 0) {
+    int32_t *seg_seq = c->at<int32_t>(c->lay.seg_seq), *seg_start = c->at<int32_t>(c->lay.seg_start);
+    SJD_CUDA(cudaMemcpyAsync(seg_seq, c->seg_seq.data(), (size_t)n_segs * 4, cudaMemcpyHostToDevice, stream));
+    SJD_CUDA(cudaMemcpyAsync(seg_start, c->seg_start.data(), (size_t)n_segs * 4, cudaMemcpyHostToDevice, stream));
+    const int cap = (int)prefill_rows(c->cfg, tc) / rows;   // segments of one pass
+    const int passes = (n_segs + cap - 1) / cap;
+    for (int i = 0; i < passes; ++i) {
+      const int s0 = (int)((long)n_segs * i / passes), n = (int)((long)n_segs * (i + 1) / passes) - s0;
+      if (tc) add_x_maps(c, n * rows);
+      prefill_inputs_kernel<<<n, 64, 0, stream>>>(prompt, row_stride, st.prompt_lens, seg_seq + s0, seg_start + s0, rows,
+                                                  st.in_tok, st.in_pos);
+      SJD_CHECK_LAUNCH();
+      rc = forward(c, n, RowSegs{rows, seg_seq + s0}, nullptr, stream);
+      if (rc != SJD_OK) return rc;
+    }
   }
   // first window: no rows to verify (w_eff = 0), the slide initialises every slot (Sec. 4.2) with the
   // initial-window step tag and bumps the step index to 0
@@ -824,7 +870,7 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
 namespace {
 // forward pass + verification of one step, enqueued on `stream`
 int enqueue_step(sjd_ctx *c, const sjd_step_out *out, int cur, cudaStream_t stream) {
-  int rc = forward(c, c->window, c->ws + c->lay.logits[cur], stream);
+  int rc = forward(c, c->batch, RowSegs{c->window, nullptr}, c->ws + c->lay.logits[cur], stream);
   if (rc != SJD_OK) return rc;
   c->tracer.begin(TC_VERIFY, stream);
   g_pdl = !c->tracer.on;
@@ -928,7 +974,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   if (!c || !info) return SJD_ERR_BAD_ARG;
   if (!c->prefilled) return SJD_ERR_STATE;
   const int M = c->batch * c->window;
-  const bool tc = c->use_tc && c->all_tc && M <= 1024 && c->xmaps.count((M + 15) / 16 * 16) != 0;
+  const bool tc = c->use_tc && c->all_tc && M <= kMaxTcRows && c->xmaps.count((M + 15) / 16 * 16) != 0;
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
       (tc && c->kv_map_valid && attention_mma_supported(c->cfg.head_dim, c->window)) ? 1 : 0;

@@ -30,14 +30,8 @@ __device__ __forceinline__ float sum_planes(const PlaneSet &ps, size_t idx) {
 // Per-row RMS scale from the partial sums of squares a resid_gain launch left:
 // scale(m) = 1 / sqrt(mean(x[m]^2) + eps).  The scale is a per-row scalar, so it commutes with the
 // projection that follows the normalisation and is applied by that projection's consumer.
-__device__ __forceinline__ float row_scale(const RowScale &rs, int m) {
-  if (!rs.ss_part) return 1.0f;
-  float tot = 0.0f;
-  for (int j = 0; j < rs.n_part; ++j) tot += __ldg(rs.ss_part + (size_t)m * rs.n_part + j);
-  return rsqrtf(tot * rs.inv_d + rs.eps);
-}
-// the same for a row index that is uniform over the (full) warp: lanes share the loads.  The partials
-// are added in a fixed tree order, so every caller gets the same bits.
+// The row index is uniform over the (full) warp: lanes share the loads.  The partials are added in a fixed
+// tree order, so every caller gets the same bits.
 __device__ __forceinline__ float row_scale_warp(const RowScale &rs, int m) {
   if (!rs.ss_part) return 1.0f;
   const int lane = threadIdx.x & 31;
@@ -88,7 +82,7 @@ __global__ void __launch_bounds__(RG_THREADS) resid_gain_kernel(float *__restric
 // slots per block.
 template <typename T>
 __global__ void qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__restrict__ in_pos,
-                                  const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, int rows_per_seq,
+                                  const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, RowSegs segs,
                                   int n_heads, QkNorm qkn) {
   __shared__ float s_ss[8];   // QK-norm: per-warp sums of squares of a head (two warps per 64-thread group)
   pdl_trigger();
@@ -96,7 +90,7 @@ __global__ void qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__res
   pdl_wait();
   SJD_TL(TL_QKV, 1, threadIdx.x == 0);
   const int m = blockIdx.x, lt = threadIdx.x & 63;
-  const int b = m / rows_per_seq;
+  const int b = seg_sequence(segs, m / segs.rows);
   const int hd = kv.head_dim, half = hd >> 1, nkv = kv.n_kv_heads;
   const int nq = n_heads * hd, nk = nkv * hd;
   const size_t rbase = (size_t)m * ps.ld;
@@ -162,50 +156,6 @@ __global__ void qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__res
   }
 }
 
-// act = silu(scale * sum gate planes) * (scale * sum up planes) as bf16 hi/lo planes; planes [S][M][2F]
-__global__ void swiglu_finish_kernel(PlaneSet ps, RowScale rs, HiLoOut act, int M, int F) {
-  pdl_trigger();
-  SJD_TL(TL_SWIGLU, 0, threadIdx.x == 0);
-  pdl_wait();
-  SJD_TL(TL_SWIGLU, 1, threadIdx.x == 0);
-  if ((F & 3) == 0 && (ps.ld & 3) == 0 && (ps.plane_stride & 3) == 0) {
-    // grid (column chunks, rows): a thread handles groups of four adjacent columns of one row
-    const int m = blockIdx.y;
-    const float sc = row_scale_warp(rs, m);
-    const float *row = ps.base + (size_t)m * ps.ld;
-    for (int f = (blockIdx.x * blockDim.x + threadIdx.x) * 4; f < F; f += gridDim.x * blockDim.x * 4) {
-      float4 g = make_float4(0.f, 0.f, 0.f, 0.f), u = g;
-      for (int sp = 0; sp < ps.splits; ++sp) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(row + (size_t)sp * ps.plane_stride + f));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(row + (size_t)sp * ps.plane_stride + F + f));
-        g.x += a.x; g.y += a.y; g.z += a.z; g.w += a.w;
-        u.x += b.x; u.y += b.y; u.z += b.z; u.w += b.w;
-      }
-      const float gv[4] = {sc * g.x, sc * g.y, sc * g.z, sc * g.w}, uv[4] = {sc * u.x, sc * u.y, sc * u.z, sc * u.w};
-      __nv_bfloat16 hi[4], lo[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float v = gv[i] / (1.0f + expf(-gv[i])) * uv[i];
-        hi[i] = __float2bfloat16_rn(v);
-        lo[i] = __float2bfloat16_rn(v - __bfloat162float(hi[i]));
-      }
-      const size_t idx = (size_t)m * F + f;   // multiple of 4: 8-byte aligned stores
-      *reinterpret_cast<uint2 *>(act.base + idx) = *reinterpret_cast<const uint2 *>(hi);
-      *reinterpret_cast<uint2 *>(act.base + act.lo_offset + idx) = *reinterpret_cast<const uint2 *>(lo);
-    }
-  } else {
-    const size_t total = (size_t)M * F;
-    const size_t nthreads = (size_t)gridDim.x * gridDim.y * blockDim.x;
-    for (size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += nthreads) {
-      const size_t m = i / F, f = i % F;
-      const float sc = row_scale(rs, (int)m);
-      const float g = sc * sum_planes(ps, m * ps.ld + f), u = sc * sum_planes(ps, m * ps.ld + F + f);
-      put_hilo(act, i, g / (1.0f + expf(-g)) * u);
-    }
-  }
-  SJD_TL(TL_SWIGLU, 2, threadIdx.x == 0);
-}
-
 }  // namespace
 
 int resid_gain_parts(int d) { return (d + 127) / 128; }
@@ -227,7 +177,7 @@ int launch_resid_gain(int dtype, float *x, PlaneSet ps, const void *gain, HiLoOu
 }
 
 int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
-                      KvLayout kv, int M, int rows_per_seq, int n_heads, QkNorm qkn, cudaStream_t stream) {
+                      KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream) {
   if (kv.head_dim > 128) return SJD_ERR_UNSUPPORTED;
   // a block per four head slots for a few dozen rows; fewer blocks per row (each walking more slots) as
   // the rows grow, about eight blocks per SM in all
@@ -237,23 +187,12 @@ int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos
   const dim3 grid(M, per_row);
   if (dtype == SJD_F32)
     SJD_CUDA(launch_kernel(qkv_finish_kernel<float>, grid, dim3(256), 0, stream, ps, rs, in_pos, rope_table, q, kv,
-                           rows_per_seq, n_heads, qkn));
+                           segs, n_heads, qkn));
   else if (dtype == SJD_BF16)
     SJD_CUDA(launch_kernel(qkv_finish_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, ps, rs, in_pos, rope_table, q, kv,
-                           rows_per_seq, n_heads, qkn));
+                           segs, n_heads, qkn));
   else
     return SJD_ERR_UNSUPPORTED;
-  SJD_CHECK_LAUNCH();
-  return SJD_OK;
-}
-
-int launch_swiglu_finish(PlaneSet ps, RowScale rs, HiLoOut act, int M, int F, cudaStream_t stream) {
-  // Few enough blocks that (for windows of a few dozen rows) the whole grid is resident at once and
-  // leaves thread slots free: only then is the next kernel scheduled early under dependent launch.
-  int per_row = (F / 4 + 255) / 256;
-  const int cap = 296 / (M < 296 ? M : 296);
-  per_row = per_row > cap ? (cap > 0 ? cap : 1) : per_row;
-  SJD_CUDA(launch_kernel(swiglu_finish_kernel, dim3(per_row, M), dim3(256), 0, stream, ps, rs, act, M, F));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

@@ -519,7 +519,7 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   int tiles = 0;
   for (int j = 0; j < 3; ++j) {
     if (j < g.n_mats && !(gu && j == 1)) {
-      if (g.M < 1 || g.M > 1024 || g.K % TILE_K != 0 || g.n_out[j] < 1) return SJD_ERR_UNSUPPORTED;
+      if (g.M < 1 || g.K % TILE_K != 0 || g.n_out[j] < 1) return SJD_ERR_UNSUPPORTED;
       if (R == TILE_N && g.n_out[j] % TILE_N != 0) return SJD_ERR_UNSUPPORTED;
       tiles += (g.n_out[j] + R - 1) / R;
     }

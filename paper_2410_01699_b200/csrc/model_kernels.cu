@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float *__restrict__ 
 // ------------------------------------------------------------------------------------ RoPE + KV append
 template <typename T>
 __global__ void rope_append_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ in_pos,
-                                   const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, int rows_per_seq,
+                                   const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, RowSegs segs,
                                    int n_heads, QkNorm qkn) {
   const int m = blockIdx.x;
   const int pos = in_pos[m];
   if (pos < 0) return;
-  const int b = m / rows_per_seq;
+  const int b = seg_sequence(segs, m / segs.rows);
   const int hd = kv.head_dim, half = hd >> 1, nkv = kv.n_kv_heads;
   const int nq = n_heads * hd, nk = nkv * hd;
   const float *row = qkv + (size_t)m * (nq + 2 * nk);
@@ -214,8 +214,8 @@ int launch_rmsnorm(int dtype, const float *x, const void *gain, float *h, int M,
 }
 
 int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const float2 *rope_table, float *q,
-                       KvLayout kv, int M, int rows_per_seq, int n_heads, QkNorm qkn, cudaStream_t stream) {
-  SJD_DISPATCH(dtype, (rope_append_kernel<T><<<M, 256, 0, stream>>>(qkv, in_pos, rope_table, q, kv, rows_per_seq,
+                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream) {
+  SJD_DISPATCH(dtype, (rope_append_kernel<T><<<M, 256, 0, stream>>>(qkv, in_pos, rope_table, q, kv, segs,
                                                                    n_heads, qkn)));
   SJD_CHECK_LAUNCH();
   return SJD_OK;

@@ -413,6 +413,17 @@ def test_small_bf16_many_rows():
         assert s.stats.flagged <= max(3, 0.03 * s.stats.decisions), s.stats
 
 
+@pytest.mark.parametrize("name,batch,prompt_len", [
+    ("small-bf16", 1, 1300),   # 21 segments of 64 positions: two passes of the tensor-core pipeline
+    ("small-bf16", 3, 66),     # 65 rows each: segments of 32 or 16, several per sequence in one pass
+    ("small-bf16", 2, 2),      # a single row per sequence
+    ("tiny", 2, 200),          # generic pipeline: two passes of at most 256 rows
+])
+def test_prefill_passes(name, batch, prompt_len):
+    """Pre-fill packs segments of the prompts into passes: segment and pass boundaries, one-row prompts."""
+    run_lockstep(WORKLOADS[name].with_(prompt_len=prompt_len), batch=batch, n_generate=40, max_steps=2)
+
+
 def report_depth(label, seq):
     """One line per cache reading of the checker, for the depth table of the design notes."""
     print()
