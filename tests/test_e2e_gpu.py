@@ -460,6 +460,20 @@ def test_sweep_points_two_layers(batch, window, prompt_len, init, steps):
         assert s.max_logit_excess <= 2e-2
 
 
+@pytest.mark.parametrize("name,batch,window,prompt_len", [
+    ("7b-2l", 3, 5, 90),        # 15 rows: eight key groups over seven tile slots, several tiles per slot
+    ("7b-2l", 1, 9, 530),       # one sequence whose keys are spread over several CTAs and merged
+    ("8b-gqa-2l", 2, 31, 70),   # 62 rows, four query heads per K/V head, two accumulators per tile
+])
+def test_one_launch_pass(name, batch, window, prompt_len):
+    """Passes of at most 64 rows on wide layers run as one launch: row counts off the 16-row grid, every key-group
+    layout of its attention."""
+    ctx, seqs, n, _ = run_lockstep(WORKLOADS[name].with_(prompt_len=prompt_len), batch=batch, window=window, max_steps=2,
+                                   gain_jitter=0.1)
+    for s in seqs:
+        assert s.max_logit_excess <= 2e-2
+
+
 @pytest.mark.parametrize("name,steps", [("7b", 2), ("8b-gqa", 1)])
 def test_full_depth(name, steps):
     """The full configurations (7B: 32 layers, vocab 65536, W = 32, the step the benchmark times; 8B with
