@@ -337,7 +337,7 @@ int sjd_attention(int batch, int window, int n_heads, int n_kv_heads, int head_d
 typedef struct {
   int32_t tensor_core_projections; /* 1: tcgen05 weight-streaming GEMM + fused consumers; 0: generic kernels */
   int32_t tensor_core_attention;   /* 1: TMA-staged split-KV tensor-core attention; 0: generic kernel       */
-  int32_t step_graph;              /* 1: a step is replayed as one captured CUDA graph                       */
+  int32_t step_graph;              /* 1: the forward pass of a step is replayed as one captured CUDA graph   */
   int32_t rows_per_step;           /* batch * window rows per forward pass                                    */
 } sjd_info;
 int sjd_get_info(sjd_ctx *ctx, sjd_info *info);

@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(NWARPS * 32) attention_partial_kernel(
   __shared__ int s_pos[64];
   __shared__ int s_len;
 
+  pdl_trigger();
+  pdl_wait();
   const int h = blockIdx.x, seg = blockIdx.y, s = blockIdx.z;
   const int b = seg_sequence(segs, seg);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -245,12 +247,10 @@ int attention_t(const float *q, KvLayout kv, const int32_t *in_pos, float *out, 
   if (smem > 48 * 1024)
     SJD_CUDA(cudaFuncSetAttribute(attention_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid(n_heads, M / W, splits);
-  attention_partial_kernel<T><<<grid, NWARPS * 32, smem, stream>>>(q, kv, in_pos, partial,
-                                                                  segs, n_heads, splits);
+  SJD_CUDA(launch_kernel(attention_partial_kernel<T>, grid, dim3(NWARPS * 32), smem, stream, q, kv, in_pos, partial, segs,
+                         n_heads, splits));
   SJD_CHECK_LAUNCH();
-  attention_combine_kernel<<<dim3(M, n_heads), 128, 0, stream>>>(partial, in_pos, out, n_heads, hd, splits, hilo);
-  SJD_CHECK_LAUNCH();
-  return SJD_OK;
+  return launch_attention_combine(partial, in_pos, out, M, n_heads, hd, splits, stream, hilo);
 }
 
 }  // namespace

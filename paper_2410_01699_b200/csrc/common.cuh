@@ -230,12 +230,24 @@ size_t verify_scratch_bytes(int batch, int window);
 int check_sample_cfg(const sjd_sample_cfg *s, int vocab);
 
 // ---- model forward (model_kernels.cu, attention.cu); `dtype` selects float / bf16 storage
-enum GemmEpilogue { EPI_STORE_F32 = 0, EPI_STORE_T = 1, EPI_ADD_F32 = 2 };
-
-// C[M][N] (epilogue) = A[M][K] * Wt[N][K]^T, fp32 accumulation.  A is fp32, Wt is of `dtype`;
-// C is fp32 (EPI_STORE_F32, EPI_ADD_F32: C += product) or `dtype` (EPI_STORE_T).  lda/ldc in elements.
-int launch_gemm_simt(int dtype, const void *A, int lda, const void *Wt, void *C, int ldc, int M, int N, int K,
-                     int epilogue, cudaStream_t stream);
+enum RowsEpilogue { RG_STORE = 0, RG_ADD = 1, RG_LOGITS = 2, RG_SWIGLU = 3 };
+// One launch of the generic projections: out[m][n] (epilogue) = s(m) * sum_k x[m][k] * gain[k] * W[n][k], fp32 sums.  The
+// rows of up to three matrices of `dtype` (n[j] rows each, N in all) follow one another; gain (of `dtype`) null: s = gain = 1,
+// else s(m) = 1 / sqrt(mean(x[m]^2) + eps).  RG_ADD: out += product; RG_LOGITS: out is of `dtype`; RG_SWIGLU: w[0] gate,
+// w[1] up, N features, out = silu(gate) * up.
+struct RowsGemm {
+  const float *x;
+  int ldx;
+  const void *w[3];
+  int n[3];
+  const void *gain;
+  float eps;
+  void *out;
+  int ldc;
+  int M, N, K;
+  int epilogue;
+};
+int launch_gemm_rows(int dtype, const RowsGemm &g, cudaStream_t stream);
 // ---- tensor-core weight-streaming GEMM (gemm_tc.cu), bf16 weights
 struct alignas(64) TensorMap {   // an encoded TMA descriptor (same size and alignment as the driver's)
   unsigned char bytes[128];
@@ -313,9 +325,6 @@ int launch_resid_gain(int dtype, float *x, PlaneSet ps, const void *gain, HiLoOu
 // x[m][:] = tok_emb[tok[m]][:]  (fp32 residual stream)
 int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, int M, int d, int vocab,
                  cudaStream_t stream);
-// h[m][:] = x[m][:] * gain[:] / sqrt(mean(x[m]^2) + eps)  (gain of `dtype`)
-int launch_rmsnorm(int dtype, const float *x, const void *gain, float *h, int M, int d, float eps, cudaStream_t stream,
-                   HiLoOut hilo = HiLoOut{nullptr, 0});
 // How the M rows of a pass map to sequences: segment m / rows holds consecutive positions of sequence
 // seq[m / rows] (null: of sequence m / rows).  A step has one segment per sequence (its window); a pre-fill pass
 // packs as many segments of the prompts as fit, several of one sequence among them.
@@ -354,8 +363,6 @@ int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const
                        KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
 int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
-// act[m][f] = silu(gu[m][f]) * gu[m][F + f]
-int launch_swiglu(const float *gu, float *act, int M, int F, cudaStream_t stream, HiLoOut hilo = HiLoOut{nullptr, 0});
 // Window-causal attention: query row m (position in_pos[m] of its segment's sequence) attends cache rows
 // 0 .. in_pos[m].  q, out: fp32 [M][H*hd]; cache of `dtype`.  partial: fp32 scratch [M][H][splits][hd + 2].
 int launch_attention(int dtype, const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial,

@@ -36,7 +36,7 @@ constexpr int kGuRows = 64;
 // Rows of one pre-fill pass: enough that a pass is bound by the tensor pipe and not by streaming the weights
 // once more (13.5 GB of weights take 2.1 ms, 1152 rows of the 7B layers about 30 ms), few enough that the
 // activations of a pass (157 KB per row at the 7B shapes) stay below 200 MB.  (Passes of max_window rows streamed the
-// weights once per 32 prompt tokens: 1063 tokens and one step took 124.2 ms on the 7B shapes, 37.3 ms this way.)  The generic pipeline keeps four
+// weights once per 32 prompt tokens: 1063 tokens and one step took 124.2 ms on the 7B shapes, 37.3 ms this way.)  The generic pipeline keeps three
 // more fp32 buffers per row and is not bound by the weights: 256 rows.
 constexpr int kPrefillRowsTc = 1152, kPrefillRowsGeneric = 256;
 constexpr int kMaxTcRows = 1152;     // largest pass of the tensor-core pipeline
@@ -59,7 +59,7 @@ struct XMaps {
 
 struct Layout {
   size_t kv, logits[2], stats[2], row_out, counters, step, status;
-  size_t x, h, qkv, q, attn, gu, act, partial, rope;
+  size_t x, qkv, q, attn, act, partial, rope;
   size_t xs_h, xs_attn, xs_act, gemm_planes, ss_part;
   size_t pass_layers, pass_loc, pass_counter;   // pass_kernel.cu: per-layer table, column locations, grid-barrier counters
   size_t committed, n, w_eff, draft, q_kind, q_row, q_draft, in_tok, in_pos;
@@ -97,6 +97,9 @@ size_t prefill_rows(const sjd_model_cfg &c, bool tc) {
 // segments (of at least 16 positions) the prompts of a full batch can make
 size_t prefill_segments(const sjd_model_cfg &c) { return (size_t)c.max_batch * ((c.max_seq + 15) / 16); }
 
+// row stride of the generic pipeline's SwiGLU output: rows start on 16 bytes
+int act_stride(const sjd_model_cfg &c) { return (c.ffn_hidden + 3) / 4 * 4; }
+
 Layout make_layout(const sjd_model_cfg &c) {
   Layout L;
   const size_t es = esize(c.dtype);
@@ -127,16 +130,13 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.x = take(Mp * c.d_model * 4);
   L.q = take((Mp + 15) / 16 * 16 * nq * 4);   // fp32, or (pass_kernel.cu) two bf16 planes
   {   // a context runs one of the two pipelines: the generic one's buffers share their memory with the other's planes
-    const size_t generic = align256(Mg * c.d_model * 4) + align256(Mg * (nq + 2 * nk) * 4) + align256(Mg * nq * 4) +
-                           align256(Mg * 2 * c.ffn_hidden * 4) + align256(Mg * c.ffn_hidden * 4);
+    const size_t generic = align256(Mg * (nq + 2 * nk) * 4) + align256(Mg * nq * 4) + align256(Mg * act_stride(c) * 4);
     const size_t Ma = (Mp + 15) / 16 * 16;
     const size_t planes = tc ? align256(2 * Ma * c.d_model * 2) + align256(2 * Ma * nq * 2) + align256(2 * Ma * c.ffn_hidden * 2) : 0;
     const size_t base = off;
-    L.h = take(Mg * c.d_model * 4);
     L.qkv = take(Mg * (nq + 2 * nk) * 4);
     L.attn = take(Mg * nq * 4);
-    L.gu = take(Mg * 2 * c.ffn_hidden * 4);
-    L.act = take(Mg * c.ffn_hidden * 4);
+    L.act = take(Mg * act_stride(c) * 4);
     off = base;   // bf16 hi/lo planes of the GEMM inputs
     L.xs_h = take(tc ? 2 * Ma * c.d_model * 2 : 0);
     L.xs_attn = take(tc ? 2 * Ma * nq * 2 : 0);
@@ -320,12 +320,11 @@ struct sjd_ctx {
   bool prefilled;
   uint32_t host_step;  // number of sjd_step calls since prefill == device step index
   cudaStream_t last_stream;
-  // One captured CUDA graph per logits-buffer parity: a step is ~330 launches, and replaying a graph
-  // takes the host out of the critical path.  Keyed by the caller's output pointers.
+  // One captured CUDA graph of the forward pass per logits-buffer parity (up to 290 launches: replaying a graph takes the
+  // host out of the critical path).  It holds nothing that belongs to a call: the verification, which takes the caller's
+  // output pointers, is launched behind it, so that the graphs serve every pre-fill with the same batch and window.
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
-    sjd_step_out out;
-    bool has_out = false;
     long long launches = 0;
   } graphs[2];
   cudaStream_t capture_stream = nullptr;
@@ -414,46 +413,50 @@ int forward_generic(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cuda
   const int nq = g.n_heads * g.head_dim, nk = g.n_kv_heads * g.head_dim, nqkv = nq + 2 * nk;
   const SeqState st = c->state();
   float *x = c->at<float>(c->lay.x);
-  float *h = c->at<float>(c->lay.h);
   float *qkv = c->at<float>(c->lay.qkv);
   float *q = c->at<float>(c->lay.q);
   float *attn = c->at<float>(c->lay.attn);
-  float *gu = c->at<float>(c->lay.gu);
   float *act = c->at<float>(c->lay.act);
   float *partial = c->at<float>(c->lay.partial);
   const float2 *rope = c->at<float2>(c->lay.rope);
   const int splits = attention_splits(g.n_heads, n_segs);
   int rc;
   Tracer &tr = c->tracer;
-  const double es = (double)esize(dt);
-  auto gemm = [&](const void *w, const float *a, int lda, void *out, int ldc, int n_out, int k_in, int epi) -> int {
-    if (tr.on) tr.gemm_weight_bytes += (double)n_out * (double)k_in * es;
+  auto gemm = [&](const float *a, int lda, const void *gain, const void *w0, int n0, const void *w1, int n1, const void *w2, int n2,
+                  void *out, int ldc, int k_in, int epilogue) -> int {
+    RowsGemm r;
+    r.x = a;
+    r.ldx = lda;
+    r.w[0] = w0; r.w[1] = w1; r.w[2] = w2;
+    r.n[0] = n0; r.n[1] = n1; r.n[2] = n2;
+    r.gain = gain;
+    r.eps = g.rms_eps;
+    r.out = out;
+    r.ldc = ldc;
+    r.M = M;
+    r.N = epilogue == RG_SWIGLU ? n0 : n0 + n1 + n2;
+    r.K = k_in;
+    r.epilogue = epilogue;
+    if (tr.on) tr.gemm_weight_bytes += (double)(n0 + n1 + n2) * (double)k_in * (double)esize(dt);
     tr.begin(TC_GEMM, stream);
-    const int r = launch_gemm_simt(dt, a, lda, w, out, ldc, M, n_out, k_in, epi, stream);
+    const int rcg = launch_gemm_rows(dt, r, stream);
     tr.end(stream);
-    return r;
+    return rcg;
   };
+  const int lda = act_stride(g);
   SJD_TR(TC_OTHER, launch_embed(dt, c->tok_emb, st.in_tok, x, M, d, g.vocab, stream));
   for (int l = 0; l < g.n_layers; ++l) {
-    SJD_TR(TC_OTHER, launch_rmsnorm(dt, x, c->attn_norm[l], h, M, d, g.rms_eps, stream));
-    SJD_TRY(gemm(c->wq[l], h, d, qkv, nqkv, nq, d, EPI_STORE_F32));
-    SJD_TRY(gemm(c->wk[l], h, d, qkv + nq, nqkv, nk, d, EPI_STORE_F32));
-    SJD_TRY(gemm(c->wv[l], h, d, qkv + nq + nk, nqkv, nk, d, EPI_STORE_F32));
+    SJD_TRY(gemm(x, d, c->attn_norm[l], c->wq[l], nq, c->wk[l], nk, c->wv[l], nk, qkv, nqkv, d, RG_STORE));
     const KvLayout kv = c->kv_layer(l);
     SJD_TR(TC_OTHER, launch_rope_append(dt, qkv, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
     if (!logits_out && l == g.n_layers - 1) break;
     SJD_TR(TC_ATTENTION, launch_attention(dt, q, kv, st.in_pos, attn, partial, M, segs, g.n_heads, splits, stream));
-    SJD_TRY(gemm(c->wo[l], attn, nq, x, d, d, nq, EPI_ADD_F32));
-    SJD_TR(TC_OTHER, launch_rmsnorm(dt, x, c->ffn_norm[l], h, M, d, g.rms_eps, stream));
-    SJD_TRY(gemm(c->w_gate[l], h, d, gu, 2 * F, F, d, EPI_STORE_F32));
-    SJD_TRY(gemm(c->w_up[l], h, d, gu + F, 2 * F, F, d, EPI_STORE_F32));
-    SJD_TR(TC_OTHER, launch_swiglu(gu, act, M, F, stream));
-    SJD_TRY(gemm(c->w_down[l], act, F, x, d, d, F, EPI_ADD_F32));
+    SJD_TRY(gemm(attn, nq, nullptr, c->wo[l], d, nullptr, 0, nullptr, 0, x, d, nq, RG_ADD));
+    SJD_TRY(gemm(x, d, c->ffn_norm[l], c->w_gate[l], F, c->w_up[l], F, nullptr, 0, act, lda, d, RG_SWIGLU));
+    SJD_TRY(gemm(act, lda, nullptr, c->w_down[l], d, nullptr, 0, nullptr, 0, x, d, F, RG_ADD));
   }
-  if (logits_out) {
-    SJD_TR(TC_OTHER, launch_rmsnorm(dt, x, c->final_norm, h, M, d, g.rms_eps, stream));
-    SJD_TRY(gemm(c->lm_head, h, d, logits_out, g.vocab, g.vocab, d, EPI_STORE_T));
-  }
+  if (logits_out)
+    SJD_TRY(gemm(x, d, c->final_norm, c->lm_head, g.vocab, nullptr, 0, nullptr, 0, logits_out, g.vocab, d, RG_LOGITS));
   return SJD_OK;
 }
 
@@ -653,12 +656,17 @@ int forward_one_launch(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, vo
   return rc;
 }
 
+// whether a pass of M rows is one cooperative launch
+bool one_launch(const sjd_ctx *c, int M) {
+  return c->use_tc && c->all_tc && c->use_pass && M <= kPassMaxRows && c->xmaps.count((M + 15) / 16 * 16) != 0;
+}
+
 int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const int M = n_segs * segs.rows;
   if (c->use_tc && c->all_tc && M <= kMaxTcRows) {
     auto it = c->xmaps.find((M + 15) / 16 * 16);
     if (it != c->xmaps.end()) {
-      if (c->use_pass && M <= kPassMaxRows) return forward_one_launch(c, it->second, n_segs, segs, logits_out, stream);
+      if (one_launch(c, M)) return forward_one_launch(c, it->second, n_segs, segs, logits_out, stream);
       // every kernel of this pipeline waits for its predecessor itself: launch them overlapped
       g_pdl = !c->tracer.on;
       const int rc = forward_tc(c, it->second, n_segs, segs, logits_out, stream);
@@ -666,7 +674,10 @@ int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t
       return rc;
     }
   }
-  return forward_generic(c, n_segs, segs, logits_out, stream);
+  g_pdl = !c->tracer.on;
+  const int rc = forward_generic(c, n_segs, segs, logits_out, stream);
+  g_pdl = false;
+  return rc;
 }
 
 int run_verify(sjd_ctx *c, const sjd_step_out *out, cudaStream_t stream) {
@@ -916,6 +927,7 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   if (sample->init == SJD_INIT_RESAMPLE_ABOVE && c->cfg.max_ring < sample->grid_stride + sample->window)
     return SJD_ERR_CAPACITY;   // a retained row must outlive the window that draws from it
   cudaStream_t stream = (cudaStream_t)cuda_stream;
+  if (batch != c->batch || sample->window != c->window) c->drop_graphs();   // what a pass depends on
   c->sample = *sample;
   c->batch = batch;
   c->prompt_len = prompt_len;
@@ -941,7 +953,6 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   c->host_step = 0;
   c->last_stream = stream;
   c->prefilled = false;
-  c->drop_graphs();
   const bool tc = c->use_tc && c->all_tc;
   if (tc) add_x_maps(c, batch * sample->window);
   const SeqState st = c->state();
@@ -994,38 +1005,17 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   return SJD_OK;
 }
 
-namespace {
-// forward pass + verification of one step, enqueued on `stream`
-int enqueue_step(sjd_ctx *c, const sjd_step_out *out, int cur, cudaStream_t stream) {
-  int rc = forward(c, c->batch, RowSegs{c->window, nullptr}, c->ws + c->lay.logits[cur], stream);
-  if (rc != SJD_OK) return rc;
-  c->tracer.begin(TC_VERIFY, stream);
-  g_pdl = !c->tracer.on;
-  rc = run_verify(c, out, stream);
-  g_pdl = false;
-  c->tracer.end(stream);
-  return rc;
-}
-
-bool same_out(const sjd_step_out &a, const sjd_step_out *b) {
-  sjd_step_out z;
-  memset(&z, 0, sizeof(z));
-  return memcmp(&a, b ? b : &z, sizeof(sjd_step_out)) == 0;
-}
-}  // namespace
-
 extern "C" int sjd_step(sjd_ctx *c, const sjd_step_out *out, void *cuda_stream) {
   if (!c) return SJD_ERR_BAD_ARG;
   if (!c->prefilled) return SJD_ERR_STATE;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   c->last_stream = stream;
   const int cur = (int)(c->host_step & 1u);
-  if (c->graphs_enabled && c->use_tc && !c->tracer.on) {
+  const RowSegs segs{c->window, nullptr};
+  void *logits = c->ws + c->lay.logits[cur];
+  bool replayed = false;
+  if (c->graphs_enabled && !c->tracer.on && !one_launch(c, c->batch * c->window)) {
     sjd_ctx::StepGraph &g = c->graphs[cur];
-    if (g.exec && !(g.has_out && same_out(g.out, out))) {
-      cudaGraphExecDestroy(g.exec);
-      g.exec = nullptr;
-    }
     if (!g.exec) {
       // capture on a private stream (the caller's may be the legacy default stream), replay on the caller's
       if (!c->capture_stream && cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -1035,7 +1025,7 @@ extern "C" int sjd_step(sjd_ctx *c, const sjd_step_out *out, void *cuda_stream) 
         cudaGraph_t graph = nullptr;
         bool ok = cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
-          const int rc = enqueue_step(c, out, cur, c->capture_stream);
+          const int rc = forward(c, c->batch, segs, logits, c->capture_stream);
           const cudaError_t e = cudaStreamEndCapture(c->capture_stream, &graph);
           ok = rc == SJD_OK && e == cudaSuccess && graph != nullptr;
         }
@@ -1044,9 +1034,6 @@ extern "C" int sjd_step(sjd_ctx *c, const sjd_step_out *out, void *cuda_stream) 
         if (ok) ok = cudaGraphInstantiate(&g.exec, graph, 0) == cudaSuccess;
         if (graph) cudaGraphDestroy(graph);
         if (ok) {
-          memset(&g.out, 0, sizeof(g.out));
-          if (out) g.out = *out;
-          g.has_out = true;
           g.launches = captured;
         } else {
           g.exec = nullptr;
@@ -1058,11 +1045,17 @@ extern "C" int sjd_step(sjd_ctx *c, const sjd_step_out *out, void *cuda_stream) 
     if (g.exec) {
       SJD_CUDA(cudaGraphLaunch(g.exec, stream));
       g_launch_count.fetch_add(g.launches, std::memory_order_relaxed);
-      c->host_step += 1;
-      return SJD_OK;
+      replayed = true;
     }
   }
-  const int rc = enqueue_step(c, out, cur, stream);
+  int rc = SJD_OK;
+  if (!replayed) rc = forward(c, c->batch, segs, logits, stream);
+  if (rc != SJD_OK) return rc;
+  c->tracer.begin(TC_VERIFY, stream);
+  g_pdl = !c->tracer.on && !replayed;
+  rc = run_verify(c, out, stream);
+  g_pdl = false;
+  c->tracer.end(stream);
   if (rc != SJD_OK) return rc;
   c->host_step += 1;
   return c->tracer.flush(stream);
@@ -1105,7 +1098,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
       (tc && c->kv_map_valid && attention_mma_supported(c->cfg.head_dim, c->window)) ? 1 : 0;
-  info->step_graph = (c->graphs_enabled && c->use_tc) ? 1 : 0;
+  info->step_graph = c->graphs_enabled && !one_launch(c, M) ? 1 : 0;
   info->rows_per_step = M;
   return SJD_OK;
 }

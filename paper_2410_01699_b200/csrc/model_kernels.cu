@@ -14,6 +14,21 @@ template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// E = 4 adjacent entries (aligned) or one
+template <typename T, int E>
+__device__ __forceinline__ void load_group(const T *p, float *v) {
+  if constexpr (E == 1) {
+    v[0] = to_f<T>(p[0]);
+  } else if constexpr (sizeof(T) == 4) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else {
+    const uint2 t = *reinterpret_cast<const uint2 *>(p);
+    v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xFFFF0000u);
+  }
+}
+
 __device__ __forceinline__ void store_hilo(const HiLoOut &o, size_t idx, float v) {
   if (!o.base) return;
   const __nv_bfloat16 hi = __float2bfloat16_rn(v);
@@ -21,72 +36,173 @@ __device__ __forceinline__ void store_hilo(const HiLoOut &o, size_t idx, float v
   o.base[o.lo_offset + idx] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// ------------------------------------------------------------------------------------ GEMM (FMA)
-// 32 x 64 output tile per block of 256 threads, K in slices of 32; every access is bounds-checked so
-// any M, N, K (683, 1408, ...) works.  Sums run over k in increasing order: deterministic.
-constexpr int GM = 32, GN = 64, GK = 32;
+// ------------------------------------------------------------------------------------ projections (FMA)
+// A projection of a few rows through small or odd-shaped matrices, where a step is a chain of launches that each cost their
+// own latency (two layers of d 256 and 16 rows: 29 launches, 418 us of projections in a 476 us step with 32 x 64 tiles that
+// walked K in slices of 32, one dependent load after the other; 14 launches and 101 us a step now).  Hence: one CTA per 16 rows x 8 * NJ weight rows, the
+// eight warps split every 256-column chunk of K between them, so that a whole chunk is one round trip to memory, and the
+// next chunk is on its way while this one is multiplied.  The RMS normalisation before a projection (its row scale
+// commutes with the product), the residual add and SwiGLU are part of the launch.  Any M, N, K; the sums have one fixed order.
+constexpr int RG_M = 16, RG_K = 256, RG_LD = RG_K + 4;   // + 4: rows eight apart meet in different banks
 
-template <typename T, int EPI>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const float *__restrict__ A, int lda, const T *__restrict__ Wt,
-                                                        void *__restrict__ Cv, int ldc, int M, int N, int K) {
-  __shared__ float As[GM][GK + 1];
-  __shared__ float Ws[GN][GK + 1];
-  const int tid = threadIdx.x;
-  const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
-  const int ty = tid >> 4, tx = tid & 15;  // rows ty*2..+1, cols tx*4..+3
-  float acc[2][4] = {};
-  for (int k0 = 0; k0 < K; k0 += GK) {
-    for (int i = tid; i < GM * GK; i += 256) {
-      const int r = i / GK, c = i % GK;
-      const int m = m0 + r, k = k0 + c;
-      As[r][c] = (m < M && k < K) ? A[(size_t)m * lda + k] : 0.0f;
+// VEC: rows of x and of every matrix can be read in groups of four entries
+template <typename T, int NJ, bool VEC>
+__global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
+  constexpr int BN = 8 * NJ;
+  extern __shared__ float smem[];
+  float *xs = smem, *ws = smem + RG_M * RG_LD;
+  __shared__ float s_ss[RG_M][8];
+  pdl_trigger();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.y * RG_M, t0 = blockIdx.x;
+  const bool glu = g.epilogue == RG_SWIGLU;
+  const T *gain = reinterpret_cast<const T *>(g.gain);
+  // weight row r of this tile: under SwiGLU the first half of the rows are gate features, the second the same up features
+  auto wrow = [&](int r) -> const T * {
+    int n, j = 0;
+    if (glu) {
+      j = r >= BN / 2;
+      n = t0 * (BN / 2) + r - j * (BN / 2);
+    } else {
+      n = t0 * BN + r;
+      while (j < 2 && n >= g.n[j]) n -= g.n[j++];
     }
-    for (int i = tid; i < GN * GK; i += 256) {
-      const int r = i / GK, c = i % GK;
-      const int n = n0 + r, k = k0 + c;
-      Ws[r][c] = (n < N && k < K) ? to_f<T>(Wt[(size_t)n * K + k]) : 0.0f;
+    return n < g.n[j] ? reinterpret_cast<const T *>(g.w[j]) + (size_t)n * g.K : nullptr;
+  };
+  constexpr int E = VEC ? 4 : 1, PER = 256 / (RG_K / E);        // entries per load, rows per round of the block
+  constexpr int NXL = RG_M / PER, NWL = BN / PER;
+  const int col = tid % (RG_K / E) * E, r0 = tid / (RG_K / E);
+  float xr[NXL][E], wr[NWL][E], gr[E], ss[NXL];
+#pragma unroll
+  for (int i = 0; i < NXL; ++i) ss[i] = 0.0f;
+  auto load_w = [&](int k0) {
+    const int k = k0 + col;
+#pragma unroll
+    for (int i = 0; i < NWL; ++i) {
+      const T *row = wrow(r0 + i * PER);
+#pragma unroll
+      for (int e = 0; e < E; ++e) wr[i][e] = 0.0f;
+      if (row && k < g.K) load_group<T, E>(row + k, wr[i]);
     }
-    __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      const float a0 = As[ty * 2][kk], a1 = As[ty * 2 + 1][kk];
+    for (int e = 0; e < E; ++e) gr[e] = 1.0f;
+    if (gain && k < g.K) load_group<T, E>(gain + k, gr);
+  };
+  auto load_x = [&](int k0) {
+    const int k = k0 + col;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float w = Ws[tx * 4 + j][kk];
-        acc[0][j] = fmaf(a0, w, acc[0][j]);
-        acc[1][j] = fmaf(a1, w, acc[1][j]);
+    for (int i = 0; i < NXL; ++i) {
+      const int m = m0 + r0 + i * PER;
+#pragma unroll
+      for (int e = 0; e < E; ++e) xr[i][e] = 0.0f;
+      if (m < g.M && k < g.K) load_group<float, E>(g.x + (size_t)m * g.ldx + k, xr[i]);
+    }
+  };
+  load_w(0);     // the weights do not depend on the kernel before
+  pdl_wait();
+  load_x(0);
+  const int lm = lane >> 3, ln = lane & 7;
+  float acc[4][NJ];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0f;
+  for (int k0 = 0; k0 < g.K; k0 += RG_K) {
+    if (k0) __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NXL; ++i)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        ss[i] = fmaf(xr[i][e], xr[i][e], ss[i]);
+        xs[(r0 + i * PER) * RG_LD + col + e] = xr[i][e] * gr[e];
       }
-    }
+#pragma unroll
+    for (int i = 0; i < NWL; ++i)
+#pragma unroll
+      for (int e = 0; e < E; ++e) ws[(r0 + i * PER) * RG_LD + col + e] = wr[i][e];
     __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int m = m0 + ty * 2 + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      const size_t idx = (size_t)m * ldc + n;
-      if (EPI == EPI_STORE_F32) reinterpret_cast<float *>(Cv)[idx] = acc[i][j];
-      else if (EPI == EPI_ADD_F32) reinterpret_cast<float *>(Cv)[idx] += acc[i][j];
-      else reinterpret_cast<T *>(Cv)[idx] = from_f<T>(acc[i][j]);
+    if (k0 + RG_K < g.K) {
+      load_w(k0 + RG_K);
+      load_x(k0 + RG_K);
     }
+    const int kw = warp * (RG_K / 8);
+#pragma unroll
+    for (int k = 0; k < RG_K / 8; k += 4) {
+      float4 xv[4], wv[NJ];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) xv[i] = *reinterpret_cast<const float4 *>(xs + (lm + 4 * i) * RG_LD + kw + k);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) wv[j] = *reinterpret_cast<const float4 *>(ws + (ln + 8 * j) * RG_LD + kw + k);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          acc[i][j] = fmaf(xv[i].w, wv[j].w, fmaf(xv[i].z, wv[j].z, fmaf(xv[i].y, wv[j].y, fmaf(xv[i].x, wv[j].x, acc[i][j]))));
+    }
+  }
+  // sums of squares of the rows (their columns lie over 256 / PER threads, whole warps of one row each)
+  if (gain) {
+#pragma unroll
+    for (int i = 0; i < NXL; ++i) {
+      const float t = warp_sum(ss[i]);
+      if (lane == 0) s_ss[r0 + i * PER][warp % (8 / PER)] = t;
+    }
+  }
+  __syncthreads();
+  float *red = smem;   // [warp][row][BN + 1]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) red[(warp * RG_M + lm + 4 * i) * (BN + 1) + ln + 8 * j] = acc[i][j];
+  __syncthreads();
+  auto total = [&](int r, int c) {
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += red[(w * RG_M + r) * (BN + 1) + c];
+    return t;
+  };
+  const int cols = glu ? BN / 2 : BN;
+  for (int i = tid; i < RG_M * cols; i += 256) {
+    const int r = i / cols, c = i - r * cols, m = m0 + r, n = t0 * cols + c;
+    if (m >= g.M || n >= g.N) continue;
+    float scale = 1.0f;
+    if (gain) {
+      float t = 0.0f;
+#pragma unroll
+      for (int w = 0; w < 8 / PER; ++w) t += s_ss[r][w];
+      scale = rsqrtf(t / (float)g.K + g.eps);
+    }
+    float v = total(r, c) * scale;
+    if (glu) {
+      const float u = total(r, c + BN / 2) * scale;
+      v = v / (1.0f + expf(-v)) * u;
+    }
+    const size_t idx = (size_t)m * g.ldc + n;
+    if (g.epilogue == RG_ADD) reinterpret_cast<float *>(g.out)[idx] += v;
+    else if (g.epilogue == RG_LOGITS) reinterpret_cast<T *>(g.out)[idx] = from_f<T>(v);
+    else reinterpret_cast<float *>(g.out)[idx] = v;
   }
 }
 
 template <typename T>
-int gemm_simt_t(const void *A, int lda, const void *Wt, void *C, int ldc, int M, int N, int K, int epi,
-                cudaStream_t stream) {
-  dim3 grid((N + GN - 1) / GN, (M + GM - 1) / GM);
-  const float *a = reinterpret_cast<const float *>(A);
-  const T *w = reinterpret_cast<const T *>(Wt);
-  if (epi == EPI_STORE_F32) gemm_simt_kernel<T, EPI_STORE_F32><<<grid, 256, 0, stream>>>(a, lda, w, C, ldc, M, N, K);
-  else if (epi == EPI_STORE_T) gemm_simt_kernel<T, EPI_STORE_T><<<grid, 256, 0, stream>>>(a, lda, w, C, ldc, M, N, K);
-  else if (epi == EPI_ADD_F32) gemm_simt_kernel<T, EPI_ADD_F32><<<grid, 256, 0, stream>>>(a, lda, w, C, ldc, M, N, K);
-  else return SJD_ERR_BAD_ARG;
-  SJD_CHECK_LAUNCH();
-  return SJD_OK;
+int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
+  const int mt = (g.M + RG_M - 1) / RG_M;
+  const int wide = g.epilogue == RG_SWIGLU ? 16 : 32;   // output columns of a CTA with four weight rows per lane
+  // two weight rows per lane while that still leaves the grid within one wave (half the work per CTA)
+  const bool narrow = mt * ((g.N + wide / 2 - 1) / (wide / 2)) <= 148;
+  bool vec = g.K % 4 == 0 && g.ldx % 4 == 0 && ((uintptr_t)g.x & 15u) == 0 && ((uintptr_t)g.gain & (4 * sizeof(T) - 1)) == 0;
+  for (int j = 0; j < 3; ++j) vec = vec && ((uintptr_t)g.w[j] & (4 * sizeof(T) - 1)) == 0;
+  const int cols = narrow ? wide / 2 : wide, bn = narrow ? 16 : 32;
+  const size_t smem = (size_t)(RG_M + bn) * RG_LD * sizeof(float);
+  const dim3 grid((g.N + cols - 1) / cols, mt);
+  auto launch = [&](auto kernel) -> int {
+    if (smem > 40 * 1024) SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SJD_CUDA(launch_kernel(kernel, grid, dim3(256), smem, stream, g));
+    SJD_CHECK_LAUNCH();
+    return SJD_OK;
+  };
+  if (narrow) return vec ? launch(gemm_rows_kernel<T, 2, true>) : launch(gemm_rows_kernel<T, 2, false>);
+  return vec ? launch(gemm_rows_kernel<T, 4, true>) : launch(gemm_rows_kernel<T, 4, false>);
 }
 
 // ------------------------------------------------------------------------------------ embedding
@@ -102,34 +218,13 @@ __global__ void embed_kernel(const T *__restrict__ emb, const int32_t *__restric
   for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)m * d + i] = to_f<T>(row[i]);
 }
 
-// ------------------------------------------------------------------------------------ RMSNorm
-template <typename T>
-__global__ void __launch_bounds__(256) rmsnorm_kernel(const float *__restrict__ x, const T *__restrict__ gain,
-                                                      float *__restrict__ h, int d, float eps, HiLoOut hilo) {
-  __shared__ float red[8];
-  const int m = blockIdx.x, tid = threadIdx.x;
-  const float *row = x + (size_t)m * d;
-  float ss = 0.0f;
-  for (int i = tid; i < d; i += 256) ss = fmaf(row[i], row[i], ss);
-  ss = warp_sum(ss);
-  if ((tid & 31) == 0) red[tid >> 5] = ss;
-  __syncthreads();
-  float tot = 0.0f;
-#pragma unroll
-  for (int w = 0; w < 8; ++w) tot += red[w];
-  const float scale = rsqrtf(tot / (float)d + eps);
-  for (int i = tid; i < d; i += 256) {
-    const float v = row[i] * scale * to_f<T>(gain[i]);
-    h[(size_t)m * d + i] = v;
-    store_hilo(hilo, (size_t)m * d + i, v);
-  }
-}
-
 // ------------------------------------------------------------------------------------ RoPE + KV append
 template <typename T>
 __global__ void rope_append_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ in_pos,
                                    const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, RowSegs segs,
                                    int n_heads, QkNorm qkn) {
+  pdl_trigger();
+  pdl_wait();
   const int m = blockIdx.x;
   const int pos = in_pos[m];
   if (pos < 0) return;
@@ -171,18 +266,6 @@ __global__ void rope_append_kernel(const float *__restrict__ qkv, const int32_t 
   }
 }
 
-// ------------------------------------------------------------------------------------ SwiGLU
-__global__ void swiglu_kernel(const float *__restrict__ gu, float *__restrict__ act, int M, int F, HiLoOut hilo) {
-  const size_t total = (size_t)M * F;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t m = i / F, f = i % F;
-    const float g = gu[m * 2 * F + f], u = gu[m * 2 * F + F + f];
-    const float v = g / (1.0f + expf(-g)) * u;
-    act[i] = v;
-    store_hilo(hilo, i, v);
-  }
-}
-
 }  // namespace
 
 #define SJD_DISPATCH(dtype, CALL)                         \
@@ -192,10 +275,9 @@ __global__ void swiglu_kernel(const float *__restrict__ gu, float *__restrict__ 
     else return SJD_ERR_UNSUPPORTED;                      \
   } while (0)
 
-int launch_gemm_simt(int dtype, const void *A, int lda, const void *Wt, void *C, int ldc, int M, int N, int K,
-                     int epilogue, cudaStream_t stream) {
-  if (M <= 0 || N <= 0 || K <= 0) return SJD_ERR_BAD_ARG;
-  SJD_DISPATCH(dtype, return gemm_simt_t<T>(A, lda, Wt, C, ldc, M, N, K, epilogue, stream));
+int launch_gemm_rows(int dtype, const RowsGemm &g, cudaStream_t stream) {
+  if (g.M <= 0 || g.N <= 0 || g.K <= 0) return SJD_ERR_BAD_ARG;
+  SJD_DISPATCH(dtype, return gemm_rows_t<T>(g, stream));
 }
 
 int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, int M, int d, int vocab,
@@ -206,25 +288,10 @@ int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, i
   return SJD_OK;
 }
 
-int launch_rmsnorm(int dtype, const float *x, const void *gain, float *h, int M, int d, float eps, cudaStream_t stream,
-                   HiLoOut hilo) {
-  SJD_DISPATCH(dtype, (rmsnorm_kernel<T><<<M, 256, 0, stream>>>(x, reinterpret_cast<const T *>(gain), h, d, eps, hilo)));
-  SJD_CHECK_LAUNCH();
-  return SJD_OK;
-}
-
 int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const float2 *rope_table, float *q,
                        KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream) {
-  SJD_DISPATCH(dtype, (rope_append_kernel<T><<<M, 256, 0, stream>>>(qkv, in_pos, rope_table, q, kv, segs,
-                                                                   n_heads, qkn)));
-  SJD_CHECK_LAUNCH();
-  return SJD_OK;
-}
-
-int launch_swiglu(const float *gu, float *act, int M, int F, cudaStream_t stream, HiLoOut hilo) {
-  const size_t total = (size_t)M * F;
-  const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
-  swiglu_kernel<<<blocks, 256, 0, stream>>>(gu, act, M, F, hilo);
+  SJD_DISPATCH(dtype, SJD_CUDA(launch_kernel(rope_append_kernel<T>, dim3(M), dim3(256), 0, stream, qkv, in_pos, rope_table, q, kv,
+                                             segs, n_heads, qkn)));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

@@ -460,6 +460,17 @@ def test_sweep_points_two_layers(batch, window, prompt_len, init, steps):
         assert s.max_logit_excess <= 2e-2
 
 
+@pytest.mark.parametrize("name,over,batch,window", [
+    ("tiny", dict(n_heads=3, n_kv_heads=3, head_dim=62, d_model=250, vocab=1021), 1, 5),   # rows off 16 bytes, widths off the tiles
+    ("tiny", {}, 5, 31),                                                                    # 155 rows: four weight rows per lane
+    ("small-bf16", dict(ffn_hidden=1003, vocab=1001), 2, 7),                                # bf16, some matrices unaligned
+])
+def test_generic_projections(name, over, batch, window):
+    """The generic pipeline (fused normalisation, residual and SwiGLU) on row counts and widths off its tiles."""
+    ctx, seqs, n, _ = run_lockstep(WORKLOADS[name].with_(**over), batch=batch, window=window, n_generate=30, max_steps=3)
+    assert ctx.info()["tensor_core_projections"] == 0
+
+
 @pytest.mark.parametrize("name,batch,window,prompt_len", [
     ("7b-2l", 3, 5, 90),        # 15 rows: eight key groups over seven tile slots, several tiles per slot
     ("7b-2l", 1, 9, 530),       # one sequence whose keys are spread over several CTAs and merged
