@@ -1554,140 +1554,151 @@ __device__ void finalize_sequence(const VerifyParams &p, int b, uint32_t step, S
   }
 }
 
-// ------------------------------------------------------------------------------------ kernel
-// STREAM: the instantiation launched for bf16 rows too long for the registers of a block (see long_statistics)
-template <typename T, int MAXT, bool STREAM = false>
-__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1) verify_rows_kernel(const VerifyParams p) {
+// ------------------------------------------------------------------------------------ what a row is verified with
+template <typename T>
+struct RowJob {
+  int b, k, r;             // sequence (image), window slot, row record
+  int kind, d, qr;         // law of the draft, the draft, row that produced it
+  bool q_ring, jacobi;
+  uint32_t step;
+  int cur;
+  float inv_t, u_acc, u_res, u_draft;
+  RowRefs<T> rows;
+};
+// false: slot k is not in use
+template <typename T>
+__device__ __forceinline__ bool row_job(const VerifyParams &p, int r, RowJob<T> &j) {
+  j.r = r;
+  j.b = r / p.W;
+  j.k = r - j.b * p.W;
+  const int sb = p.paired ? 2 * j.b : j.b;   // sequence whose state describes the window (under guidance both streams' do)
+  const int rs = sb * p.W + j.k;
+  j.step = p.step_ptr ? *p.step_ptr : p.step;
+  j.cur = p.step_ptr ? (int)(j.step & 1u) : 0;
+  j.inv_t = 1.0f / p.temperature;
+  if (j.k >= (p.w_eff ? p.w_eff[sb] : p.W)) return false;
+  // (the Jacobi schedule compares tokens and uses no q: treat every draft as a copied one)
+  const int kind_raw = p.q_kind ? p.q_kind[rs] : SJD_Q_ROW;
+  j.q_ring = kind_raw == SJD_Q_RING;   // a retained row: the same law as a row of the other buffer
+  j.jacobi = p.schedule == SJD_SCHEDULE_JACOBI;
+  j.kind = j.jacobi ? SJD_Q_ONEHOT : (j.q_ring ? SJD_Q_ROW : kind_raw);
+  j.d = p.draft[rs];
+  j.qr = p.q_row ? p.q_row[rs] : j.k;
+  const int base = p.e2e ? p.st.n[sb] : (p.base_pos ? p.base_pos[j.b] : 0);
+  const Philox4 rnd = philox4x32_10((uint32_t)(base + j.k), j.step, p.seq_base + (uint32_t)j.b, kStreamVerify, p.seed_lo, p.seed_hi);
+  j.u_acc = u24(rnd.w[0]);
+  j.u_res = u24(rnd.w[1]);
+  j.u_draft = u24(rnd.w[2]);
+  if (j.jacobi)   // Sec. 3.2: the draw of a position uses the same uniform in every pass (step index 0)
+    j.u_draft = u24(philox4x32_10((uint32_t)(base + j.k), 0u, p.seq_base + (uint32_t)j.b, kStreamVerify, p.seed_lo, p.seed_hi).w[2]);
+  j.rows = row_refs<T>(p, j.b, j.k, j.qr, j.cur, j.q_ring);
+  return true;
+}
+
+// Eq. 2 by the functors of the general route: residual weights, or p itself where nothing is left
+template <typename T>
+__device__ void general_residual(const ResidualWeights<T> &rf, const PRowWeights<T> &pf, float u_res, Scratch &sc, uint32_t &flags) {
   using E = Elt<T>;
-  extern __shared__ uint4 dyn_smem[];
-  __shared__ Scratch sc;
-  uint4 *stage = p.staged ? dyn_smem : nullptr;
-  pdl_trigger();
-  SJD_TL(TL_VERIFY, 0, threadIdx.x == 0);
-  pdl_wait();   // the logits come from the preceding kernel
-  SJD_TL(TL_VERIFY, 1, threadIdx.x == 0);
-
-  const int r = blockIdx.x;
-  const int b = r / p.W, k = r % p.W;
-  const int sb = p.paired ? 2 * b : b;   // sequence whose state describes the window (under guidance both streams' do)
-  const int rs = sb * p.W + k;
-  const int tid = threadIdx.x;
-  const int w_eff = p.w_eff ? p.w_eff[sb] : p.W;
-  const uint32_t step = p.step_ptr ? *p.step_ptr : p.step;
-  const int cur = p.step_ptr ? (int)(step & 1u) : 0;
-  const float inv_t = 1.0f / p.temperature;
-
-  if (k < w_eff) {
-    // (the Jacobi schedule compares tokens and uses no q: treat every draft as a copied one)
-    const int kind_raw = p.q_kind ? p.q_kind[rs] : SJD_Q_ROW;
-    const bool q_ring = kind_raw == SJD_Q_RING;   // a retained row: the same law as a row of the other buffer
-    const int kind = p.schedule == SJD_SCHEDULE_JACOBI ? SJD_Q_ONEHOT : (q_ring ? SJD_Q_ROW : kind_raw);
-    const int d = p.draft[rs];
-    const bool d_ok = d >= 0 && d < p.V;
-    const int qr = p.q_row ? p.q_row[rs] : k;
-    const int base = p.e2e ? p.st.n[sb] : (p.base_pos ? p.base_pos[b] : 0);
-    const Philox4 rnd = philox4x32_10((uint32_t)(base + k), step, p.seq_base + (uint32_t)b, kStreamVerify,
-                                      p.seed_lo, p.seed_hi);
-    const float u_acc = u24(rnd.w[0]), u_res = u24(rnd.w[1]);
-    float u_draft = u24(rnd.w[2]);
-    const bool jacobi = p.schedule == SJD_SCHEDULE_JACOBI;
-    if (jacobi)   // Sec. 3.2: the draw of a position uses the same uniform in every pass (step index 0)
-      u_draft = u24(philox4x32_10((uint32_t)(base + k), 0u, p.seq_base + (uint32_t)b, kStreamVerify, p.seed_lo, p.seed_hi).w[2]);
-    const RowRefs<T> rows = row_refs<T>(p, b, k, qr, cur, q_ring);
-
-    RowOut fast_out;
-    const bool fast_done = p.fast && (((uintptr_t)rows.q | (uintptr_t)rows.p) & 15u) == 0 &&
-                           fast_row<T, STREAM>(p, sc, r, b, kind, d, qr, cur, rows, inv_t, u_acc, u_res, u_draft, fast_out);
-    if (fast_done) {
-      if (tid == 0) p.row_out[r] = fast_out;
-    } else {
+  const int NV = rf.prow.NV, off = rf.prow.off;
+  chunk_sums<E::VEC>(rf, NV, sc);
+  if (sc.chunk_excl[(NV + 31) >> 5] > 0.0) {
+    sample_icdf<E::VEC>(rf, NV, off, sc, u_res);
+  } else {
+    flags |= SJD_FLAG_RESIDUAL_EMPTY;
     __syncthreads();
-    // ---- the law of the draft
-    Row<T> qrow;
-    qrow.init(rows.q, p.V, rows.q2, p.guidance);
-    RowStats qs;
-    qs.tau_key = 0; qs.xmax = 0.0f; qs.z = 1.0f; qs.flags = 0;
-    PRowWeights<T> qf;
-    float q_d;
-    if (kind == SJD_Q_ROW) {
-      if (p.prev_stats_valid) {
-        qs = *rows.qstats;
-      } else {
-        qs = row_statistics<T>(qrow, stage, sc, p.top_k, inv_t, qf);
-        if (tid == 0) p.stats[cur ^ 1][r] = qs;
-        __syncthreads();
-        qrow.s = nullptr;  // the staging buffer is about to be reused
-      }
-      qf.row = qrow;
-      qf.pw.init(qs, inv_t);
-      q_d = d_ok ? qf.pw.one(qrow.element(d), d) / qs.z : 1.0f;
-    } else if (kind == SJD_Q_UNIFORM) {
-      q_d = 1.0f / (float)p.V;
+    chunk_sums<E::VEC>(pf, NV, sc);
+    sample_icdf<E::VEC>(pf, NV, off, sc, u_res);
+  }
+}
+
+// the general route: any row, block-wide
+template <typename T>
+__device__ void general_row(const VerifyParams &p, const RowJob<T> &j, uint4 *stage, Scratch &sc) {
+  using E = Elt<T>;
+  const int tid = threadIdx.x, kind = j.kind, d = j.d;
+  const bool d_ok = d >= 0 && d < p.V;
+  __syncthreads();
+  // ---- the law of the draft
+  Row<T> qrow;
+  qrow.init(j.rows.q, p.V, j.rows.q2, p.guidance);
+  RowStats qs;
+  qs.tau_key = 0; qs.xmax = 0.0f; qs.z = 1.0f; qs.flags = 0;
+  PRowWeights<T> qf;
+  float q_d;
+  if (kind == SJD_Q_ROW) {
+    if (p.prev_stats_valid) {
+      qs = *j.rows.qstats;
     } else {
-      q_d = 1.0f;
+      qs = row_statistics<T>(qrow, stage, sc, p.top_k, j.inv_t, qf);
+      if (tid == 0) p.stats[j.cur ^ 1][j.r] = qs;
+      __syncthreads();
+      qrow.s = nullptr;  // the staging buffer is about to be reused
     }
-
-    SJD_TL(TL_VERIFY, 10, tid == 0);   // the draft's law is known
-    // ---- this iteration's distribution
-    Row<T> prow;
-    prow.init(rows.p, p.V, rows.p2, p.guidance);
-    PRowWeights<T> pf;
-    const RowStats ps = row_statistics<T>(prow, stage, sc, p.top_k, inv_t, pf);
-    if (tid == 0) p.stats[cur][r] = ps;
-    const float p_d = d_ok ? pf.pw.one(prow.element(d), d) / ps.z : 0.0f;
-
-    SJD_TL(TL_VERIFY, 11, tid == 0);   // this row's statistics are known
-    // ---- Eq. 1
-    float ratio;
-    if (q_d > 0.0f) ratio = p_d / q_d;
-    else ratio = p_d > 0.0f ? INFINITY : 0.0f;
-    float thr = fminf(1.0f, ratio);
-    bool accept = u_acc < thr;
-    uint32_t flags = ps.flags | (kind == SJD_Q_ROW ? qs.flags : 0u);
-    if (thr < 1.0f && fabsf(u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
-
-    // ---- Eq. 3: re-draft from p (used if an earlier row rejects)
-    sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, u_draft);
-    const int redraft_tok = sc.tok;
-    const float redraft_p = sc.tok_w / ps.z;
-    __syncthreads();
-
-    SJD_TL(TL_VERIFY, 12, tid == 0);   // re-draft token drawn
-    // ---- Eq. 2: residual resample (used if this is the first rejected row)
-    int resample_tok = -1;
-    if (jacobi) {   // deterministic criterion instead of Eqs. 1-2
-      accept = d_ok && redraft_tok == d;
-      thr = accept ? 1.0f : 0.0f;
-      flags &= ~SJD_FLAG_NEAR_TIE_ACCEPT;
-      resample_tok = accept ? -1 : redraft_tok;
-    } else if (!accept) {
-      ResidualWeights<T> rf;
-      rf.prow = prow; rf.qrow = qrow; rf.pw = pf.pw; rf.qw = qf.pw;
-      rf.inv_zp = 1.0f / ps.z; rf.inv_zq = 1.0f / qs.z;
-      rf.kind = kind; rf.draft = d; rf.V = p.V;
-      if (kind != SJD_Q_ROW) rf.qw = pf.pw;
-      chunk_sums<E::VEC>(rf, prow.NV, sc);
-      if (sc.chunk_excl[(prow.NV + 31) >> 5] > 0.0) {
-        sample_icdf<E::VEC>(rf, prow.NV, prow.off, sc, u_res);
-      } else {
-        flags |= SJD_FLAG_RESIDUAL_EMPTY;
-        __syncthreads();
-        chunk_sums<E::VEC>(pf, prow.NV, sc);
-        sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, u_res);
-      }
-      resample_tok = sc.tok;
-    }
-    SJD_TL(TL_VERIFY, 13, tid == 0);   // residual token drawn
-    if (tid == 0) {
-      RowOut ro;
-      ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
-      ro.redraft_tok = redraft_tok; ro.redraft_p = redraft_p; ro.resample_tok = resample_tok; ro.flags = flags;
-      p.row_out[r] = ro;
-    }
-    }   // general route
+    qf.row = qrow;
+    qf.pw.init(qs, j.inv_t);
+    q_d = d_ok ? qf.pw.one(qrow.element(d), d) / qs.z : 1.0f;
+  } else if (kind == SJD_Q_UNIFORM) {
+    q_d = 1.0f / (float)p.V;
+  } else {
+    q_d = 1.0f;
   }
 
-  // ---- ticket: the last block of the sequence slides the window
+  SJD_TL(TL_VERIFY, 10, tid == 0);   // the draft's law is known
+  // ---- this iteration's distribution
+  Row<T> prow;
+  prow.init(j.rows.p, p.V, j.rows.p2, p.guidance);
+  PRowWeights<T> pf;
+  const RowStats ps = row_statistics<T>(prow, stage, sc, p.top_k, j.inv_t, pf);
+  if (tid == 0) p.stats[j.cur][j.r] = ps;
+  const float p_d = d_ok ? pf.pw.one(prow.element(d), d) / ps.z : 0.0f;
+
+  SJD_TL(TL_VERIFY, 11, tid == 0);   // this row's statistics are known
+  // ---- Eq. 1
+  float ratio;
+  if (q_d > 0.0f) ratio = p_d / q_d;
+  else ratio = p_d > 0.0f ? INFINITY : 0.0f;
+  float thr = fminf(1.0f, ratio);
+  bool accept = j.u_acc < thr;
+  uint32_t flags = ps.flags | (kind == SJD_Q_ROW ? qs.flags : 0u);
+  if (thr < 1.0f && fabsf(j.u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
+
+  // ---- Eq. 3: re-draft from p (used if an earlier row rejects)
+  sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, j.u_draft);
+  const int redraft_tok = sc.tok;
+  const float redraft_p = sc.tok_w / ps.z;
+  __syncthreads();
+
+  SJD_TL(TL_VERIFY, 12, tid == 0);   // re-draft token drawn
+  // ---- Eq. 2: residual resample (used if this is the first rejected row)
+  int resample_tok = -1;
+  if (j.jacobi) {   // deterministic criterion instead of Eqs. 1-2
+    accept = d_ok && redraft_tok == d;
+    thr = accept ? 1.0f : 0.0f;
+    flags &= ~SJD_FLAG_NEAR_TIE_ACCEPT;
+    resample_tok = accept ? -1 : redraft_tok;
+  } else if (!accept) {
+    ResidualWeights<T> rf;
+    rf.prow = prow; rf.qrow = qrow; rf.pw = pf.pw; rf.qw = qf.pw;
+    rf.inv_zp = 1.0f / ps.z; rf.inv_zq = 1.0f / qs.z;
+    rf.kind = kind; rf.draft = d; rf.V = p.V;
+    if (kind != SJD_Q_ROW) rf.qw = pf.pw;
+    general_residual<T>(rf, pf, j.u_res, sc, flags);
+    resample_tok = sc.tok;
+  }
+  SJD_TL(TL_VERIFY, 13, tid == 0);   // residual token drawn
+  if (tid == 0) {
+    RowOut ro;
+    ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
+    ro.redraft_tok = redraft_tok; ro.redraft_p = redraft_p; ro.resample_tok = resample_tok; ro.flags = flags;
+    p.row_out[j.r] = ro;
+  }
+}
+
+// After a block's row record is written (block-wide): a ticket; the last block of the sequence slides the window.
+// `deferred(...)`: makes the Eq. 2 draw that the rows of the sequence have left open.
+template <typename T, typename F>
+__device__ void ticket_and_slide(const VerifyParams &p, int b, uint32_t step, int cur, Scratch &sc, F deferred) {
+  const int tid = threadIdx.x;
   __syncthreads();
   if (tid == 0) {
     __threadfence();
@@ -1698,9 +1709,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1)
   if (!sc.is_last) return;
   __threadfence();
   SJD_TL(TL_VERIFY, 14, tid == 0);
-  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-    if (p.fast && p.defer_residual) deferred_residual_bf16<STREAM>(p, b, step, cur, sc);
-  }
+  deferred();
   if (p.e2e && (p.st.init == SJD_INIT_RESAMPLE_LEFT || p.st.init == SJD_INIT_RESAMPLE_ABOVE))
     draw_fresh_slots<T>(p, b, step, cur, sc);
   finalize_sequence(p, b, step, sc);
@@ -1715,6 +1724,737 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1)
       if (p.step_ptr) *p.step_ptr = step + 1u;
     }
   }
+}
+
+// ------------------------------------------------------------------------------------ kernel: a block per row
+// STREAM: the instantiation launched for bf16 rows too long for the registers of a block (see long_statistics)
+template <typename T, int MAXT, bool STREAM = false>
+__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1) verify_rows_kernel(const VerifyParams p) {
+  extern __shared__ uint4 dyn_smem[];
+  __shared__ Scratch sc;
+  uint4 *stage = p.staged ? dyn_smem : nullptr;
+  pdl_trigger();
+  SJD_TL(TL_VERIFY, 0, threadIdx.x == 0);
+  pdl_wait();   // the logits come from the preceding kernel
+  SJD_TL(TL_VERIFY, 1, threadIdx.x == 0);
+
+  RowJob<T> j;
+  if (row_job<T>(p, blockIdx.x, j)) {
+    RowOut fast_out;
+    const bool fast_done = p.fast && (((uintptr_t)j.rows.q | (uintptr_t)j.rows.p) & 15u) == 0 &&
+                           fast_row<T, STREAM>(p, sc, j.r, j.b, j.kind, j.d, j.qr, j.cur, j.rows, j.inv_t, j.u_acc, j.u_res, j.u_draft,
+                                               fast_out);
+    if (fast_done) {
+      if (threadIdx.x == 0) p.row_out[j.r] = fast_out;
+    } else {
+      general_row<T>(p, j, stage, sc);
+    }
+  }
+  ticket_and_slide<T>(p, j.b, j.step, j.cur, sc, [&]() {
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+      if (p.fast && p.defer_residual) deferred_residual_bf16<STREAM>(p, j.b, j.step, j.cur, sc);
+    }
+  });
+}
+
+// ------------------------------------------------------------------------------------ kernel: a thread-block cluster per row
+// For few rows (latency counts, most SMs would idle) and for every fp32 row: CS blocks hold a row and the row its draft was
+// drawn from in shared memory, a contiguous slice each, and meet in distributed shared memory: once for the maxima, once for
+// the histograms, once for the sums.  The threshold is exact: a histogram of the distances below the maximum in the top 16
+// bits of the key (as on the register route); for fp32 the entries in the bin found are then listed (usually some hundred)
+// and every block selects among their low 16 bits.  Bound by the chain of barriers, block scans and round trips (each about
+// a microsecond) and by instruction fetch: every phase runs once, so its loops are kept rolled.
+constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClVecs = 8, kClList = 4096;
+
+template <int CS>
+struct ClScratch {
+  alignas(16) uint32_t hist[2][4096];          // p row, q row
+  union {
+    uint32_t coarse[2][CS][kClThreads];        // sums of eight adjacent bins of every block
+    unsigned short list[2][kClList];           // then, fp32: low 16 bits of the keys in the threshold's bin
+  };
+  double part[2][CS];                          // sums of the blocks' slices
+  double wsum[2][kClWarps];
+  uint32_t kmax[2][CS], bad[CS];
+  uint32_t scan[2][kClWarps], redu[2][kClWarps];
+  uint32_t sel_bin[2], sel_above[2], n_list[2], hist16[2][16];
+  float chunk_sum[kClWarps * kClVecs];
+  int tok[2];                                  // redraft, resample: written in block 0's copy by the block that finds it
+  float tok_w;
+};
+
+__device__ __forceinline__ uint32_t cl_map(const void *p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ uint4 cl_load4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cl_store(uint32_t a, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void cl_store(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+template <int CS>
+__device__ __forceinline__ void cl_sync() {
+  if constexpr (CS == 1) {
+    __syncthreads();
+  } else {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
+// vector of the entries i0 .. of a row, in the vector space of the p row: whatever its alignment; outside the row -inf
+template <typename T>
+__device__ __forceinline__ uint4 cl_vec(const T *g, const T *g2, float gw, int i0, int V, bool aligned) {
+  using E = Elt<T>;
+  if (aligned && i0 >= 0 && i0 + E::VEC <= V) {
+    const uint4 c = __ldg(reinterpret_cast<const uint4 *>(g + i0));
+    if (!g2) return c;
+    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(g2 + i0));
+    uint4 o;
+#pragma unroll
+    for (int t = 0; t < E::VEC; ++t) {
+      const float cf = E::val(E::get(c, t)), uf = E::val(E::get(u, t));
+      if (t % (E::VEC / 4) == 0 && E::VEC == 8) reinterpret_cast<uint32_t *>(&o)[t / 2] = 0u;
+      E::set(o, t, E::bits(fmaf(gw, cf - uf, uf)));
+    }
+    return o;
+  }
+  uint4 v = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int t = 0; t < E::VEC; ++t) {
+    const int i = i0 + t;
+    uint32_t b = E::NEG_INF;
+    if (i >= 0 && i < V) {
+      b = E::load_bits(g + i);
+      if (g2) {
+        const float cf = E::val(b), uf = E::val(E::load_bits(g2 + i));
+        b = E::bits(fmaf(gw, cf - uf, uf));
+      }
+    }
+    E::set(v, t, b);
+  }
+  return v;
+}
+
+// Block-wide: the thread whose eight bins hold the K-th entry (own: the entries in a thread's bins); `fine(x)` of that thread
+// picks the bin.  Two block barriers; sel_bin 4096 where K is not reached.
+template <int CS, typename F>
+__device__ __forceinline__ void cl_scan(ClScratch<CS> &cs, bool second, const uint32_t *own, const uint32_t *K, const F &fine) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t incl[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    uint32_t t = own[x];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    incl[x] = t;
+    if (lane == 31) cs.scan[x][warp] = t;
+  }
+  if (tid < 2) cs.sel_bin[tid] = 4096u;
+  __syncthreads();
+#pragma unroll 1
+  for (int x = 0; x < (second ? 2 : 1); ++x) {
+    const uint32_t t = x ? incl[1] : incl[0], o = x ? own[1] : own[0], k = x ? K[1] : K[0];
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? cs.scan[x][lane] : 0u);
+    uint32_t acc = before + t - o;
+    if (acc < k && k <= acc + o) {
+      const uint4 a = fine(x, 0), b = fine(x, 1);
+      const uint32_t c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (acc < k && k <= acc + c[i]) {
+          cs.sel_bin[x] = (uint32_t)(tid * 8 + i);
+          cs.sel_above[x] = acc;
+        }
+        acc += c[i];
+      }
+    }
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ uint4 add4(const uint4 &a, const uint4 &b) { return make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ uint32_t sum4(const uint4 &a) { return a.x + a.y + a.z + a.w; }
+
+// The histograms are complete in this block (a barrier ago): the bin, counted from bin 0, that holds the K-th entry of a row
+// over all blocks, and the entries before it.  One cluster barrier; every block finds it for itself.
+template <int CS>
+__device__ __forceinline__ void cl_find(ClScratch<CS> &cs, int rank, bool second, const uint32_t *K) {
+  const int tid = threadIdx.x;
+  uint32_t own[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const uint4 *h = reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8]);
+    own[x] = sum4(h[0]) + sum4(h[1]);
+    if constexpr (CS > 1) {
+#pragma unroll
+      for (int r = 0; r < CS; ++r) cl_store(cl_map(&cs.coarse[x][rank][tid], r), own[x]);
+    }
+  }
+  if constexpr (CS > 1) {
+    cl_sync<CS>();
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      own[x] = 0;
+#pragma unroll
+      for (int r = 0; r < CS; ++r) own[x] += cs.coarse[x][r][tid];
+    }
+  }
+  cl_scan<CS>(cs, second, own, K, [&](int x, int half) {
+    uint4 t = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int r = 0; r < CS; ++r) {
+      if constexpr (CS == 1) t = *reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8 + half * 4]);
+      else t = add4(t, cl_load4(cl_map(&cs.hist[x][tid * 8 + half * 4], r)));
+    }
+    return t;
+  });
+}
+
+// Sums of the slices' weights, chunk by chunk in token order: this block's chunk sums in cs.chunk_sum (of row x = 0 when
+// `chunks`), its total in part[x] of every block.  A cluster barrier completes it (the caller's).
+template <int CS, typename F>
+__device__ __forceinline__ void cl_sums(ClScratch<CS> &cs, int x, int ni, int rank, bool chunks, const F &wf) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double tot = 0.0;
+#pragma unroll 2
+  for (int i = 0; i < ni; ++i) {
+    const float t = warp_sum(wf(i));
+    if (chunks && lane == 0) cs.chunk_sum[warp * ni + i] = t;
+    tot += (double)t;
+  }
+  if (lane == 0) cs.wsum[x][warp] = tot;
+  __syncthreads();
+  if (tid < CS) {
+    double t = 0.0;
+    for (int w = 0; w < kClWarps; ++w) t += cs.wsum[x][w];
+    if constexpr (CS == 1) cs.part[x][0] = t;
+    else cl_store(cl_map(&cs.part[x][rank], tid), t);
+  }
+}
+
+// Inverse CDF over row x = 0's sums (same rules as sample_icdf): the block whose slice holds the target finds the token and
+// stores it in block 0's cs.tok[which] (and its weight).  No barrier.
+template <typename T, int CS, typename F>
+__device__ __forceinline__ void cl_icdf(ClScratch<CS> &cs, int which, int ni, int rank, int vec0, int off, float u, const F &wf) {
+  using E = Elt<T>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double total = 0.0, base = 0.0;
+  int hit = -1, last = -1;
+  double base_last = 0.0;
+  for (int r = 0; r < CS; ++r) total += cs.part[0][r];
+  const double target = (double)u * total;
+  double run = 0.0;
+  for (int r = 0; r < CS; ++r) {
+    const double t = cs.part[0][r], nxt = run + t;
+    if (t > 0.0) {
+      if (hit < 0 && run <= target && target < nxt) {
+        hit = r;
+        base = run;
+      }
+      last = r;
+      base_last = run;
+    }
+    run = nxt;
+  }
+  bool fallback = hit < 0;
+  const int owner = fallback ? (last < 0 ? 0 : last) : hit;
+  if (fallback) base = base_last;
+  if (rank != owner) return;
+  auto publish = [&](int tok, float w) {
+    if constexpr (CS == 1) {
+      cs.tok[which] = tok;
+      if (which == 0) cs.tok_w = w;
+    } else {
+      cl_store(cl_map(&cs.tok[which], 0), (uint32_t)tok);
+      if (which == 0) cl_store(cl_map(&cs.tok_w, 0), __float_as_uint(w));
+    }
+  };
+  if (last < 0) {   // no mass at all
+    if (tid == 0) publish(0, 0.0f);
+    return;
+  }
+  // every warp: the owning block's warps in order, then the chunks of the warp that holds the target
+  int c = -1, wl = -1;
+  double at = base, c_base = 0.0, l_base = 0.0;
+  int cl = -1;
+  for (int w = 0; w < kClWarps; ++w) {
+    const double t = cs.wsum[0][w];
+    if (t > 0.0) {
+      if (!fallback && c < 0 && target < at + t) {
+        c = w;
+        c_base = at;
+      }
+      wl = w;
+      l_base = at;
+    }
+    at += t;
+  }
+  if (c < 0) {   // rounding at the end of the slice: its last warp with mass
+    fallback = true;
+    c = wl;
+    c_base = l_base;
+  }
+  if (warp != c) return;
+  at = c_base;
+  int chunk = -1;
+  double chunk_base = 0.0, cl_base = 0.0;
+  for (int i = 0; i < ni; ++i) {
+    const float t = cs.chunk_sum[warp * ni + i];
+    if (t > 0.0f) {
+      if (!fallback && chunk < 0 && target < at + (double)t) {
+        chunk = i;
+        chunk_base = at;
+      }
+      cl = i;
+      cl_base = at;
+    }
+    at += (double)t;
+  }
+  bool take_last = fallback;
+  if (chunk < 0) {
+    chunk = cl;
+    chunk_base = cl_base;
+    take_last = true;
+  }
+  if (chunk < 0) return;
+  float w[E::VEC], sum = 0.0f;
+  wf(chunk, w);
+#pragma unroll
+  for (int t = 0; t < E::VEC; ++t) sum += w[t];
+  float incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+  if (lane == 0) excl = 0.0f;
+  const uint32_t ballot = __ballot_sync(0xffffffffu, !take_last && chunk_base + (double)incl > target && sum > 0.0f);
+  const uint32_t pos = __ballot_sync(0xffffffffu, sum > 0.0f);
+  const int sel = ballot ? __ffs(ballot) - 1 : pos ? 31 - __clz(pos) : 0;
+  if (lane == sel) {
+    double acc = chunk_base + (double)excl;
+    int found = -1, lt = 0;
+#pragma unroll
+    for (int t = 0; t < E::VEC; ++t) {
+      if (w[t] > 0.0f) {
+        acc += (double)w[t];
+        lt = t;
+        if (found < 0 && ballot && acc > target) found = t;
+      }
+    }
+    const int t_sel = found >= 0 ? found : lt;
+    float ws = 0.0f;
+#pragma unroll
+    for (int t = 0; t < E::VEC; ++t)
+      if (t == t_sel) ws = w[t];
+    publish((vec0 + (warp * ni + chunk) * 32 + lane) * E::VEC + t_sel - off, ws);
+  }
+}
+
+// largest key of a vector and whether it holds a NaN or +inf
+__device__ __forceinline__ void cl_max(const uint4 &v, float &mx, bool &bad, float) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const float f = __uint_as_float(word_of(v, t));
+    bad = bad || !(f < INFINITY);
+    mx = fmaxf(mx, f);
+  }
+}
+__device__ __forceinline__ void cl_max(const uint4 &v, float &mx, bool &bad, __nv_bfloat16) {
+  __nv_bfloat162 m = __hmax2_nan(__hmax2_nan(as_bf2(v.x), as_bf2(v.y)), __hmax2_nan(as_bf2(v.z), as_bf2(v.w)));
+  const float a = __low2float(m), b = __high2float(m);
+  bad = bad || !(a < INFINITY) || !(b < INFINITY);
+  mx = fmaxf(mx, fmaxf(a, b));
+}
+
+template <typename T, int CS>
+__device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch<CS> &cs, uint4 *slice, int rank) {
+  using E = Elt<T>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int V = p.V, d = j.d;
+  const int off = (int)(((uintptr_t)j.rows.p & 15u) / sizeof(T));
+  const int NV = (off + V + E::VEC - 1) / E::VEC;
+  const int ni = ((NV + CS - 1) / CS + kClThreads - 1) / kClThreads;    // chunks of 32 vectors per warp
+  const int vec0 = rank * ni * kClThreads;
+  const bool q_row = j.kind == SJD_Q_ROW, q_stat = q_row && !p.prev_stats_valid;
+  const bool need_select = p.top_k < V, d_ok = d >= 0 && d < V;
+  const bool aligned_p = !j.rows.p2 || (((uintptr_t)j.rows.p2 & 15u) == ((uintptr_t)j.rows.p & 15u));
+  const bool aligned_q = ((uintptr_t)j.rows.q & 15u) == ((uintptr_t)j.rows.p & 15u) &&
+                         (!j.rows.q2 || (((uintptr_t)j.rows.q2 & 15u) == ((uintptr_t)j.rows.p & 15u)));
+  const uint32_t fill = sizeof(T) == 4 ? E::NEG_INF : E::NEG_INF * 0x10001u;
+  // ---- both slices into shared memory (a thread reads back only what it wrote); the entries at the draft
+  uint4 *pv = slice + tid, *qv = slice + ni * kClThreads + tid;   // vector i of this thread: [i * kClThreads]
+  auto vec_index = [&](int i) { return vec0 + (warp * ni + i) * 32 + lane; };
+  auto fetch = [&](uint4 *dst, const T *g, const T *g2, int v, bool aligned) {
+    const int i0 = v * E::VEC - off;
+    if (v >= NV) *dst = make_uint4(fill, fill, fill, fill);
+    else if (aligned && !g2 && i0 >= 0 && i0 + E::VEC <= V)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(g + i0) : "memory");
+    else *dst = cl_vec<T>(g, g2, p.guidance, i0, V, aligned);
+  };
+#pragma unroll 1
+  for (int i = 0; i < ni; ++i) {
+    fetch(pv + i * kClThreads, j.rows.p, j.rows.p2, vec_index(i), aligned_p);
+    if (q_row) fetch(qv + i * kClThreads, j.rows.q, j.rows.q2, vec_index(i), aligned_q);
+  }
+  RowStats qs;
+  qs.tau_key = 0; qs.xmax = 0.0f; qs.z = 1.0f; qs.flags = 0;
+  if (q_row && !q_stat) qs = *j.rows.qstats;
+  uint32_t dp = E::NEG_INF, dq = E::NEG_INF;
+  if (d_ok) {
+    Row<T> r;
+    r.init(j.rows.p, V, j.rows.p2, p.guidance);
+    dp = r.raw_bits(d);
+    if (q_row) {
+      r.init(j.rows.q, V, j.rows.q2, p.guidance);
+      dq = r.raw_bits(d);
+    }
+  }
+  if (need_select)
+    for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 2) cs.n_list[tid] = 0;
+  if (tid < 32) cs.hist16[tid >> 4][tid & 15] = 0;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  float mx[2] = {-INFINITY, -INFINITY};
+  bool bad = false;
+#pragma unroll 1
+  for (int i = 0; i < ni; ++i) {
+    cl_max(pv[i * kClThreads], mx[0], bad, T());
+    if (q_row) cl_max(qv[i * kClThreads], mx[1], bad, T());
+  }
+  uint32_t km[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    km[x] = __reduce_max_sync(0xffffffffu, E::key(E::bits(mx[x])));
+    if (lane == 0) cs.redu[x][warp] = km[x];
+  }
+  const int any_bad = __syncthreads_or((int)bad);
+  if (warp < CS) {
+    const uint32_t a = __reduce_max_sync(0xffffffffu, lane < kClWarps ? cs.redu[0][lane] : 0u);
+    const uint32_t b = __reduce_max_sync(0xffffffffu, lane < kClWarps ? cs.redu[1][lane] : 0u);
+    if (lane == 0) {
+      if constexpr (CS == 1) {
+        cs.kmax[0][0] = a; cs.kmax[1][0] = b; cs.bad[0] = (uint32_t)any_bad;
+      } else {
+        cl_store(cl_map(&cs.kmax[0][rank], warp), a);
+        cl_store(cl_map(&cs.kmax[1][rank], warp), b);
+        cl_store(cl_map(&cs.bad[rank], warp), (uint32_t)any_bad);
+      }
+    }
+  }
+  cl_sync<CS>();
+  uint32_t not_ok = 0;
+  km[0] = km[1] = 0;
+#pragma unroll
+  for (int r = 0; r < CS; ++r) {
+    km[0] = max(km[0], cs.kmax[0][r]);
+    km[1] = max(km[1], cs.kmax[1][r]);
+    not_ok |= cs.bad[r];
+  }
+  const uint32_t key_ninf = E::key(E::NEG_INF);
+  if (not_ok || qs.flags != 0 || km[0] <= key_ninf || (q_stat && km[1] <= key_ninf) || (q_row && !q_stat && !(qs.xmax > -FLT_MAX)))
+    return false;   // the same in every block of the cluster
+
+  // ---- thresholds
+  uint32_t tau[2] = {0, 0};
+  if (need_select) {
+    constexpr int HI = E::KEYBITS - 16;   // bits below the top 16 of a key
+    uint32_t K[2] = {(uint32_t)p.top_k, (uint32_t)p.top_k};
+    const uint32_t top[2] = {km[0] >> HI, km[1] >> HI};
+#pragma unroll 1
+    for (int i = 0; i < ni; ++i) {
+      if (vec_index(i) >= NV) break;
+      const uint4 a = pv[i * kClThreads];
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) atomicAdd(&cs.hist[0][min(top[0] - (E::key(E::get(a, t)) >> HI), 4095u)], 1u);
+      if (q_stat) {
+        const uint4 b = qv[i * kClThreads];
+#pragma unroll
+        for (int t = 0; t < E::VEC; ++t) atomicAdd(&cs.hist[1][min(top[1] - (E::key(E::get(b, t)) >> HI), 4095u)], 1u);
+      }
+    }
+    __syncthreads();
+    cl_find<CS>(cs, rank, q_stat, K);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      if (x && !q_stat) break;
+      if (cs.sel_bin[x] >= 4095u) return false;   // too far below the maximum: the general route decides
+      tau[x] = (top[x] - cs.sel_bin[x]) << HI;
+      K[x] -= cs.sel_above[x];
+    }
+    if constexpr (HI == 16) {   // fp32: the entries in those bins are listed, then selected by their low 16 bits
+#pragma unroll 1
+      for (int i = 0; i < ni; ++i) {
+        const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
+#pragma unroll
+        for (int t = 0; t < E::VEC; ++t) {
+          const uint32_t ka = E::key(E::get(a, t)), kb = E::key(E::get(b, t));
+          if ((ka >> 16) == (tau[0] >> 16)) {
+            const uint32_t at = atomicAdd(&cs.n_list[0], 1u);
+            if (at < kClList) cs.list[0][at] = (unsigned short)ka;
+          }
+          if (q_stat && (kb >> 16) == (tau[1] >> 16)) {
+            const uint32_t at = atomicAdd(&cs.n_list[1], 1u);
+            if (at < kClList) cs.list[1][at] = (unsigned short)kb;
+          }
+        }
+      }
+      cl_sync<CS>();
+      for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+      bool over = false;
+      // low 16 bits of entry e of block r's list of row x; f(value)
+      auto for_list = [&](int x, auto f) {
+#pragma unroll 1
+        for (int r = 0; r < CS; ++r) {
+          uint32_t n;
+          if constexpr (CS == 1) n = cs.n_list[x];
+          else asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(cl_map(&cs.n_list[x], r)) : "memory");
+          over = over || n > (uint32_t)kClList;
+          n = min(n, (uint32_t)kClList);
+          const uint32_t base = CS == 1 ? 0u : cl_map(cs.list[x], r);
+          for (uint32_t e = tid; e < n; e += kClThreads) {
+            unsigned short v;
+            if constexpr (CS == 1) v = cs.list[x][e];
+            else asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(base + e * 2) : "memory");
+            f((uint32_t)v);
+          }
+        }
+      };
+#pragma unroll 1
+      for (int x = 0; x < (q_stat ? 2 : 1); ++x) for_list(x, [&](uint32_t v) { atomicAdd(&cs.hist[x][4095u - (v >> 4)], 1u); });
+      __syncthreads();
+      if (over) return false;   // (the same everywhere) more entries than the list holds
+      uint32_t own[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const uint4 *h = reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8]);
+        own[x] = sum4(h[0]) + sum4(h[1]);
+      }
+      cl_scan<CS>(cs, q_stat, own, K, [&](int x, int half) { return *reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8 + half * 4]); });
+      uint32_t mid[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        mid[x] = 4095u - cs.sel_bin[x];
+        K[x] -= cs.sel_above[x];
+      }
+#pragma unroll 1
+      for (int x = 0; x < (q_stat ? 2 : 1); ++x) {
+        const uint32_t m = x ? mid[1] : mid[0];
+        for_list(x, [&](uint32_t v) { if ((v >> 4) == m) atomicAdd(&cs.hist16[x][15u - (v & 15u)], 1u); });
+      }
+      __syncthreads();
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (x && !q_stat) break;
+        uint32_t acc = 0, low = 0;
+        for (int i = 0; i < 16; ++i) {
+          acc += cs.hist16[x][i];
+          if (acc >= K[x]) {
+            low = 15u - i;
+            break;
+          }
+        }
+        tau[x] |= mid[x] << 4 | low;
+      }
+    }
+  }
+  // ---- denominators: weights 2^((x - max) * scale) of the entries at or above the threshold
+  const float scale = j.inv_t * 1.4426950408889634f;
+  RowStats ps;
+  ps.tau_key = tau[0];
+  ps.xmax = E::val(E::unkey(km[0]));
+  ps.flags = 0;
+  if (q_stat) {
+    qs.tau_key = tau[1];
+    qs.xmax = E::val(E::unkey(km[1]));
+  }
+  auto weight = [&](uint32_t bits, uint32_t tau_key, float xmax) {
+    return E::key(bits) >= tau_key ? exp2_neg((E::val(bits) - xmax) * scale) : 0.0f;
+  };
+  auto p_w = [&](int i, float *w) {
+    const uint4 v = pv[i * kClThreads];
+#pragma unroll
+    for (int t = 0; t < E::VEC; ++t) w[t] = weight(E::get(v, t), ps.tau_key, ps.xmax);
+  };
+  auto sum_of = [](const float *w) {
+    float t = 0.0f;
+#pragma unroll
+    for (int e = 0; e < E::VEC; ++e) t += w[e];
+    return t;
+  };
+  if (q_stat)
+    cl_sums<CS>(cs, 1, ni, rank, false, [&](int i) {
+      float w[E::VEC];
+      const uint4 v = qv[i * kClThreads];
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) w[t] = weight(E::get(v, t), qs.tau_key, qs.xmax);
+      return sum_of(w);
+    });
+  cl_sums<CS>(cs, 0, ni, rank, true, [&](int i) {
+    float w[E::VEC];
+    p_w(i, w);
+    return sum_of(w);
+  });
+  cl_sync<CS>();
+  double zp = 0.0, zq = 0.0;
+#pragma unroll
+  for (int r = 0; r < CS; ++r) {
+    zp += cs.part[0][r];
+    if (q_stat) zq += cs.part[1][r];
+  }
+  ps.z = (float)zp;
+  if (q_stat) qs.z = (float)zq;
+  if (rank == 0 && tid == 0) {
+    p.stats[j.cur][j.r] = ps;
+    if (q_stat) p.stats[j.cur ^ 1][j.r] = qs;
+  }
+  // ---- Eq. 1
+  const float p_d = d_ok ? weight(dp, ps.tau_key, ps.xmax) / ps.z : 0.0f;
+  float q_d = 1.0f;
+  if (q_row) q_d = d_ok ? weight(dq, qs.tau_key, qs.xmax) / qs.z : 1.0f;
+  else if (j.kind == SJD_Q_UNIFORM) q_d = 1.0f / (float)V;
+  float ratio;
+  if (q_d > 0.0f) ratio = p_d / q_d;
+  else ratio = p_d > 0.0f ? INFINITY : 0.0f;
+  float thr = fminf(1.0f, ratio);
+  bool accept = j.u_acc < thr;
+  uint32_t flags = 0;
+  if (thr < 1.0f && fabsf(j.u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
+  // ---- Eq. 3
+  cl_icdf<T, CS>(cs, 0, ni, rank, vec0, off, j.u_draft, p_w);
+  // ---- Eq. 2
+  int resample = accept ? -1 : kResampleDeferred;
+  const bool residual = !accept && !p.defer_residual && !j.jacobi;
+  if (residual) {
+    cl_sync<CS>();   // every block has read the sums
+    const float ip = 1.0f / ps.z, iq = 1.0f / qs.z, qu = 1.0f / (float)V;
+    auto r_w = [&](int i, float *w) {
+      const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
+      const int i0 = (vec0 + (warp * ni + i) * 32 + lane) * E::VEC - off;
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) {
+        // both products rounded: contracted into the difference, equal rows would leave rounding residue instead of zero
+        const float pp = __fmul_rn(weight(E::get(a, t), ps.tau_key, ps.xmax), ip);
+        const float qq = q_row ? __fmul_rn(weight(E::get(b, t), qs.tau_key, qs.xmax), iq) : j.kind == SJD_Q_UNIFORM ? qu : i0 + t == d ? 1.0f : 0.0f;
+        w[t] = fmaxf(0.0f, pp - qq);
+      }
+    };
+    cl_sums<CS>(cs, 0, ni, rank, true, [&](int i) {
+      float w[E::VEC];
+      r_w(i, w);
+      return sum_of(w);
+    });
+    cl_sync<CS>();
+    double zr = 0.0;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) zr += cs.part[0][r];
+    if (zr > 0.0) {
+      cl_icdf<T, CS>(cs, 1, ni, rank, vec0, off, j.u_res, r_w);
+    } else {
+      flags |= SJD_FLAG_RESIDUAL_EMPTY;
+      cl_sync<CS>();
+      cl_sums<CS>(cs, 0, ni, rank, true, [&](int i) {
+        float w[E::VEC];
+        p_w(i, w);
+        return sum_of(w);
+      });
+      cl_sync<CS>();
+      cl_icdf<T, CS>(cs, 1, ni, rank, vec0, off, j.u_res, p_w);
+    }
+  }
+  cl_sync<CS>();   // the tokens are in block 0; nobody reads another block's memory from here on
+  if (rank == 0 && tid == 0) {
+    RowOut ro;
+    ro.redraft_tok = cs.tok[0];
+    ro.redraft_p = cs.tok_w / ps.z;
+    if (residual) resample = cs.tok[1];
+    if (j.jacobi) {   // deterministic criterion instead of Eqs. 1-2
+      accept = d_ok && ro.redraft_tok == d;
+      thr = accept ? 1.0f : 0.0f;
+      flags = 0;
+      resample = accept ? -1 : ro.redraft_tok;
+    }
+    ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
+    ro.resample_tok = resample;
+    ro.flags = flags;
+    p.row_out[j.r] = ro;
+  }
+  return true;
+}
+
+template <typename T, int CS>
+__global__ void __launch_bounds__(kClThreads, 2) verify_cluster_kernel(const VerifyParams p) {
+  extern __shared__ uint4 dyn_smem[];
+  ClScratch<CS> &cs = *reinterpret_cast<ClScratch<CS> *>(dyn_smem);
+  __shared__ Scratch sc;
+  pdl_trigger();
+  cl_sync<CS>();   // every block of the cluster has started: its shared memory may be written
+  pdl_wait();
+  const int rank = (int)(blockIdx.x % CS);
+  RowJob<T> j;
+  if (row_job<T>(p, (int)(blockIdx.x / CS), j)) {
+    const bool done = cluster_row<T, CS>(p, j, cs, dyn_smem + (sizeof(ClScratch<CS>) + 15) / 16, rank);
+    if (!done) {
+      cl_sync<CS>();   // no block leaves while another may still store into it
+      if (rank == 0) general_row<T>(p, j, nullptr, sc);
+    }
+  }
+  if (rank != 0) return;
+  ticket_and_slide<T>(p, j.b, j.step, j.cur, sc, [&]() {
+    if (!p.defer_residual) return;
+    // the first rejected row of the sequence, if it left Eq. 2 open
+    const int w_eff = p.w_eff ? p.w_eff[p.paired ? 2 * j.b : j.b] : p.W;
+    RowOut *ro = p.row_out + (size_t)j.b * p.W;
+    if (threadIdx.x < 32) {
+      int first = w_eff;
+      for (int k = threadIdx.x; k < w_eff; k += 32)
+        if (!__ldcg(&ro[k].accept)) first = min(first, k);
+      first = __reduce_min_sync(0xffffffffu, first);
+      if (threadIdx.x == 0) sc.sel_chunk = (first < w_eff && __ldcg(&ro[first].resample_tok) == kResampleDeferred) ? first : -1;
+    }
+    __syncthreads();
+    const int a = sc.sel_chunk;
+    __syncthreads();
+    if (a < 0) return;
+    RowJob<T> f;
+    row_job<T>(p, j.b * p.W + a, f);
+    auto stats = [](const RowStats *g) {
+      const uint4 u = __ldcg(reinterpret_cast<const uint4 *>(g));
+      RowStats st;
+      st.tau_key = u.x; st.xmax = __uint_as_float(u.y); st.z = __uint_as_float(u.z); st.flags = u.w;
+      return st;
+    };
+    const RowStats ps = stats(&p.stats[f.cur][f.r]);
+    RowStats qs = ps;
+    qs.z = 1.0f;
+    if (f.kind == SJD_Q_ROW) qs = stats(f.rows.qstats);
+    ResidualWeights<T> rf;
+    rf.prow.init(f.rows.p, p.V, f.rows.p2, p.guidance);
+    rf.qrow.init(f.rows.q, p.V, f.rows.q2, p.guidance);
+    rf.pw.init(ps, f.inv_t);
+    rf.qw.init(qs, f.inv_t);
+    rf.inv_zp = 1.0f / ps.z; rf.inv_zq = 1.0f / qs.z;
+    rf.kind = f.kind; rf.draft = f.d; rf.V = p.V;
+    PRowWeights<T> pf;
+    pf.row = rf.prow;
+    pf.pw = rf.pw;
+    uint32_t flags = 0;
+    general_residual<T>(rf, pf, f.u_res, sc, flags);
+    if (threadIdx.x == 0) {
+      ro[a].resample_tok = sc.tok;
+      ro[a].flags = __ldcg(&ro[a].flags) | flags;
+      __threadfence();
+    }
+    __syncthreads();
+  });
 }
 
 // Sec. 4.2 (d): keep the rows of the window just verified (as the verification saw them: mixed under
@@ -1764,12 +2504,65 @@ size_t verify_scratch_bytes(int batch, int window) {
   return (b + 255) / 256 * 256;
 }
 
+static int sm_count() {
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 148;
+  return v;
+}
+
+template <typename T, int CS>
+static int launch_cluster(const VerifyParams &p, long nv, cudaStream_t stream) {
+  auto kernel = verify_cluster_kernel<T, CS>;
+  const long ni = ((nv + CS - 1) / CS + kClThreads - 1) / kClThreads;
+  const size_t smem = (sizeof(ClScratch<CS>) + 15) / 16 * 16 + (size_t)2 * ni * kClThreads * 16;
+  SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(p.B * p.W * CS);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CS;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = g_pdl ? 2 : 1;
+  SJD_CUDA(cudaLaunchKernelEx(&cfg, kernel, p));
+  SJD_CHECK_LAUNCH();
+  return SJD_OK;
+}
+
 template <typename T>
 static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
   VerifyParams p = p_in;
   constexpr int VEC = Elt<T>::VEC;
   const long nv_max = ((long)p.V + 2 * VEC - 2) / VEC + 1;
   if ((nv_max + 31) / 32 > kMaxChunks) return SJD_ERR_CAPACITY;
+  // A cluster per row, with as many blocks as the rows leave SMs for: whenever the grid is resident at once (us a call, block per
+  // row -> cluster: fp32 1 x 27 x 65536 155 -> 40, 1 x 16 x 1024 24.7 -> 18.5; bf16 1 x 32 x 65536 40 -> 29, 3 x 16 x 4096 24.6 ->
+  // 18.5, 4 x 32 x 16384 26.7 -> 24.7), and for fp32 rows of more than 2048 entries in any number (8 x 32 x 16384 67 -> 56,
+  // 32 x 32 x 16384 180 -> 149, 26 x 33 x 4096 60 -> 55).  bf16 rows in several waves are better off a block per row
+  // (1 x 64 x 184320: 89 against 157 us), and so are short fp32 rows (32 x 18 x 1096: 31 against 36 us).
+  const int n_sms = sm_count();
+  {
+    const bool whole = p.V % VEC == 0 && ((uintptr_t)p.logits[0] & 15u) == 0;   // every row starts on a vector
+    const long nv = whole ? p.V / VEC : nv_max;
+    int cs = 1;
+    while (cs < 8 && (long)cs * kClThreads * kClVecs < nv) cs *= 2;
+    const bool fits = (long)cs * kClThreads * kClVecs >= nv;
+    while (cs < 8 && p.B * p.W * cs * 2 <= n_sms && nv > (long)cs * kClThreads) cs *= 2;
+    const bool few = (long)p.B * p.W * cs <= n_sms;
+    const bool wide = std::is_same<T, float>::value && nv > kClThreads;
+    if (fits && (few || wide)) {
+      p.staged = p.fast = 0;
+      p.defer_residual = p.B * p.W * cs > n_sms ? 1 : 0;
+      return cs == 1 ? launch_cluster<T, 1>(p, nv, stream) : cs == 2 ? launch_cluster<T, 2>(p, nv, stream)
+             : cs == 4 ? launch_cluster<T, 4>(p, nv, stream) : launch_cluster<T, 8>(p, nv, stream);
+    }
+  }
   const size_t stage_bytes = (size_t)nv_max * 16;
   p.staged = stage_bytes <= 160 * 1024 ? 1 : 0;
   int threads = nv_max <= 1024 ? 128 : nv_max <= 4096 ? 256 : nv_max <= 16384 ? 512 : 1024;
@@ -1786,13 +2579,7 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
     // threshold out of the histogram's reach) re-reads global memory instead, and more blocks fit an SM
     p.staged = 0;
     // more blocks than can be resident at once: rejected rows leave the Eq. 2 draw to the sequence's last block
-    static int n_sms = 0;
-    if (n_sms == 0) {
-      int dev = 0, v = 0;
-      if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-        n_sms = v;
-    }
-    const int resident = (n_sms > 0 ? n_sms : 148) * (threads <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1);
+    const int resident = n_sms * (threads <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1);
     p.defer_residual = p.B * p.W > resident ? 1 : 0;
   }
   const size_t dyn = p.staged ? stage_bytes : 0;

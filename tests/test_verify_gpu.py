@@ -108,6 +108,28 @@ def test_verify_shapes(dtype, vocab, window, top_k):
     _check_case(case, max_flag_frac=0.06)
 
 
+@pytest.mark.parametrize("batch,window,vocab,dtype,top_k", [
+    (1, 3, 65537, "f32", 900),       # rows that start off 16 bytes, the last vector partly outside
+    (1, 2, 131056, "f32", 2000),     # close to the longest row: eight blocks, eight vectors per thread
+    (2, 2, 513, "f32", 1),           # two vectors past a block's first chunk row
+    (5, 32, 3000, "f32", 100),       # more rows than SMs: Eq. 2 left to the sequence's last block
+    (2, 5, 60001, "bf16", 700),      # bf16 rows at four alignments
+    (1, 3, 32776, "bf16", 40000),    # no filter (top-k above the vocabulary), odd tail
+])
+def test_verify_cluster_rows(batch, window, vocab, dtype, top_k):
+    """A thread-block cluster per row: slice sizes, alignments and the rules between it and a block per row."""
+    _check_case(make_verify_case(batch, window=window, vocab=vocab, dtype=dtype, top_k=top_k, mixed_kinds=True, seed=9))
+
+
+@pytest.mark.parametrize("levels", [3, 4000])
+def test_verify_cluster_ties(levels):
+    """fp32 rows of few distinct values: thousands of entries tie at the threshold (more than a block lists at 3 levels)."""
+    case = make_verify_case(1, window=3, vocab=40000, dtype="f32", top_k=1500, seed=11)
+    for rows in (case.logits_cur, case.logits_prev):
+        rows[...] = np.floor(rows * (levels / 60.0)) * np.float32(60.0 / levels)
+    _check_case(case)
+
+
 def test_verify_mixed_laws():
     """Slots whose draft came from a uniform initialisation (q = 1/V) or a copy (point mass)."""
     case = make_verify_case(6, window=16, vocab=4096, top_k=300, seed=11, mixed_kinds=True)
