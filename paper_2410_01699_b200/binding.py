@@ -234,7 +234,7 @@ def sjd_gemm(x, w, out=None, accumulate=False):
     m, k = x.shape
     n = w.shape[0]
     if out is None:
-        out = torch.zeros(m, n, dtype=torch.float32, device=x.device)
+        out = (torch.zeros if accumulate else torch.empty)(m, n, dtype=torch.float32, device=x.device)
     nbytes = int(lib().sjd_gemm_workspace_bytes(m, n, k))
     if nbytes == 0:
         raise SJDError(SJD_ERR_UNSUPPORTED, "sjd_gemm_workspace_bytes")

@@ -110,7 +110,7 @@ constexpr int kGemmSmsMax = 160;
 extern "C" size_t sjd_gemm_workspace_bytes(int M, int N, int K) {
   if (!gemm_tc_supported(M, N, K)) return 0;
   const int mp = (M + 15) / 16 * 16;
-  const int splits = gemm_tc_splits(gemm_tc_plan(M), N / 128, K / 64, kGemmSmsMax);
+  const int splits = gemm_tc_splits_max(gemm_tc_plan(M), N / 128, K / 64);
   return 256 + up256((size_t)splits * M * N * 4) + up256((size_t)2 * mp * K * 2);
 }
 
@@ -130,14 +130,13 @@ extern "C" int sjd_gemm(int M, int N, int K, const float *x, const void *w, floa
   const int mp = (M + 15) / 16 * 16;
   const GemmTcPlan plan = gemm_tc_plan(M);
   const int splits = gemm_tc_splits(plan, N / 128, K / 64, sms);
-  const int splits_max = gemm_tc_splits(plan, N / 128, K / 64, kGemmSmsMax);
+  const int splits_max = gemm_tc_splits_max(plan, N / 128, K / 64);
   char *p = (char *)ws;
   int *status = (int *)p;
   float *planes = (float *)(p + 256);
   __nv_bfloat16 *xs = (__nv_bfloat16 *)(p + 256 + up256((size_t)splits_max * M * N * 4));
-  SJD_CUDA(cudaMemsetAsync(p, 0, 256, stream));
-  SJD_CUDA(cudaMemsetAsync(xs, 0, (size_t)2 * mp * K * 2, stream));
-  int rc = launch_split_hilo(x, HiLoOut{xs, (size_t)mp * K}, (size_t)M * K, stream);
+  // (token rows past M stay as they are: a row of x reaches its own output row only)
+  int rc = launch_split_hilo(x, HiLoOut{xs, (size_t)mp * K}, (size_t)M * K, status, stream);
   if (rc != SJD_OK) return rc;
   TensorMap wm, xm;
   rc = make_tensor_map_bf16(&wm, w, N, K, 128);
@@ -154,15 +153,18 @@ extern "C" int sjd_gemm(int M, int N, int K, const float *x, const void *w, floa
   g.M = M;
   g.K = K;
   g.splits = splits;
-  g.out = planes;
+  const bool direct = splits == 1 && !accumulate;   // the product is the result: no plane, no sum
+  g.out = direct ? out : planes;
   g.plane_stride = (size_t)M * N;
   g.ldc = N;
   g.store_bf16 = 0;
   g.status = status;
   g.n_sms = sms;
+  g_pdl = true;   // each of the two launches waits for the one before it
   rc = launch_gemm_tc(g, stream);
-  if (rc != SJD_OK) return rc;
-  return launch_sum_planes(planes, (size_t)M * N, splits, out, (size_t)M * N, accumulate, stream);
+  if (rc == SJD_OK && !direct) rc = launch_sum_planes(planes, (size_t)M * N, splits, out, (size_t)M * N, accumulate, stream);
+  g_pdl = false;
+  return rc;
 }
 
 #ifdef SJD_TIMELINE

@@ -261,6 +261,9 @@ struct GemmTcPlan {
   int n_slabs, slab_rows;
 };
 GemmTcPlan gemm_tc_plan(int M);
+// more than 64 rows run on CTA pairs
+inline bool gemm_tc_pairs(const GemmTcPlan &pl) { return pl.n_slabs * pl.slab_rows > 64; }
+int gemm_tc_splits_max(const GemmTcPlan &pl, int tiles, int k_blocks);   // over every SM count that scratch is sized for
 int gemm_tc_splits(const GemmTcPlan &pl, int tiles, int k_blocks, int n_sms);   // tiles: 128-row weight tiles of the launch
 // One launch over up to three weight matrices that share the activation operand X (two bf16 planes:
 // hi at row 0, lo at row x_lo_row of x_map, each [rows][K]).  Matrix j has n_out[j] rows and writes
@@ -309,7 +312,7 @@ struct HiLoOut {
   size_t lo_offset;
 };
 
-int launch_split_hilo(const float *x, HiLoOut o, size_t total, cudaStream_t stream);
+int launch_split_hilo(const float *x, HiLoOut o, size_t total, int *status, cudaStream_t stream);   // also clears *status
 // consumer kernels of the tensor-core path (fused_kernels.cu)
 struct KvLayout;
 // partial sums of squares of the residual rows: scale(m) = 1/sqrt(sum_j ss_part[m][j] * inv_d + eps)

@@ -162,8 +162,7 @@ Layout make_layout(const sjd_model_cfg &c) {
     for (int i = 0; i < 3 && tc; ++i) {
       for (size_t rows = 16; rows < Mp + 16 && rows <= kMaxTcRows; rows += 16) {   // splits shrink as the token slabs grow
         const size_t m = rows < Mp ? rows : Mp;
-        const size_t n = (size_t)gemm_tc_splits(gemm_tc_plan((int)m), tiles[i] > 0 ? tiles[i] : 1, kbs[i],
-                                                 kMaxGemmCtas) * m * cols[i];
+        const size_t n = (size_t)gemm_tc_splits_max(gemm_tc_plan((int)m), tiles[i] > 0 ? tiles[i] : 1, kbs[i]) * m * cols[i];
         need = n > need ? n : need;
       }
     }

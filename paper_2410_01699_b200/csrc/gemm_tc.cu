@@ -1,15 +1,10 @@
 // Weight-streaming projection GEMM for sm_100a:  P[s][m][n] = sum_{k in split s} X[m][k] * W[n][k]
 // (Sec. 4.1 Step 2: the one forward pass over the window; every projection of the decoder).
 //
-// Shape of the problem: M = batch * window is 8..128 rows, the weight matrices (bf16) are tens to
+// Shape of the problem: M = batch * window is mostly 8..64 rows, the weight matrices (bf16) are tens to
 // hundreds of MB and are read exactly once per step, so the kernel is bound by HBM bandwidth and its
-// job is to keep every SM's TMA queue full.  Larger M (batches of images with wide windows, up to
-// 1024 rows) is cut into token slabs of at most 128 rows; the CTAs of the slabs of one weight tile
-// are neighbours in the grid, so the tile comes from HBM once and from L2 for the other slabs.  With
-// several slabs the kernel is bound by the tensor pipe (both activation planes are multiplied) and, in
-// this tiling, by shared-memory bandwidth: a 128 x 256 MMA tile moves 96 KB through shared memory per 512
-// tensor clocks.  (Measured and removed: two adjacent weight tiles per CTA against one activation tile,
-// 10-15 % slower than two independent CTAs per SM.)
+// job is to keep every SM's TMA queue full.  More rows (batches of images, pre-fill passes) run on CTA
+// pairs, see gemm_pair_kernel.
 //   * W is the 128-row operand of tcgen05.mma (M = 128), the tokens are the N dimension.  The fp32
 //     activations arrive split into two bf16 planes, hi = bf16(x) and lo = bf16(x - hi); both planes
 //     are columns of the same MMA (N = 2 * Mp), and the epilogue adds the two halves: activations keep
@@ -68,7 +63,7 @@ struct GemmParams {
   int ldc;
   int M;                  // valid token rows
   int Mp;                 // token rows of one slab, a multiple of 16 (MMA N = 2 * Mp: hi and lo plane)
-  int n_slabs;            // token slabs; CTA blockIdx.x = weight tile * n_slabs + slab
+  int n_slabs;            // token slabs (CTA pairs only: more than one)
   int x_lo_row;           // row of the lo plane inside the activation tensor map
   int k_blocks, splits;   // K / 64, K splits (gridDim.y)
   int tile_end[3];        // matrix j owns tiles [tile_end[j-1], tile_end[j])
@@ -125,6 +120,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
     if (global_ns() - t0 > kWaitNs) return false;
   }
 }
+
+// One lane of a converged warp.  The producer and issuer warps run converged and elect a lane for the copies and MMAs only:
+// their addresses and descriptors then stay in uniform registers (one lane running the whole loop is up to a quarter slower).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity)); }
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar,
                                             uint64_t policy) {
@@ -197,6 +201,32 @@ __device__ __forceinline__ bool epilogue_all(bool pred) {
   return r != 0;
 }
 
+// 16 tokens of one output column: out[i * ld] = hi[i] + lo[i] (times scale[i], if any), the first n of them.  Nothing but
+// independent adds and stores: an epilogue has a warp or two per scheduler, so every dependent instruction costs its latency
+// (with bounds, type and scale tested per element, 128 tokens took 7 us).
+template <typename O>
+__device__ __forceinline__ void store_column(O *out, size_t ld, const uint32_t *hi, const uint32_t *lo, const float *scale, int n) {
+  float v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+  if (scale) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] *= scale[i];
+  }
+  auto put = [&](int i) {
+    if constexpr (sizeof(O) == 2) out[i * ld] = __float2bfloat16_rn(v[i]);
+    else out[i * ld] = v[i];
+  };
+  if (n >= 16) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) put(i);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < n) put(i);
+  }
+}
+
 // ---------------------------------------------------------------------------------- kernel
 // GU: the gate|up launch that applies SwiGLU in its epilogue
 template <bool GU>
@@ -208,20 +238,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   __shared__ uint32_t s_tmem_base;
   __shared__ float s_scale[TILE_N];   // per-row output scales of this CTA's token slab (epilogue)
 
-  constexpr int WT = 1;   // weight tiles (accumulators) per CTA
-  constexpr int XP = 2;   // activation planes multiplied: hi and lo
   pdl_trigger();   // the next kernel in the stream may be scheduled as soon as every CTA got here
   SJD_TL(TL_GEMM, 0, threadIdx.x == 0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int unit = (int)blockIdx.x / p.n_slabs, split = blockIdx.y;
-  const int tile = unit * WT;                         // first weight tile of this CTA
-  const int m_base = ((int)blockIdx.x - unit * p.n_slabs) * p.Mp;   // first token row of this CTA's slab
-  const int NN = XP * p.Mp;                          // MMA N
+  const int tile = blockIdx.x, split = blockIdx.y;
+  constexpr int m_base = 0;   // one slab: more rows run on CTA pairs
+  const int NN = 2 * p.Mp;                           // MMA N
   const int x_tile_bytes = NN * TILE_K * 2;
-  const int w_bytes = WT * W_TILE_BYTES;
-  const int stage_bytes = w_bytes + x_tile_bytes;
+  const int stage_bytes = W_TILE_BYTES + x_tile_bytes;
   const int R = p.tile_rows;
-  const uint32_t stage_tx = (uint32_t)((GU ? 2 : WT) * R * TILE_K * 2 + x_tile_bytes);   // bytes the copies of a stage deliver
+  const uint32_t stage_tx = (uint32_t)((GU ? 2 : 1) * R * TILE_K * 2 + x_tile_bytes);   // bytes the copies of a stage deliver
   uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
 
   // which weight matrix this tile belongs to
@@ -234,7 +260,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   const int n_kb = kb_end - kb_begin;
 
   uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < WT * NN) tmem_cols <<= 1;
+  while ((int)tmem_cols < NN) tmem_cols <<= 1;
 
   if (tid == 0) {
     tma_prefetch_desc(w_map);
@@ -260,90 +286,82 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint64_t policy;
-      asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-      // The weights do not depend on the preceding kernel: fill the ring with W tiles right away,
-      // then wait for the predecessor before fetching the activation tiles it produced.
-      const int pre = n_kb < p.stages ? n_kb : p.stages;
-      for (int i = 0; i < pre; ++i) {
-        mbar_expect_tx(&bar_full[i], stage_tx);
-        if (GU) {
-          tma_load_2d(smem + i * stage_bytes, &w_map0, (kb_begin + i) * TILE_K, tile * R, &bar_full[i], policy);
-          tma_load_2d(smem + i * stage_bytes + W_TILE_BYTES / 2, &w_map1, (kb_begin + i) * TILE_K, tile * R, &bar_full[i],
-                      policy);
-        } else {
-#pragma unroll
-          for (int j = 0; j < WT; ++j)
-            tma_load_2d(smem + i * stage_bytes + j * W_TILE_BYTES, w_map, (kb_begin + i) * TILE_K, (tile_in_mat + j) * R,
-                        &bar_full[i], policy);
-        }
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    auto load_w = [&](int kcol, int s) {
+      uint8_t *dst = smem + s * stage_bytes;
+      mbar_expect_tx(&bar_full[s], stage_tx);
+      if (GU) {
+        tma_load_2d(dst, &w_map0, kcol, tile * R, &bar_full[s], policy);
+        tma_load_2d(dst + W_TILE_BYTES / 2, &w_map1, kcol, tile * R, &bar_full[s], policy);
+      } else {
+        tma_load_2d(dst, w_map, kcol, tile_in_mat * R, &bar_full[s], policy);
       }
-      SJD_TL(TL_GEMM, 3, true);
-      pdl_wait();
-      SJD_TL(TL_GEMM, 1, true);
-      for (int i = 0; i < pre; ++i) {
-        uint8_t *dst = smem + i * stage_bytes;
-        const int kcol = (kb_begin + i) * TILE_K;
-        tma_load_2d_nohint(dst + w_bytes, &x_map, kcol, m_base, &bar_full[i]);
-        if (XP == 2)
-          tma_load_2d_nohint(dst + w_bytes + x_tile_bytes / 2, &x_map, kcol, p.x_lo_row + m_base, &bar_full[i]);
+    };
+    auto load_x = [&](int kcol, int s) {
+      uint8_t *dst = smem + s * stage_bytes + W_TILE_BYTES;
+      tma_load_2d_nohint(dst, &x_map, kcol, m_base, &bar_full[s]);
+      tma_load_2d_nohint(dst + x_tile_bytes / 2, &x_map, kcol, p.x_lo_row + m_base, &bar_full[s]);
+    };
+    // The weights do not depend on the preceding kernel: fill the ring with W tiles right away,
+    // then wait for the predecessor before fetching the activation tiles it produced.
+    const int pre = n_kb < p.stages ? n_kb : p.stages;
+    for (int i = 0; i < pre; ++i) {
+      if (elect_one()) load_w((kb_begin + i) * TILE_K, i);
+      __syncwarp();
+    }
+    SJD_TL(TL_GEMM, 3, lane == 0);
+    pdl_wait();
+    SJD_TL(TL_GEMM, 1, lane == 0);
+    for (int i = 0; i < pre; ++i) {
+      if (elect_one()) load_x((kb_begin + i) * TILE_K, i);
+      __syncwarp();
+    }
+    int s = pre == p.stages ? 0 : pre;
+    uint32_t ph = pre == p.stages ? 1u : 0u;
+    bool ok = true;
+    int it = pre;
+    for (; it < n_kb; ++it) {
+      if (!warp_wait(&bar_empty[s], ph ^ 1u)) { ok = false; break; }
+      if (elect_one()) {
+        load_w((kb_begin + it) * TILE_K, s);
+        load_x((kb_begin + it) * TILE_K, s);
       }
-      int s = pre == p.stages ? 0 : pre;
-      uint32_t ph = pre == p.stages ? 1u : 0u;
-      bool ok = true;
-      int it = pre;
-      for (; it < n_kb; ++it) {
-        if (!mbar_wait(&bar_empty[s], ph ^ 1u)) { ok = false; break; }
-        uint8_t *dst = smem + s * stage_bytes;
-        const int kcol = (kb_begin + it) * TILE_K;
-        mbar_expect_tx(&bar_full[s], stage_tx);
-        if (GU) {
-          tma_load_2d(dst, &w_map0, kcol, tile * R, &bar_full[s], policy);
-          tma_load_2d(dst + W_TILE_BYTES / 2, &w_map1, kcol, tile * R, &bar_full[s], policy);
-        } else {
-#pragma unroll
-          for (int j = 0; j < WT; ++j)
-            tma_load_2d(dst + j * W_TILE_BYTES, w_map, kcol, (tile_in_mat + j) * R, &bar_full[s], policy);
-        }
-        tma_load_2d_nohint(dst + w_bytes, &x_map, kcol, m_base, &bar_full[s]);
-        if (XP == 2)
-          tma_load_2d_nohint(dst + w_bytes + x_tile_bytes / 2, &x_map, kcol, p.x_lo_row + m_base, &bar_full[s]);
-        if (++s == p.stages) { s = 0; ph ^= 1u; }
-      }
-      if (!ok) {
-        atomicExch(p.status, 1);
-        // leave no copy in flight: wait (bounded) for the stages armed most recently
-        const int armed = it < p.stages ? it : p.stages;
-        for (int j = it - armed; j < it; ++j) mbar_wait(&bar_full[j % p.stages], (uint32_t)((j / p.stages) & 1));
-      }
+      __syncwarp();
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
+    }
+    if (!ok) {
+      if (lane == 0) atomicExch(p.status, 1);
+      // leave no copy in flight: wait (bounded) for the stages armed most recently
+      const int armed = it < p.stages ? it : p.stages;
+      for (int j = it - armed; j < it; ++j) mbar_wait(&bar_full[j % p.stages], (uint32_t)((j / p.stages) & 1));
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(NN);
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int it = 0; it < n_kb; ++it) {
-        if (!mbar_wait(&bar_full[s], ph)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t a_addr = smem_u32(smem + s * stage_bytes);
-        const uint32_t b_addr = a_addr + w_bytes;
+    const uint32_t idesc = umma_idesc_bf16(NN);
+    const uint64_t desc0 = umma_desc_sw128(0);
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int it = 0; it < n_kb; ++it) {
+      if (!warp_wait(&bar_full[s], ph)) { ok = false; break; }
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t at = smem_u32(smem + s * stage_bytes);
+        const uint64_t a = desc0 | (uint64_t)(at >> 4), b = desc0 | (uint64_t)((at + W_TILE_BYTES) >> 4);
 #pragma unroll
-        for (int k = 0; k < TILE_K / UMMA_K; ++k) {
-          const uint64_t bdesc = umma_desc_sw128(b_addr + k * UMMA_K * 2);
-  #pragma unroll
-        for (int j = 0; j < WT; ++j)
-            umma_bf16(tmem_base + j * NN, umma_desc_sw128(a_addr + j * W_TILE_BYTES + k * UMMA_K * 2), bdesc, idesc,
-                      !(it == 0 && k == 0));
-        }
+        for (int k = 0; k < TILE_K / UMMA_K; ++k) umma_bf16(tmem_base, a + k * 2, b + k * 2, idesc, !(it == 0 && k == 0));
         umma_commit(&bar_empty[s]);   // frees the stage once these MMAs have read it
-        if (++s == p.stages) { s = 0; ph ^= 1u; }
       }
-      if (ok) umma_commit(&bar_acc_full);
-      else atomicExch(p.status, 2);
+      __syncwarp();
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
     }
+    if (ok) {
+      if (elect_one()) umma_commit(&bar_acc_full);
+    } else if (lane == 0) {
+      atomicExch(p.status, 2);
+    }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue warps (2..5)
     const int quarter = warp & 3;                 // TMEM lane quarter this warp may read
@@ -388,43 +406,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
         const int e = tid - 64, fr = e & 63;
         const int f = tile * R + fr;
         if (fr < R && f < p.F) {
-          for (int mm = e >> 6; mm < p.Mp; mm += 2) {
-            const int m = m_base + mm;
-            if (m >= p.M) break;
+#pragma unroll 8
+          for (int mm = e >> 6; mm < p.M; mm += 2) {
             const float g = ex[fr * ldx + mm], u = ex[(64 + fr) * ldx + mm];
             const float v = g / (1.0f + expf(-g)) * u;
             const __nv_bfloat16 vh = __float2bfloat16_rn(v);
-            p.act_hi[(size_t)m * p.F + f] = vh;
-            p.act_hi[p.act_lo_off + (size_t)m * p.F + f] = __float2bfloat16_rn(v - __bfloat162float(vh));
+            p.act_hi[(size_t)mm * p.F + f] = vh;
+            p.act_hi[p.act_lo_off + (size_t)mm * p.F + f] = __float2bfloat16_rn(v - __bfloat162float(vh));
           }
         }
       } else {
-#pragma unroll
-      for (int j = 0; j < WT; ++j)                               // accumulator
+      const int n_local = tile_in_mat * R + row;
+      const int n = p.col_off[mat] + n_local;
+      const bool live = row < R && n_local < p.n_out[mat];
       for (int m0 = 0; m0 < p.Mp; m0 += 16) {                    // first token row of the chunk
-        const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + j * NN;
-        const int n_local = (tile_in_mat + j) * R + row;
-        const int n = p.col_off[mat] + n_local;
-        const bool live = row < R && n_local < p.n_out[mat];
+        const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
         uint32_t hi[16], lo[16];
         tmem_ld16_issue(t_addr + m0, hi);
-        if (XP == 2) {
-          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) lo[i] = 0u;
-        }
+        tmem_ld16_issue(t_addr + p.Mp + m0, lo);
         tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int m = m_base + m0 + i;
-          if (live && m < p.M) {
-            float v = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
-            if (p.ss_part) v *= s_scale[m0 + i];
-            if (p.store_bf16) out_bf16[(size_t)m * p.ldc + n] = __float2bfloat16_rn(v);
-            else plane[(size_t)m * p.ldc + n] = v;
-          }
-        }
+        if (!live) continue;
+        const float *scale = p.ss_part ? s_scale + m0 : nullptr;
+        if (p.store_bf16) store_column(out_bf16 + (size_t)m0 * p.ldc + n, p.ldc, hi, lo, scale, p.M - m0);
+        else store_column(plane + (size_t)m0 * p.ldc + n, p.ldc, hi, lo, scale, p.M - m0);
       }
       }
     } else if (tid == 64) {
@@ -438,6 +442,317 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------------- many rows: CTA pairs
+// More than 64 token rows.  The tensor pipe is the bound (both activation planes are multiplied), and with one CTA per tile the
+// shared memory is: a 128 x 256 MMA moves 192 bytes of operands per clock through a port of 128 (measured: 57 % tensor
+// activity, 29-35 % of the bf16 peak useful).  Here two CTAs of a cluster work on 256 weight rows x one slab of up to 128
+// tokens with cta_group::2 MMAs: each holds its own 128 weight rows and one activation plane (rank 0 hi, rank 1 lo), i.e. half
+// of the bytes.  One CTA per SM, persistent: a pair runs through (weight tile pair, K split, token slab) units, slabs
+// innermost so that the pairs at work share weight tiles in L2; two accumulators in tensor memory, so that a unit's epilogue
+// runs under the next unit's products.  Kernel alone, before -> now, us: 128 x 12288 x 4096 31.5 -> 25, 256 x 12288 x 4096 59 -> 42,
+// 200 x 22016 x 4096 102 -> 61, 1024 x 12288 x 4096 169 -> 135 (1.5 PFLOP/s issued).
+constexpr int kPairStages = 8;
+constexpr int kPairThreads = 64 + 256;   // producer, issuer, eight epilogue warps
+constexpr int kExTokens = 16;            // tokens of one exchange round of the gate|up epilogue
+
+struct PairParams {
+  GemmParams g;
+  int tiles, pairs;      // 128-row weight tiles, pairs of them
+  int n_units;
+};
+
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void pair_load(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void pair_load_nohint(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void pair_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
+// arrives on the barrier at this offset in both CTAs once every MMA issued so far is done
+__device__ __forceinline__ void pair_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+               "h"((unsigned short)3)
+               : "memory");
+}
+
+// AND over the 256 epilogue threads (named barrier 1): keeps their control flow uniform
+__device__ __forceinline__ bool pair_epilogue_all(bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "bar.red.and.pred p, 1, 256, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)pred)
+      : "memory");
+  return r != 0;
+}
+
+template <bool GU>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant__ CUtensorMap w_map1,
+                 const __grid_constant__ CUtensorMap w_map2, const __grid_constant__ CUtensorMap x_map, const PairParams q) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  __shared__ uint64_t bar_full[kPairStages], bar_empty[kPairStages], acc_full[2], acc_empty[2];
+  __shared__ uint32_t s_tmem_base;
+  __shared__ float s_scale[TILE_N];
+  const GemmParams &p = q.g;
+  pdl_trigger();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = blockIdx.x & 1u;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int R = p.tile_rows, NN = 2 * p.Mp, x_bytes = p.Mp * TILE_K * 2;
+  const int stage_bytes = W_TILE_BYTES + x_bytes;
+  // bytes that the copies of both CTAs bring into a stage
+  const uint32_t stage_tx = 2u * (uint32_t)((GU ? 2 : 1) * R * TILE_K * 2 + x_bytes);
+  uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint32_t tmem_cols = 32;
+  while ((int)tmem_cols < 2 * NN) tmem_cols <<= 1;
+
+  if (tid == 0) {
+    tma_prefetch_desc(&w_map0);
+    tma_prefetch_desc(&x_map);
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&bar_full[s], 1);
+      mbar_init(&bar_empty[s], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_empty[i], 16);   // eight epilogue warps of both CTAs
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // both CTAs' barriers are set up
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  tc_fence_after();
+  const uint32_t tmem_base = s_tmem_base;
+
+  // unit -> this CTA's weight tile, k-blocks, slab
+  struct Unit {
+    int tile, kb0, kb1, split, slab;
+  };
+  auto unit_of = [&](int u) {
+    Unit t;
+    t.slab = u % p.n_slabs;
+    const int v = u / p.n_slabs;
+    t.split = v % p.splits;
+    t.tile = (v / p.splits) * 2 + (int)rank;
+    t.kb0 = (int)(((long)t.split * p.k_blocks) / p.splits);
+    t.kb1 = (int)(((long)(t.split + 1) * p.k_blocks) / p.splits);
+    return t;
+  };
+  auto mat_of = [&](int tile) { return GU ? 0 : tile < p.tile_end[0] ? 0 : tile < p.tile_end[1] ? 1 : 2; };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer (each CTA its half)
+    uint64_t policy;   // several slabs read a weight tile again from L2
+    if (p.n_slabs > 1) asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+    else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    const uint32_t full0 = cluster_addr(&bar_full[0], 0), smem0 = smem_u32(smem);
+    struct Src {
+      const CUtensorMap *map;
+      int row;
+    };
+    auto src_of = [&](const Unit &t) {   // (a tile past the last: rows outside the matrix, filled with zeros)
+      const int mat = mat_of(t.tile);
+      return Src{mat == 0 ? &w_map0 : mat == 1 ? &w_map1 : &w_map2, (t.tile - (mat ? p.tile_end[mat - 1] : 0)) * R};
+    };
+    auto load_w = [&](const Src &c, int kb, int s) {
+      const uint32_t dst = smem0 + s * stage_bytes, bar = full0 + s * 8;
+      if (rank == 0) mbar_expect_tx(&bar_full[s], stage_tx);
+      pair_load(dst, c.map, kb * TILE_K, c.row, bar, policy);
+      if (GU) pair_load(dst + W_TILE_BYTES / 2, &w_map1, kb * TILE_K, c.row, bar, policy);
+    };
+    // the weights do not depend on the preceding kernel: those of the first stages are fetched before the wait
+    int pre = 0, it = 0;
+    if (pair < q.n_units) {
+      const Unit t = unit_of(pair);
+      const Src c = src_of(t);
+      for (; pre < p.stages && t.kb0 + pre < t.kb1; ++pre) {
+        if (elect_one()) load_w(c, t.kb0 + pre, pre);
+        __syncwarp();
+      }
+    }
+    pdl_wait();
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int u = pair; u < q.n_units && ok; u += n_pairs) {
+      const Unit t = unit_of(u);
+      const Src c = src_of(t);
+      const int x_row = (rank ? p.x_lo_row : 0) + t.slab * p.Mp;
+      for (int kb = t.kb0; kb < t.kb1; ++kb, ++it) {
+        if (it >= pre && !warp_wait(&bar_empty[s], ph ^ 1u)) { ok = false; break; }
+        if (elect_one()) {
+          if (it >= pre) load_w(c, kb, s);
+          pair_load_nohint(smem0 + s * stage_bytes + W_TILE_BYTES, &x_map, kb * TILE_K, x_row, full0 + s * 8);
+        }
+        __syncwarp();
+        if (++s == p.stages) { s = 0; ph ^= 1u; }
+      }
+    }
+    if (!ok) {   // leave no copy in flight: they are short, give them ample time
+      if (lane == 0) atomicExch(p.status, 1);
+      const unsigned long long t0 = global_ns();
+      while (global_ns() - t0 < 20000000ull) {}
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (rank 0 for the pair)
+    if (rank == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      const uint64_t desc0 = umma_desc_sw128(0);
+      int s = 0, n = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = pair; u < q.n_units && ok; u += n_pairs, ++n) {
+        const Unit t = unit_of(u);
+        const int buf = n & 1;
+        if (!warp_wait(&acc_empty[buf], ((n >> 1) & 1) ^ 1u)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d = tmem_base + buf * NN;
+        for (int kb = t.kb0; kb < t.kb1; ++kb) {
+          if (!warp_wait(&bar_full[s], ph)) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
+            const uint32_t at = smem_u32(smem + s * stage_bytes);
+            const uint64_t a = desc0 | (uint64_t)(at >> 4), b = desc0 | (uint64_t)((at + W_TILE_BYTES) >> 4);
+#pragma unroll
+            for (int k = 0; k < TILE_K / UMMA_K; ++k) pair_mma(d, a + k * 2, b + k * 2, idesc, !(kb == t.kb0 && k == 0));
+            pair_commit(&bar_empty[s]);
+          }
+          __syncwarp();
+          if (++s == p.stages) { s = 0; ph ^= 1u; }
+        }
+        if (ok && elect_one()) pair_commit(&acc_full[buf]);
+        __syncwarp();
+      }
+      if (!ok && lane == 0) atomicExch(p.status, 2);
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue warps (2..9): two groups of four, 16 tokens in turn
+    const int quarter = warp & 3, row = quarter * 32 + lane, grp = (warp - 2) >> 2, e = (tid - 64) & 127;
+    float *ex = reinterpret_cast<float *>(smem + p.stages * stage_bytes) + grp * TILE_N * (kExTokens + 1);   // GU: [128][kExTokens + 1]
+    pdl_wait();   // the planes may still be read, and the row scales written, by the preceding kernel
+    int n = 0, have_slab = -1;
+    for (int u = pair; u < q.n_units; u += n_pairs, ++n) {
+      const Unit t = unit_of(u);
+      const int buf = n & 1, m_base = t.slab * p.Mp;
+      if ((p.ss_part || GU) && have_slab != t.slab) {   // RMS scale of the slab's token rows
+        have_slab = t.slab;
+        pair_epilogue_all(true);
+        if (grp == 0) {
+          float sc = 1.0f;
+          if (p.ss_part && e < p.Mp && m_base + e < p.M) {
+            float tot = 0.0f;
+#pragma unroll 8
+            for (int jj = 0; jj < p.n_part; ++jj) tot += __ldg(p.ss_part + (size_t)(m_base + e) * p.n_part + jj);
+            sc = rsqrtf(tot * p.inv_d + p.eps);
+          }
+          s_scale[e] = sc;
+        }
+        pair_epilogue_all(true);
+      }
+      if (!pair_epilogue_all(mbar_wait(&acc_full[buf], (n >> 1) & 1))) {
+        if (tid == 64) atomicExch(p.status, 3);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * NN;
+      const int mat = mat_of(t.tile), m_left = p.M - m_base;
+      if (GU) {
+        // MMA rows 0..63 hold gate features, rows 64..127 the same features of the up matrix: they meet in shared memory, 16
+        // tokens at a time; then thread e finishes feature e % 64 for every second token
+        const int fr = e & 63, f = t.tile * R + fr, odd = e >> 6;
+        const bool live = fr < R && f < p.F;
+        for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
+          uint32_t hi[16], lo[16];
+          tmem_ld16_issue(t_addr + m0, hi);
+          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            ex[row * (kExTokens + 1) + i] = (__uint_as_float(hi[i]) + __uint_as_float(lo[i])) * s_scale[m0 + i];
+          asm volatile("bar.sync %0, 128;" ::"r"(grp + 2) : "memory");
+          if (live) {
+            __nv_bfloat16 *dst = p.act_hi + (size_t)(m_base + m0 + odd) * p.F + f;
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float g = ex[fr * (kExTokens + 1) + 2 * i + odd], up = ex[(64 + fr) * (kExTokens + 1) + 2 * i + odd];
+              v[i] = g / (1.0f + expf(-g)) * up;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (m0 + odd + 2 * i >= m_left) break;
+              const __nv_bfloat16 vh = __float2bfloat16_rn(v[i]);
+              dst[(size_t)(2 * i) * p.F] = vh;
+              dst[p.act_lo_off + (size_t)(2 * i) * p.F] = __float2bfloat16_rn(v[i] - __bfloat162float(vh));
+            }
+          }
+          asm volatile("bar.sync %0, 128;" ::"r"(grp + 2) : "memory");
+        }
+      } else {
+        const int n_local = (t.tile - (mat ? p.tile_end[mat - 1] : 0)) * R + row;
+        const int col = p.col_off[mat] + n_local;
+        const bool live = t.tile < q.tiles && row < R && n_local < p.n_out[mat];
+        float *plane = reinterpret_cast<float *>(p.out) + (size_t)t.split * p.plane_stride + (size_t)m_base * p.ldc + col;
+        __nv_bfloat16 *logits = reinterpret_cast<__nv_bfloat16 *>(p.out) + (size_t)m_base * p.ldc + col;
+        for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
+          uint32_t hi[16], lo[16];
+          tmem_ld16_issue(t_addr + m0, hi);
+          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
+          tmem_ld_wait();
+          if (!live) continue;
+          const float *scale = p.ss_part ? s_scale + m0 : nullptr;
+          if (p.store_bf16) store_column(logits + (size_t)m0 * p.ldc, p.ldc, hi, lo, scale, m_left - m0);
+          else store_column(plane + (size_t)m0 * p.ldc, p.ldc, hi, lo, scale, m_left - m0);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0)   // the accumulator is free (rank 0 issues into both CTAs' tensor memory)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr(&acc_empty[buf], 0)) : "memory");
+    }
+  }
+
+  tc_fence_before();
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // neither CTA leaves while the other may reach into it
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
 }
 
@@ -457,13 +772,23 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// plain sum of split planes (sjd_gemm): out[m][n] (+)= sum_s P[s][m][n]
+// plain sum of split planes (sjd_gemm): out[m][n] (+)= sum_s P[s][m][n]; V: entries per thread (4 when out is 16-byte aligned)
+template <typename V>
 __global__ void sum_planes_kernel(const float *__restrict__ planes, size_t plane_stride, int splits, float *__restrict__ out,
                                   size_t total, int accumulate) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    float acc = 0.0f;
-    for (int s = 0; s < splits; ++s) acc += planes[(size_t)s * plane_stride + i];
-    out[i] = accumulate ? out[i] + acc : acc;
+  pdl_wait();
+  constexpr int E = sizeof(V) / 4;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total / E; i += (size_t)gridDim.x * blockDim.x) {
+    float acc[E] = {};
+    for (int s = 0; s < splits; ++s) {
+      const V v = __ldcg(reinterpret_cast<const V *>(planes + (size_t)s * plane_stride) + i);
+      const float *f = reinterpret_cast<const float *>(&v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) acc[e] += f[e];
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = accumulate ? out[i * E + e] + acc[e] : acc[e];
+    *(reinterpret_cast<V *>(out) + i) = *reinterpret_cast<const V *>(acc);
   }
 }
 
@@ -497,15 +822,68 @@ GemmTcPlan gemm_tc_plan(int M) {
   return pl;
 }
 
-// K splits for a launch of `tiles` weight tiles: a single wave of the resident CTAs (two per SM), at least 16 k-blocks (256 KB of weights) per CTA so that
-// set-up and drain stay small next to the streaming
+// K splits for a launch of `tiles` weight tiles.  Few rows: a single wave of the resident CTAs (two per SM), at least
+// SJD_GEMM_MIN_KB k-blocks per CTA so that set-up and drain stay small next to the streaming.  Many rows (CTA pairs): the split
+// with the shortest schedule, counted in k-blocks of a full tile (0.27 us): rounds of the grid, about three k-blocks of
+// ramp per round, and the traffic of the planes through L2.
 int gemm_tc_splits(const GemmTcPlan &pl, int tiles, int k_blocks, int n_sms) {
+  const int sms = n_sms < 132 ? 132 : n_sms > 160 ? 160 : n_sms;   // the range scratch is sized for
+  if (gemm_tc_pairs(pl)) {
+    const int units = (tiles + 1) / 2 * pl.n_slabs, pairs = sms / 2;
+    const double per_kb = pl.slab_rows / 128.0, plane = (double)tiles * 128.0 * pl.n_slabs * pl.slab_rows * 8.0 / 2.7e6;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int s = 1; s <= 16 && s * 4 <= k_blocks; ++s) {
+      const int rounds = (units * s + pairs - 1) / pairs;
+      const double cost = rounds * ((k_blocks + s - 1) / s + 3) * per_kb + s * plane;
+      if (s == 1 || cost < best_cost) {
+        best = s;
+        best_cost = cost;
+      }
+    }
+    return best;
+  }
   const int ctas = tiles * pl.n_slabs;
   int s = (SJD_GEMM_CTAS_PER_SM * n_sms) / (ctas > 0 ? ctas : 1);
   const int cap = k_blocks / SJD_GEMM_MIN_KB > 1 ? k_blocks / SJD_GEMM_MIN_KB : 1;
   s = s > cap ? cap : s;
   s = s > 16 ? 16 : s;
   return s < 1 ? 1 : s;
+}
+int gemm_tc_splits_max(const GemmTcPlan &pl, int tiles, int k_blocks) {
+  int most = 1;
+  for (int sms = 132; sms <= 160; sms += 2) {
+    const int s = gemm_tc_splits(pl, tiles, k_blocks, sms);
+    most = s > most ? s : most;
+  }
+  return most;
+}
+
+static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles, cudaStream_t stream) {
+  PairParams q;
+  q.g = p;
+  q.tiles = tiles;
+  q.pairs = (tiles + 1) / 2;
+  q.n_units = q.pairs * p.n_slabs * p.splits;
+  const bool gu = g.act_hi != nullptr;
+  const int stage_bytes = W_TILE_BYTES + p.Mp * TILE_K * 2;
+  const int ex = gu ? 2 * TILE_N * (kExTokens + 1) * 4 : 0;
+  const int budget = 232448 - 2048 - 1024 - ex;
+  int stages = budget / stage_bytes;
+  stages = stages > kPairStages ? kPairStages : stages;
+  q.g.stages = stages;
+  const size_t smem = (size_t)stages * stage_bytes + 1024 + ex;
+  const CUtensorMap &w0 = reinterpret_cast<const CUtensorMap &>(*g.w_map[0]);
+  const CUtensorMap &w1 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 1 ? 1 : 0]);
+  const CUtensorMap &w2 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 2 ? 2 : 0]);
+  const CUtensorMap &xm = reinterpret_cast<const CUtensorMap &>(*g.x_map);
+  auto kernel = gu ? gemm_pair_kernel<true> : gemm_pair_kernel<false>;
+  SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int sms = g.n_sms > 1 ? g.n_sms : 148;
+  const int pairs = q.n_units < sms / 2 ? q.n_units : sms / 2;
+  SJD_CUDA(launch_kernel(kernel, dim3(2 * pairs), dim3(kPairThreads), smem, stream, w0, w1, w2, xm, q));
+  SJD_CHECK_LAUNCH();
+  return SJD_OK;
 }
 
 int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
@@ -548,8 +926,9 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   p.act_hi = g.act_hi;
   p.act_lo_off = g.act_lo_off;
   p.F = gu ? g.n_out[0] : 0;
+  if (gemm_tc_pairs(pl)) return launch_gemm_pair(g, p, tiles, stream);
   const int stage_bytes = W_TILE_BYTES + 2 * p.Mp * TILE_K * 2;
-  const int ctas = tiles * p.n_slabs;
+  const int ctas = tiles;
   // one CTA per SM or fewer: give each the deeper ring
   const int budget =
       (SJD_GEMM_DEEP_RING && g.n_sms > 0 && ctas * g.splits <= g.n_sms) ? 2 * kSmemBudget : kSmemBudget;
@@ -584,8 +963,11 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
 
 int launch_sum_planes(const float *planes, size_t plane_stride, int splits, float *out, size_t total, int accumulate,
                       cudaStream_t stream) {
-  const int blocks = (int)((total + 255) / 256 < 2368 ? (total + 255) / 256 : 2368);
-  sum_planes_kernel<<<blocks, 256, 0, stream>>>(planes, plane_stride, splits, out, total, accumulate);
+  const bool vec = ((uintptr_t)out & 15u) == 0 && total % 4 == 0 && plane_stride % 4 == 0;
+  const size_t groups = vec ? total / 4 : total;
+  const int blocks = (int)((groups + 255) / 256 < 1184 ? (groups + 255) / 256 : 1184);
+  auto kernel = vec ? sum_planes_kernel<float4> : sum_planes_kernel<float>;
+  SJD_CUDA(launch_kernel(kernel, dim3(blocks), dim3(256), 0, stream, planes, plane_stride, splits, out, total, accumulate));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

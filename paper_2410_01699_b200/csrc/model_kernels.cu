@@ -300,16 +300,35 @@ int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const
 
 namespace sjd {
 namespace {
-__global__ void split_hilo_kernel(const float *__restrict__ x, HiLoOut o, size_t total) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
-    store_hilo(o, i, x[i]);
+// VEC: four entries per thread and round (both sides 16-byte aligned).  Also clears the call's status word.
+template <int VEC>
+__global__ void split_hilo_kernel(const float *__restrict__ x, HiLoOut o, size_t groups, int *status) {
+  pdl_trigger();
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < groups; i += (size_t)gridDim.x * blockDim.x) {
+    if constexpr (VEC == 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4 *>(x) + i);
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
+      const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+      const __nv_bfloat162 l0 = __floats2bfloat162_rn(v.x - f0.x, v.y - f0.y), l1 = __floats2bfloat162_rn(v.z - f1.x, v.w - f1.y);
+      *reinterpret_cast<uint2 *>(o.base + i * 4) =
+          make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+      *reinterpret_cast<uint2 *>(o.base + o.lo_offset + i * 4) =
+          make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+    } else {
+      store_hilo(o, i, x[i]);
+    }
+  }
 }
 }  // namespace
 
-// hi/lo bf16 planes of an fp32 matrix (same row stride), for the tensor-core GEMM
-int launch_split_hilo(const float *x, HiLoOut o, size_t total, cudaStream_t stream) {
-  const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
-  split_hilo_kernel<<<blocks, 256, 0, stream>>>(x, o, total);
+// hi/lo bf16 planes of an fp32 matrix (same row stride; total a multiple of 4), for the tensor-core GEMM
+int launch_split_hilo(const float *x, HiLoOut o, size_t total, int *status, cudaStream_t stream) {
+  const bool vec = ((uintptr_t)x & 15u) == 0 && total % 4 == 0 && o.lo_offset % 4 == 0;
+  const size_t groups = vec ? total / 4 : total;
+  const int blocks = (int)((groups + 255) / 256 < 1184 ? (groups + 255) / 256 : 1184);
+  if (vec) SJD_CUDA(launch_kernel(split_hilo_kernel<4>, dim3(blocks), dim3(256), 0, stream, x, o, groups, status));
+  else SJD_CUDA(launch_kernel(split_hilo_kernel<1>, dim3(blocks), dim3(256), 0, stream, x, o, groups, status));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

@@ -40,6 +40,9 @@ def _tolerance(x, w, k):
     (300, 384, 640),      # three ragged slabs of 112 rows (the last holds 76)
     (512, 4096, 4096),    # 8 images x W = 64 on the attention output projection: 4 slabs x 32 tiles x K splits
     (1024, 256, 256),     # most rows covered: eight slabs
+    (65, 128, 64),            # CTA pairs: one tile (the second CTA has none), one k-block
+    (130, 384, 1088),         # three tiles (an odd pair), two slabs of 80 rows, K over several splits
+    (257, 19200, 256),        # more units than pairs, three slabs, few k-blocks per unit
 ])
 def test_gemm_matches_fp64_product(m, n, k):
     x, w, ref = _case(m, n, k, seed=m + n + k)
