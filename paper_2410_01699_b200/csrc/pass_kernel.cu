@@ -866,28 +866,36 @@ __device__ __forceinline__ void epilogue(const Ctx &x, const PassGemm &g, int ki
     ++acc_n;
     fence_tc_after();
     const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + buf * 2 * NN;
+    // (stores of 8 or 16 tokens without a test between them: two warps per scheduler cannot hide dependent instructions)
     if (kind == PK_GU) {
       const bool live = row < t.R && row < n_left;
       __nv_bfloat16 *dst = p.act.base + t.row0 + row;
 #pragma unroll 1
-      for (int m0 = grp * 8; m0 < p.Mp; m0 += 16) {
+      for (int m0 = grp * 8; m0 < p.M; m0 += 16) {
         uint32_t gh[8], gl[8], uh[8], ul[8];
         tmem_ld8(base + m0, gh);
         tmem_ld8(base + p.Mp + m0, gl);
         tmem_ld8(base + NN + m0, uh);
         tmem_ld8(base + NN + p.Mp + m0, ul);
         tmem_wait_ld();
+        __nv_bfloat16 hi[8], lo[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const int m = m0 + i;
-          const float sc = x.sh.scale[m & 63];
+          const float sc = x.sh.scale[m0 + i];
           const float gv = (__uint_as_float(gh[i]) + __uint_as_float(gl[i])) * sc;
           const float uv = (__uint_as_float(uh[i]) + __uint_as_float(ul[i])) * sc;
           const float v = gv / (1.0f + expf(-gv)) * uv;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-          if (live && m < p.M) {
-            dst[(size_t)m * p.F] = hi;
-            dst[p.act.lo_offset + (size_t)m * p.F] = __float2bfloat16_rn(v - __bfloat162float(hi));
+          hi[i] = __float2bfloat16_rn(v);
+          lo[i] = __float2bfloat16_rn(v - __bfloat162float(hi[i]));
+        }
+        if (!live) continue;
+        __nv_bfloat16 *o = dst + (size_t)m0 * p.F;
+        const int n = p.M - m0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (i < n) {
+            o[(size_t)i * p.F] = hi[i];
+            o[p.act.lo_offset + (size_t)i * p.F] = lo[i];
           }
         }
       }
@@ -898,19 +906,26 @@ __device__ __forceinline__ void epilogue(const Ctx &x, const PassGemm &g, int ki
       float *dst = p.part + (size_t)(s.tile * g.max_pieces + s.piece) * p.M * p.part_ld + r;
       __nv_bfloat16 *lg = p.logits + (size_t)t.row0 + r;
 #pragma unroll 1
-      for (int m0 = t.two ? 0 : grp * 16; m0 < p.Mp; m0 += t.two ? 16 : 32) {
+      for (int m0 = t.two ? 0 : grp * 16; m0 < p.M; m0 += t.two ? 16 : 32) {
         uint32_t hi[16], lo[16];
         tmem_ld16(base + half * NN + m0, hi);
         tmem_ld16(base + half * NN + p.Mp + m0, lo);
         tmem_wait_ld();
+        if (!live) continue;
+        const int n = p.M - m0;
+        float v[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int m = m0 + i;
-          const float v = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
-          if (live && m < p.M) {
-            if (kind == PK_LOGITS) lg[(size_t)m * p.vocab] = __float2bfloat16_rn(v * x.sh.scale[m & 63]);
-            else dst[(size_t)m * p.part_ld] = v;
-          }
+        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+        if (kind == PK_LOGITS) {
+          __nv_bfloat16 *o = lg + (size_t)m0 * p.vocab;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (i < n) o[(size_t)i * p.vocab] = __float2bfloat16_rn(v[i] * x.sh.scale[m0 + i]);
+        } else {
+          float *o = dst + (size_t)m0 * p.part_ld;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (i < n) o[(size_t)i * p.part_ld] = v[i];
         }
       }
     }
