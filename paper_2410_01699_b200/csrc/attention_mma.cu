@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constan
   SJD_TL(TL_ATTN, 0, threadIdx.x == 0);
   pdl_wait();   // keys/values of this step were written by the preceding kernel
   SJD_TL(TL_ATTN, 1, threadIdx.x == 0);
-  const int h = blockIdx.x, seg = blockIdx.y, split = blockIdx.z;
+  // (later segments of a prompt see more keys: they start first)
+  const int h = blockIdx.x, seg = gridDim.y - 1 - blockIdx.y, split = blockIdx.z;
   const int b = seg_sequence(p.segs, seg);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int W = p.segs.rows;

@@ -322,7 +322,7 @@ struct RowScale {
   float inv_d, eps;
 };
 int resid_gain_parts(int d);
-int launch_resid_gain(int dtype, float *x, PlaneSet ps, const void *gain, HiLoOut h, float *ss_part, int M, int d,
+int launch_resid_gain(float *x, PlaneSet ps, const void *gain, HiLoOut h, float *ss_part, int M, int d,
                       cudaStream_t stream);
 
 // x[m][:] = tok_emb[tok[m]][:]  (fp32 residual stream)
@@ -364,7 +364,7 @@ struct QkNorm {
 };
 int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const float2 *rope_table, float *q,
                        KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
-int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
+int launch_qkv_finish(PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
 // Window-causal attention: query row m (position in_pos[m] of its segment's sequence) attends cache rows
 // 0 .. in_pos[m].  q, out: fp32 [M][H*hd]; cache of `dtype`.  partial: fp32 scratch [M][H][splits][hd + 2].

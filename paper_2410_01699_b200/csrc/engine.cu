@@ -532,14 +532,14 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
   for (int l = 0; l < g.n_layers; ++l) {
     const LayerMaps &lm = c->wmaps[l];
     PlaneSet ps;
-    SJD_TR(TC_OTHER, launch_resid_gain(dt, x, pending, c->attn_norm[l], hl_h, ss_part, M, d, stream));
+    SJD_TR(TC_OTHER, launch_resid_gain(x, pending, c->attn_norm[l], hl_h, ss_part, M, d, stream));
     {
       const WMap *wm[3] = {&lm.wq, &lm.wk, &lm.wv};
       const int n_out[3] = {nq, nk, nk};
       SJD_TRY(gemm(wm, 3, n_out, xm.h, d, nqkv, planes, false, &ps));
     }
     const KvLayout kv = c->kv_layer(l);
-    SJD_TR(TC_OTHER, launch_qkv_finish(dt, ps, rs, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
+    SJD_TR(TC_OTHER, launch_qkv_finish(ps, rs, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
     if (!logits_out && l == g.n_layers - 1) break;
     if (c->kv_map_valid && attention_mma_supported(g.head_dim, segs.rows)) {
       SJD_TR(TC_ATTENTION, launch_attention_mma(c->kv_map, l * g.max_batch * 2 * g.n_kv_heads, kv, q, st.in_pos, partial, nullptr,
@@ -557,7 +557,7 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
       const int n_out[1] = {d};
       SJD_TRY(gemm(wm, 1, n_out, xm.attn, nq, d, planes, false, &ps));
     }
-    SJD_TR(TC_OTHER, launch_resid_gain(dt, x, ps, c->ffn_norm[l], hl_h, ss_part, M, d, stream));
+    SJD_TR(TC_OTHER, launch_resid_gain(x, ps, c->ffn_norm[l], hl_h, ss_part, M, d, stream));
     {
       const WMap *wm[2] = {&lm.gate_gu, &lm.up_gu};
       const int n_out[2] = {F, F};
@@ -570,7 +570,7 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
     }
   }
   if (logits_out) {
-    SJD_TR(TC_OTHER, launch_resid_gain(dt, x, pending, c->final_norm, hl_h, ss_part, M, d, stream));
+    SJD_TR(TC_OTHER, launch_resid_gain(x, pending, c->final_norm, hl_h, ss_part, M, d, stream));
     const WMap *wm[1] = {&c->wmap_head};
     const int n_out[1] = {g.vocab};
     SJD_TRY(gemm(wm, 1, n_out, xm.h, d, g.vocab, logits_out, true, nullptr));

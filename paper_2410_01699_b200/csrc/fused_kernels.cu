@@ -15,16 +15,28 @@ template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
-__device__ __forceinline__ void put_hilo(const HiLoOut &o, size_t idx, float v) {
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  o.base[idx] = hi;
-  o.base[o.lo_offset + idx] = __float2bfloat16_rn(v - __bfloat162float(hi));
+// two adjacent values -> packed bf16 hi pair and lo pair (lo = value - hi, rounded)
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t &hi, uint32_t &lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  const float2 f = __bfloat1622float2(h);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(a - f.x, b - f.y);
+  hi = *reinterpret_cast<const uint32_t *>(&h);
+  lo = *reinterpret_cast<const uint32_t *>(&l);
 }
-
-__device__ __forceinline__ float sum_planes(const PlaneSet &ps, size_t idx) {
-  float acc = 0.0f;
-  for (int s = 0; s < ps.splits; ++s) acc += __ldg(ps.base + (size_t)s * ps.plane_stride + idx);
-  return acc;
+// N adjacent entries (4 or 2, aligned) as fp32
+template <int N>
+__device__ __forceinline__ void load_gain(const float *p, float *v) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = __ldg(p + i);
+}
+template <int N>
+__device__ __forceinline__ void load_gain(const __nv_bfloat16 *p, float *v) {
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    const float2 f = __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162 *>(p + i)));
+    v[i] = f.x;
+    v[i + 1] = f.y;
+  }
 }
 
 // Per-row RMS scale from the partial sums of squares a resid_gain launch left:
@@ -59,7 +71,14 @@ __global__ void __launch_bounds__(RG_THREADS) resid_gain_kernel(float *__restric
   const int m = blockIdx.x, chunk = blockIdx.y, tid = threadIdx.x;
   const int c0 = chunk * RG_COLS + tid * 4;
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  if (c0 < d) {   // d is a multiple of 4
+  if (c0 < d) {   // d is a multiple of 4; the gain row may start on any element of its dtype
+    float gv[4];
+    if (((uintptr_t)gain & 3u) == 0) {
+      load_gain<4>(gain + c0, gv);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) gv[i] = to_f<T>(gain[c0 + i]);
+    }
     const float4 t = *reinterpret_cast<const float4 *>(x + (size_t)m * d + c0);
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
     for (int s = 0; s < ps.splits; ++s) {
@@ -67,8 +86,11 @@ __global__ void __launch_bounds__(RG_THREADS) resid_gain_kernel(float *__restric
       v[0] += pv.x; v[1] += pv.y; v[2] += pv.z; v[3] += pv.w;
     }
     if (ps.splits > 0) *reinterpret_cast<float4 *>(x + (size_t)m * d + c0) = make_float4(v[0], v[1], v[2], v[3]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) put_hilo(h, (size_t)m * d + c0 + i, v[i] * to_f<T>(gain[c0 + i]));
+    uint2 hi, lo;
+    split_pair(v[0] * gv[0], v[1] * gv[1], hi.x, lo.x);
+    split_pair(v[2] * gv[2], v[3] * gv[3], hi.y, lo.y);
+    *reinterpret_cast<uint2 *>(h.base + (size_t)m * d + c0) = hi;
+    *reinterpret_cast<uint2 *>(h.base + h.lo_offset + (size_t)m * d + c0) = lo;
   }
   float ss = v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
   ss = warp_sum(ss);
@@ -78,80 +100,103 @@ __global__ void __launch_bounds__(RG_THREADS) resid_gain_kernel(float *__restric
 }
 
 // q,k,v = scale * sum of the QKV planes; rotate q and k (pairs i, i + hd/2) by the row's absolute
-// position; q -> fp32 [M][H*hd]; k, v -> cache row in_pos[m].  64 threads per (row, head slot), four
-// slots per block.
-template <typename T>
-__global__ void qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__restrict__ in_pos,
-                                  const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, RowSegs segs,
-                                  int n_heads, QkNorm qkn) {
-  __shared__ float s_ss[8];   // QK-norm: per-warp sums of squares of a head (two warps per 64-thread group)
+// position; q -> fp32 [M][H*hd]; k, v -> cache row in_pos[m].  A warp per (row, head slot), eight slots per block;
+// a lane holds up to two entries of each half of the head: adjacent ones at head_dim 128 (VEC), so that planes, q and cache are
+// accessed in 8-byte (cache: 4-byte) groups, else those 32 apart (any even head_dim up to 128).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__restrict__ in_pos,
+                                                         const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv,
+                                                         RowSegs segs, int n_heads, QkNorm qkn) {
   pdl_trigger();
   SJD_TL(TL_QKV, 0, threadIdx.x == 0);
   pdl_wait();
   SJD_TL(TL_QKV, 1, threadIdx.x == 0);
-  const int m = blockIdx.x, lt = threadIdx.x & 63;
-  const int b = seg_sequence(segs, m / segs.rows);
-  const int hd = kv.head_dim, half = hd >> 1, nkv = kv.n_kv_heads;
-  const int nq = n_heads * hd, nk = nkv * hd;
-  const size_t rbase = (size_t)m * ps.ld;
+  constexpr int PER = 2;
+  const int HD = VEC ? 128 : kv.head_dim, HALF = HD >> 1;
+  const int m = blockIdx.x, lane = threadIdx.x & 31;
+  auto at = [&](int i) { return VEC ? lane * 2 + i : lane + 32 * i; };   // entry i of this lane in a half
+  auto on = [&](int i) { return VEC || at(i) < HALF; };
+  const int nkv = kv.n_kv_heads, nq = n_heads * HD;
+  const float *row = ps.base + (size_t)m * ps.ld;
   T *cache = reinterpret_cast<T *>(kv.base);
   // The loads of the projection planes depend on nothing, the row's position and RMS scale are loads of their
   // own and the rotary entry depends on the position: the plane loads of a slot are issued first, so that the
   // kernel waits for two memory round trips in a row and not three.
-  int pos = 0;
+  int pos = 0, b = 0;
   float sc = 0.0f;
   bool first = true;
-  // the block's 64-thread groups walk over the head slots of the row (one pass when the grid has a
-  // block for every four slots, several when many rows share fewer blocks per row)
-  const int stride = gridDim.y * (blockDim.x >> 6);
-  for (int slot = blockIdx.y * (blockDim.x >> 6) + (threadIdx.x >> 6); slot < n_heads + 2 * nkv; slot += stride) {
-    const bool is_v = slot >= n_heads + nkv;
-    const bool is_q = slot < n_heads;
-    // head_dim <= 128: a thread of the group owns at most one rotary pair (j, j + half) of a q or k head,
-    // or the entries j and j + 64 of a v head
-    const int col0 = is_q ? slot * hd : is_v ? nq + nk + (slot - n_heads - nkv) * hd : nq + (slot - n_heads) * hd;
-    const int ja = lt, jb = is_v ? lt + 64 : lt + half;
-    const bool has_a = is_v ? ja < hd : ja < half, has_b = is_v ? jb < hd : ja < half;
-    float x1 = 0.0f, x2 = 0.0f;
-    if (has_a) x1 = sum_planes(ps, rbase + col0 + ja);
-    if (has_b) x2 = sum_planes(ps, rbase + col0 + jb);
-    if (first) {   // uniform over the block
+  for (int slot = blockIdx.y * 8 + (threadIdx.x >> 5); slot < n_heads + 2 * nkv; slot += gridDim.y * 8) {
+    float v[2][PER];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i) v[h][i] = 0.0f;
+      const float *src = row + slot * HD + h * HALF;
+#pragma unroll 4
+      for (int s = 0; s < ps.splits; ++s) {
+        const float *a = src + (size_t)s * ps.plane_stride;
+        if constexpr (VEC) {
+          const float2 f = __ldg(reinterpret_cast<const float2 *>(a) + lane);
+          v[h][0] += f.x;
+          v[h][1] += f.y;
+        } else {
+#pragma unroll
+          for (int i = 0; i < PER; ++i)
+            if (on(i)) v[h][i] += __ldg(a + at(i));
+        }
+      }
+    }
+    if (first) {
       pos = in_pos[m];
-      sc = row_scale_warp(rs, m);   // before any thread leaves: the warp shares the loads
+      b = seg_sequence(segs, m / segs.rows);
+      sc = row_scale_warp(rs, m);
       first = false;
       if (pos < 0) return;
     }
-    x1 *= sc;
-    x2 *= sc;
-    if (is_v) {
-      T *dst = cache + kv_row_offset(kv, b, 1, slot - n_heads - nkv, pos);
-      if (has_a) dst[ja] = from_f<T>(x1);
-      if (has_b) dst[jb] = from_f<T>(x2);
-      continue;
-    }
-    if (qkn.q_gain) {   // QK-norm: RMS over the head's entries, held by the 64 threads of this group
-      const int grp = threadIdx.x >> 6;
-      const float ws = warp_sum(x1 * x1 + x2 * x2);
-      if ((threadIdx.x & 31) == 0) s_ss[threadIdx.x >> 5] = ws;
-      asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
-      const float rinv = rsqrtf((s_ss[2 * grp] + s_ss[2 * grp + 1]) / (float)hd + qkn.eps);
-      asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");   // the sums are reused by the group's next head
-      if (has_a) {
+    const bool is_q = slot < n_heads, is_v = slot >= n_heads + nkv;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < PER; ++i) v[h][i] *= sc;
+    if (!is_v) {
+      if (qkn.q_gain) {   // QK-norm: RMS over the head's entries
+        float ss = 0.0f;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) ss += v[0][i] * v[0][i] + v[1][i] * v[1][i];
+        const float rinv = rsqrtf(warp_sum(ss) / (float)HD + qkn.eps);
         const T *gain = reinterpret_cast<const T *>(is_q ? qkn.q_gain : qkn.k_gain);
-        x1 *= rinv * to_f<T>(gain[ja]);
-        x2 *= rinv * to_f<T>(gain[jb]);
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+          if (!on(i)) continue;
+          v[0][i] *= rinv * to_f<T>(gain[at(i)]);
+          v[1][i] *= rinv * to_f<T>(gain[at(i) + HALF]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if (!on(i)) continue;
+        const float2 c = rope[(size_t)pos * HALF + at(i)];
+        const float r1 = v[0][i] * c.x - v[1][i] * c.y, r2 = v[1][i] * c.x + v[0][i] * c.y;
+        v[0][i] = r1;
+        v[1][i] = r2;
       }
     }
-    if (!has_a) continue;
-    const float2 c = rope[(size_t)pos * half + ja];
-    const float r1 = x1 * c.x - x2 * c.y, r2 = x2 * c.x + x1 * c.y;
-    if (is_q) {
-      q[(size_t)m * nq + slot * hd + ja] = r1;
-      q[(size_t)m * nq + slot * hd + jb] = r2;
-    } else {
-      T *dst = cache + kv_row_offset(kv, b, 0, slot - n_heads, pos);
-      dst[ja] = from_f<T>(r1);
-      dst[jb] = from_f<T>(r2);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      T *kvd = nullptr;
+      if (!is_q) kvd = cache + kv_row_offset(kv, b, is_v ? 1 : 0, slot - n_heads - (is_v ? nkv : 0), pos) + h * HALF;
+      float *qd = q + (size_t)m * nq + slot * HD + h * HALF;
+      if constexpr (VEC && sizeof(T) == 2) {
+        if (is_q) reinterpret_cast<float2 *>(qd)[lane] = make_float2(v[h][0], v[h][1]);
+        else reinterpret_cast<__nv_bfloat162 *>(kvd)[lane] = __floats2bfloat162_rn(v[h][0], v[h][1]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+          if (!on(i)) continue;
+          if (is_q) qd[at(i)] = v[h][i];
+          else kvd[at(i)] = from_f<T>(v[h][i]);
+        }
+      }
     }
   }
 }
@@ -160,39 +205,26 @@ __global__ void qkv_finish_kernel(PlaneSet ps, RowScale rs, const int32_t *__res
 
 int resid_gain_parts(int d) { return (d + 127) / 128; }
 
-int launch_resid_gain(int dtype, float *x, PlaneSet ps, const void *gain, HiLoOut h, float *ss_part, int M, int d,
+int launch_resid_gain(float *x, PlaneSet ps, const void *gain, HiLoOut h, float *ss_part, int M, int d,
                       cudaStream_t stream) {
   if (d % 4 != 0) return SJD_ERR_UNSUPPORTED;
   const dim3 grid(M, (d + RG_COLS - 1) / RG_COLS);
-  if (dtype == SJD_F32)
-    SJD_CUDA(launch_kernel(resid_gain_kernel<float>, grid, dim3(RG_THREADS), 0, stream, x, ps,
-                           reinterpret_cast<const float *>(gain), h, ss_part, d));
-  else if (dtype == SJD_BF16)
-    SJD_CUDA(launch_kernel(resid_gain_kernel<__nv_bfloat16>, grid, dim3(RG_THREADS), 0, stream, x, ps,
-                           reinterpret_cast<const __nv_bfloat16 *>(gain), h, ss_part, d));
-  else
-    return SJD_ERR_UNSUPPORTED;
+  SJD_CUDA(launch_kernel(resid_gain_kernel<__nv_bfloat16>, grid, dim3(RG_THREADS), 0, stream, x, ps,
+                         reinterpret_cast<const __nv_bfloat16 *>(gain), h, ss_part, d));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }
 
-int launch_qkv_finish(int dtype, PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
+int launch_qkv_finish(PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream) {
   if (kv.head_dim > 128) return SJD_ERR_UNSUPPORTED;
-  // a block per four head slots for a few dozen rows; fewer blocks per row (each walking more slots) as
+  // a block per eight head slots for a few dozen rows; fewer blocks per row (each walking more slots) as
   // the rows grow, about eight blocks per SM in all
-  int per_row = (n_heads + 2 * kv.n_kv_heads + 3) / 4;
+  int per_row = (n_heads + 2 * kv.n_kv_heads + 7) / 8;
   const int cap = 1184 / M > 0 ? 1184 / M : 1;
   per_row = per_row < cap ? per_row : cap;
-  const dim3 grid(M, per_row);
-  if (dtype == SJD_F32)
-    SJD_CUDA(launch_kernel(qkv_finish_kernel<float>, grid, dim3(256), 0, stream, ps, rs, in_pos, rope_table, q, kv,
-                           segs, n_heads, qkn));
-  else if (dtype == SJD_BF16)
-    SJD_CUDA(launch_kernel(qkv_finish_kernel<__nv_bfloat16>, grid, dim3(256), 0, stream, ps, rs, in_pos, rope_table, q, kv,
-                           segs, n_heads, qkn));
-  else
-    return SJD_ERR_UNSUPPORTED;
+  auto kernel = kv.head_dim == 128 ? qkv_finish_kernel<__nv_bfloat16, true> : qkv_finish_kernel<__nv_bfloat16, false>;
+  SJD_CUDA(launch_kernel(kernel, dim3(M, per_row), dim3(256), 0, stream, ps, rs, in_pos, rope_table, q, kv, segs, n_heads, qkn));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

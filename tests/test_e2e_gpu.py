@@ -471,6 +471,16 @@ def test_generic_projections(name, over, batch, window):
     assert ctx.info()["tensor_core_projections"] == 0
 
 
+@pytest.mark.parametrize("over,qk_norm", [
+    (dict(head_dim=96, n_heads=4, n_kv_heads=4, d_model=512), True),    # halves of 48 entries: two per lane, some idle
+    (dict(head_dim=32, n_heads=16, n_kv_heads=4), False),              # halves of 16
+])
+def test_rotary_step_of_other_head_sizes(over, qk_norm):
+    """The cache append of the tensor-core pipeline at head sizes without tensor-core attention."""
+    ctx, seqs, n, _ = run_lockstep(WORKLOADS["small-bf16"].with_(**over), batch=2, n_generate=40, max_steps=2, qk_norm=qk_norm)
+    assert ctx.info()["tensor_core_projections"] == 1 and ctx.info()["tensor_core_attention"] == 0
+
+
 @pytest.mark.parametrize("name,batch,window,prompt_len", [
     ("7b-2l", 3, 5, 90),        # 15 rows: eight key groups over seven tile slots, several tiles per slot
     ("7b-2l", 1, 9, 530),       # one sequence whose keys are spread over several CTAs and merged
