@@ -294,7 +294,12 @@ struct GemmTcCall {
   // hi/lo planes [M][n_out[0]], the lo plane act_lo_off elements after the hi plane.
   __nv_bfloat16 *act_hi;
   size_t act_lo_off;
+  // scratch of gemm_tc_share_floats() entries and 160 zeroed counters with which CTA pairs may share the units of a partial last
+  // round (null: they do not)
+  float *share;
+  int *share_flags;
 };
+size_t gemm_tc_share_floats();
 int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream);
 int launch_sum_planes(const float *planes, size_t plane_stride, int splits, float *out, size_t total, int accumulate,
                       cudaStream_t stream);

@@ -61,7 +61,7 @@ struct Layout {
   size_t kv, logits[2], stats[2], row_out, counters, step, status;
   size_t x, qkv, q, attn, act, partial, rope;
   size_t xs_h, xs_attn, xs_act, gemm_planes, ss_part;
-  size_t pass_layers, pass_loc, pass_counter;   // pass_kernel.cu: per-layer table, column locations, grid-barrier counters
+  size_t pass_layers, pass_loc, pass_counter, share_flags;   // pass_kernel.cu: per-layer table, column locations, grid-barrier counters
   size_t committed, n, w_eff, draft, q_kind, q_row, q_draft, in_tok, in_pos;
   size_t ring, ring_stats, n_prev, w_prev;   // Sec. 4.2 (d): retained logits rows (max_ring > 0)
   size_t prompt_lens;                        // [max_batch] prompt length of every sequence
@@ -167,6 +167,7 @@ Layout make_layout(const sjd_model_cfg &c) {
       }
     }
     size_t bytes = need * 4;
+    if (tc && Mp > 64 && bytes < gemm_tc_share_floats() * 4) bytes = gemm_tc_share_floats() * 4;   // shared units use the planes' memory
     for (int sms = 1; sms <= kMaxGemmCtas && tc; ++sms) {   // the one-launch pass of few rows keeps its planes in the same place
       PassPlan pl;
       if (pass_plan(c, sms, &pl) && pl.part_bytes > bytes && sms >= 100) bytes = pl.part_bytes;
@@ -176,6 +177,7 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.pass_layers = take(tc ? (size_t)(c.n_layers + 1) * sizeof(PassLayer) : 0);
   L.pass_loc = take(tc ? (nq + 2 * nk + 2 * c.d_model) / 8 * sizeof(int2) : 0);
   L.pass_counter = take(8);
+  L.share_flags = take(tc ? 160 * 4 : 0);
   L.ss_part = take(Mp * (size_t)resid_gain_parts(c.d_model) * 4);
   L.rope = take((size_t)c.max_seq * (c.head_dim / 2) * sizeof(float2));
   L.committed = take((size_t)c.max_batch * c.max_seq * 4);
@@ -514,6 +516,10 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
     call.store_bf16 = bf16_out ? 1 : 0;
     call.status = status;
     call.n_sms = c->n_ctas;
+    if ((bf16_out || act) && M > 64) {   // nobody reads the planes while one of these launches runs
+      call.share = planes;
+      call.share_flags = c->at<int>(c->lay.share_flags);
+    }
     if (bf16_out || act) {   // the logits projection and the gate|up launch apply the pending row scale themselves
       call.ss_part = rs.ss_part;
       call.n_part = rs.n_part;
@@ -797,6 +803,7 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.counters, 0, ((size_t)cfg->max_batch + 1) * 4);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.status, 0, 4);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.pass_counter, 0, 8);
+  if (e == cudaSuccess && tc_shapes(*cfg)) e = cudaMemset(c->ws + lay.share_flags, 0, 160 * 4);
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     delete c;

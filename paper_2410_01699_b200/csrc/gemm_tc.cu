@@ -201,14 +201,11 @@ __device__ __forceinline__ bool epilogue_all(bool pred) {
   return r != 0;
 }
 
-// 16 tokens of one output column: out[i * ld] = hi[i] + lo[i] (times scale[i], if any), the first n of them.  Nothing but
+// 16 tokens of one output column: out[i * ld] = v[i] (times scale[i], if any), the first n of them.  Nothing but
 // independent adds and stores: an epilogue has a warp or two per scheduler, so every dependent instruction costs its latency
 // (with bounds, type and scale tested per element, 128 tokens took 7 us).
 template <typename O>
-__device__ __forceinline__ void store_column(O *out, size_t ld, const uint32_t *hi, const uint32_t *lo, const float *scale, int n) {
-  float v[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+__device__ __forceinline__ void store_column(O *out, size_t ld, float *v, const float *scale, int n) {
   if (scale) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] *= scale[i];
@@ -427,8 +424,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
         tmem_ld_wait();
         if (!live) continue;
         const float *scale = p.ss_part ? s_scale + m0 : nullptr;
-        if (p.store_bf16) store_column(out_bf16 + (size_t)m0 * p.ldc + n, p.ldc, hi, lo, scale, p.M - m0);
-        else store_column(plane + (size_t)m0 * p.ldc + n, p.ldc, hi, lo, scale, p.M - m0);
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+        if (p.store_bf16) store_column(out_bf16 + (size_t)m0 * p.ldc + n, p.ldc, v, scale, p.M - m0);
+        else store_column(plane + (size_t)m0 * p.ldc + n, p.ldc, v, scale, p.M - m0);
       }
       }
     } else if (tid == 64) {
@@ -456,12 +456,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
 // 200 x 22016 x 4096 102 -> 61, 1024 x 12288 x 4096 169 -> 135 (1.5 PFLOP/s issued).
 constexpr int kPairStages = 8;
 constexpr int kPairThreads = 64 + 256;   // producer, issuer, eight epilogue warps
+constexpr int kShareParts = 4;           // most pairs that share a unit
 constexpr int kExTokens = 16;            // tokens of one exchange round of the gate|up epilogue
 
 struct PairParams {
   GemmParams g;
-  int tiles, pairs;      // 128-row weight tiles, pairs of them
+  int tiles;             // 128-row weight tiles
   int n_units;
+  // Units of the last, partial round (from unit `full` on) that several pairs share: `parts` pairs take a range of K each;
+  // the first adds the others' sums (scratch [unit][part - 1][rank][token][128]) to its own before the epilogue.  The grid is
+  // resident at once and the others wait for nothing.
+  int full, parts;
+  float *scratch;
+  int *flags;            // [unit][rank] arrivals, zero before and after a launch
 };
 
 __device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
@@ -558,18 +565,29 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
   tc_fence_after();
   const uint32_t tmem_base = s_tmem_base;
 
-  // unit -> this CTA's weight tile, k-blocks, slab
+  // the n-th unit of this pair: this CTA's weight tile, k-blocks, slab; part of a shared unit
   struct Unit {
-    int tile, kb0, kb1, split, slab;
+    int tile, kb0, kb1, split, slab, part, shared;   // shared: index among the shared units, -1: not one
   };
-  auto unit_of = [&](int u) {
+  const int n_full = q.parts > 1 ? q.full / n_pairs : (q.n_units - pair + n_pairs - 1) / n_pairs;
+  const int n_local = n_full + (q.parts > 1 && pair < (q.n_units - q.full) * q.parts ? 1 : 0);
+  auto unit_of = [&](int n) {
     Unit t;
+    t.part = 0;
+    t.shared = -1;
+    int u = pair + n * n_pairs;
+    if (n >= n_full) {
+      t.shared = pair / q.parts;
+      t.part = pair - t.shared * q.parts;
+      u = q.full + t.shared;
+    }
     t.slab = u % p.n_slabs;
     const int v = u / p.n_slabs;
     t.split = v % p.splits;
     t.tile = (v / p.splits) * 2 + (int)rank;
-    t.kb0 = (int)(((long)t.split * p.k_blocks) / p.splits);
-    t.kb1 = (int)(((long)(t.split + 1) * p.k_blocks) / p.splits);
+    const int at = t.shared >= 0 ? t.part : t.split, of = t.shared >= 0 ? q.parts : p.splits;
+    t.kb0 = (int)(((long)at * p.k_blocks) / of);
+    t.kb1 = (int)(((long)(at + 1) * p.k_blocks) / of);
     return t;
   };
   auto mat_of = [&](int tile) { return GU ? 0 : tile < p.tile_end[0] ? 0 : tile < p.tile_end[1] ? 1 : 2; };
@@ -596,8 +614,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
     };
     // the weights do not depend on the preceding kernel: those of the first stages are fetched before the wait
     int pre = 0, it = 0;
-    if (pair < q.n_units) {
-      const Unit t = unit_of(pair);
+    if (n_local > 0) {
+      const Unit t = unit_of(0);
       const Src c = src_of(t);
       for (; pre < p.stages && t.kb0 + pre < t.kb1; ++pre) {
         if (elect_one()) load_w(c, t.kb0 + pre, pre);
@@ -608,8 +626,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
     int s = 0;
     uint32_t ph = 0;
     bool ok = true;
-    for (int u = pair; u < q.n_units && ok; u += n_pairs) {
-      const Unit t = unit_of(u);
+    for (int n = 0; n < n_local && ok; ++n) {
+      const Unit t = unit_of(n);
       const Src c = src_of(t);
       const int x_row = (rank ? p.x_lo_row : 0) + t.slab * p.Mp;
       for (int kb = t.kb0; kb < t.kb1; ++kb, ++it) {
@@ -632,11 +650,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
     if (rank == 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       const uint64_t desc0 = umma_desc_sw128(0);
-      int s = 0, n = 0;
+      int s = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int u = pair; u < q.n_units && ok; u += n_pairs, ++n) {
-        const Unit t = unit_of(u);
+      for (int n = 0; n < n_local && ok; ++n) {
+        const Unit t = unit_of(n);
         const int buf = n & 1;
         if (!warp_wait(&acc_empty[buf], ((n >> 1) & 1) ^ 1u)) { ok = false; break; }
         tc_fence_after();
@@ -664,9 +682,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
     const int quarter = warp & 3, row = quarter * 32 + lane, grp = (warp - 2) >> 2, e = (tid - 64) & 127;
     float *ex = reinterpret_cast<float *>(smem + p.stages * stage_bytes) + grp * TILE_N * (kExTokens + 1);   // GU: [128][kExTokens + 1]
     pdl_wait();   // the planes may still be read, and the row scales written, by the preceding kernel
-    int n = 0, have_slab = -1;
-    for (int u = pair; u < q.n_units; u += n_pairs, ++n) {
-      const Unit t = unit_of(u);
+    int have_slab = -1;
+    for (int n = 0; n < n_local; ++n) {
+      const Unit t = unit_of(n);
       const int buf = n & 1, m_base = t.slab * p.Mp;
       if ((p.ss_part || GU) && have_slab != t.slab) {   // RMS scale of the slab's token rows
         have_slab = t.slab;
@@ -690,19 +708,72 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * NN;
       const int mat = mat_of(t.tile), m_left = p.M - m_base;
-      if (GU) {
+      const bool helper = t.part > 0;
+      const int n_add = t.shared >= 0 && !helper ? q.parts - 1 : 0;   // sums to add
+      const size_t piece = (size_t)2 * p.Mp * TILE_N;
+      float *share = q.scratch + (size_t)(t.shared < 0 ? 0 : t.shared) * (q.parts - 1) * piece + (size_t)rank * p.Mp * TILE_N + row;
+      int *flag = q.flags + (t.shared < 0 ? 0 : t.shared) * 2 + rank;
+      if (n_add) {
+        bool there = true;
+        if (tid == 64) {
+          const unsigned long long t0 = global_ns();
+          for (int i = 0;; ++i) {
+            int v;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+            if (v == n_add) break;
+            if ((i & 255) == 255 && global_ns() - t0 > kWaitNs) { there = false; break; }
+          }
+          *flag = 0;
+        }
+        if (!pair_epilogue_all(there)) {
+          if (tid == 64) atomicExch(p.status, 5);
+          break;
+        }
+      }
+      // 16 tokens of this thread's row: hi + lo plane, and the other parts of a shared unit
+      auto sums = [&](int m0, float *v) {
+        uint32_t hi[16], lo[16];
+        tmem_ld16_issue(t_addr + m0, hi);
+        tmem_ld16_issue(t_addr + p.Mp + m0, lo);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+        if (n_add) {   // all loads in flight at once: one round trip per 16 tokens
+          float w[kShareParts - 1][16];
+#pragma unroll
+          for (int k = 0; k < kShareParts - 1; ++k)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[k][i] = k < n_add ? __ldcg(share + k * piece + (size_t)(m0 + i) * TILE_N) : 0.0f;
+#pragma unroll
+          for (int k = 0; k < kShareParts - 1; ++k)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] += w[k][i];
+        }
+      };
+      if (helper) {
+        float *dst = share + (t.part - 1) * piece;
+        for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
+          float v[16];
+          sums(m0, v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) dst[(size_t)(m0 + i) * TILE_N] = v[i];
+        }
+        __threadfence();
+        pair_epilogue_all(true);
+        if (tid == 64) {
+          __threadfence();
+          atomicAdd(flag, 1);
+        }
+      } else if (GU) {
         // MMA rows 0..63 hold gate features, rows 64..127 the same features of the up matrix: they meet in shared memory, 16
         // tokens at a time; then thread e finishes feature e % 64 for every second token
         const int fr = e & 63, f = t.tile * R + fr, odd = e >> 6;
         const bool live = fr < R && f < p.F;
         for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
-          uint32_t hi[16], lo[16];
-          tmem_ld16_issue(t_addr + m0, hi);
-          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
-          tmem_ld_wait();
+          float a[16];
+          sums(m0, a);
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            ex[row * (kExTokens + 1) + i] = (__uint_as_float(hi[i]) + __uint_as_float(lo[i])) * s_scale[m0 + i];
+          for (int i = 0; i < 16; ++i) ex[row * (kExTokens + 1) + i] = a[i] * s_scale[m0 + i];
           asm volatile("bar.sync %0, 128;" ::"r"(grp + 2) : "memory");
           if (live) {
             __nv_bfloat16 *dst = p.act_hi + (size_t)(m_base + m0 + odd) * p.F + f;
@@ -729,14 +800,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
         float *plane = reinterpret_cast<float *>(p.out) + (size_t)t.split * p.plane_stride + (size_t)m_base * p.ldc + col;
         __nv_bfloat16 *logits = reinterpret_cast<__nv_bfloat16 *>(p.out) + (size_t)m_base * p.ldc + col;
         for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
-          uint32_t hi[16], lo[16];
-          tmem_ld16_issue(t_addr + m0, hi);
-          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
-          tmem_ld_wait();
+          float v[16];
+          sums(m0, v);
           if (!live) continue;
           const float *scale = p.ss_part ? s_scale + m0 : nullptr;
-          if (p.store_bf16) store_column(logits + (size_t)m0 * p.ldc, p.ldc, hi, lo, scale, m_left - m0);
-          else store_column(plane + (size_t)m0 * p.ldc, p.ldc, hi, lo, scale, m_left - m0);
+          if (p.store_bf16) store_column(logits + (size_t)m0 * p.ldc, p.ldc, v, scale, m_left - m0);
+          else store_column(plane + (size_t)m0 * p.ldc, p.ldc, v, scale, m_left - m0);
         }
       }
       tc_fence_before();
@@ -850,6 +919,8 @@ int gemm_tc_splits(const GemmTcPlan &pl, int tiles, int k_blocks, int n_sms) {
   s = s > 16 ? 16 : s;
   return s < 1 ? 1 : s;
 }
+size_t gemm_tc_share_floats() { return (size_t)(160 / 2) * 2 * 128 * TILE_N; }   // a shared part per pair: 128 tokens of both CTAs
+
 int gemm_tc_splits_max(const GemmTcPlan &pl, int tiles, int k_blocks) {
   int most = 1;
   for (int sms = 132; sms <= 160; sms += 2) {
@@ -863,8 +934,7 @@ static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles,
   PairParams q;
   q.g = p;
   q.tiles = tiles;
-  q.pairs = (tiles + 1) / 2;
-  q.n_units = q.pairs * p.n_slabs * p.splits;
+  q.n_units = (tiles + 1) / 2 * p.n_slabs * p.splits;
   const bool gu = g.act_hi != nullptr;
   const int stage_bytes = W_TILE_BYTES + p.Mp * TILE_K * 2;
   const int ex = gu ? 2 * TILE_N * (kExTokens + 1) * 4 : 0;
@@ -880,7 +950,21 @@ static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles,
   auto kernel = gu ? gemm_pair_kernel<true> : gemm_pair_kernel<false>;
   SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int sms = g.n_sms > 1 ? g.n_sms : 148;
-  const int pairs = q.n_units < sms / 2 ? q.n_units : sms / 2;
+  // The units of a partial last round are shared where K may not be split otherwise and the launch has few rounds: one token slab
+  // (7B gate|up at 128 rows: 86 units for 74 pairs, 2 rounds without, 1.25 with; 8 layers 1131 -> 1084 us at 80 rows, 1280 ->
+  // 1240 at 128; at 192 and 256 rows, 3 rounds against 2.4, nothing to 2 % slower).
+  int pairs = sms / 2;
+  q.full = q.n_units / pairs * pairs;
+  const int tail = q.n_units - q.full;
+  q.parts = tail > 0 ? pairs / tail : 1;
+  if (q.parts > p.k_blocks / 4) q.parts = p.k_blocks / 4;
+  if (q.parts > kShareParts) q.parts = kShareParts;
+  q.scratch = g.share;
+  q.flags = g.share_flags;
+  if (!g.share || p.splits != 1 || p.n_slabs > 1 || q.parts < 2) {
+    q.parts = 1;
+    pairs = q.n_units < pairs ? q.n_units : pairs;
+  }
   SJD_CUDA(launch_kernel(kernel, dim3(2 * pairs), dim3(kPairThreads), smem, stream, w0, w1, w2, xm, q));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
