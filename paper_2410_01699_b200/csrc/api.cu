@@ -175,7 +175,6 @@ void timeline_set_gemm(TimelineBuf *);
 void timeline_set_attn(TimelineBuf *);
 void timeline_set_combine(TimelineBuf *);
 void timeline_set_verify(TimelineBuf *);
-void timeline_set_pass(TimelineBuf *);
 }  // namespace sjd
 extern "C" int sjd_timeline_attach(void *device_buf) {
   TimelineBuf *b = (TimelineBuf *)device_buf;
@@ -184,7 +183,6 @@ extern "C" int sjd_timeline_attach(void *device_buf) {
   timeline_set_attn(b);
   timeline_set_combine(b);
   timeline_set_verify(b);
-  timeline_set_pass(b);
   return SJD_OK;
 }
 extern "C" size_t sjd_timeline_bytes(void) { return sizeof(TimelineBuf); }

@@ -390,8 +390,8 @@ typedef CUresult (*EncodeTiledFn3)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 
 }  // namespace
 
-// bf16 cache [planes][max_seq][head_dim] as boxes of `keys` rows x 64 dims, 128-byte swizzle
-int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim, int keys) {
+// bf16 cache [planes][max_seq][head_dim] as boxes of 64 keys x 64 dims, 128-byte swizzle
+int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim) {
   static EncodeTiledFn3 fn = nullptr;
   if (!fn) {
     void *sym = nullptr;
@@ -404,7 +404,7 @@ int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_s
   if (((uintptr_t)base & 15u) != 0 || (head_dim != 64 && head_dim != 128)) return SJD_ERR_UNSUPPORTED;
   cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)max_seq, (cuuint64_t)planes};
   cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, (cuuint64_t)max_seq * head_dim * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)keys, 1};
+  cuuint32_t box[3] = {64, (cuuint32_t)KT, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = fn(reinterpret_cast<CUtensorMap *>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base),
                         dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,

@@ -379,56 +379,13 @@ int launch_attention(int dtype, const float *q, KvLayout kv, const int32_t *in_p
 // merge of the split-KV partials only (used after launch_attention_mma); out may be null when only the hi/lo planes are wanted
 int launch_attention_combine(const float *partial, const int32_t *in_pos, float *out, int M, int n_heads, int head_dim,
                              int splits, cudaStream_t stream, HiLoOut hilo);
-// tensor-core split-KV attention for bf16 caches (attention_mma.cu); the map's boxes hold `keys` rows of 64 entries
-int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim, int keys = KV_PAGE);
+// tensor-core split-KV attention for bf16 caches (attention_mma.cu)
+int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim);
 bool attention_mma_supported(int head_dim, int rows_per_seq);
 // plane0: first plane of this layer in the contiguous map [planes][max_seq][hd]; with kv.page_table set the map is
 // the pool's [planes][KV_PAGE][hd] and the plane of a tile comes from the page table.
 int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const float *q, const int32_t *in_pos, float *partial,
                          float *out, HiLoOut hilo, int *status, int M, RowSegs segs, int n_heads, int n_kv_heads,
                          int head_dim, int splits, cudaStream_t stream);
-
-// ---- a whole forward pass of at most kPassMaxRows rows as one cooperative launch (pass_kernel.cu)
-constexpr int kPassMaxRows = 64, kPassMaxPieces = 10;
-struct PassGemm {        // one projection: tiles of rows[j] weight rows of up to three matrices, kb k-blocks of 64
-  int kb, tiles, full;   // full: tiles dealt whole to the CTAs; else tiles * kb units cut evenly
-  int rows[3], n_out[3], tile_end[3];
-  int max_pieces;        // partial planes per tile
-};
-struct PassPlan {
-  PassGemm gemm[5];      // Q|K|V, O, gate|up, down, logits
-  int slot_bytes, n_w;   // weight ring
-  int part_ld;           // row stride of the partial planes
-  size_t part_bytes;
-};
-struct PassLayer {       // device table, one entry per layer; one more holds the logits matrix (w[0]) and the final norm (attn_norm)
-  TensorMap w[7];        // wq, wk, wv, wo, gate, up, down
-  const __nv_bfloat16 *attn_norm, *ffn_norm, *q_norm, *k_norm;
-};
-struct PassParams {
-  TensorMap h_map, attn_map, act_map, kv_map, q_map;
-  PassGemm gemm[5];
-  int slot_bytes, n_w, part_ld;
-  const PassLayer *layers;
-  const __nv_bfloat16 *tok_emb;
-  const int32_t *in_tok, *in_pos, *seg_seq;
-  const int2 *loc_qkv, *loc_o, *loc_down;   // where a column's partial planes are, an entry per 8 columns
-  float *x, *part, *partial, *partial_ml, *ss_part;   // partial: [M][H][splits][hd], partial_ml: [M][H][splits] (max, sum)
-  HiLoOut h, attn, act, qs;   // qs: queries times log2(e) / sqrt(head_dim)
-  __nv_bfloat16 *logits;   // null: pre-fill
-  const float2 *rope;
-  void *kv_base;
-  const int32_t *page_table;
-  int pages_per_seq, planes_per_layer, max_seq;
-  int n_layers, d, F, vocab, n_heads, n_kv_heads, head_dim;
-  int M, Mp, n_segs, rows, x_lo_row;
-  int splits, key_groups;
-  float eps;
-  uint32_t *counter;       // [0] arrivals at the grid barriers so far, [1] their number before this launch
-  int *status;
-};
-bool pass_plan(const sjd_model_cfg &c, int n_sms, PassPlan *plan);   // false: the model is not covered
-void pass_locations(const PassPlan &plan, int n_sms, int2 *out);   // (nq + 2 nk + 2 d) / 8 entries
-int launch_pass(const PassParams &p, int n_sms, cudaStream_t stream);
 
 }  // namespace sjd

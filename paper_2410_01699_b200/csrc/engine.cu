@@ -40,10 +40,6 @@ constexpr int kGuRows = 64;
 // more fp32 buffers per row and is not bound by the weights: 256 rows.
 constexpr int kPrefillRowsTc = 1152, kPrefillRowsGeneric = 256;
 constexpr int kMaxTcRows = 1152;     // largest pass of the tensor-core pipeline
-// Passes of at most kPassMaxRows rows run as one launch when a layer streams enough weights to hide its chain behind: per
-// step, 4 layers of 405 MB take 417 / 444 / 555 us at 8 / 32 / 64 rows (separate launches: 438 / 488 / 566), 8 layers of
-// 101 MB 553 / 625 / 739 us (457 / 534 / 656).  Two points of one family: the line is between them.
-constexpr double kOneLaunchLayerBytes = 192e6;
 
 struct WMap {
   TensorMap map;
@@ -61,7 +57,7 @@ struct Layout {
   size_t kv, logits[2], stats[2], row_out, counters, step, status;
   size_t x, qkv, q, attn, act, partial, rope;
   size_t xs_h, xs_attn, xs_act, gemm_planes, ss_part;
-  size_t pass_layers, pass_loc, pass_counter, share_flags;   // pass_kernel.cu: per-layer table, column locations, grid-barrier counters
+  size_t share_flags;                        // counters of CTA pairs that share a tile (gemm_tc.cu)
   size_t committed, n, w_eff, draft, q_kind, q_row, q_draft, in_tok, in_pos;
   size_t ring, ring_stats, n_prev, w_prev;   // Sec. 4.2 (d): retained logits rows (max_ring > 0)
   size_t prompt_lens;                        // [max_batch] prompt length of every sequence
@@ -128,7 +124,7 @@ Layout make_layout(const sjd_model_cfg &c) {
   L.step = take(4);
   L.status = take(4);
   L.x = take(Mp * c.d_model * 4);
-  L.q = take((Mp + 15) / 16 * 16 * nq * 4);   // fp32, or (pass_kernel.cu) two bf16 planes
+  L.q = take(Mp * nq * 4);
   {   // a context runs one of the two pipelines: the generic one's buffers share their memory with the other's planes
     const size_t generic = align256(Mg * (nq + 2 * nk) * 4) + align256(Mg * nq * 4) + align256(Mg * act_stride(c) * 4);
     const size_t Ma = (Mp + 15) / 16 * 16;
@@ -168,15 +164,8 @@ Layout make_layout(const sjd_model_cfg &c) {
     }
     size_t bytes = need * 4;
     if (tc && Mp > 64 && bytes < gemm_tc_share_floats() * 4) bytes = gemm_tc_share_floats() * 4;   // shared units use the planes' memory
-    for (int sms = 1; sms <= kMaxGemmCtas && tc; ++sms) {   // the one-launch pass of few rows keeps its planes in the same place
-      PassPlan pl;
-      if (pass_plan(c, sms, &pl) && pl.part_bytes > bytes && sms >= 100) bytes = pl.part_bytes;
-    }
     L.gemm_planes = take(bytes);
   }
-  L.pass_layers = take(tc ? (size_t)(c.n_layers + 1) * sizeof(PassLayer) : 0);
-  L.pass_loc = take(tc ? (nq + 2 * nk + 2 * c.d_model) / 8 * sizeof(int2) : 0);
-  L.pass_counter = take(8);
   L.share_flags = take(tc ? 160 * 4 : 0);
   L.ss_part = take(Mp * (size_t)resid_gain_parts(c.d_model) * 4);
   L.rope = take((size_t)c.max_seq * (c.head_dim / 2) * sizeof(float2));
@@ -323,7 +312,9 @@ struct sjd_ctx {
   cudaStream_t last_stream;
   // One captured CUDA graph of the forward pass per logits-buffer parity (up to 290 launches: replaying a graph takes the
   // host out of the critical path).  It holds nothing that belongs to a call: the verification, which takes the caller's
-  // output pointers, is launched behind it, so that the graphs serve every pre-fill with the same batch and window.
+  // output pointers, is launched behind it, so that the graphs serve every pre-fill with the same batch and window.  The first
+  // two steps after a pre-fill are launched directly unless there are graphs already: the capture (0.7 ms of host time each at 32
+  // layers) then runs while they do.
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     long long launches = 0;
@@ -349,10 +340,6 @@ struct sjd_ctx {
   std::map<int, XMaps> xmaps;   // keyed by padded row count
   TensorMap kv_map;             // whole KV cache as [planes][max_seq][head_dim]
   bool kv_map_valid = false;
-  bool use_pass = false;        // passes of at most kPassMaxRows rows run as one launch (pass_kernel.cu)
-  PassPlan pass;
-  TensorMap kv_map16;           // the cache in boxes of 16 keys
-  std::map<int, TensorMap> q_maps;   // hi/lo planes of the queries in boxes of a segment's rows
   int rows_alloc() const { return ((int)lay.pass_rows + 15) / 16 * 16; }
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
@@ -586,92 +573,11 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
 #undef SJD_TR
 #undef SJD_TRY
 
-// the same pass as one cooperative launch
-int forward_one_launch(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
-  const sjd_model_cfg &g = c->cfg;
-  const int M = n_segs * segs.rows, Ma = c->rows_alloc();
-  const SeqState st = c->state();
-  PassParams p;
-  memset(&p, 0, sizeof(p));
-  p.h_map = xm.h;
-  p.attn_map = xm.attn;
-  p.act_map = xm.act;
-  p.kv_map = c->kv_map16;
-  auto qm = c->q_maps.find(segs.rows);
-  if (qm == c->q_maps.end()) {
-    TensorMap m;
-    const int rc = make_tensor_map_bf16(&m, c->ws + c->lay.q, 2L * Ma, (long)g.n_heads * g.head_dim, segs.rows);
-    if (rc != SJD_OK) return rc;
-    qm = c->q_maps.emplace(segs.rows, m).first;
-  }
-  p.q_map = qm->second;
-  memcpy(p.gemm, c->pass.gemm, sizeof(p.gemm));
-  p.slot_bytes = c->pass.slot_bytes;
-  p.n_w = c->pass.n_w;
-  p.part_ld = c->pass.part_ld;
-  p.layers = c->at<PassLayer>(c->lay.pass_layers);
-  p.tok_emb = (const __nv_bfloat16 *)c->tok_emb;
-  p.in_tok = st.in_tok;
-  p.in_pos = st.in_pos;
-  p.seg_seq = segs.seq;
-  p.x = c->at<float>(c->lay.x);
-  const size_t nq = (size_t)g.n_heads * g.head_dim, nk = (size_t)g.n_kv_heads * g.head_dim;
-  p.loc_qkv = c->at<int2>(c->lay.pass_loc);
-  p.loc_o = p.loc_qkv + (nq + 2 * nk) / 8;
-  p.loc_down = p.loc_o + g.d_model / 8;
-  p.part = c->at<float>(c->lay.gemm_planes);
-  p.partial = c->at<float>(c->lay.partial);
-  p.ss_part = c->at<float>(c->lay.ss_part);
-  p.h = HiLoOut{c->at<__nv_bfloat16>(c->lay.xs_h), (size_t)Ma * g.d_model};
-  p.attn = HiLoOut{c->at<__nv_bfloat16>(c->lay.xs_attn), (size_t)Ma * nq};
-  p.qs = HiLoOut{c->at<__nv_bfloat16>(c->lay.q), (size_t)Ma * nq};
-  p.act = HiLoOut{c->at<__nv_bfloat16>(c->lay.xs_act), (size_t)Ma * g.ffn_hidden};
-  p.logits = (__nv_bfloat16 *)logits_out;
-  p.rope = c->at<float2>(c->lay.rope);
-  p.kv_base = c->ws + c->lay.kv;
-  p.page_table = g.kv_pages > 0 ? c->at<int32_t>(c->lay.page_table) : nullptr;
-  p.pages_per_seq = g.kv_pages > 0 ? c->pages_per_seq() : 0;
-  p.planes_per_layer = g.max_batch * 2 * g.n_kv_heads;
-  p.max_seq = g.max_seq;
-  p.n_layers = g.n_layers;
-  p.d = g.d_model;
-  p.F = g.ffn_hidden;
-  p.vocab = g.vocab;
-  p.n_heads = g.n_heads;
-  p.n_kv_heads = g.n_kv_heads;
-  p.head_dim = g.head_dim;
-  p.M = M;
-  p.Mp = (M + 15) / 16 * 16;
-  p.n_segs = n_segs;
-  p.rows = segs.rows;
-  p.x_lo_row = Ma;
-  const int s = c->n_ctas / (g.n_heads * n_segs);   // key ranges per head: no more than the grid has CTAs for
-  p.splits = s < 1 ? 1 : s > 16 ? 16 : s;
-  p.partial_ml = p.partial + (size_t)M * g.n_heads * p.splits * g.head_dim;
-  p.key_groups = segs.rows <= 16 ? 8 : segs.rows <= 32 ? 4 : 2;
-  p.eps = g.rms_eps;
-  p.counter = c->at<uint32_t>(c->lay.pass_counter);
-  p.status = c->at<int>(c->lay.status);
-  Tracer &tr = c->tracer;
-  if (tr.on) tr.gemm_weight_bytes += 2.0 * ((double)g.n_layers * ((double)g.d_model * (2.0 * g.n_heads + 2.0 * g.n_kv_heads) * g.head_dim +
-                                             3.0 * (double)g.ffn_hidden * g.d_model) + (logits_out ? (double)g.vocab * g.d_model : 0.0));
-  tr.begin(TC_GEMM, stream);
-  const int rc = launch_pass(p, c->n_ctas, stream);
-  tr.end(stream);
-  return rc;
-}
-
-// whether a pass of M rows is one cooperative launch
-bool one_launch(const sjd_ctx *c, int M) {
-  return c->use_tc && c->all_tc && c->use_pass && M <= kPassMaxRows && c->xmaps.count((M + 15) / 16 * 16) != 0;
-}
-
 int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const int M = n_segs * segs.rows;
   if (c->use_tc && c->all_tc && M <= kMaxTcRows) {
     auto it = c->xmaps.find((M + 15) / 16 * 16);
     if (it != c->xmaps.end()) {
-      if (one_launch(c, M)) return forward_one_launch(c, it->second, n_segs, segs, logits_out, stream);
       // every kernel of this pipeline waits for its predecessor itself: launch them overlapped
       g_pdl = !c->tracer.on;
       const int rc = forward_tc(c, it->second, n_segs, segs, logits_out, stream);
@@ -802,7 +708,6 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
   cudaError_t e = cudaMemcpy(c->ws + lay.rope, table.data(), table.size() * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.counters, 0, ((size_t)cfg->max_batch + 1) * 4);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.status, 0, 4);
-  if (e == cudaSuccess) e = cudaMemset(c->ws + lay.pass_counter, 0, 8);
   if (e == cudaSuccess && tc_shapes(*cfg)) e = cudaMemset(c->ws + lay.share_flags, 0, 160 * 4);
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
@@ -846,39 +751,6 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
         make_kv_tensor_map(&c->kv_map, c->ws + lay.kv, planes, plane_rows, cfg->head_dim) == SJD_OK &&
         cudaMemset(c->ws + lay.kv, 0, (size_t)planes * plane_rows * cfg->head_dim * 2) == cudaSuccess)
       c->kv_map_valid = true;
-    // passes of few rows as one launch: per-layer tensor maps with the tile heights of its plan
-    int coop = 0;
-    const double layer_bytes = 2.0 * ((double)d * (2 * nq + 2 * nk) + 3.0 * (double)F * d);
-    if (tc_shapes(*cfg) && layer_bytes >= kOneLaunchLayerBytes && c->kv_map_valid && sms <= kMaxGemmCtas && pass_plan(*cfg, sms, &c->pass) &&
-        c->pass.part_bytes <= lay.pass_layers - lay.gemm_planes &&
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        make_kv_tensor_map(&c->kv_map16, c->ws + lay.kv, planes, plane_rows, cfg->head_dim, 16) == SJD_OK) {
-      std::vector<PassLayer> pls((size_t)L + 1);
-      memset((void *)pls.data(), 0, pls.size() * sizeof(PassLayer));
-      bool ok = true;
-      auto map = [&](TensorMap &m, const void *w, int n, int k, int rows) { ok = ok && make_tensor_map_bf16(&m, w, n, k, rows) == SJD_OK; };
-      const PassPlan &pp = c->pass;
-      for (int l = 0; l < L; ++l) {
-        PassLayer &pl = pls[l];
-        map(pl.w[0], c->wq[l], nq, d, pp.gemm[0].rows[0]);
-        map(pl.w[1], c->wk[l], nk, d, pp.gemm[0].rows[1]);
-        map(pl.w[2], c->wv[l], nk, d, pp.gemm[0].rows[2]);
-        map(pl.w[3], c->wo[l], d, nq, pp.gemm[1].rows[0]);
-        map(pl.w[4], c->w_gate[l], F, d, pp.gemm[2].rows[0]);
-        map(pl.w[5], c->w_up[l], F, d, pp.gemm[2].rows[0]);
-        map(pl.w[6], c->w_down[l], d, F, pp.gemm[3].rows[0]);
-        pl.attn_norm = (const __nv_bfloat16 *)c->attn_norm[l];
-        pl.ffn_norm = (const __nv_bfloat16 *)c->ffn_norm[l];
-        pl.q_norm = (const __nv_bfloat16 *)c->q_norm[l];
-        pl.k_norm = (const __nv_bfloat16 *)c->k_norm[l];
-      }
-      map(pls[L].w[0], c->lm_head, cfg->vocab, d, pp.gemm[4].rows[0]);
-      pls[L].attn_norm = (const __nv_bfloat16 *)c->final_norm;
-      std::vector<int2> loc(((size_t)nq + 2 * nk + 2 * d) / 8);
-      pass_locations(pp, sms, loc.data());
-      ok = ok && cudaMemcpy(c->ws + lay.pass_loc, loc.data(), loc.size() * sizeof(int2), cudaMemcpyHostToDevice) == cudaSuccess;
-      c->use_pass = ok && cudaMemcpy(c->ws + lay.pass_layers, pls.data(), pls.size() * sizeof(PassLayer), cudaMemcpyHostToDevice) == cudaSuccess;
-    }
     for (int l = 0; l < L; ++l) {
       const LayerMaps &lm = c->wmaps[l];
       c->all_tc = c->all_tc && lm.wq.valid && lm.wk.valid && lm.wv.valid && lm.wo.valid && lm.gate_gu.valid &&
@@ -1020,7 +892,7 @@ extern "C" int sjd_step(sjd_ctx *c, const sjd_step_out *out, void *cuda_stream) 
   const RowSegs segs{c->window, nullptr};
   void *logits = c->ws + c->lay.logits[cur];
   bool replayed = false;
-  if (c->graphs_enabled && !c->tracer.on && !one_launch(c, c->batch * c->window)) {
+  if (c->graphs_enabled && !c->tracer.on && (c->host_step >= 2 || c->graphs[cur].exec)) {
     sjd_ctx::StepGraph &g = c->graphs[cur];
     if (!g.exec) {
       // capture on a private stream (the caller's may be the legacy default stream), replay on the caller's
@@ -1104,7 +976,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
       (tc && c->kv_map_valid && attention_mma_supported(c->cfg.head_dim, c->window)) ? 1 : 0;
-  info->step_graph = c->graphs_enabled && !one_launch(c, M) ? 1 : 0;
+  info->step_graph = c->graphs_enabled ? 1 : 0;
   info->rows_per_step = M;
   return SJD_OK;
 }

@@ -482,13 +482,12 @@ def test_rotary_step_of_other_head_sizes(over, qk_norm):
 
 
 @pytest.mark.parametrize("name,batch,window,prompt_len", [
-    ("7b-2l", 3, 5, 90),        # 15 rows: eight key groups over seven tile slots, several tiles per slot
+    ("7b-2l", 3, 5, 90),        # 15 rows
     ("7b-2l", 1, 9, 530),       # one sequence whose keys are spread over several CTAs and merged
-    ("8b-gqa-2l", 2, 31, 70),   # 62 rows, four query heads per K/V head, two accumulators per tile
+    ("8b-gqa-2l", 2, 31, 70),   # 62 rows, four query heads per K/V head
 ])
-def test_one_launch_pass(name, batch, window, prompt_len):
-    """Passes of at most 64 rows on wide layers run as one launch: row counts off the 16-row grid, every key-group
-    layout of its attention."""
+def test_wide_layers_ragged_rows(name, batch, window, prompt_len):
+    """Row counts off the 16-row grid on the 7B / 8B layer shapes."""
     ctx, seqs, n, _ = run_lockstep(WORKLOADS[name].with_(prompt_len=prompt_len), batch=batch, window=window, max_steps=2,
                                    gain_jitter=0.1)
     for s in seqs:
