@@ -2396,8 +2396,10 @@ __global__ void __launch_bounds__(kClThreads, 2) verify_cluster_kernel(const Ver
   ClScratch<CS> &cs = *reinterpret_cast<ClScratch<CS> *>(dyn_smem);
   __shared__ Scratch sc;
   pdl_trigger();
+  SJD_TL(TL_VERIFY, 0, threadIdx.x == 0);
   cl_sync<CS>();   // every block of the cluster has started: its shared memory may be written
   pdl_wait();
+  SJD_TL(TL_VERIFY, 1, threadIdx.x == 0);
   const int rank = (int)(blockIdx.x % CS);
   RowJob<T> j;
   if (row_job<T>(p, (int)(blockIdx.x / CS), j)) {
