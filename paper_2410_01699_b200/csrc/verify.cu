@@ -25,6 +25,9 @@
 // threshold) or next to +-0 use the general route above; both routes produce the same threshold and
 // the same weights.  Longer bf16 rows (the 184320-entry head) take the same route streamed: a full block
 // passes the row through its registers in segments of 65536 entries, once per phase (long_statistics).
+//
+// Few rows, and fp32 rows of more than 2048 entries, are verified by a thread-block cluster per row instead
+// (verify_cluster_kernel; the rule is in launch_verify_t).
 #include <float.h>
 
 #include <type_traits>
