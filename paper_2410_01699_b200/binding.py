@@ -292,22 +292,24 @@ class Context:
     def prefill(self, prompt, sample: sjd_sample_cfg):
         """prompt: int32 cuda tensor [B][P]."""
         assert prompt.dtype == torch.int32 and prompt.is_cuda and prompt.is_contiguous()
-        self._prompt = prompt
-        self.batch, self.window = int(prompt.shape[0]), int(sample.window)
-        self._guided = float(sample.guidance) != 0.0
-        _check(lib().sjd_prefill(self._ctx, self.batch, _ptr(prompt), int(prompt.shape[1]), C.byref(sample),
+        _check(lib().sjd_prefill(self._ctx, int(prompt.shape[0]), _ptr(prompt), int(prompt.shape[1]), C.byref(sample),
                                  _stream()), "sjd_prefill")
+        self._prefilled(prompt, sample)
 
     def prefill_ragged(self, prompt, prompt_lens, sample: sjd_sample_cfg):
         """prompt: int32 cuda tensor [B][row_stride]; prompt_lens: B host integers (sequence b uses the first
         prompt_lens[b] tokens of its row)."""
         assert prompt.dtype == torch.int32 and prompt.is_cuda and prompt.is_contiguous()
+        batch = int(prompt.shape[0])
+        lens = (C.c_int32 * batch)(*[int(x) for x in prompt_lens])
+        _check(lib().sjd_prefill_ragged(self._ctx, batch, _ptr(prompt), lens, int(prompt.shape[1]), C.byref(sample),
+                                        _stream()), "sjd_prefill_ragged")
+        self._prefilled(prompt, sample)
+
+    def _prefilled(self, prompt, sample):   # (a refused call changes nothing: the generation under way can go on)
         self._prompt = prompt
         self.batch, self.window = int(prompt.shape[0]), int(sample.window)
         self._guided = float(sample.guidance) != 0.0
-        lens = (C.c_int32 * self.batch)(*[int(x) for x in prompt_lens])
-        _check(lib().sjd_prefill_ragged(self._ctx, self.batch, _ptr(prompt), lens, int(prompt.shape[1]), C.byref(sample),
-                                        _stream()), "sjd_prefill_ragged")
 
     def step(self, out: StepOut | None = None):
         _check(lib().sjd_step(self._ctx, C.byref(out.c) if out is not None else None, _stream()), "sjd_step")

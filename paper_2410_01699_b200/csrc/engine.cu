@@ -804,23 +804,26 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   }
   if (sample->init == SJD_INIT_RESAMPLE_ABOVE && c->cfg.max_ring < sample->grid_stride + sample->window)
     return SJD_ERR_CAPACITY;   // a retained row must outlive the window that draws from it
+  // every sequence gets the pages its own prompt and generated tokens need
+  auto pages_of = [&](int b) { return (prompt_lens[b] + sample->n_generate + KV_PAGE - 1) / KV_PAGE; };
+  if (c->cfg.kv_pages > 0) {
+    long need = 0;
+    for (int b = 0; b < batch; ++b) need += pages_of(b);
+    if (need > c->cfg.kv_pages) return SJD_ERR_CAPACITY;
+  }
+  // (a call refused above leaves the context as it was: its generation can go on)
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   if (batch != c->batch || sample->window != c->window) c->drop_graphs();   // what a pass depends on
   c->sample = *sample;
   c->batch = batch;
   c->prompt_len = prompt_len;
   if (c->cfg.kv_pages > 0) {
-    // every sequence gets the pages its own prompt and generated tokens need, in order, from page 0; entries
-    // past a sequence's last page point to the spare page
+    // in order, from page 0; entries past a sequence's last page point to the spare page
     const int pps = c->pages_per_seq();
     c->page_table.assign((size_t)c->cfg.max_batch * pps, c->cfg.kv_pages);
-    long next = 0;
-    for (int b = 0; b < batch; ++b) {
-      const int need = (prompt_lens[b] + sample->n_generate + KV_PAGE - 1) / KV_PAGE;
-      if (next + need > c->cfg.kv_pages) return SJD_ERR_CAPACITY;
-      for (int i = 0; i < need; ++i) c->page_table[(size_t)b * pps + i] = (int32_t)(next + i);
-      next += need;
-    }
+    int next = 0;
+    for (int b = 0; b < batch; ++b)
+      for (int i = 0, n = pages_of(b); i < n; ++i) c->page_table[(size_t)b * pps + i] = next++;
     SJD_CUDA(cudaMemcpyAsync(c->ws + c->lay.page_table, c->page_table.data(), c->page_table.size() * sizeof(int32_t),
                              cudaMemcpyHostToDevice, stream));
   }

@@ -547,3 +547,31 @@ def test_api_errors_and_state():
     with pytest.raises(B.SJDError):
         B.Context(B.make_model_cfg(wl.with_(head_dim=63), 1, 64, 8), weights)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("refused", [
+    dict(batch=1, seed=5, n_generate=250),   # five pages needed, four there
+    dict(batch=2, seed=2, n_generate=120),   # six pages for a larger batch
+])
+def test_refused_prefill_leaves_the_generation_alone(refused):
+    """A pre-fill that the paged cache cannot hold is refused before anything of the context changes: the generation
+    under way goes on to the tokens that it yields undisturbed."""
+    wl = WORKLOADS["small-bf16"]
+    weights = B.weights_to_device(make_weights(wl))
+    prompt = torch.from_numpy(make_prompt(wl, 2)).cuda()
+    tokens = []
+    for disturbed in (False, True):
+        ctx = B.Context(B.make_model_cfg(wl, 2, 320, wl.window, 0, 4), weights)
+        ctx.prefill(prompt[:1].contiguous(), B.make_sample_cfg(top_k=wl.top_k, seed=2, window=wl.window, n_generate=100))
+        out = B.StepOut(1, wl.window)
+        for step in range(40):
+            if disturbed and step in (1, 7):
+                with pytest.raises(B.SJDError) as e:
+                    ctx.prefill(prompt[:refused["batch"]].contiguous(),
+                                B.make_sample_cfg(top_k=wl.top_k, seed=refused["seed"], window=wl.window,
+                                                  n_generate=refused["n_generate"]))
+                assert e.value.status == B.SJD_ERR_CAPACITY
+            ctx.step(out)
+        tokens.append([t.cpu() for t in (*ctx.get_tokens(), ctx.peek_logits())])
+    for a, b in zip(*tokens):
+        assert torch.equal(a, b)
