@@ -244,8 +244,9 @@ int attention_t(const float *q, KvLayout kv, const int32_t *in_pos, float *out, 
   const int hd = kv.head_dim, W = segs.rows;
   if (W > NWARPS * MAXQ || hd > 32 * MAXD || M % W != 0) return SJD_ERR_UNSUPPORTED;
   const size_t smem = sizeof(float) * ((size_t)W * hd + TK * (hd + 1) + TK * hd + (size_t)W * TK);
-  if (smem > 48 * 1024)
-    SJD_CUDA(cudaFuncSetAttribute(attention_partial_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  constexpr int WM = NWARPS * MAXQ, HM = 32 * MAXD;   // the most rows and head entries
+  const int rc = allow_smem(attention_partial_kernel<T>, sizeof(float) * (WM * HM + TK * (HM + 1) + TK * HM + WM * TK));
+  if (rc != SJD_OK) return rc;
   dim3 grid(n_heads, M / W, splits);
   SJD_CUDA(launch_kernel(attention_partial_kernel<T>, grid, dim3(NWARPS * 32), smem, stream, q, kv, in_pos, partial, segs,
                          n_heads, splits));

@@ -445,7 +445,8 @@ int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const
   const CUtensorMap &km = reinterpret_cast<const CUtensorMap &>(kv_map);
   const size_t smem = (size_t)kStagesAttn * 2 * KT * head_dim * 2 + 1024;
   auto launch = [&](auto kernel) -> int {
-    SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int rc = allow_smem(kernel, smem);   // (the size follows from the kernel's head_dim)
+    if (rc != SJD_OK) return rc;
     SJD_CUDA(launch_kernel(kernel, grid, dim3(threads), smem, stream, km, p));
     SJD_CHECK_LAUNCH();
     return SJD_OK;

@@ -56,6 +56,14 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
   cfg.numAttrs = g_pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+// Lets launches of a kernel ask for up to `bytes` of dynamic shared memory.  The limit belongs to the function and not to a
+// launch, so it is the most that any call can need and never a call's own size: a thread with a smaller call would lower it
+// between another thread's setting and its launch, which then fails.
+template <typename K>
+inline int allow_smem(K kernel, size_t bytes) {
+  SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return SJD_OK;
+}
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

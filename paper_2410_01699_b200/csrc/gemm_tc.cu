@@ -26,6 +26,8 @@
 #include <cuda.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace sjd {
@@ -456,6 +458,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
 // 200 x 22016 x 4096 102 -> 61, 1024 x 12288 x 4096 169 -> 135 (1.5 PFLOP/s issued).
 constexpr int kPairStages = 8;
 constexpr int kPairThreads = 64 + 256;   // producer, issuer, eight epilogue warps
+constexpr int kPairSmem = 232448 - 2048; // most dynamic shared memory of a CTA, beside its static part
 constexpr int kShareParts = 4;           // most pairs that share a unit
 constexpr int kExTokens = 16;            // tokens of one exchange round of the gate|up epilogue
 
@@ -930,6 +933,22 @@ int gemm_tc_splits_max(const GemmTcPlan &pl, int tiles, int k_blocks) {
   return most;
 }
 
+// every kernel here may ask for as much shared memory as its largest launch needs; set once per device
+static int allow_gemm_smem() {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  SJD_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return SJD_ERR_UNSUPPORTED;
+  if (done.load() >> dev & 1) return SJD_OK;
+  constexpr size_t kMost = 2 * kSmemBudget + 2048;   // stages * stage_bytes + 1024 is at most that
+  int rc = allow_smem(gemm_tc_kernel<false>, kMost);
+  if (rc == SJD_OK) rc = allow_smem(gemm_tc_kernel<true>, kMost);
+  if (rc == SJD_OK) rc = allow_smem(gemm_pair_kernel<false>, kPairSmem);
+  if (rc == SJD_OK) rc = allow_smem(gemm_pair_kernel<true>, kPairSmem);
+  if (rc == SJD_OK) done.fetch_or(1ull << dev);
+  return rc;
+}
+
 static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles, cudaStream_t stream) {
   PairParams q;
   q.g = p;
@@ -938,7 +957,7 @@ static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles,
   const bool gu = g.act_hi != nullptr;
   const int stage_bytes = W_TILE_BYTES + p.Mp * TILE_K * 2;
   const int ex = gu ? 2 * TILE_N * (kExTokens + 1) * 4 : 0;
-  const int budget = 232448 - 2048 - 1024 - ex;
+  const int budget = kPairSmem - 1024 - ex;
   int stages = budget / stage_bytes;
   stages = stages > kPairStages ? kPairStages : stages;
   q.g.stages = stages;
@@ -948,7 +967,6 @@ static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles,
   const CUtensorMap &w2 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 2 ? 2 : 0]);
   const CUtensorMap &xm = reinterpret_cast<const CUtensorMap &>(*g.x_map);
   auto kernel = gu ? gemm_pair_kernel<true> : gemm_pair_kernel<false>;
-  SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int sms = g.n_sms > 1 ? g.n_sms : 148;
   // The units of a partial last round are shared where K may not be split otherwise and the launch has few rounds: one token slab
   // (7B gate|up at 128 rows: 86 units for 74 pairs, 2 rounds without, 1.25 with; 8 layers 1131 -> 1084 us at 80 rows, 1280 ->
@@ -1010,6 +1028,8 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   p.act_hi = g.act_hi;
   p.act_lo_off = g.act_lo_off;
   p.F = gu ? g.n_out[0] : 0;
+  const int rc = allow_gemm_smem();
+  if (rc != SJD_OK) return rc;
   if (gemm_tc_pairs(pl)) return launch_gemm_pair(g, p, tiles, stream);
   const int stage_bytes = W_TILE_BYTES + 2 * p.Mp * TILE_K * 2;
   const int ctas = tiles;
@@ -1025,17 +1045,6 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   const CUtensorMap &w1 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 1 ? 1 : 0]);
   const CUtensorMap &w2 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 2 ? 2 : 0]);
   const CUtensorMap &xm = reinterpret_cast<const CUtensorMap &>(*g.x_map);
-  // opt in to > 48 KB of dynamic shared memory, once per device
-  static bool configured[64] = {};
-  int dev = 0;
-  SJD_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return SJD_ERR_UNSUPPORTED;
-  if (!configured[dev]) {
-    const int max_dyn = 2 * kSmemBudget + 2048;
-    SJD_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
-    SJD_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
-    configured[dev] = true;
-  }
   const dim3 grid(ctas, g.splits);
   if (gu)
     SJD_CUDA(launch_kernel(gemm_tc_kernel<true>, grid, dim3(kThreads), smem, stream, w0, w1, w2, xm, p));

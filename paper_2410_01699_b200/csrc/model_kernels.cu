@@ -196,7 +196,8 @@ int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
   const size_t smem = (size_t)(RG_M + bn) * RG_LD * sizeof(float);
   const dim3 grid((g.N + cols - 1) / cols, mt);
   auto launch = [&](auto kernel) -> int {
-    if (smem > 40 * 1024) SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int rc = smem > 40 * 1024 ? allow_smem(kernel, smem) : SJD_OK;   // (the size follows from the kernel's tile)
+    if (rc != SJD_OK) return rc;
     SJD_CUDA(launch_kernel(kernel, grid, dim3(256), smem, stream, g));
     SJD_CHECK_LAUNCH();
     return SJD_OK;

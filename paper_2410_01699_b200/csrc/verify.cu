@@ -2519,8 +2519,10 @@ template <typename T, int CS>
 static int launch_cluster(const VerifyParams &p, long nv, cudaStream_t stream) {
   auto kernel = verify_cluster_kernel<T, CS>;
   const long ni = ((nv + CS - 1) / CS + kClThreads - 1) / kClThreads;
-  const size_t smem = (sizeof(ClScratch<CS>) + 15) / 16 * 16 + (size_t)2 * ni * kClThreads * 16;
-  SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  auto smem_of = [](long n) { return (sizeof(ClScratch<CS>) + 15) / 16 * 16 + (size_t)2 * n * kClThreads * 16; };
+  const size_t smem = smem_of(ni);
+  const int rc = allow_smem(kernel, smem_of(kClVecs));
+  if (rc != SJD_OK) return rc;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(p.B * p.W * CS);
@@ -2569,7 +2571,8 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
     }
   }
   const size_t stage_bytes = (size_t)nv_max * 16;
-  p.staged = stage_bytes <= 160 * 1024 ? 1 : 0;
+  constexpr size_t kMostStaged = 160 * 1024;
+  p.staged = stage_bytes <= kMostStaged ? 1 : 0;
   int threads = nv_max <= 1024 ? 128 : nv_max <= 4096 ? 256 : nv_max <= 16384 ? 512 : 1024;
   // rows a block can hold in registers, eight vectors per thread
   p.fast = 0;
@@ -2590,7 +2593,8 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
   const size_t dyn = p.staged ? stage_bytes : 0;
   auto launch = [&](auto kernel) -> int {
     // static scratch (about 30 KB) + the staged row: opt in as soon as the sum can pass 48 KB
-    if (dyn > 16 * 1024) SJD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    const int rc = dyn > 16 * 1024 ? allow_smem(kernel, kMostStaged) : SJD_OK;
+    if (rc != SJD_OK) return rc;
     SJD_CUDA(launch_kernel(kernel, dim3(p.B * p.W), dim3(threads), dyn, stream, p));
     SJD_CHECK_LAUNCH();
     return SJD_OK;

@@ -266,3 +266,29 @@ class LockStepSequence:
         st.qdescs = [QDesc(Q_ROW, row=np.array(gpu_logits_rows[a + 1 + s], dtype=np.float64)) for s in range(redrawn)]
         _fill_window(st, scfg, vocab, st.step - 1)
         self.check_window(out_b["draft"], out_b["q_kind"], out_b["q_draft"], out_b["total_committed"])
+
+
+def run_in_threads(*work):
+    """Runs every callable in a thread of its own, on a CUDA stream of its own, all at once; re-raises the first error."""
+    import threading
+
+    import torch
+    errors, gate = [], threading.Barrier(len(work))
+
+    def body(f):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                gate.wait()
+                f()
+                torch.cuda.current_stream().synchronize()
+        except BaseException as e:   # noqa: BLE001 (handed to the caller)
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=body, args=(f,)) for f in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]

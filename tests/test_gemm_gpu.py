@@ -1,10 +1,13 @@
 """GPU parity of the tensor-core weight-streaming GEMM (sjd_gemm through the C-ABI) against a plain
 fp64 matrix product of the same bf16 weights and fp32 activations."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2410_01699_b200 import binding as B
+from tests.parity_util import run_in_threads
 
 pytestmark = pytest.mark.gpu
 
@@ -83,3 +86,22 @@ def test_gemm_rejects_uncovered_shapes():
         B.sjd_gemm(x, w)                      # K not a multiple of 64
     assert e.value.status == B.SJD_ERR_UNSUPPORTED
     assert B.lib().sjd_gemm_workspace_bytes(1025, 128, 64) == 0
+
+
+def test_gemm_threads_with_different_sizes():
+    """Threads whose launches ask for different amounts of shared memory (80 and 128 token rows: rings of eight and of seven
+    stages): none lowers the limit under another's launch."""
+    x, w, _ = _case(128, 256, 512, seed=3)
+    x, w = x.cuda(), w.cuda()
+    want = {m: B.sjd_gemm(x[:m], w)[0] for m in (80, 128)}
+
+    def calls(m):
+        out = torch.empty(m, 256, device="cuda")
+        ws = torch.empty(int(B.lib().sjd_gemm_workspace_bytes(m, 256, 512)), dtype=torch.uint8, device="cuda")
+        args = [m, 256, 512, *(C.c_void_p(t.data_ptr()) for t in (x, w, out)), 0, C.c_void_p(ws.data_ptr()), ws.numel(),
+                C.c_void_p(torch.cuda.current_stream().cuda_stream)]
+        call = B.lib().sjd_gemm
+        assert all(call(*args) == B.SJD_OK for _ in range(10000))
+        assert torch.equal(out, want[m])
+
+    run_in_threads(*[lambda m=m: calls(m) for m in (80, 128, 80, 128)])

@@ -1,12 +1,14 @@
 """GPU parity of the fused verify-and-resample kernel (sjd_verify through the C-ABI) against the
 CPU checker, element by element on the same seeded inputs."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2410_01699_b200 import binding as B
 from paper_2410_01699_b200.inputs import make_verify_case, round_bf16
-from tests.parity_util import ParityStats, compare_window, oracle_verify_case
+from tests.parity_util import ParityStats, compare_window, oracle_verify_case, run_in_threads
 
 pytestmark = pytest.mark.gpu
 
@@ -214,6 +216,30 @@ def test_verify_is_deterministic():
     a, b = _run_gpu(case), _run_gpu(case)
     for k in a:
         assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("rows,dtype", [((4096, 16000), "f32"), ((12001, 30001), "bf16")])   # a cluster, a block per row
+def test_verify_threads_with_different_rows(rows, dtype):
+    """Two threads whose rows need different amounts of shared memory in the same kernel."""
+    def calls(vocab):
+        case = make_verify_case(20, window=8, vocab=vocab, dtype=dtype, top_k=100, seed=4)
+        dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+        args = [torch.from_numpy(a).cuda() for a in (case.logits_cur, case.logits_prev, case.draft, case.q_kind.astype(np.int32),
+                                                     case.base_pos)]
+        args[:2] = [a.to(dt) for a in args[:2]]
+        sample = B.make_sample_cfg(temperature=case.temperature, top_k=case.top_k, seed=case.seed, window=case.window)
+        outs = [B.StepOut(case.batch, case.window) for _ in range(2)]
+        ws = torch.empty(B.sjd_verify_workspace_bytes(case.batch, case.window), dtype=torch.uint8, device="cuda")
+        stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        call = [(case.batch, case.window, vocab, B.SJD_BF16 if dtype == "bf16" else B.SJD_F32,
+                 *(C.c_void_p(a.data_ptr()) for a in args), C.byref(sample), case.step, C.byref(o.c), C.c_void_p(ws.data_ptr()),
+                 ws.numel(), stream) for o in outs]
+        verify = B.lib().sjd_verify
+        assert all(verify(*call[i > 0]) == B.SJD_OK for i in range(5000))
+        a, b = outs[0].host(), outs[1].host()
+        assert all(np.array_equal(a[k], b[k]) for k in a)
+
+    run_in_threads(*[lambda v=v: calls(v) for v in rows * 2])
 
 
 def test_verify_argument_errors():
