@@ -40,6 +40,7 @@ constexpr int kGuRows = 64;
 // more fp32 buffers per row and is not bound by the weights: 256 rows.
 constexpr int kPrefillRowsTc = 1152, kPrefillRowsGeneric = 256;
 constexpr int kMaxTcRows = 1152;     // largest pass of the tensor-core pipeline
+constexpr int kShareFlags = 160;     // arrival counters of a projection's shared units: two per CTA pair
 
 struct WMap {
   TensorMap map;
@@ -166,7 +167,7 @@ Layout make_layout(const sjd_model_cfg &c) {
     if (tc && Mp > 64 && bytes < gemm_tc_share_floats() * 4) bytes = gemm_tc_share_floats() * 4;   // shared units use the planes' memory
     L.gemm_planes = take(bytes);
   }
-  L.share_flags = take(tc ? 160 * 4 : 0);
+  L.share_flags = take(tc ? kShareFlags * 4 : 0);
   L.ss_part = take(Mp * (size_t)resid_gain_parts(c.d_model) * 4);
   L.rope = take((size_t)c.max_seq * (c.head_dim / 2) * sizeof(float2));
   L.committed = take((size_t)c.max_batch * c.max_seq * 4);
@@ -239,8 +240,9 @@ struct Tracer {
 };
 
 // prompt: [B][ld] token ids, sequence b uses the first st.prompt_lens[b] of its row
+// share_flags (tensor-core pipeline, else null): every launch leaves them zero, but one in which a wait ran out may not
 __global__ void prefill_setup_kernel(const int32_t *prompt, int ld, SeqState st, uint32_t *step, int32_t *counters,
-                                     int B) {
+                                     int *share_flags, int B) {
   const int b = blockIdx.x;
   const int P = st.prompt_lens[b];
   for (int i = threadIdx.x; i < P; i += blockDim.x) st.committed[(size_t)b * st.max_seq + i] = prompt[(size_t)b * ld + i];
@@ -253,6 +255,8 @@ __global__ void prefill_setup_kernel(const int32_t *prompt, int ld, SeqState st,
       *step = kStepInitialWindow;
     }
   }
+  if (b == 0 && share_flags)
+    for (int i = threadIdx.x; i < kShareFlags; i += blockDim.x) share_flags[i] = 0;
 }
 
 // one block per segment of a pre-fill pass: its tokens and positions (the last prompt token is not among them)
@@ -708,7 +712,6 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
   cudaError_t e = cudaMemcpy(c->ws + lay.rope, table.data(), table.size() * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.counters, 0, ((size_t)cfg->max_batch + 1) * 4);
   if (e == cudaSuccess) e = cudaMemset(c->ws + lay.status, 0, 4);
-  if (e == cudaSuccess && tc_shapes(*cfg)) e = cudaMemset(c->ws + lay.share_flags, 0, 160 * 4);
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     delete c;
@@ -838,7 +841,8 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
   if (tc) add_x_maps(c, batch * sample->window);
   const SeqState st = c->state();
   prefill_setup_kernel<<<batch, 128, 0, stream>>>(prompt, row_stride, st, c->at<uint32_t>(c->lay.step),
-                                                  c->at<int32_t>(c->lay.counters), batch);
+                                                  c->at<int32_t>(c->lay.counters),
+                                                  tc ? c->at<int>(c->lay.share_flags) : nullptr, batch);
   SJD_CHECK_LAUNCH();
   // Cache keys/values of c[0..P-1): the prompts are cut into segments of `rows` positions, which are packed into as
   // few passes as the activation buffers allow.  Short segments waste fewer padding rows, long ones re-read fewer

@@ -466,9 +466,9 @@ struct PairParams {
   GemmParams g;
   int tiles;             // 128-row weight tiles
   int n_units;
-  // Units of the last, partial round (from unit `full` on) that several pairs share: `parts` pairs take a range of K each;
-  // the first adds the others' sums (scratch [unit][part - 1][rank][token][128]) to its own before the epilogue.  The grid is
-  // resident at once and the others wait for nothing.
+  // Units of the last, partial round (from unit `full` on) that several pairs share: `parts` pairs take a range of K each and
+  // leave their sums in scratch [unit][part][rank][token][128].  The one that arrives last adds them, in the order of the parts,
+  // and goes on to the epilogue: nobody waits for another pair, so it does not matter which of them are resident.
   int full, parts;
   float *scratch;
   int *flags;            // [unit][rank] arrivals, zero before and after a launch
@@ -711,62 +711,55 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * NN;
       const int mat = mat_of(t.tile), m_left = p.M - m_base;
-      const bool helper = t.part > 0;
-      const int n_add = t.shared >= 0 && !helper ? q.parts - 1 : 0;   // sums to add
       const size_t piece = (size_t)2 * p.Mp * TILE_N;
-      float *share = q.scratch + (size_t)(t.shared < 0 ? 0 : t.shared) * (q.parts - 1) * piece + (size_t)rank * p.Mp * TILE_N + row;
-      int *flag = q.flags + (t.shared < 0 ? 0 : t.shared) * 2 + rank;
-      if (n_add) {
-        bool there = true;
+      float *share = q.scratch + (size_t)(t.shared < 0 ? 0 : t.shared) * q.parts * piece + (size_t)rank * p.Mp * TILE_N + row;
+      bool finish = true, gather = false;   // this CTA does the unit's epilogue; from the parts' sums
+      if (t.shared >= 0) {
+        float *dst = share + t.part * piece;
+        for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
+          uint32_t hi[16], lo[16];
+          tmem_ld16_issue(t_addr + m0, hi);
+          tmem_ld16_issue(t_addr + p.Mp + m0, lo);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) dst[(size_t)(m0 + i) * TILE_N] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+        }
+        __threadfence();
+        pair_epilogue_all(true);
+        bool last = true;
         if (tid == 64) {
-          const unsigned long long t0 = global_ns();
-          for (int i = 0;; ++i) {
-            int v;
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-            if (v == n_add) break;
-            if ((i & 255) == 255 && global_ns() - t0 > kWaitNs) { there = false; break; }
-          }
-          *flag = 0;
+          int *flag = q.flags + t.shared * 2 + rank;
+          last = atomicAdd(flag, 1) == q.parts - 1;
+          if (last) *flag = 0;
+          __threadfence();
         }
-        if (!pair_epilogue_all(there)) {
-          if (tid == 64) atomicExch(p.status, 5);
-          break;
-        }
+        finish = gather = pair_epilogue_all(last);
       }
-      // 16 tokens of this thread's row: hi + lo plane, and the other parts of a shared unit
+      // 16 tokens of this thread's row: hi + lo plane, or the sums of a shared unit's parts
       auto sums = [&](int m0, float *v) {
+        if (gather) {   // all loads in flight at once: one round trip per 16 tokens
+          float w[kShareParts][16];
+#pragma unroll
+          for (int k = 0; k < kShareParts; ++k)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[k][i] = k < q.parts ? __ldcg(share + k * piece + (size_t)(m0 + i) * TILE_N) : 0.0f;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            v[i] = w[0][i];
+#pragma unroll
+            for (int k = 1; k < kShareParts; ++k) v[i] += w[k][i];
+          }
+          return;
+        }
         uint32_t hi[16], lo[16];
         tmem_ld16_issue(t_addr + m0, hi);
         tmem_ld16_issue(t_addr + p.Mp + m0, lo);
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
-        if (n_add) {   // all loads in flight at once: one round trip per 16 tokens
-          float w[kShareParts - 1][16];
-#pragma unroll
-          for (int k = 0; k < kShareParts - 1; ++k)
-#pragma unroll
-            for (int i = 0; i < 16; ++i) w[k][i] = k < n_add ? __ldcg(share + k * piece + (size_t)(m0 + i) * TILE_N) : 0.0f;
-#pragma unroll
-          for (int k = 0; k < kShareParts - 1; ++k)
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] += w[k][i];
-        }
       };
-      if (helper) {
-        float *dst = share + (t.part - 1) * piece;
-        for (int m0 = grp * 16; m0 < p.Mp; m0 += 32) {
-          float v[16];
-          sums(m0, v);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) dst[(size_t)(m0 + i) * TILE_N] = v[i];
-        }
-        __threadfence();
-        pair_epilogue_all(true);
-        if (tid == 64) {
-          __threadfence();
-          atomicAdd(flag, 1);
-        }
+      if (!finish) {
+        // (another pair finishes this unit)
       } else if (GU) {
         // MMA rows 0..63 hold gate features, rows 64..127 the same features of the up matrix: they meet in shared memory, 16
         // tokens at a time; then thread e finishes feature e % 64 for every second token

@@ -10,7 +10,7 @@ from oracle.sjd import (INIT_COPY_ABOVE, INIT_COPY_LEFT, INIT_RANDOM, INIT_RESAM
                         SampleCfg)
 from paper_2410_01699_b200 import binding as B
 from paper_2410_01699_b200.inputs import WORKLOADS, make_prompt, make_weights
-from tests.parity_util import LockStepSequence
+from tests.parity_util import LockStepSequence, run_in_threads
 
 pytestmark = pytest.mark.gpu
 
@@ -575,3 +575,27 @@ def test_refused_prefill_leaves_the_generation_alone(refused):
         tokens.append([t.cpu() for t in (*ctx.get_tokens(), ctx.peek_logits())])
     for a, b in zip(*tokens):
         assert torch.equal(a, b)
+
+
+def test_contexts_on_two_streams():
+    """Two contexts of 80 rows per pass (projections on CTA pairs that share the units of a partial last round) step at the
+    same time on two streams: each yields what it yields alone."""
+    wl = WORKLOADS["small-bf16"]
+    weights = B.weights_to_device(make_weights(wl))
+    prompt = torch.from_numpy(make_prompt(wl, 5)).cuda()
+
+    def run(seed, got):
+        ctx = B.Context(B.make_model_cfg(wl, 5, 320, wl.window), weights)
+        ctx.prefill(prompt, B.make_sample_cfg(top_k=wl.top_k, seed=seed, window=wl.window, n_generate=250))
+        for _ in range(150):
+            ctx.step()
+        got[seed] = [t.cpu() for t in (*ctx.get_tokens(), ctx.peek_logits())]
+        assert ctx.device_status() == B.SJD_OK
+
+    alone, together = {}, {}
+    for seed in (1, 2):
+        run(seed, alone)
+    run_in_threads(*[lambda seed=seed: run(seed, together) for seed in (1, 2)])
+    for seed in (1, 2):
+        for a, b in zip(alone[seed], together[seed]):
+            assert torch.equal(a, b)
