@@ -65,6 +65,7 @@ struct Layout {
   size_t page_table;                         // [max_batch][pages_per_seq] (paged cache, kv_pages > 0)
   size_t seg_seq, seg_start;                 // [prefill_segments] pre-fill: sequence and first position of every segment
   size_t pass_rows;                          // rows of the largest pass (a step or a pre-fill chunk)
+  size_t generic_rows;                       // and of the largest one that the generic kernels have room for
   size_t total;
 };
 
@@ -105,6 +106,7 @@ Layout make_layout(const sjd_model_cfg &c) {
   const size_t Rg = prefill_rows(c, false), Mg = Mx > Rg ? Mx : Rg;          // of the largest pass, generic pipeline
   const size_t Rp = prefill_rows(c, tc), Mp = Mx > Rp ? Mx : Rp;             // and of either pipeline
   L.pass_rows = Mp;
+  L.generic_rows = Mg;
   const size_t nq = (size_t)c.n_heads * c.head_dim, nk = (size_t)c.n_kv_heads * c.head_dim;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -344,6 +346,12 @@ struct sjd_ctx {
   std::map<int, XMaps> xmaps;   // keyed by padded row count
   TensorMap kv_map;             // whole KV cache as [planes][max_seq][head_dim]
   bool kv_map_valid = false;
+  // a pass of M rows may take the tensor-core pipeline (given its activation descriptors).  Without the cache's descriptor
+  // (one that could not be encoded) the generic attention has to have room for the rows.
+  bool tc_pass(int M) const {
+    return use_tc && all_tc && M <= kMaxTcRows &&
+           (kv_map_valid || !attention_mma_supported(cfg.head_dim, 64) || (size_t)M <= lay.generic_rows);
+  }
   int rows_alloc() const { return ((int)lay.pass_rows + 15) / 16 * 16; }
 
   template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
@@ -579,7 +587,7 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
 
 int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const int M = n_segs * segs.rows;
-  if (c->use_tc && c->all_tc && M <= kMaxTcRows) {
+  if (c->tc_pass(M)) {
     auto it = c->xmaps.find((M + 15) / 16 * 16);
     if (it != c->xmaps.end()) {
       // every kernel of this pipeline waits for its predecessor itself: launch them overlapped
@@ -589,6 +597,7 @@ int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t
       return rc;
     }
   }
+  if ((size_t)M > c->lay.generic_rows) return SJD_ERR_UNSUPPORTED;
   g_pdl = !c->tracer.on;
   const int rc = forward_generic(c, n_segs, segs, logits_out, stream);
   g_pdl = false;
@@ -765,10 +774,11 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
 }
 
 namespace {
-// activation descriptors for passes of `rows` rows (once per padded row count and context)
-void add_x_maps(sjd_ctx *c, int rows) {
+// activation descriptors for passes of `rows` rows (once per padded row count and context); false: no such pass
+bool add_x_maps(sjd_ctx *c, int rows) {
   const int Mp = (rows + 15) / 16 * 16;
-  if (rows > kMaxTcRows || c->xmaps.count(Mp)) return;
+  if (!c->tc_pass(rows)) return false;
+  if (c->xmaps.count(Mp)) return true;
   const int Ma = c->rows_alloc();
   const int nq = c->cfg.n_heads * c->cfg.head_dim;
   XMaps xm;
@@ -777,6 +787,7 @@ void add_x_maps(sjd_ctx *c, int rows) {
                   make_tensor_map_bf16(&xm.attn, c->ws + c->lay.xs_attn, 2L * Ma, nq, box) == SJD_OK &&
                   make_tensor_map_bf16(&xm.act, c->ws + c->lay.xs_act, 2L * Ma, c->cfg.ffn_hidden, box) == SJD_OK;
   if (ok) c->xmaps[Mp] = xm;
+  return ok;
 }
 }  // namespace
 
@@ -870,11 +881,18 @@ extern "C" int sjd_prefill_ragged(sjd_ctx *c, int batch, const int32_t *prompt, 
     int32_t *seg_seq = c->at<int32_t>(c->lay.seg_seq), *seg_start = c->at<int32_t>(c->lay.seg_start);
     SJD_CUDA(cudaMemcpyAsync(seg_seq, c->seg_seq.data(), (size_t)n_segs * 4, cudaMemcpyHostToDevice, stream));
     SJD_CUDA(cudaMemcpyAsync(seg_start, c->seg_start.data(), (size_t)n_segs * 4, cudaMemcpyHostToDevice, stream));
-    const int cap = (int)prefill_rows(c->cfg, tc) / rows;   // segments of one pass
-    const int passes = (n_segs + cap - 1) / cap;
+    // segments of one pass; a pass that finds no descriptors goes to the generic kernels and has to fit their buffers
+    auto passes_for = [&](bool tensor) {
+      const int cap = (int)prefill_rows(c->cfg, tensor) / rows;
+      return (n_segs + cap - 1) / cap;
+    };
+    auto first_of = [&](int i, int n) { return (int)((long)n_segs * i / n); };
+    int passes = passes_for(tc);
+    bool mapped = tc;
+    for (int i = 0; i < passes && mapped; ++i) mapped = add_x_maps(c, (first_of(i + 1, passes) - first_of(i, passes)) * rows);
+    if (tc && !mapped) passes = passes_for(false);
     for (int i = 0; i < passes; ++i) {
-      const int s0 = (int)((long)n_segs * i / passes), n = (int)((long)n_segs * (i + 1) / passes) - s0;
-      if (tc) add_x_maps(c, n * rows);
+      const int s0 = first_of(i, passes), n = first_of(i + 1, passes) - s0;
       prefill_inputs_kernel<<<n, 64, 0, stream>>>(prompt, row_stride, st.prompt_lens, seg_seq + s0, seg_start + s0, rows,
                                                   st.in_tok, st.in_pos);
       SJD_CHECK_LAUNCH();
@@ -979,7 +997,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   if (!c || !info) return SJD_ERR_BAD_ARG;
   if (!c->prefilled) return SJD_ERR_STATE;
   const int M = c->batch * c->window;
-  const bool tc = c->use_tc && c->all_tc && M <= kMaxTcRows && c->xmaps.count((M + 15) / 16 * 16) != 0;
+  const bool tc = c->tc_pass(M) && c->xmaps.count((M + 15) / 16 * 16) != 0;
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
       (tc && c->kv_map_valid && attention_mma_supported(c->cfg.head_dim, c->window)) ? 1 : 0;
