@@ -1764,10 +1764,17 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1)
 // For few rows (latency counts, most SMs would idle) and for every fp32 row: CS blocks hold a row and the row its draft was
 // drawn from in shared memory, a contiguous slice each, and meet in distributed shared memory: once for the maxima, once for
 // the histograms, once for the sums.  The threshold is exact: a histogram of the distances below the maximum in the top 16
-// bits of the key (as on the register route); for fp32 the entries in the bin found are then listed (usually some hundred)
-// and every block selects among their low 16 bits.  Bound by the chain of barriers, block scans and round trips (each about
+// bits of the key (as on the register route; a threshold beyond its 4095 codes takes further windows, cl_further); for fp32 the
+// entries in the bin found are then listed (usually some hundred) and every block selects among their low 16 bits (from the
+// slices where they are many, cl_ties).  Only a row without a finite entry is left to the general route: a block that tries
+// this one first and then reads its row again is slower than a block per row was (us a call with a block per row / with such
+// rows left to it / decided here: fp32 1 x 27 x 65536, threshold below zero 154 / 216 / 48, most entries masked with one value
+// 163 / 231 / 52, a NaN in each row 156 / 214 / 43; bf16 1 x 16 x 184320, threshold below zero 292 / 320 / 66).
+// Bound by the chain of barriers, block scans and round trips (each about
 // a microsecond) and by instruction fetch: every phase runs once, so its loops are kept rolled.
 constexpr int kClThreads = 512, kClWarps = kClThreads / 32, kClVecs = 8, kClList = 4096;
+constexpr uint32_t kClMany = 1024;   // entries in a threshold's bin beyond which they are not listed (26 x 33 x 4096, most entries
+                                     // masked with one value: 94 us a call with 4096, 81 with 1024)
 
 template <int CS>
 struct ClScratch {
@@ -1780,7 +1787,7 @@ struct ClScratch {
   double wsum[2][kClWarps];
   uint32_t kmax[2][CS], bad[CS];
   uint32_t scan[2][kClWarps], redu[2][kClWarps];
-  uint32_t sel_bin[2], sel_above[2], n_list[2], hist16[2][16];
+  uint32_t sel_bin[2], sel_above[2], sel_count[2], n_list[2], hist16[2][16], low16[2][16];
   float chunk_sum[kClWarps * kClVecs];
   int tok[2];                                  // redraft, resample: written in block 0's copy by the block that finds it
   float tok_w;
@@ -1874,6 +1881,7 @@ __device__ __forceinline__ void cl_scan(ClScratch<CS> &cs, bool second, const ui
         if (acc < k && k <= acc + c[i]) {
           cs.sel_bin[x] = (uint32_t)(tid * 8 + i);
           cs.sel_above[x] = acc;
+          cs.sel_count[x] = c[i];
         }
         acc += c[i];
       }
@@ -1885,7 +1893,7 @@ __device__ __forceinline__ uint4 add4(const uint4 &a, const uint4 &b) { return m
 __device__ __forceinline__ uint32_t sum4(const uint4 &a) { return a.x + a.y + a.z + a.w; }
 
 // The histograms are complete in this block (a barrier ago): the bin, counted from bin 0, that holds the K-th entry of a row
-// over all blocks, and the entries before it.  One cluster barrier; every block finds it for itself.
+// over all blocks, the entries before it and those in it.  One cluster barrier; every block finds it for itself.
 template <int CS>
 __device__ __forceinline__ void cl_find(ClScratch<CS> &cs, int rank, bool second, const uint32_t *K) {
   const int tid = threadIdx.x;
@@ -2077,6 +2085,231 @@ __device__ __forceinline__ void cl_max(const uint4 &v, float &mx, bool &bad, __n
   mx = fmaxf(mx, fmaxf(a, b));
 }
 
+// What few rows need is kept out of line: the kernel is bound by instruction fetch as well.  pv, qv: the slices, vector i of a
+// thread at [i * kClThreads]; qv null: no q row.
+
+// The largest keys of the two rows and the union of `bad` over all blocks.  One block and one cluster barrier; the arrays may
+// be shared again after another cluster barrier.
+template <int CS>
+__device__ __forceinline__ uint3 cl_share_max(ClScratch<CS> &cs, int rank, uint32_t key_p, uint32_t key_q, uint32_t bad) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  key_p = __reduce_max_sync(0xffffffffu, key_p);
+  key_q = __reduce_max_sync(0xffffffffu, key_q);
+  bad = __reduce_or_sync(0xffffffffu, bad);
+  if (lane == 0) {
+    cs.redu[0][warp] = key_p;
+    cs.redu[1][warp] = key_q;
+    cs.scan[0][warp] = bad;
+  }
+  __syncthreads();
+  if (warp < CS) {
+    const uint32_t a = __reduce_max_sync(0xffffffffu, lane < kClWarps ? cs.redu[0][lane] : 0u);
+    const uint32_t b = __reduce_max_sync(0xffffffffu, lane < kClWarps ? cs.redu[1][lane] : 0u);
+    const uint32_t c = __reduce_or_sync(0xffffffffu, lane < kClWarps ? cs.scan[0][lane] : 0u);
+    if (lane == 0) {
+      if constexpr (CS == 1) {
+        cs.kmax[0][0] = a; cs.kmax[1][0] = b; cs.bad[0] = c;
+      } else {
+        cl_store(cl_map(&cs.kmax[0][rank], warp), a);
+        cl_store(cl_map(&cs.kmax[1][rank], warp), b);
+        cl_store(cl_map(&cs.bad[rank], warp), c);
+      }
+    }
+  }
+  cl_sync<CS>();
+  uint3 all = make_uint3(0u, 0u, 0u);
+#pragma unroll
+  for (int r = 0; r < CS; ++r) {
+    all.x = max(all.x, cs.kmax[0][r]);
+    all.y = max(all.y, cs.kmax[1][r]);
+    all.z |= cs.bad[r];
+  }
+  return all;
+}
+
+// As in the general route, a NaN or +inf counts as -inf: replaces them in the slices.  The largest keys of both rows, and a bit
+// for each row that held one.
+template <typename T, int CS>
+__device__ __noinline__ uint3 cl_replace_bad(ClScratch<CS> &cs, int rank, int ni, uint4 *pv, uint4 *qv) {
+  using E = Elt<T>;
+  uint32_t km[2] = {0u, 0u}, bad = 0;
+#pragma unroll 1
+  for (int i = 0; i < (qv ? 2 : 1) * ni; ++i) {
+    uint4 &at = i < ni ? pv[i * kClThreads] : qv[(i - ni) * kClThreads];
+    const int x = i < ni ? 0 : 1;
+    uint4 v = at;
+#pragma unroll
+    for (int t = 0; t < E::VEC; ++t) {
+      if (E::bad(E::get(v, t))) {
+        E::set(v, t, E::NEG_INF);
+        bad |= 1u << x;
+      }
+      const uint32_t k = E::key(E::get(v, t));
+      if (x) km[1] = max(km[1], k);
+      else km[0] = max(km[0], k);
+    }
+    at = v;
+  }
+  cl_sync<CS>();   // every block has read the first maxima
+  return cl_share_max<CS>(cs, rank, km[0], km[1], bad);
+}
+
+// The threshold lies further below the maximum than the histogram's 4095 codes, in row 0 and / or 1 (bits of `open`): window after
+// window of 4095 codes, each from the largest entry that is further down.  K: the entries left to count.  Returns the
+// thresholds (their top 16 bits) and the entries left to count in the thresholds' bins; sel_count: the entries in those.
+template <typename T, int CS>
+__device__ __noinline__ uint4 cl_further(ClScratch<CS> &cs, int rank, int ni, const uint4 *pv, const uint4 *qv, uint32_t open,
+                                         uint32_t top_p, uint32_t top_q, uint32_t K_p, uint32_t K_q) {
+  using E = Elt<T>;
+  constexpr int HI = E::KEYBITS - 16;
+  const int tid = threadIdx.x;
+  uint32_t top[2] = {top_p, top_q}, K[2] = {K_p, K_q}, tau[2] = {0u, 0u}, count[2] = {cs.sel_count[0], cs.sel_count[1]};
+  // (17 windows cover the 65536 codes, and entries outside the row, which count as -inf, end the search at the latest)
+#pragma unroll 1
+  for (int round = 0; round < 17 && open; ++round) {
+    uint32_t next[2] = {0u, 0u};
+#pragma unroll 1
+    for (int i = 0; i < ni; ++i) {
+      const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) {
+        const uint32_t ha = E::key(E::get(a, t)) >> HI, hb = E::key(E::get(b, t)) >> HI;
+        if (ha + 4095u <= top[0]) next[0] = max(next[0], ha);
+        if (hb + 4095u <= top[1]) next[1] = max(next[1], hb);
+      }
+    }
+    const uint3 m = cl_share_max<CS>(cs, rank, next[0], next[1], 0u);   // (its barrier: nobody reads the histograms any more)
+    top[0] = m.x;
+    top[1] = m.y;
+    for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    uint32_t equal[2] = {0u, 0u};   // entries at the top of the window: many at once where a row is masked with one value
+#pragma unroll 1
+    for (int i = 0; i < ni; ++i) {
+      const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) {
+        // (entries above the window wrap to its last bin, as those below it)
+        const uint32_t da = top[0] - (E::key(E::get(a, t)) >> HI), db = top[1] - (E::key(E::get(b, t)) >> HI);
+        if (da == 0u) ++equal[0];
+        else atomicAdd(&cs.hist[0][min(da, 4095u)], 1u);
+        if (db == 0u) ++equal[1];
+        else atomicAdd(&cs.hist[1][min(db, 4095u)], 1u);
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const uint32_t n = __reduce_add_sync(0xffffffffu, equal[x]);
+      if ((tid & 31) == 0) atomicAdd(&cs.hist[x][0], n);
+    }
+    __syncthreads();
+    cl_find<CS>(cs, rank, true, K);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      if (!(open >> x & 1u)) continue;
+      K[x] -= cs.sel_above[x];
+      if (cs.sel_bin[x] < 4095u) {
+        tau[x] = (top[x] - cs.sel_bin[x]) << HI;
+        count[x] = cs.sel_count[x];
+        open &= ~(1u << x);
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < 2) cs.sel_count[tid] = tid ? count[1] : count[0];
+  __syncthreads();
+  return make_uint4(tau[0], tau[1], K[0], K[1]);
+}
+
+// fp32: the low 16 bits of the thresholds where more entries share their top 16 bits than a list holds.  Usually they are all
+// equal (a row masked with one value); else they are counted from the slices, 12 bits and then 4.
+template <int CS>
+__device__ __noinline__ uint2 cl_ties(ClScratch<CS> &cs, int rank, int ni, const uint4 *pv, const uint4 *qv, uint32_t tau_p, uint32_t tau_q,
+                                      uint32_t K_p, uint32_t K_q) {
+  using E = Elt<float>;
+  const int tid = threadIdx.x, rows = qv ? 2 : 1;
+  uint32_t K[2] = {K_p, K_q}, tau[2] = {tau_p, tau_q};
+  auto in_bin = [&](int x, auto f) {
+#pragma unroll 1
+    for (int i = 0; i < ni; ++i) {
+      const uint4 v = (x ? qv : pv)[i * kClThreads];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const uint32_t key = E::key(E::get(v, t));
+        if ((key >> 16) == ((x ? tau_q : tau_p) >> 16)) f(key);
+      }
+    }
+  };
+  uint32_t lo[2] = {0u, 0u}, hi[2] = {0u, 0u};   // largest complement and largest key of the bins
+#pragma unroll 1
+  for (int i = 0; i < ni; ++i) {
+    const uint4 a = pv[i * kClThreads], b = (qv ? qv : pv)[i * kClThreads];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const uint32_t ka = E::key(E::get(a, t)), kb = E::key(E::get(b, t));
+      if ((ka >> 16) == (tau_p >> 16)) {
+        lo[0] = max(lo[0], ~ka);
+        hi[0] = max(hi[0], ka);
+      }
+      if ((kb >> 16) == (tau_q >> 16)) {
+        lo[1] = max(lo[1], ~kb);
+        hi[1] = max(hi[1], kb);
+      }
+    }
+  }
+  const uint3 m = cl_share_max<CS>(cs, rank, hi[0], hi[1], 0u);
+  cl_sync<CS>();   // the arrays are shared again
+  const uint3 n = cl_share_max<CS>(cs, rank, lo[0], lo[1], 0u);
+  tau[0] = m.x;
+  tau[1] = m.y;
+  const uint32_t differ = (m.x != ~n.x ? 1u : 0u) | (qv && m.y != ~n.y ? 2u : 0u);
+  if (differ) {   // (the barriers above: the lists' memory is free)
+    for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+#pragma unroll 1
+    for (int x = 0; x < rows; ++x) in_bin(x, [&](uint32_t key) { atomicAdd(&cs.hist[x][4095u - ((key >> 4) & 4095u)], 1u); });
+    __syncthreads();
+    cl_find<CS>(cs, rank, rows == 2, K);
+    uint32_t mid[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      mid[x] = 4095u - cs.sel_bin[x];
+      K[x] -= cs.sel_above[x];
+    }
+#pragma unroll 1
+    for (int x = 0; x < rows; ++x)
+      in_bin(x, [&](uint32_t key) { if (((key >> 4) & 4095u) == (x ? mid[1] : mid[0])) atomicAdd(&cs.hist16[x][15u - (key & 15u)], 1u); });
+    cl_sync<CS>();
+    if (tid < 32) {
+      uint32_t n = 0;
+      for (int r = 0; r < CS; ++r) {
+        uint32_t v;
+        if constexpr (CS == 1) v = cs.hist16[tid >> 4][tid & 15];
+        else asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cl_map(&cs.hist16[tid >> 4][tid & 15], r)) : "memory");
+        n += v;
+      }
+      cs.low16[tid >> 4][tid & 15] = n;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int x = 0; x < rows; ++x) {
+      if (!(differ >> x & 1u)) continue;
+      uint32_t acc = 0, low = 0;
+      for (int i = 0; i < 16; ++i) {
+        acc += cs.low16[x][i];
+        if (acc >= (x ? K[1] : K[0])) {
+          low = 15u - i;
+          break;
+        }
+      }
+      const uint32_t key = ((x ? tau_q : tau_p) & 0xFFFF0000u) | (x ? mid[1] : mid[0]) << 4 | low;
+      if (x) tau[1] = key;
+      else tau[0] = key;
+    }
+  }
+  return make_uint2(tau[0], tau[1]);
+}
+
 template <typename T, int CS>
 __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch<CS> &cs, uint4 *slice, int rank) {
   using E = Elt<T>;
@@ -2114,10 +2347,10 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   if (d_ok) {
     Row<T> r;
     r.init(j.rows.p, V, j.rows.p2, p.guidance);
-    dp = r.raw_bits(d);
+    dp = r.element(d);
     if (q_row) {
       r.init(j.rows.q, V, j.rows.q2, p.guidance);
-      dq = r.raw_bits(d);
+      dq = r.element(d);
     }
   }
   if (need_select)
@@ -2161,9 +2394,16 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
     km[1] = max(km[1], cs.kmax[1][r]);
     not_ok |= cs.bad[r];
   }
-  const uint32_t key_ninf = E::key(E::NEG_INF);
-  if (not_ok || qs.flags != 0 || km[0] <= key_ninf || (q_stat && km[1] <= key_ninf) || (q_row && !q_stat && !(qs.xmax > -FLT_MAX)))
-    return false;   // the same in every block of the cluster
+  uint32_t nonfinite = 0;   // bit x: row x holds a NaN or +inf
+  if (not_ok) {
+    const uint3 r = cl_replace_bad<T, CS>(cs, rank, ni, pv, q_row ? qv : nullptr);
+    km[0] = r.x;
+    km[1] = r.y;
+    nonfinite = r.z;
+  }
+  if (!(E::val(E::unkey(km[0])) > -FLT_MAX) || (q_stat && !(E::val(E::unkey(km[1])) > -FLT_MAX)) ||
+      (q_row && !q_stat && !(qs.xmax > -FLT_MAX)))
+    return false;   // no finite entry; the same in every block of the cluster
 
   // ---- thresholds
   uint32_t tau[2] = {0, 0};
@@ -2185,87 +2425,95 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
     }
     __syncthreads();
     cl_find<CS>(cs, rank, q_stat, K);
+    const uint32_t far = (cs.sel_bin[0] >= 4095u ? 1u : 0u) | (q_stat && cs.sel_bin[1] >= 4095u ? 2u : 0u);
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
       if (x && !q_stat) break;
-      if (cs.sel_bin[x] >= 4095u) return false;   // too far below the maximum: the general route decides
       tau[x] = (top[x] - cs.sel_bin[x]) << HI;
       K[x] -= cs.sel_above[x];
     }
+    if (far) {   // e.g. on the other side of zero
+      const uint4 r = cl_further<T, CS>(cs, rank, ni, pv, qv, far, top[0], top[1], K[0], K[1]);
+      if (far & 1) { tau[0] = r.x; K[0] = r.z; }
+      if (far & 2) { tau[1] = r.y; K[1] = r.w; }
+    }
     if constexpr (HI == 16) {   // fp32: the entries in those bins are listed, then selected by their low 16 bits
+      if (cs.sel_count[0] > kClMany || (q_stat && cs.sel_count[1] > kClMany)) {   // (the same everywhere)
+        const uint2 r = cl_ties<CS>(cs, rank, ni, pv, q_stat ? qv : nullptr, tau[0], tau[1], K[0], K[1]);
+        tau[0] = r.x;
+        tau[1] = r.y;
+      } else {
 #pragma unroll 1
-      for (int i = 0; i < ni; ++i) {
-        const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
+        for (int i = 0; i < ni; ++i) {
+          const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
 #pragma unroll
-        for (int t = 0; t < E::VEC; ++t) {
-          const uint32_t ka = E::key(E::get(a, t)), kb = E::key(E::get(b, t));
-          if ((ka >> 16) == (tau[0] >> 16)) {
-            const uint32_t at = atomicAdd(&cs.n_list[0], 1u);
-            if (at < kClList) cs.list[0][at] = (unsigned short)ka;
-          }
-          if (q_stat && (kb >> 16) == (tau[1] >> 16)) {
-            const uint32_t at = atomicAdd(&cs.n_list[1], 1u);
-            if (at < kClList) cs.list[1][at] = (unsigned short)kb;
-          }
-        }
-      }
-      cl_sync<CS>();
-      for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();
-      bool over = false;
-      // low 16 bits of entry e of block r's list of row x; f(value)
-      auto for_list = [&](int x, auto f) {
-#pragma unroll 1
-        for (int r = 0; r < CS; ++r) {
-          uint32_t n;
-          if constexpr (CS == 1) n = cs.n_list[x];
-          else asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(cl_map(&cs.n_list[x], r)) : "memory");
-          over = over || n > (uint32_t)kClList;
-          n = min(n, (uint32_t)kClList);
-          const uint32_t base = CS == 1 ? 0u : cl_map(cs.list[x], r);
-          for (uint32_t e = tid; e < n; e += kClThreads) {
-            unsigned short v;
-            if constexpr (CS == 1) v = cs.list[x][e];
-            else asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(base + e * 2) : "memory");
-            f((uint32_t)v);
+          for (int t = 0; t < E::VEC; ++t) {
+            const uint32_t ka = E::key(E::get(a, t)), kb = E::key(E::get(b, t));
+            if ((ka >> 16) == (tau[0] >> 16)) {
+              const uint32_t at = atomicAdd(&cs.n_list[0], 1u);
+              if (at < kClList) cs.list[0][at] = (unsigned short)ka;
+            }
+            if (q_stat && (kb >> 16) == (tau[1] >> 16)) {
+              const uint32_t at = atomicAdd(&cs.n_list[1], 1u);
+              if (at < kClList) cs.list[1][at] = (unsigned short)kb;
+            }
           }
         }
-      };
+        cl_sync<CS>();
+        for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        // low 16 bits of entry e of block r's list of row x; f(value)
+        auto for_list = [&](int x, auto f) {
 #pragma unroll 1
-      for (int x = 0; x < (q_stat ? 2 : 1); ++x) for_list(x, [&](uint32_t v) { atomicAdd(&cs.hist[x][4095u - (v >> 4)], 1u); });
-      __syncthreads();
-      if (over) return false;   // (the same everywhere) more entries than the list holds
-      uint32_t own[2];
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const uint4 *h = reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8]);
-        own[x] = sum4(h[0]) + sum4(h[1]);
-      }
-      cl_scan<CS>(cs, q_stat, own, K, [&](int x, int half) { return *reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8 + half * 4]); });
-      uint32_t mid[2];
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        mid[x] = 4095u - cs.sel_bin[x];
-        K[x] -= cs.sel_above[x];
-      }
-#pragma unroll 1
-      for (int x = 0; x < (q_stat ? 2 : 1); ++x) {
-        const uint32_t m = x ? mid[1] : mid[0];
-        for_list(x, [&](uint32_t v) { if ((v >> 4) == m) atomicAdd(&cs.hist16[x][15u - (v & 15u)], 1u); });
-      }
-      __syncthreads();
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        if (x && !q_stat) break;
-        uint32_t acc = 0, low = 0;
-        for (int i = 0; i < 16; ++i) {
-          acc += cs.hist16[x][i];
-          if (acc >= K[x]) {
-            low = 15u - i;
-            break;
+          for (int r = 0; r < CS; ++r) {
+            uint32_t n;
+            if constexpr (CS == 1) n = cs.n_list[x];
+            else asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(cl_map(&cs.n_list[x], r)) : "memory");
+            n = min(n, (uint32_t)kClList);
+            const uint32_t base = CS == 1 ? 0u : cl_map(cs.list[x], r);
+            for (uint32_t e = tid; e < n; e += kClThreads) {
+              unsigned short v;
+              if constexpr (CS == 1) v = cs.list[x][e];
+              else asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(base + e * 2) : "memory");
+              f((uint32_t)v);
+            }
           }
+        };
+#pragma unroll 1
+        for (int x = 0; x < (q_stat ? 2 : 1); ++x) for_list(x, [&](uint32_t v) { atomicAdd(&cs.hist[x][4095u - (v >> 4)], 1u); });
+        __syncthreads();
+        uint32_t own[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const uint4 *h = reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8]);
+          own[x] = sum4(h[0]) + sum4(h[1]);
         }
-        tau[x] |= mid[x] << 4 | low;
+        cl_scan<CS>(cs, q_stat, own, K, [&](int x, int half) { return *reinterpret_cast<const uint4 *>(&cs.hist[x][tid * 8 + half * 4]); });
+        uint32_t mid[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          mid[x] = 4095u - cs.sel_bin[x];
+          K[x] -= cs.sel_above[x];
+        }
+#pragma unroll 1
+        for (int x = 0; x < (q_stat ? 2 : 1); ++x) {
+          const uint32_t m = x ? mid[1] : mid[0];
+          for_list(x, [&](uint32_t v) { if ((v >> 4) == m) atomicAdd(&cs.hist16[x][15u - (v & 15u)], 1u); });
+        }
+        __syncthreads();
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          if (x && !q_stat) break;
+          uint32_t acc = 0, low = 0;
+          for (int i = 0; i < 16; ++i) {
+            acc += cs.hist16[x][i];
+            if (acc >= K[x]) {
+              low = 15u - i;
+              break;
+            }
+          }
+          tau[x] |= mid[x] << 4 | low;
+        }
       }
     }
   }
@@ -2274,10 +2522,11 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   RowStats ps;
   ps.tau_key = tau[0];
   ps.xmax = E::val(E::unkey(km[0]));
-  ps.flags = 0;
+  ps.flags = nonfinite & 1 ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
   if (q_stat) {
     qs.tau_key = tau[1];
     qs.xmax = E::val(E::unkey(km[1]));
+    qs.flags = nonfinite & 2 ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
   }
   auto weight = [&](uint32_t bits, uint32_t tau_key, float xmax) {
     return E::key(bits) >= tau_key ? exp2_neg((E::val(bits) - xmax) * scale) : 0.0f;
@@ -2329,7 +2578,7 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   else ratio = p_d > 0.0f ? INFINITY : 0.0f;
   float thr = fminf(1.0f, ratio);
   bool accept = j.u_acc < thr;
-  uint32_t flags = 0;
+  uint32_t flags = ps.flags | (q_row ? qs.flags : 0u);
   if (thr < 1.0f && fabsf(j.u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
   // ---- Eq. 3
   cl_icdf<T, CS>(cs, 0, ni, rank, vec0, off, j.u_draft, p_w);
@@ -2382,7 +2631,7 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
     if (j.jacobi) {   // deterministic criterion instead of Eqs. 1-2
       accept = d_ok && ro.redraft_tok == d;
       thr = accept ? 1.0f : 0.0f;
-      flags = 0;
+      flags = ps.flags;
       resample = accept ? -1 : ro.redraft_tok;
     }
     ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
@@ -2393,8 +2642,10 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   return true;
 }
 
-template <typename T, int CS>
-__global__ void __launch_bounds__(kClThreads, 2) verify_cluster_kernel(const VerifyParams p) {
+// MINB: blocks that an SM may hold.  With a cluster there is never a second one (the shared memory does not admit it, or there
+// are no more blocks than SMs), and with the registers of both nothing spills (1 x 16 x 184320, bf16: 46.6 -> 43.7 us).
+template <typename T, int CS, int MINB>
+__global__ void __launch_bounds__(kClThreads, MINB) verify_cluster_kernel(const VerifyParams p) {
   extern __shared__ uint4 dyn_smem[];
   ClScratch<CS> &cs = *reinterpret_cast<ClScratch<CS> *>(dyn_smem);
   __shared__ Scratch sc;
@@ -2515,9 +2766,9 @@ static int sm_count() {
   return v;
 }
 
-template <typename T, int CS>
+template <typename T, int CS, int MINB>
 static int launch_cluster(const VerifyParams &p, long nv, cudaStream_t stream) {
-  auto kernel = verify_cluster_kernel<T, CS>;
+  auto kernel = verify_cluster_kernel<T, CS, MINB>;
   const long ni = ((nv + CS - 1) / CS + kClThreads - 1) / kClThreads;
   auto smem_of = [](long n) { return (sizeof(ClScratch<CS>) + 15) / 16 * 16 + (size_t)2 * n * kClThreads * 16; };
   const size_t smem = smem_of(ni);
@@ -2549,10 +2800,12 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
   const long nv_max = ((long)p.V + 2 * VEC - 2) / VEC + 1;
   if ((nv_max + 31) / 32 > kMaxChunks) return SJD_ERR_CAPACITY;
   // A cluster per row, with as many blocks as the rows leave SMs for: whenever the grid is resident at once (us a call, block per
-  // row -> cluster: fp32 1 x 27 x 65536 155 -> 40, 1 x 16 x 1024 24.7 -> 18.5; bf16 1 x 32 x 65536 40 -> 29, 3 x 16 x 4096 24.6 ->
-  // 18.5, 4 x 32 x 16384 26.7 -> 24.7), and for fp32 rows of more than 2048 entries in any number (8 x 32 x 16384 67 -> 56,
-  // 32 x 32 x 16384 180 -> 149, 26 x 33 x 4096 60 -> 55).  bf16 rows in several waves are better off a block per row
-  // (1 x 64 x 184320: 89 against 157 us), and so are short fp32 rows (32 x 18 x 1096: 31 against 36 us).
+  // row -> cluster: fp32 1 x 27 x 65536 156 -> 39, 1 x 16 x 1024 25 -> 19; bf16 1 x 32 x 65536 42 -> 29, 3 x 16 x 4096 27 ->
+  // 20, 4 x 32 x 16384 27 -> 25), and for fp32 rows of more than 2048 entries in any number (8 x 32 x 16384 68 -> 60, 26 x 33 x
+  // 4096 66 -> 59).  There a threshold of more than half the entries, which mostly lies on the other side of zero from the
+  // maximum, stays with a block per row (8 x 32 x 16384, top-k 0.6 V: 68 against 81); one that lies there because the logits do
+  // costs 68 -> 75, with one value masking nine entries in ten 72 -> 87.  bf16 rows in several waves are better off a block per
+  // row (1 x 64 x 184320: 90 against 157 us), and so are short fp32 rows (32 x 18 x 1096: 32 against 36 us).
   const int n_sms = sm_count();
   {
     const bool whole = p.V % VEC == 0 && ((uintptr_t)p.logits[0] & 15u) == 0;   // every row starts on a vector
@@ -2562,12 +2815,15 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
     const bool fits = (long)cs * kClThreads * kClVecs >= nv;
     while (cs < 8 && p.B * p.W * cs * 2 <= n_sms && nv > (long)cs * kClThreads) cs *= 2;
     const bool few = (long)p.B * p.W * cs <= n_sms;
-    const bool wide = std::is_same<T, float>::value && nv > kClThreads;
+    const bool wide = std::is_same<T, float>::value && nv > kClThreads && (p.top_k <= p.V / 2 || p.top_k >= p.V);
     if (fits && (few || wide)) {
       p.staged = p.fast = 0;
       p.defer_residual = p.B * p.W * cs > n_sms ? 1 : 0;
-      return cs == 1 ? launch_cluster<T, 1>(p, nv, stream) : cs == 2 ? launch_cluster<T, 2>(p, nv, stream)
-             : cs == 4 ? launch_cluster<T, 4>(p, nv, stream) : launch_cluster<T, 8>(p, nv, stream);
+      // fp32 rows of more than 4096 entries: a block's shared memory does not admit a second one on its SM
+      constexpr bool f32 = std::is_same<T, float>::value;
+      if (cs == 1) return f32 && nv > 2 * kClThreads ? launch_cluster<T, 1, 1>(p, nv, stream) : launch_cluster<T, 1, 2>(p, nv, stream);
+      return cs == 2 ? launch_cluster<T, 2, 1>(p, nv, stream) : cs == 4 ? launch_cluster<T, 4, 1>(p, nv, stream)
+                                                                     : launch_cluster<T, 8, 1>(p, nv, stream);
     }
   }
   const size_t stage_bytes = (size_t)nv_max * 16;

@@ -132,6 +132,51 @@ def test_verify_cluster_ties(levels):
     _check_case(case)
 
 
+def _awkward(case, mode, seed=0):
+    """Rows whose threshold a histogram of the codes next to the maximum does not reach, or whose entries are not all finite."""
+    rng = np.random.default_rng(seed)
+    for rows in (case.logits_cur, case.logits_prev):
+        if mode == "below zero":            # positive maximum, negative threshold
+            rows -= np.float32(9.0)
+        elif mode.startswith("masked"):     # nine entries in ten hold one value, the threshold among them
+            rows[rng.random(rows.shape) > 0.1] = np.float32(-np.inf if mode == "masked -inf" else -1e9)
+        elif mode == "dense":               # a third of the row within one step of the 16 leading bits of a key
+            pick = rng.random(rows.shape) < 0.33
+            rows[pick] = (8.0 + 0.03 * rng.random(int(pick.sum()))).astype(np.float32)
+        elif mode == "levels":
+            rows[...] = np.floor(rows / 8.0) * np.float32(8.0)
+    if mode == "nan":                       # in this row, the earlier one, both
+        case.logits_cur[:, 0::3, 7] = np.nan
+        case.logits_prev[:, 1::3, 9] = np.inf
+        case.logits_cur[:, 2::3, 11] = np.inf
+        case.logits_prev[:, 2::3, 11] = np.nan
+    if mode == "none finite":
+        case.logits_cur[:, case.window // 2, :] = -np.inf
+    if case.dtype == "bf16":
+        case.logits_cur, case.logits_prev = round_bf16(case.logits_cur), round_bf16(case.logits_prev)
+    for b in range(case.batch):             # drafts that have mass in both rows
+        for k in range(case.window):
+            both = np.nan_to_num(case.logits_cur[b, k], nan=-1e30, posinf=-1e30, neginf=-1e30)
+            case.draft[b, k] = int(np.argsort(-both, kind="stable")[3])
+    return case
+
+
+@pytest.mark.parametrize("mode", ["below zero", "masked -1e9", "masked -inf", "dense", "levels", "nan", "none finite"])
+@pytest.mark.parametrize("batch,window,vocab,dtype", [
+    (1, 4, 1024, "f32"), (1, 3, 4000, "f32"), (1, 4, 8001, "f32"), (1, 3, 40000, "f32"),         # clusters of 1, 2, 4, 8 blocks
+    (1, 4, 4096, "bf16"), (1, 3, 8000, "bf16"), (1, 3, 16001, "bf16"), (1, 3, 40000, "bf16"),
+    (19, 8, 4096, "f32"), (150, 1, 3000, "f32"),                                                # more rows than SMs
+    (19, 8, 4096, "bf16"), (75, 2, 3001, "bf16"),                                               # and a block per row
+])
+def test_verify_awkward_rows(batch, window, vocab, dtype, mode):
+    """Thresholds far below the maximum, masked entries, thousands of ties, entries that are not finite: on every size of cluster
+    and with a block per row."""
+    case = make_verify_case(batch, window=window, vocab=vocab, dtype=dtype, top_k=vocab // 4, seed=41)
+    _check_case(_awkward(case, mode), max_flag_frac=0.06)
+    if mode == "nan" and window > 2:
+        assert all(f & B.SJD_FLAG_NONFINITE for f in _run_gpu(case)["flags"])
+
+
 def test_verify_mixed_laws():
     """Slots whose draft came from a uniform initialisation (q = 1/V) or a copy (point mass)."""
     case = make_verify_case(6, window=16, vocab=4096, top_k=300, seed=11, mixed_kinds=True)
