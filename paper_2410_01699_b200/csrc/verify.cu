@@ -30,6 +30,7 @@
 // (verify_cluster_kernel; the rule is in launch_verify_t).
 #include <float.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1614,89 +1615,6 @@ __device__ void general_residual(const ResidualWeights<T> &rf, const PRowWeights
   }
 }
 
-// the general route: any row, block-wide
-template <typename T>
-__device__ void general_row(const VerifyParams &p, const RowJob<T> &j, uint4 *stage, Scratch &sc) {
-  using E = Elt<T>;
-  const int tid = threadIdx.x, kind = j.kind, d = j.d;
-  const bool d_ok = d >= 0 && d < p.V;
-  __syncthreads();
-  // ---- the law of the draft
-  Row<T> qrow;
-  qrow.init(j.rows.q, p.V, j.rows.q2, p.guidance);
-  RowStats qs;
-  qs.tau_key = 0; qs.xmax = 0.0f; qs.z = 1.0f; qs.flags = 0;
-  PRowWeights<T> qf;
-  float q_d;
-  if (kind == SJD_Q_ROW) {
-    if (p.prev_stats_valid) {
-      qs = *j.rows.qstats;
-    } else {
-      qs = row_statistics<T>(qrow, stage, sc, p.top_k, j.inv_t, qf);
-      if (tid == 0) p.stats[j.cur ^ 1][j.r] = qs;
-      __syncthreads();
-      qrow.s = nullptr;  // the staging buffer is about to be reused
-    }
-    qf.row = qrow;
-    qf.pw.init(qs, j.inv_t);
-    q_d = d_ok ? qf.pw.one(qrow.element(d), d) / qs.z : 1.0f;
-  } else if (kind == SJD_Q_UNIFORM) {
-    q_d = 1.0f / (float)p.V;
-  } else {
-    q_d = 1.0f;
-  }
-
-  SJD_TL(TL_VERIFY, 10, tid == 0);   // the draft's law is known
-  // ---- this iteration's distribution
-  Row<T> prow;
-  prow.init(j.rows.p, p.V, j.rows.p2, p.guidance);
-  PRowWeights<T> pf;
-  const RowStats ps = row_statistics<T>(prow, stage, sc, p.top_k, j.inv_t, pf);
-  if (tid == 0) p.stats[j.cur][j.r] = ps;
-  const float p_d = d_ok ? pf.pw.one(prow.element(d), d) / ps.z : 0.0f;
-
-  SJD_TL(TL_VERIFY, 11, tid == 0);   // this row's statistics are known
-  // ---- Eq. 1
-  float ratio;
-  if (q_d > 0.0f) ratio = p_d / q_d;
-  else ratio = p_d > 0.0f ? INFINITY : 0.0f;
-  float thr = fminf(1.0f, ratio);
-  bool accept = j.u_acc < thr;
-  uint32_t flags = ps.flags | (kind == SJD_Q_ROW ? qs.flags : 0u);
-  if (thr < 1.0f && fabsf(j.u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
-
-  // ---- Eq. 3: re-draft from p (used if an earlier row rejects)
-  sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, j.u_draft);
-  const int redraft_tok = sc.tok;
-  const float redraft_p = sc.tok_w / ps.z;
-  __syncthreads();
-
-  SJD_TL(TL_VERIFY, 12, tid == 0);   // re-draft token drawn
-  // ---- Eq. 2: residual resample (used if this is the first rejected row)
-  int resample_tok = -1;
-  if (j.jacobi) {   // deterministic criterion instead of Eqs. 1-2
-    accept = d_ok && redraft_tok == d;
-    thr = accept ? 1.0f : 0.0f;
-    flags &= ~SJD_FLAG_NEAR_TIE_ACCEPT;
-    resample_tok = accept ? -1 : redraft_tok;
-  } else if (!accept) {
-    ResidualWeights<T> rf;
-    rf.prow = prow; rf.qrow = qrow; rf.pw = pf.pw; rf.qw = qf.pw;
-    rf.inv_zp = 1.0f / ps.z; rf.inv_zq = 1.0f / qs.z;
-    rf.kind = kind; rf.draft = d; rf.V = p.V;
-    if (kind != SJD_Q_ROW) rf.qw = pf.pw;
-    general_residual<T>(rf, pf, j.u_res, sc, flags);
-    resample_tok = sc.tok;
-  }
-  SJD_TL(TL_VERIFY, 13, tid == 0);   // residual token drawn
-  if (tid == 0) {
-    RowOut ro;
-    ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
-    ro.redraft_tok = redraft_tok; ro.redraft_p = redraft_p; ro.resample_tok = resample_tok; ro.flags = flags;
-    p.row_out[j.r] = ro;
-  }
-}
-
 // After a block's row record is written (block-wide): a ticket; the last block of the sequence slides the window.
 // `deferred(...)`: makes the Eq. 2 draw that the rows of the sequence have left open.
 template <typename T, typename F>
@@ -1733,6 +1651,7 @@ __device__ void ticket_and_slide(const VerifyParams &p, int b, uint32_t step, in
 // STREAM: the instantiation launched for bf16 rows too long for the registers of a block (see long_statistics)
 template <typename T, int MAXT, bool STREAM = false>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1) verify_rows_kernel(const VerifyParams p) {
+  using E = Elt<T>;
   extern __shared__ uint4 dyn_smem[];
   __shared__ Scratch sc;
   uint4 *stage = p.staged ? dyn_smem : nullptr;
@@ -1741,21 +1660,129 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1)
   pdl_wait();   // the logits come from the preceding kernel
   SJD_TL(TL_VERIFY, 1, threadIdx.x == 0);
 
-  RowJob<T> j;
-  if (row_job<T>(p, blockIdx.x, j)) {
+  const int r = blockIdx.x;
+  const int b = r / p.W, k = r % p.W;
+  const int sb = p.paired ? 2 * b : b;   // sequence whose state describes the window (under guidance both streams' do)
+  const int rs = sb * p.W + k;
+  const int tid = threadIdx.x;
+  const int w_eff = p.w_eff ? p.w_eff[sb] : p.W;
+  const uint32_t step = p.step_ptr ? *p.step_ptr : p.step;
+  const int cur = p.step_ptr ? (int)(step & 1u) : 0;
+  const float inv_t = 1.0f / p.temperature;
+
+  if (k < w_eff) {
+    // (the Jacobi schedule compares tokens and uses no q: treat every draft as a copied one)
+    const int kind_raw = p.q_kind ? p.q_kind[rs] : SJD_Q_ROW;
+    const bool q_ring = kind_raw == SJD_Q_RING;   // a retained row: the same law as a row of the other buffer
+    const int kind = p.schedule == SJD_SCHEDULE_JACOBI ? SJD_Q_ONEHOT : (q_ring ? SJD_Q_ROW : kind_raw);
+    const int d = p.draft[rs];
+    const bool d_ok = d >= 0 && d < p.V;
+    const int qr = p.q_row ? p.q_row[rs] : k;
+    const int base = p.e2e ? p.st.n[sb] : (p.base_pos ? p.base_pos[b] : 0);
+    const Philox4 rnd = philox4x32_10((uint32_t)(base + k), step, p.seq_base + (uint32_t)b, kStreamVerify,
+                                      p.seed_lo, p.seed_hi);
+    const float u_acc = u24(rnd.w[0]), u_res = u24(rnd.w[1]);
+    float u_draft = u24(rnd.w[2]);
+    const bool jacobi = p.schedule == SJD_SCHEDULE_JACOBI;
+    if (jacobi)   // Sec. 3.2: the draw of a position uses the same uniform in every pass (step index 0)
+      u_draft = u24(philox4x32_10((uint32_t)(base + k), 0u, p.seq_base + (uint32_t)b, kStreamVerify, p.seed_lo, p.seed_hi).w[2]);
+    const RowRefs<T> rows = row_refs<T>(p, b, k, qr, cur, q_ring);
+
     RowOut fast_out;
-    const bool fast_done = p.fast && (((uintptr_t)j.rows.q | (uintptr_t)j.rows.p) & 15u) == 0 &&
-                           fast_row<T, STREAM>(p, sc, j.r, j.b, j.kind, j.d, j.qr, j.cur, j.rows, j.inv_t, j.u_acc, j.u_res, j.u_draft,
-                                               fast_out);
+    const bool fast_done = p.fast && (((uintptr_t)rows.q | (uintptr_t)rows.p) & 15u) == 0 &&
+                           fast_row<T, STREAM>(p, sc, r, b, kind, d, qr, cur, rows, inv_t, u_acc, u_res, u_draft, fast_out);
     if (fast_done) {
-      if (threadIdx.x == 0) p.row_out[j.r] = fast_out;
+      if (tid == 0) p.row_out[r] = fast_out;
     } else {
-      general_row<T>(p, j, stage, sc);
+    __syncthreads();
+    // ---- the law of the draft
+    Row<T> qrow;
+    qrow.init(rows.q, p.V, rows.q2, p.guidance);
+    RowStats qs;
+    qs.tau_key = 0; qs.xmax = 0.0f; qs.z = 1.0f; qs.flags = 0;
+    PRowWeights<T> qf;
+    float q_d;
+    if (kind == SJD_Q_ROW) {
+      if (p.prev_stats_valid) {
+        qs = *rows.qstats;
+      } else {
+        qs = row_statistics<T>(qrow, stage, sc, p.top_k, inv_t, qf);
+        if (tid == 0) p.stats[cur ^ 1][r] = qs;
+        __syncthreads();
+        qrow.s = nullptr;  // the staging buffer is about to be reused
+      }
+      qf.row = qrow;
+      qf.pw.init(qs, inv_t);
+      q_d = d_ok ? qf.pw.one(qrow.element(d), d) / qs.z : 1.0f;
+    } else if (kind == SJD_Q_UNIFORM) {
+      q_d = 1.0f / (float)p.V;
+    } else {
+      q_d = 1.0f;
     }
+
+    SJD_TL(TL_VERIFY, 10, tid == 0);   // the draft's law is known
+    // ---- this iteration's distribution
+    Row<T> prow;
+    prow.init(rows.p, p.V, rows.p2, p.guidance);
+    PRowWeights<T> pf;
+    const RowStats ps = row_statistics<T>(prow, stage, sc, p.top_k, inv_t, pf);
+    if (tid == 0) p.stats[cur][r] = ps;
+    const float p_d = d_ok ? pf.pw.one(prow.element(d), d) / ps.z : 0.0f;
+
+    SJD_TL(TL_VERIFY, 11, tid == 0);   // this row's statistics are known
+    // ---- Eq. 1
+    float ratio;
+    if (q_d > 0.0f) ratio = p_d / q_d;
+    else ratio = p_d > 0.0f ? INFINITY : 0.0f;
+    float thr = fminf(1.0f, ratio);
+    bool accept = u_acc < thr;
+    uint32_t flags = ps.flags | (kind == SJD_Q_ROW ? qs.flags : 0u);
+    if (thr < 1.0f && fabsf(u_acc - thr) < 1e-4f) flags |= SJD_FLAG_NEAR_TIE_ACCEPT;
+
+    // ---- Eq. 3: re-draft from p (used if an earlier row rejects)
+    sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, u_draft);
+    const int redraft_tok = sc.tok;
+    const float redraft_p = sc.tok_w / ps.z;
+    __syncthreads();
+
+    SJD_TL(TL_VERIFY, 12, tid == 0);   // re-draft token drawn
+    // ---- Eq. 2: residual resample (used if this is the first rejected row)
+    int resample_tok = -1;
+    if (jacobi) {   // deterministic criterion instead of Eqs. 1-2
+      accept = d_ok && redraft_tok == d;
+      thr = accept ? 1.0f : 0.0f;
+      flags &= ~SJD_FLAG_NEAR_TIE_ACCEPT;
+      resample_tok = accept ? -1 : redraft_tok;
+    } else if (!accept) {
+      ResidualWeights<T> rf;
+      rf.prow = prow; rf.qrow = qrow; rf.pw = pf.pw; rf.qw = qf.pw;
+      rf.inv_zp = 1.0f / ps.z; rf.inv_zq = 1.0f / qs.z;
+      rf.kind = kind; rf.draft = d; rf.V = p.V;
+      if (kind != SJD_Q_ROW) rf.qw = pf.pw;
+      chunk_sums<E::VEC>(rf, prow.NV, sc);
+      if (sc.chunk_excl[(prow.NV + 31) >> 5] > 0.0) {
+        sample_icdf<E::VEC>(rf, prow.NV, prow.off, sc, u_res);
+      } else {
+        flags |= SJD_FLAG_RESIDUAL_EMPTY;
+        __syncthreads();
+        chunk_sums<E::VEC>(pf, prow.NV, sc);
+        sample_icdf<E::VEC>(pf, prow.NV, prow.off, sc, u_res);
+      }
+      resample_tok = sc.tok;
+    }
+    SJD_TL(TL_VERIFY, 13, tid == 0);   // residual token drawn
+    if (tid == 0) {
+      RowOut ro;
+      ro.p_draft = p_d; ro.q_draft = q_d; ro.thr = thr; ro.accept = accept ? 1 : 0;
+      ro.redraft_tok = redraft_tok; ro.redraft_p = redraft_p; ro.resample_tok = resample_tok; ro.flags = flags;
+      p.row_out[r] = ro;
+    }
+    }   // general route
   }
-  ticket_and_slide<T>(p, j.b, j.step, j.cur, sc, [&]() {
+
+  ticket_and_slide<T>(p, b, step, cur, sc, [&]() {
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-      if (p.fast && p.defer_residual) deferred_residual_bf16<STREAM>(p, j.b, j.step, j.cur, sc);
+      if (p.fast && p.defer_residual) deferred_residual_bf16<STREAM>(p, b, step, cur, sc);
     }
   });
 }
@@ -1766,9 +1793,9 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? SJD_VERIFY_MIN_BLOCKS : 1)
 // the histograms, once for the sums.  The threshold is exact: a histogram of the distances below the maximum in the top 16
 // bits of the key (as on the register route; a threshold beyond its 4095 codes takes further windows, cl_further); for fp32 the
 // entries in the bin found are then listed (usually some hundred) and every block selects among their low 16 bits (from the
-// slices where they are many, cl_ties).  Only a row without a finite entry is left to the general route: a block that tries
-// this one first and then reads its row again is slower than a block per row was (us a call with a block per row / with such
-// rows left to it / decided here: fp32 1 x 27 x 65536, threshold below zero 154 / 216 / 48, most entries masked with one value
+// slices where they are many, cl_ties).  No row is left to the general route: a block that tries this one first and then reads
+// its row again is slower than a block per row was (us a call with a block per row / with such rows left to the general route /
+// decided here: fp32 1 x 27 x 65536, threshold below zero 154 / 216 / 48, most entries masked with one value
 // 163 / 231 / 52, a NaN in each row 156 / 214 / 43; bf16 1 x 16 x 184320, threshold below zero 292 / 320 / 66).
 // Bound by the chain of barriers, block scans and round trips (each about
 // a microsecond) and by instruction fetch: every phase runs once, so its loops are kept rolled.
@@ -2085,7 +2112,7 @@ __device__ __forceinline__ void cl_max(const uint4 &v, float &mx, bool &bad, __n
   mx = fmaxf(mx, fmaxf(a, b));
 }
 
-// What few rows need is kept out of line: the kernel is bound by instruction fetch as well.  pv, qv: the slices, vector i of a
+// What only odd rows need is kept out of line: the kernel is bound by instruction fetch as well.  pv, qv: the slices, vector i of a
 // thread at [i * kClThreads]; qv null: no q row.
 
 // The largest keys of the two rows and the union of `bad` over all blocks.  One block and one cluster barrier; the arrays may
@@ -2127,22 +2154,24 @@ __device__ __forceinline__ uint3 cl_share_max(ClScratch<CS> &cs, int rank, uint3
   return all;
 }
 
-// As in the general route, a NaN or +inf counts as -inf: replaces them in the slices.  The largest keys of both rows, and a bit
-// for each row that held one.
+// Rows with a NaN or +inf, or without a finite entry, read as in the general route: what is not finite counts as -inf, and a row
+// that has nothing else has all its mass on token 0 (here: a 0 there and -inf elsewhere).  Rewrites the slices.  The largest
+// keys of both rows, and a bit for each row (1, 2) that held a NaN or +inf and (4, 8) that has no finite entry.
 template <typename T, int CS>
-__device__ __noinline__ uint3 cl_replace_bad(ClScratch<CS> &cs, int rank, int ni, uint4 *pv, uint4 *qv) {
+__device__ __noinline__ uint3 cl_repair(ClScratch<CS> &cs, int rank, int ni, int vec0, int off, uint4 *pv, uint4 *qv) {
   using E = Elt<T>;
-  uint32_t km[2] = {0u, 0u}, bad = 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = (qv ? 2 : 1) * ni;
+  uint32_t km[2] = {0u, 0u}, bits = 0;
 #pragma unroll 1
-  for (int i = 0; i < (qv ? 2 : 1) * ni; ++i) {
-    uint4 &at = i < ni ? pv[i * kClThreads] : qv[(i - ni) * kClThreads];
+  for (int i = 0; i < n; ++i) {
     const int x = i < ni ? 0 : 1;
+    uint4 &at = x ? qv[(i - ni) * kClThreads] : pv[i * kClThreads];
     uint4 v = at;
 #pragma unroll
     for (int t = 0; t < E::VEC; ++t) {
       if (E::bad(E::get(v, t))) {
         E::set(v, t, E::NEG_INF);
-        bad |= 1u << x;
+        bits |= 1u << x;
       }
       const uint32_t k = E::key(E::get(v, t));
       if (x) km[1] = max(km[1], k);
@@ -2151,7 +2180,23 @@ __device__ __noinline__ uint3 cl_replace_bad(ClScratch<CS> &cs, int rank, int ni
     at = v;
   }
   cl_sync<CS>();   // every block has read the first maxima
-  return cl_share_max<CS>(cs, rank, km[0], km[1], bad);
+  uint3 r = cl_share_max<CS>(cs, rank, km[0], km[1], bits);
+#pragma unroll 1
+  for (int x = 0; x < (qv ? 2 : 1); ++x) {
+    if (E::val(E::unkey(x ? r.y : r.x)) > -FLT_MAX) continue;
+    r.z |= 4u << x;
+    if (x) r.y = E::key(E::bits(0.0f));
+    else r.x = E::key(E::bits(0.0f));
+#pragma unroll 1
+    for (int i = 0; i < ni; ++i) {
+      const int i0 = (vec0 + (warp * ni + i) * 32 + lane) * E::VEC - off;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int t = 0; t < E::VEC; ++t) E::set(v, t, i0 + t == 0 ? E::bits(0.0f) : E::NEG_INF);
+      (x ? qv : pv)[i * kClThreads] = v;
+    }
+  }
+  return r;
 }
 
 // The threshold lies further below the maximum than the histogram's 4095 codes, in row 0 and / or 1 (bits of `open`): window after
@@ -2183,24 +2228,14 @@ __device__ __noinline__ uint4 cl_further(ClScratch<CS> &cs, int rank, int ni, co
     top[1] = m.y;
     for (int i = tid; i < 2048; i += kClThreads) reinterpret_cast<uint4 *>(cs.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    uint32_t equal[2] = {0u, 0u};   // entries at the top of the window: many at once where a row is masked with one value
 #pragma unroll 1
     for (int i = 0; i < ni; ++i) {
       const uint4 a = pv[i * kClThreads], b = qv[i * kClThreads];
 #pragma unroll
-      for (int t = 0; t < E::VEC; ++t) {
-        // (entries above the window wrap to its last bin, as those below it)
-        const uint32_t da = top[0] - (E::key(E::get(a, t)) >> HI), db = top[1] - (E::key(E::get(b, t)) >> HI);
-        if (da == 0u) ++equal[0];
-        else atomicAdd(&cs.hist[0][min(da, 4095u)], 1u);
-        if (db == 0u) ++equal[1];
-        else atomicAdd(&cs.hist[1][min(db, 4095u)], 1u);
+      for (int t = 0; t < E::VEC; ++t) {   // (entries above the window wrap to its last bin, as those below it)
+        atomicAdd(&cs.hist[0][min(top[0] - (E::key(E::get(a, t)) >> HI), 4095u)], 1u);
+        atomicAdd(&cs.hist[1][min(top[1] - (E::key(E::get(b, t)) >> HI), 4095u)], 1u);
       }
-    }
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const uint32_t n = __reduce_add_sync(0xffffffffu, equal[x]);
-      if ((tid & 31) == 0) atomicAdd(&cs.hist[x][0], n);
     }
     __syncthreads();
     cl_find<CS>(cs, rank, true, K);
@@ -2311,7 +2346,7 @@ __device__ __noinline__ uint2 cl_ties(ClScratch<CS> &cs, int rank, int ni, const
 }
 
 template <typename T, int CS>
-__device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch<CS> &cs, uint4 *slice, int rank) {
+__device__ void cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch<CS> &cs, uint4 *slice, int rank) {
   using E = Elt<T>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = p.V, d = j.d;
@@ -2347,10 +2382,10 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   if (d_ok) {
     Row<T> r;
     r.init(j.rows.p, V, j.rows.p2, p.guidance);
-    dp = r.element(d);
+    dp = r.raw_bits(d);
     if (q_row) {
       r.init(j.rows.q, V, j.rows.q2, p.guidance);
-      dq = r.element(d);
+      dq = r.raw_bits(d);
     }
   }
   if (need_select)
@@ -2394,16 +2429,22 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
     km[1] = max(km[1], cs.kmax[1][r]);
     not_ok |= cs.bad[r];
   }
-  uint32_t nonfinite = 0;   // bit x: row x holds a NaN or +inf
-  if (not_ok) {
-    const uint3 r = cl_replace_bad<T, CS>(cs, rank, ni, pv, q_row ? qv : nullptr);
+  uint32_t odd = 0;   // of cl_repair
+  constexpr uint32_t kLowest = sizeof(T) == 4 ? 0x00800000u : 0x007Fu;   // key of the lowest row maximum that counts as none: -FLT_MAX, in bf16 -inf
+  if (not_ok || km[0] <= kLowest || (q_row && km[1] <= kLowest)) {
+    const uint3 r = cl_repair<T, CS>(cs, rank, ni, vec0, off, pv, q_row ? qv : nullptr);
     km[0] = r.x;
     km[1] = r.y;
-    nonfinite = r.z;
+    odd = r.z;
+    if (E::bad(dp)) dp = E::NEG_INF;
+    if (E::bad(dq)) dq = E::NEG_INF;
+    if (odd & 4u) dp = d == 0 ? E::bits(0.0f) : E::NEG_INF;
+    if (odd & 8u) {
+      dq = d == 0 ? E::bits(0.0f) : E::NEG_INF;
+      qs.tau_key = 0u;
+      qs.xmax = 0.0f;
+    }
   }
-  if (!(E::val(E::unkey(km[0])) > -FLT_MAX) || (q_stat && !(E::val(E::unkey(km[1])) > -FLT_MAX)) ||
-      (q_row && !q_stat && !(qs.xmax > -FLT_MAX)))
-    return false;   // no finite entry; the same in every block of the cluster
 
   // ---- thresholds
   uint32_t tau[2] = {0, 0};
@@ -2522,11 +2563,11 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   RowStats ps;
   ps.tau_key = tau[0];
   ps.xmax = E::val(E::unkey(km[0]));
-  ps.flags = nonfinite & 1 ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
+  ps.flags = odd & 1u ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
   if (q_stat) {
     qs.tau_key = tau[1];
     qs.xmax = E::val(E::unkey(km[1]));
-    qs.flags = nonfinite & 2 ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
+    qs.flags = odd & 2u ? (uint32_t)SJD_FLAG_NONFINITE : 0u;
   }
   auto weight = [&](uint32_t bits, uint32_t tau_key, float xmax) {
     return E::key(bits) >= tau_key ? exp2_neg((E::val(bits) - xmax) * scale) : 0.0f;
@@ -2565,8 +2606,12 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
   ps.z = (float)zp;
   if (q_stat) qs.z = (float)zq;
   if (rank == 0 && tid == 0) {
-    p.stats[j.cur][j.r] = ps;
-    if (q_stat) p.stats[j.cur ^ 1][j.r] = qs;
+    auto keep = [](RowStats st, uint32_t none) {   // (whoever evaluates the row itself knows it by its maximum)
+      if (none) st.xmax = -INFINITY;
+      return st;
+    };
+    p.stats[j.cur][j.r] = keep(ps, odd & 4u);
+    if (q_stat) p.stats[j.cur ^ 1][j.r] = keep(qs, odd & 8u);
   }
   // ---- Eq. 1
   const float p_d = d_ok ? weight(dp, ps.tau_key, ps.xmax) / ps.z : 0.0f;
@@ -2639,7 +2684,6 @@ __device__ bool cluster_row(const VerifyParams &p, const RowJob<T> &j, ClScratch
     ro.flags = flags;
     p.row_out[j.r] = ro;
   }
-  return true;
 }
 
 // MINB: blocks that an SM may hold.  With a cluster there is never a second one (the shared memory does not admit it, or there
@@ -2657,11 +2701,7 @@ __global__ void __launch_bounds__(kClThreads, MINB) verify_cluster_kernel(const 
   const int rank = (int)(blockIdx.x % CS);
   RowJob<T> j;
   if (row_job<T>(p, (int)(blockIdx.x / CS), j)) {
-    const bool done = cluster_row<T, CS>(p, j, cs, dyn_smem + (sizeof(ClScratch<CS>) + 15) / 16, rank);
-    if (!done) {
-      cl_sync<CS>();   // no block leaves while another may still store into it
-      if (rank == 0) general_row<T>(p, j, nullptr, sc);
-    }
+    cluster_row<T, CS>(p, j, cs, dyn_smem + (sizeof(ClScratch<CS>) + 15) / 16, rank);
   }
   if (rank != 0) return;
   ticket_and_slide<T>(p, j.b, j.step, j.cur, sc, [&]() {
@@ -2760,9 +2800,14 @@ size_t verify_scratch_bytes(int batch, int window) {
   return (b + 255) / 256 * 256;
 }
 
+// of the current device
 static int sm_count() {
+  static std::atomic<int> known[64] = {};
   int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 148;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if ((v = known[dev].load(std::memory_order_relaxed)) > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) return 148;
+  known[dev].store(v, std::memory_order_relaxed);
   return v;
 }
 

@@ -151,7 +151,10 @@ def _awkward(case, mode, seed=0):
         case.logits_cur[:, 2::3, 11] = np.inf
         case.logits_prev[:, 2::3, 11] = np.nan
     if mode == "none finite":
-        case.logits_cur[:, case.window // 2, :] = -np.inf
+        case.logits_cur[::2, case.window // 2, :] = -np.inf
+        case.logits_prev[1::2, 0, :] = -np.inf
+        if case.batch == 1:
+            case.logits_prev[:, 0, :] = -np.inf
     if case.dtype == "bf16":
         case.logits_cur, case.logits_prev = round_bf16(case.logits_cur), round_bf16(case.logits_prev)
     for b in range(case.batch):             # drafts that have mass in both rows
