@@ -2846,24 +2846,39 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
   if ((nv_max + 31) / 32 > kMaxChunks) return SJD_ERR_CAPACITY;
   // A cluster per row, with as many blocks as the rows leave SMs for: whenever the grid is resident at once (us a call, block per
   // row -> cluster: fp32 1 x 27 x 65536 156 -> 39, 1 x 16 x 1024 25 -> 19; bf16 1 x 32 x 65536 42 -> 29, 3 x 16 x 4096 27 ->
-  // 20, 4 x 32 x 16384 27 -> 25), and for fp32 rows of more than 2048 entries in any number (8 x 32 x 16384 68 -> 60, 26 x 33 x
-  // 4096 66 -> 59).  There a threshold of more than half the entries, which mostly lies on the other side of zero from the
-  // maximum, stays with a block per row (8 x 32 x 16384, top-k 0.6 V: 68 against 81); one that lies there because the logits do
-  // costs 68 -> 75, with one value masking nine entries in ten 72 -> 87.  bf16 rows in several waves are better off a block per
-  // row (1 x 64 x 184320: 90 against 157 us), and so are short fp32 rows (32 x 18 x 1096: 32 against 36 us).
+  // 20, 4 x 32 x 16384 27 -> 25).  bf16 rows in several waves are better off a block per row (1 x 64 x 184320: 90 against 157 us),
+  // and so are short fp32 rows (32 x 18 x 1096: 32 against 36 us).  Longer fp32 rows in several waves:
+  //   * a wave of clusters takes less than a wave of blocks, but an SM holds fewer of them, so the waves of both decide (8 x 32 x
+  //     16384, 2 waves against 1: 68 -> 61 us; 30 x 16 x 16384, 4 against 2: 110 -> 97; 37 x 16 x 4096, 2 against 1: 44 against
+  //     54; 27 x 16 x 8192, 3 against 1: 59 against 70; 37 x 16 x 16384, 5 against 2: 126 -> 114; 14 x 16 x 60000, not staged,
+  //     7 against 1: 269 -> 241);
+  //   * a threshold among more than half the entries mostly lies on the other side of zero from the maximum and stays with a
+  //     block per row (8 x 32 x 16384, top-k 0.6 V: 68 against 77; where it lies there because of the logits, 68 -> 72).
   const int n_sms = sm_count();
+  const size_t stage_bytes = (size_t)nv_max * 16;
+  constexpr size_t kMostStaged = 160 * 1024;
+  p.staged = stage_bytes <= kMostStaged ? 1 : 0;
+  int threads = nv_max <= 1024 ? 128 : nv_max <= 4096 ? 256 : nv_max <= 16384 ? 512 : 1024;
   {
     const bool whole = p.V % VEC == 0 && ((uintptr_t)p.logits[0] & 15u) == 0;   // every row starts on a vector
-    const long nv = whole ? p.V / VEC : nv_max;
+    const long nv = whole ? p.V / VEC : nv_max, rows = (long)p.B * p.W;
     int cs = 1;
     while (cs < 8 && (long)cs * kClThreads * kClVecs < nv) cs *= 2;
     const bool fits = (long)cs * kClThreads * kClVecs >= nv;
-    while (cs < 8 && p.B * p.W * cs * 2 <= n_sms && nv > (long)cs * kClThreads) cs *= 2;
-    const bool few = (long)p.B * p.W * cs <= n_sms;
-    const bool wide = std::is_same<T, float>::value && nv > kClThreads && (p.top_k <= p.V / 2 || p.top_k >= p.V);
+    while (cs < 8 && rows * cs * 2 <= n_sms && nv > (long)cs * kClThreads) cs *= 2;
+    const bool few = rows * cs <= n_sms;
+    bool wide = std::is_same<T, float>::value && nv > kClThreads && (p.top_k <= p.V / 2 || p.top_k >= p.V);
+    if (wide && !few) {
+      const bool two = cs == 1 && nv <= 2 * kClThreads;                                       // clusters of an SM
+      const long blocks = p.staged ? 227 * 1024 / ((long)stage_bytes + 32 * 1024) : 1024 / threads;   // and blocks
+      // (a grid of long rows that fills its last wave to more than 93 % takes one more: 18 x 16 x 16384 78 us, 8 x 32 x 16384 61)
+      const long slots = two ? 2 * n_sms : nv > 4 * kClThreads ? n_sms * 93 / 100 : n_sms;
+      const long waves = (rows * cs + slots - 1) / slots, waves_b = (rows + blocks * n_sms - 1) / (blocks * n_sms);
+      wide = !p.staged ? waves <= 7 * waves_b : two ? waves < 2 * waves_b : 2 * waves <= 5 * waves_b;
+    }
     if (fits && (few || wide)) {
       p.staged = p.fast = 0;
-      p.defer_residual = p.B * p.W * cs > n_sms ? 1 : 0;
+      p.defer_residual = rows * cs > n_sms ? 1 : 0;
       // fp32 rows of more than 4096 entries: a block's shared memory does not admit a second one on its SM
       constexpr bool f32 = std::is_same<T, float>::value;
       if (cs == 1) return f32 && nv > 2 * kClThreads ? launch_cluster<T, 1, 1>(p, nv, stream) : launch_cluster<T, 1, 2>(p, nv, stream);
@@ -2871,10 +2886,6 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
                                                                      : launch_cluster<T, 8, 1>(p, nv, stream);
     }
   }
-  const size_t stage_bytes = (size_t)nv_max * 16;
-  constexpr size_t kMostStaged = 160 * 1024;
-  p.staged = stage_bytes <= kMostStaged ? 1 : 0;
-  int threads = nv_max <= 1024 ? 128 : nv_max <= 4096 ? 256 : nv_max <= 16384 ? 512 : 1024;
   // rows a block can hold in registers, eight vectors per thread
   p.fast = 0;
   // (longer rows, up to kMaxChunks chunks, stream through the registers of a full block in segments)
