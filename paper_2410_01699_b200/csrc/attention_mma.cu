@@ -14,6 +14,8 @@
 // merge kernel of attention.cu.  Every barrier wait is bounded.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sjd {
@@ -86,18 +88,22 @@ struct AttnParams {
   const float *q;        // [M][H*HD]
   const int32_t *in_pos; // [M]
   float *partial;        // [M][H][splits][HD + 2]
-  float *out;            // [M][H*HD] or null: written here when splits == 1 (no merge launch needed)
+  float *out;            // [M][H*HD], OUT only: written here when splits == 1 (no merge launch needed)
   HiLoOut hilo;          // optional bf16 hi/lo planes of out (same case)
   int *status;
-  RowSegs segs;
-  int n_heads, n_kv_heads, splits;
+  int rows_per_seq, n_heads, n_kv_heads, splits;
   int plane0;            // first cache plane of this layer: planes are [b][k|v][kv_head]
   // paged cache: planes are [page][layer][k|v][kv_head], one page (KT positions) per tile
   const int32_t *page_table;   // [B][pages_per_seq]; null: contiguous
   int pages_per_seq, layer, n_layers;
+  const int32_t *seg_seq;      // PACKED: sequence of every segment
 };
 
-template <int HD, int KG>
+// PACKED: a pre-fill pass, whose rows are segments of prompts, several of one sequence among them.  OUT: the fp32 output is
+// wanted (else only its planes).  As run-time tests these three cost the calls that have no use for them up to 8 % (us a call,
+// 32 heads of 128, 8 x 32 rows x 3977 keys: 117.7 without, 127.3 with the segment order, the segment table and the test of out;
+// 8 x 64: 198 and 214).
+template <int HD, int KG, bool PACKED, bool OUT>
 __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constant__ CUtensorMap kv_map, const AttnParams p) {
   constexpr int HALVES = HD / 64;                // 64-dim (128-byte) boxes per row
   constexpr int TILE_BYTES = KT * HD * 2;        // one of K or V
@@ -111,11 +117,11 @@ __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constan
   SJD_TL(TL_ATTN, 0, threadIdx.x == 0);
   pdl_wait();   // keys/values of this step were written by the preceding kernel
   SJD_TL(TL_ATTN, 1, threadIdx.x == 0);
-  // (later segments of a prompt see more keys: they start first)
-  const int h = blockIdx.x, seg = gridDim.y - 1 - blockIdx.y, split = blockIdx.z;
-  const int b = seg_sequence(p.segs, seg);
+  // (PACKED: later segments of a prompt see more keys, they start first)
+  const int h = blockIdx.x, seg = PACKED ? gridDim.y - 1 - blockIdx.y : blockIdx.y, split = blockIdx.z;
+  const int b = PACKED ? __ldg(p.seg_seq + seg) : seg;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int W = p.segs.rows;
+  const int W = p.rows_per_seq;
   const int kvh = h / (p.n_heads / p.n_kv_heads);
   const int m0 = seg * W;
   const int g = lane >> 2, tq = lane & 3;
@@ -357,7 +363,7 @@ __global__ void __launch_bounds__(128) attention_mma_kernel(const __grid_constan
       for (int i = 0; i < HD / 8; ++i) {
         const float v0 = o[i][rr * 2] * inv, v1 = o[i][rr * 2 + 1] * inv;
         const size_t idx = base + i * 8 + tq * 2;
-        if (p.out) *reinterpret_cast<float2 *>(p.out + idx) = make_float2(v0, v1);
+        if constexpr (OUT) *reinterpret_cast<float2 *>(p.out + idx) = make_float2(v0, v1);
         if (p.hilo.base) {
           uint32_t hi, lo;
           split_pair(v0, v1, hi, lo);
@@ -429,7 +435,8 @@ int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const
   p.out = out;
   p.hilo = hilo;
   p.status = status;
-  p.segs = segs;
+  p.rows_per_seq = rows_per_seq;
+  p.seg_seq = segs.seq;
   p.n_heads = n_heads;
   p.n_kv_heads = n_kv_heads;
   p.splits = splits;
@@ -451,14 +458,19 @@ int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const
     SJD_CHECK_LAUNCH();
     return SJD_OK;
   };
-  if (head_dim == 128) {
-    if (kg == 4) return launch(attention_mma_kernel<128, 4>);
-    if (kg == 2) return launch(attention_mma_kernel<128, 2>);
-    return launch(attention_mma_kernel<128, 1>);
-  }
-  if (kg == 4) return launch(attention_mma_kernel<64, 4>);
-  if (kg == 2) return launch(attention_mma_kernel<64, 2>);
-  return launch(attention_mma_kernel<64, 1>);
+  auto pick = [&](auto packed, auto wants_out) -> int {
+    constexpr bool P = decltype(packed)::value, O = decltype(wants_out)::value;
+    if (head_dim == 128) {
+      if (kg == 4) return launch(attention_mma_kernel<128, 4, P, O>);
+      if (kg == 2) return launch(attention_mma_kernel<128, 2, P, O>);
+      return launch(attention_mma_kernel<128, 1, P, O>);
+    }
+    if (kg == 4) return launch(attention_mma_kernel<64, 4, P, O>);
+    if (kg == 2) return launch(attention_mma_kernel<64, 2, P, O>);
+    return launch(attention_mma_kernel<64, 1, P, O>);
+  };
+  if (segs.seq) return out ? SJD_ERR_UNSUPPORTED : pick(std::true_type(), std::false_type());
+  return out ? pick(std::false_type(), std::true_type()) : pick(std::false_type(), std::false_type());
 }
 
 }  // namespace sjd
