@@ -59,12 +59,15 @@ def test_verify_full_batch():
     assert stats.sequences == 32
 
 
-def test_verify_ratio_corner_cases():
+# Few rows run on a thread-block cluster each, bf16 rows in more blocks than the device has SMs (148) on a block per row: the
+# corner cases below take both routes.
+@pytest.mark.parametrize("batch", [3, 40])
+def test_verify_ratio_corner_cases(batch):
     """Eq. 1 where q(d) or p(d) vanishes (drafts whose law is a logits row, top-k 200 of 4096):
     q(d) = 0 < p(d) accepts for any uniform, p(d) = 0 < q(d) rejects, p(d) = q(d) = 0 rejects.  Rows
     around the corner rows have identical current and previous logits (ratio exactly 1: accepted), so the
     scan reaches each corner row and the number of accepted drafts is known without any checker."""
-    case = make_verify_case(3, window=6, vocab=4096, top_k=200, seed=77)
+    case = make_verify_case(batch, window=6, vocab=4096, top_k=200, seed=77)
     case.logits_prev = case.logits_cur.copy()
     order = np.argsort(-case.logits_cur, axis=-1, kind="stable")   # tokens of each row, largest logit first
 
@@ -78,7 +81,7 @@ def test_verify_ratio_corner_cases():
             case.logits_prev[b, k, d] = np.float32(12.0)      # in q's set only
         return d
 
-    for b in range(3):
+    for b in range(batch):
         for k in range(6):
             case.draft[b, k] = int(order[b, k, 20])           # p == q on the draft: always accepted
     put(0, 2, True, False)     # q(d) = 0 < p(d): accepted, the scan goes on
@@ -87,33 +90,43 @@ def test_verify_ratio_corner_cases():
     put(1, 1, False, True)     # p(d) = 0 < q(d): rejected
     put(2, 0, False, False)    # 0 / 0 on the very first row
     got = _run_gpu(case)
-    assert list(got["n_accepted"]) == [4, 1, 0]
-    assert list(got["n_committed"]) == [5, 2, 1]
+    assert list(got["n_accepted"]) == [4, 1, 0] + [6] * (batch - 3)
+    assert list(got["n_committed"]) == [5, 2, 1] + [6] * (batch - 3)
     stats = _check_case(case)
     assert stats.flagged == 0
 
 
-@pytest.mark.parametrize("dtype,vocab,window,top_k", [
-    ("bf16", 16001, 29, 2000),   # ragged: rows not 16-byte aligned, odd window
-    ("f32", 1024, 16, 64),       # the tiny end-to-end model's head
-    ("f32", 1000, 7, 1000),      # top_k == V: no filtering
-    ("bf16", 4099, 5, 1),        # top-1
-    ("bf16", 65536, 4, 2000),    # 128 KB rows (the 7B head)
-    ("bf16", 184320, 2, 2048),   # rows longer than a block's registers: streamed in three segments (the 8B head)
-    ("bf16", 100000, 5, 2000),   # two segments, the second partial (12500 vectors against 8192)
-    ("bf16", 184320, 3, 184320), # streamed rows, top_k == V: no threshold
-    ("bf16", 262000, 2, 4000),   # the longest row the chunk table covers: four segments
-    ("f32", 50000, 3, 500),      # fp32 rows beyond the staging buffer
+@pytest.mark.parametrize("batch,dtype,vocab,window,top_k", [
+    (2, "bf16", 16001, 29, 2000),    # ragged: rows not 16-byte aligned, odd window
+    (6, "bf16", 16001, 29, 2000),    # the same, a staged block per row
+    (2, "f32", 1024, 16, 64),        # the tiny end-to-end model's head
+    (2, "f32", 1000, 7, 1000),       # top_k == V: no filtering
+    (22, "f32", 1000, 7, 1000),      # the same, a block per row
+    (2, "bf16", 4099, 5, 1),         # top-1
+    (30, "bf16", 4099, 5, 1),
+    (2, "bf16", 65536, 4, 2000),     # 128 KB rows (the 7B head)
+    (38, "bf16", 65536, 4, 2000),    # the same in the registers of a block
+    (2, "bf16", 184320, 2, 2048),    # the longest bf16 rows of a cluster (the 8B head)
+    (10, "bf16", 184320, 2, 2048),   # longer than a block's registers: streamed in three segments
+    (2, "bf16", 100000, 5, 2000),
+    (8, "bf16", 100000, 5, 2000),    # two segments, the second partial (12500 vectors against 8192)
+    (2, "bf16", 184320, 3, 184320),  # top_k == V: no threshold
+    (7, "bf16", 184320, 3, 184320),  # the same on streamed rows
+    (2, "bf16", 262000, 2, 4000),
+    (10, "bf16", 262000, 2, 4000),   # the longest row the chunk table covers: four segments
+    (2, "f32", 50000, 3, 500),       # fp32 rows beyond the staging buffer
 ])
-def test_verify_shapes(dtype, vocab, window, top_k):
-    case = make_verify_case(2, window=window, vocab=vocab, dtype=dtype, top_k=top_k, seed=7 + vocab)
+def test_verify_shapes(batch, dtype, vocab, window, top_k):
+    """Row lengths, alignments and filters at a few rows (a cluster per row) and at many (a block per row)."""
+    case = make_verify_case(batch, window=window, vocab=vocab, dtype=dtype, top_k=top_k, seed=7 + vocab)
     _check_case(case, max_flag_frac=0.06)
 
 
 @pytest.mark.parametrize("batch,window,vocab,dtype,top_k", [
     (1, 3, 65537, "f32", 900),       # rows that start off 16 bytes, the last vector partly outside
     (1, 2, 131056, "f32", 2000),     # close to the longest row: eight blocks, eight vectors per thread
-    (2, 2, 513, "f32", 1),           # two vectors past a block's first chunk row
+    (2, 2, 513, "f32", 1),           # one block, the last vector partly outside
+    (15, 5, 2050, "f32", 100),       # one block whose rows reach past the first vector of every thread
     (5, 32, 3000, "f32", 100),       # more rows than SMs: Eq. 2 left to the sequence's last block
     (2, 5, 60001, "bf16", 700),      # bf16 rows at four alignments
     (1, 3, 32776, "bf16", 40000),    # no filter (top-k above the vocabulary), odd tail
@@ -170,6 +183,7 @@ def _awkward(case, mode, seed=0):
     (1, 4, 4096, "bf16"), (1, 3, 8000, "bf16"), (1, 3, 16001, "bf16"), (1, 3, 40000, "bf16"),
     (19, 8, 4096, "f32"), (150, 1, 3000, "f32"),                                                # more rows than SMs
     (19, 8, 4096, "bf16"), (75, 2, 3001, "bf16"),                                               # and a block per row
+    (7, 3, 140000, "bf16"),                                                                     # whose rows are streamed
 ])
 def test_verify_awkward_rows(batch, window, vocab, dtype, mode):
     """Thresholds far below the maximum, masked entries, thousands of ties, entries that are not finite: on every size of cluster
@@ -186,10 +200,11 @@ def test_verify_mixed_laws():
     _check_case(case)
 
 
-def test_verify_mixed_laws_on_streamed_rows():
-    """The same on rows too long for the registers (drift 3: most drafts are rejected, so Eq. 2 runs on streamed
+@pytest.mark.parametrize("batch", [3, 7])   # a cluster per row; streamed through the registers of a block
+def test_verify_mixed_laws_on_long_rows(batch):
+    """The same on rows too long for a block's registers (drift 3: most drafts are rejected, so Eq. 2 runs on long
     rows against uniform, copied and predicted drafts)."""
-    case = make_verify_case(3, window=6, vocab=100000, top_k=2000, seed=12, mixed_kinds=True, drift=3.0)
+    case = make_verify_case(batch, window=6, vocab=100000, top_k=2000, seed=12, mixed_kinds=True, drift=3.0)
     _check_case(case, max_flag_frac=0.06)
 
 
@@ -200,35 +215,38 @@ def test_verify_streamed_rows_in_a_grid_of_several_waves():
     _check_case(case, max_flag_frac=0.06)
 
 
-def test_verify_temperature_and_ties():
-    case = make_verify_case(3, window=8, vocab=8192, top_k=500, temperature=0.7, seed=5)
+@pytest.mark.parametrize("batch", [3, 20])
+def test_verify_temperature_and_ties(batch):
+    case = make_verify_case(batch, window=8, vocab=8192, top_k=500, temperature=0.7, seed=5)
     _check_case(case)
     # coarse logits: many exact ties at the top-k threshold (all must be kept)
-    case = make_verify_case(3, window=8, vocab=8192, top_k=500, seed=6)
+    case = make_verify_case(batch, window=8, vocab=8192, top_k=500, seed=6)
     case.logits_cur = round_bf16(np.round(case.logits_cur * 2) / 2)
     case.logits_prev = round_bf16(np.round(case.logits_prev * 2) / 2)
     _check_case(case)
 
 
+@pytest.mark.parametrize("batch", [2, 26])
 @pytest.mark.parametrize("shift,top_k", [
-    (-9.0, 2000),    # positive maximum, negative threshold: more than 4095 bf16 codes apart (general route)
-    (-30.0, 2000),   # every logit negative: maximum and threshold within a few binades (register route)
+    (-9.0, 2000),    # positive maximum, negative threshold: more than 4095 bf16 codes apart
+    (-30.0, 2000),   # every logit negative: maximum and threshold within a few binades
     (0.0, 8000),     # half the row kept: threshold around zero
-    (0.0, 16384),    # top_k == V: no filtering on the register route
+    (0.0, 16384),    # top_k == V: no filtering
 ])
-def test_verify_threshold_far_from_the_maximum(shift, top_k):
-    """The register-resident route counts entries by their distance below the row maximum and hands rows
-    whose threshold is out of that reach to the general route; both must agree with the checker."""
-    case = make_verify_case(2, window=6, vocab=16384, top_k=top_k, seed=31)
+def test_verify_threshold_far_from_the_maximum(shift, top_k, batch):
+    """Entries are counted by their distance below the row maximum.  Where the threshold is out of the histogram's reach, a
+    cluster counts on in further windows and a block per row takes its general route."""
+    case = make_verify_case(batch, window=6, vocab=16384, top_k=top_k, seed=31)
     case.logits_cur = round_bf16(case.logits_cur + np.float32(shift))
     case.logits_prev = round_bf16(case.logits_prev + np.float32(shift))
     _check_case(case, max_flag_frac=0.06)
 
 
-def test_verify_zeros_at_the_threshold():
+@pytest.mark.parametrize("batch", [2, 38])
+def test_verify_zeros_at_the_threshold(batch):
     """Exact zeros of both signs around the top-k threshold (bf16 comparison cannot order +0 and -0, the
-    order-preserving keys can): such rows take the general route."""
-    case = make_verify_case(2, window=4, vocab=8192, top_k=3000, seed=33)
+    order-preserving keys can): with a block per row such rows take the general route."""
+    case = make_verify_case(batch, window=4, vocab=8192, top_k=3000, seed=33)
     for arr in (case.logits_cur, case.logits_prev):
         small = np.abs(arr) < 0.35
         arr[small] = np.where(arr[small] < 0, np.float32(-0.0), np.float32(0.0))
@@ -245,8 +263,9 @@ def test_verify_identical_rows_accept_everything():
     assert np.all(got["draft"] == -1)
 
 
-def test_verify_nonfinite_rows_are_flagged():
-    case = make_verify_case(2, window=4, vocab=2048, top_k=50, seed=9)
+@pytest.mark.parametrize("batch", [2, 38])
+def test_verify_nonfinite_rows_are_flagged(batch):
+    case = make_verify_case(batch, window=4, vocab=2048, top_k=50, seed=9)
     case.logits_cur[0, 1, 5] = np.nan
     case.logits_cur[0, 1, 9] = np.inf
     got = _check_and_flags(case)
