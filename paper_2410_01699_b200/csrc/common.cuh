@@ -100,7 +100,7 @@ struct TimelineBuf {
 #define SJD_TIMELINE_TU(name)
 #define SJD_TL(tag, phase, cond) do { } while (0)
 #endif
-enum TimelineTag { TL_EMBED = 0, TL_RESID = 1, TL_GEMM = 2, TL_QKV = 3, TL_ATTN = 4, TL_COMBINE = 5, TL_SWIGLU = 6, TL_VERIFY = 7 };
+enum TimelineTag { TL_EMBED = 0, TL_RESID = 1, TL_GEMM = 2, TL_QKV = 3, TL_ATTN = 4, TL_COMBINE = 5, TL_VERIFY = 6 };
 
 // ---------------------------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): 128-bit counter, 64-bit key, ten rounds of

@@ -36,7 +36,7 @@ constexpr int kGuRows = 64;
 // Rows of one pre-fill pass: enough that a pass is bound by the tensor pipe and not by streaming the weights
 // once more (13.5 GB of weights take 2.1 ms, 1152 rows of the 7B layers about 30 ms), few enough that the
 // activations of a pass (157 KB per row at the 7B shapes) stay below 200 MB.  (Passes of max_window rows streamed the
-// weights once per 32 prompt tokens: 1063 tokens and one step took 124.2 ms on the 7B shapes, 37.3 ms this way.)  The generic pipeline keeps three
+// weights once per 32 prompt tokens: 1063 tokens and one step took 124.2 ms on the 7B shapes, 29.8 ms this way.)  The generic pipeline keeps three
 // more fp32 buffers per row and is not bound by the weights: 256 rows.
 constexpr int kPrefillRowsTc = 1152, kPrefillRowsGeneric = 256;
 constexpr int kMaxTcRows = 1152;     // largest pass of the tensor-core pipeline
@@ -316,11 +316,13 @@ struct sjd_ctx {
   bool prefilled;
   uint32_t host_step;  // number of sjd_step calls since prefill == device step index
   cudaStream_t last_stream;
-  // One captured CUDA graph of the forward pass per logits-buffer parity (up to 290 launches: replaying a graph takes the
-  // host out of the critical path).  It holds nothing that belongs to a call: the verification, which takes the caller's
+  // One captured CUDA graph of the forward pass per logits-buffer parity (291 launches at 32 layers: replaying a graph takes
+  // the host out of the critical path).  It holds nothing that belongs to a call: the verification, which takes the caller's
   // output pointers, is launched behind it, so that the graphs serve every pre-fill with the same batch and window.  The first
-  // two steps after a pre-fill are launched directly unless there are graphs already: the capture (0.7 ms of host time each at 32
-  // layers) then runs while they do.
+  // two steps after a pre-fill are launched directly unless there are graphs already: the captures (0.8 ms of host time each at
+  // 32 layers) then run while they do.  Pre-fill and steps without and with graphs from an earlier pre-fill, W = 16: 7B, 64 prompt
+  // tokens, 2 / 4 / 8 steps 9.86 / 15.92 / 28.03 and 9.82 / 15.72 / 27.83 ms; the small bf16 model 299 / 576 / 945 and 288 / 467 /
+  // 836 us.
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     long long launches = 0;

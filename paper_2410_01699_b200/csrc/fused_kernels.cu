@@ -9,10 +9,8 @@ SJD_TIMELINE_TU(fused)
 namespace {
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
-template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 template <typename T> __device__ __forceinline__ T from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // two adjacent values -> packed bf16 hi pair and lo pair (lo = value - hi, rounded)
@@ -24,11 +22,6 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t &hi, uint3
   lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 // N adjacent entries (4 or 2, aligned) as fp32
-template <int N>
-__device__ __forceinline__ void load_gain(const float *p, float *v) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = __ldg(p + i);
-}
 template <int N>
 __device__ __forceinline__ void load_gain(const __nv_bfloat16 *p, float *v) {
 #pragma unroll

@@ -26,8 +26,8 @@
 // the same weights.  Longer bf16 rows (the 184320-entry head) take the same route streamed: a full block
 // passes the row through its registers in segments of 65536 entries, once per phase (long_statistics).
 //
-// Few rows, and fp32 rows of more than 2048 entries, are verified by a thread-block cluster per row instead
-// (verify_cluster_kernel; the rule is in launch_verify_t).
+// Few rows, and more fp32 rows of over 2048 entries where the waves of both grids speak for it, are verified by a thread-block
+// cluster per row instead (verify_cluster_kernel; the rule is in launch_verify_t).
 #include <float.h>
 
 #include <atomic>
@@ -2912,7 +2912,9 @@ static int launch_verify_t(const VerifyParams &p_in, cudaStream_t stream) {
     return SJD_OK;
   };
   if (threads <= 256) return launch(verify_rows_kernel<T, 256>);
-  if (p.fast && !in_registers) return launch(verify_rows_kernel<T, kMaxThreads, true>);
+  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+    if (p.fast && !in_registers) return launch(verify_rows_kernel<T, kMaxThreads, true>);
+  }
   return launch(verify_rows_kernel<T, kMaxThreads>);
 }
 

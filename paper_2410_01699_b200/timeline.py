@@ -26,7 +26,7 @@ from . import build as bld
 from .inputs import WORKLOADS, make_prompt, make_weights
 
 LIB_TL = os.path.join(bld.HERE, "libsjd_tl.so")
-NAMES = {0: "embed", 1: "resid_gain", 2: "gemm", 3: "qkv_finish", 4: "attention", 5: "combine", 6: "swiglu", 7: "verify"}
+NAMES = {0: "embed", 1: "resid_gain", 2: "gemm", 3: "qkv_finish", 4: "attention", 5: "combine", 6: "verify"}
 
 
 def build_instrumented() -> str:
@@ -89,7 +89,7 @@ def main():
     wl = WORKLOADS[a.workload]
     ln = links(capture(wl))
     # ln[0] is the verification of the previous step; then per layer: resid, gemm, qkv, attention(, combine), gemm,
-    # resid, gemm(, swiglu), gemm
+    # resid, gemm, gemm
     per_layer = (len(ln) - 3) // wl.n_layers
     print("step: %.1f us from one verification to the next; %d links per layer" % (ln[-1][0] - ln[0][0], per_layer))
     i0 = 1 + a.layer * per_layer
