@@ -946,6 +946,8 @@ static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles,
   PairParams q;
   q.g = p;
   q.tiles = tiles;
+  // the second half of a last pair without a tile is the tile past the last matrix: zeros, not rows of a matrix once more
+  for (int j = g.n_mats - 1; j < 3; ++j) q.g.tile_end[j] += tiles & 1;
   q.n_units = (tiles + 1) / 2 * p.n_slabs * p.splits;
   const bool gu = g.act_hi != nullptr;
   const int stage_bytes = W_TILE_BYTES + p.Mp * TILE_K * 2;
