@@ -2,6 +2,8 @@
 // Step 2: one pass over the window).  These cover every shape and both dtypes with plain FMA
 // arithmetic and fp32 accumulation.  Activations between kernels are fp32 (they are a few hundred KB);
 // only weights, the KV cache and the stored logits are in the model dtype.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sjd {
@@ -14,20 +16,33 @@ template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
-// E = 4 adjacent entries (aligned) or one
+// E = 4 adjacent entries (aligned) or one, as they are stored: they are converted where they are used, so that nothing waits for a
+// load that was issued ahead.
 template <typename T, int E>
-__device__ __forceinline__ void load_group(const T *p, float *v) {
-  if constexpr (E == 1) {
-    v[0] = to_f<T>(p[0]);
-  } else if constexpr (sizeof(T) == 4) {
-    const float4 t = *reinterpret_cast<const float4 *>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-  } else {
-    const uint2 t = *reinterpret_cast<const uint2 *>(p);
-    v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xFFFF0000u);
-    v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xFFFF0000u);
+struct Group {
+  uint32_t w[E * sizeof(T) / 4 ? E * sizeof(T) / 4 : 1];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (uint32_t &x : w) x = 0u;
   }
-}
+  __device__ __forceinline__ void load(const T *p) {
+    if constexpr (E == 1 && sizeof(T) == 4) {
+      w[0] = __float_as_uint(p[0]);
+    } else if constexpr (E == 1) {
+      w[0] = *reinterpret_cast<const unsigned short *>(p);
+    } else if constexpr (sizeof(T) == 4) {
+      const uint4 t = *reinterpret_cast<const uint4 *>(p);
+      w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+    } else {
+      const uint2 t = *reinterpret_cast<const uint2 *>(p);
+      w[0] = t.x; w[1] = t.y;
+    }
+  }
+  __device__ __forceinline__ float get(int e) const {
+    if constexpr (sizeof(T) == 4) return __uint_as_float(w[e]);
+    else return __uint_as_float(e & 1 ? w[e / 2] & 0xFFFF0000u : w[e / 2] << 16);
+  }
+};
 
 __device__ __forceinline__ void store_hilo(const HiLoOut &o, size_t idx, float v) {
   if (!o.base) return;
@@ -37,24 +52,39 @@ __device__ __forceinline__ void store_hilo(const HiLoOut &o, size_t idx, float v
 }
 
 // ------------------------------------------------------------------------------------ projections (FMA)
-// A projection of a few rows through small or odd-shaped matrices, where a step is a chain of launches that each cost their
-// own latency (two layers of d 256 and 16 rows: 29 launches, 418 us of projections in a 476 us step with 32 x 64 tiles that
-// walked K in slices of 32, one dependent load after the other; 14 launches and 101 us a step now).  Hence: one CTA per 16 rows x 8 * NJ weight rows, the
-// eight warps split every 256-column chunk of K between them, so that a whole chunk is one round trip to memory, and the
-// next chunk is on its way while this one is multiplied.  The RMS normalisation before a projection (its row scale
-// commutes with the product), the residual add and SwiGLU are part of the launch.  Any M, N, K; the sums have one fixed order.
-constexpr int RG_M = 16, RG_K = 256, RG_LD = RG_K + 4;   // + 4: rows eight apart meet in different banks
+// Small or odd-shaped matrices and fp32 models.  With few rows a step is a chain of launches that each cost their own latency (two
+// layers of d 256 and 16 rows: 29 launches, 418 us of projections in a 476 us step with 32 x 64 tiles that walked K in slices of
+// 32, one dependent load after the other; 16 launches and the verification in 107 us now).  Hence: the eight warps of a CTA
+// split every chunk of KC columns between them, so that a whole chunk is one round trip to memory, and the next chunk is
+// on its way while this one is multiplied.  The RMS normalisation before a projection (its row scale commutes with the
+// product), the residual add and SwiGLU are part of the launch.  Any M, N, K; the sums have one fixed order.
+// A tile: 4 * MI rows x 8 * NJ weight rows; BLOCKS: CTAs that an SM has registers for.  (LD: + 4, rows eight apart meet in
+// different banks.)
+template <int MI_, int NJ_, int KC_, int BLOCKS_>
+struct RowsTile {
+  static constexpr int MI = MI_, NJ = NJ_, KC = KC_, BLOCKS = BLOCKS_, BM = 4 * MI, BN = 8 * NJ, LD = KC + 4;
+  static constexpr size_t kOperands = (size_t)(BM + BN) * LD, kSums = (size_t)8 * BM * (BN + 1);
+  static constexpr size_t kSmem = (kOperands > kSums ? kOperands : kSums) * sizeof(float);
+};
+// Few rows: 16 x 16 (small matrices: half the work per CTA) or 16 x 32, with all the registers they want (two CTAs on an SM: a
+// step of the fp32 model of d 256 with 192 rows 160 us, one: 142).  More rows: 32 x 32, which loads a third less per product, with
+// two CTAs on an SM.  (With 16 x 32 alone, one CTA on an SM and the CTAs of one weight tile far apart in the grid, passes of
+// many rows were slower than the 32 x 64 tiles had been.  us, 32 x 64 / 16 x 32 / now: fp32 512 x 12288 x 4096 2655 / 2915 /
+// 1681, 256 x 8192 x 1024 234 / 265 / 158; bf16 1280 x 22016 x 4096 11460 / 17392 / 6769, 512 x 2560 x 961 168 / 345 / 148.)
+using RowsNarrow = RowsTile<4, 2, 256, 1>;
+using RowsFew = RowsTile<4, 4, 256, 1>;
+using RowsMany = RowsTile<8, 4, 128, 2>;
 
 // VEC: rows of x and of every matrix can be read in groups of four entries
-template <typename T, int NJ, bool VEC>
-__global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
-  constexpr int BN = 8 * NJ;
+template <typename T, typename Tile, bool VEC>
+__global__ void __launch_bounds__(256, Tile::BLOCKS) gemm_rows_kernel(const RowsGemm g) {
+  constexpr int MI = Tile::MI, NJ = Tile::NJ, RG_M = Tile::BM, BN = Tile::BN, RG_K = Tile::KC, RG_LD = Tile::LD;
   extern __shared__ float smem[];
   float *xs = smem, *ws = smem + RG_M * RG_LD;
   __shared__ float s_ss[RG_M][8];
   pdl_trigger();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * RG_M, t0 = blockIdx.x;
+  const int m0 = blockIdx.x * RG_M, t0 = blockIdx.y + blockIdx.z * gridDim.y;   // (blocks that share weight rows run side by side)
   const bool glu = g.epilogue == RG_SWIGLU;
   const T *gain = reinterpret_cast<const T *>(g.gain);
   // weight row r of this tile: under SwiGLU the first half of the rows are gate features, the second the same up features
@@ -72,39 +102,39 @@ __global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
   constexpr int E = VEC ? 4 : 1, PER = 256 / (RG_K / E);        // entries per load, rows per round of the block
   constexpr int NXL = RG_M / PER, NWL = BN / PER;
   const int col = tid % (RG_K / E) * E, r0 = tid / (RG_K / E);
-  float xr[NXL][E], wr[NWL][E], gr[E], ss[NXL];
+  Group<float, E> xr[NXL];
+  Group<T, E> wr[NWL], gr;
+  float ss[NXL];
+  const T *wp[NWL];   // this thread's weight rows (each is looked up on the way to its first load)
 #pragma unroll
   for (int i = 0; i < NXL; ++i) ss[i] = 0.0f;
-  auto load_w = [&](int k0) {
+  auto load_w = [&](int k0, auto first) {
     const int k = k0 + col;
 #pragma unroll
     for (int i = 0; i < NWL; ++i) {
-      const T *row = wrow(r0 + i * PER);
-#pragma unroll
-      for (int e = 0; e < E; ++e) wr[i][e] = 0.0f;
-      if (row && k < g.K) load_group<T, E>(row + k, wr[i]);
+      if constexpr (decltype(first)::value) wp[i] = wrow(r0 + i * PER);
+      wr[i].clear();
+      if (wp[i] && k < g.K) wr[i].load(wp[i] + k);
     }
-#pragma unroll
-    for (int e = 0; e < E; ++e) gr[e] = 1.0f;
-    if (gain && k < g.K) load_group<T, E>(gain + k, gr);
+    gr.clear();
+    if (gain && k < g.K) gr.load(gain + k);
   };
   auto load_x = [&](int k0) {
     const int k = k0 + col;
 #pragma unroll
     for (int i = 0; i < NXL; ++i) {
       const int m = m0 + r0 + i * PER;
-#pragma unroll
-      for (int e = 0; e < E; ++e) xr[i][e] = 0.0f;
-      if (m < g.M && k < g.K) load_group<float, E>(g.x + (size_t)m * g.ldx + k, xr[i]);
+      xr[i].clear();
+      if (m < g.M && k < g.K) xr[i].load(g.x + (size_t)m * g.ldx + k);
     }
   };
-  load_w(0);     // the weights do not depend on the kernel before
+  load_w(0, std::true_type());     // the weights do not depend on the kernel before
   pdl_wait();
   load_x(0);
   const int lm = lane >> 3, ln = lane & 7;
-  float acc[4][NJ];
+  float acc[MI][NJ];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MI; ++i)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0f;
   for (int k0 = 0; k0 < g.K; k0 += RG_K) {
@@ -113,28 +143,29 @@ __global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
     for (int i = 0; i < NXL; ++i)
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        ss[i] = fmaf(xr[i][e], xr[i][e], ss[i]);
-        xs[(r0 + i * PER) * RG_LD + col + e] = xr[i][e] * gr[e];
+        const float v = xr[i].get(e);
+        ss[i] = fmaf(v, v, ss[i]);
+        xs[(r0 + i * PER) * RG_LD + col + e] = gain ? v * gr.get(e) : v;
       }
 #pragma unroll
     for (int i = 0; i < NWL; ++i)
 #pragma unroll
-      for (int e = 0; e < E; ++e) ws[(r0 + i * PER) * RG_LD + col + e] = wr[i][e];
+      for (int e = 0; e < E; ++e) ws[(r0 + i * PER) * RG_LD + col + e] = wr[i].get(e);
     __syncthreads();
     if (k0 + RG_K < g.K) {
-      load_w(k0 + RG_K);
+      load_w(k0 + RG_K, std::false_type());
       load_x(k0 + RG_K);
     }
     const int kw = warp * (RG_K / 8);
 #pragma unroll
     for (int k = 0; k < RG_K / 8; k += 4) {
-      float4 xv[4], wv[NJ];
+      float4 xv[MI], wv[NJ];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) xv[i] = *reinterpret_cast<const float4 *>(xs + (lm + 4 * i) * RG_LD + kw + k);
+      for (int i = 0; i < MI; ++i) xv[i] = *reinterpret_cast<const float4 *>(xs + (lm + 4 * i) * RG_LD + kw + k);
 #pragma unroll
       for (int j = 0; j < NJ; ++j) wv[j] = *reinterpret_cast<const float4 *>(ws + (ln + 8 * j) * RG_LD + kw + k);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < MI; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
           acc[i][j] = fmaf(xv[i].w, wv[j].w, fmaf(xv[i].z, wv[j].z, fmaf(xv[i].y, wv[j].y, fmaf(xv[i].x, wv[j].x, acc[i][j]))));
@@ -151,7 +182,7 @@ __global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
   __syncthreads();
   float *red = smem;   // [warp][row][BN + 1]
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MI; ++i)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) red[(warp * RG_M + lm + 4 * i) * (BN + 1) + ln + 8 * j] = acc[i][j];
   __syncthreads();
@@ -184,26 +215,35 @@ __global__ void __launch_bounds__(256) gemm_rows_kernel(const RowsGemm g) {
   }
 }
 
-template <typename T>
-int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
-  const int mt = (g.M + RG_M - 1) / RG_M;
-  const int wide = g.epilogue == RG_SWIGLU ? 16 : 32;   // output columns of a CTA with four weight rows per lane
-  // two weight rows per lane while that still leaves the grid within one wave (half the work per CTA)
-  const bool narrow = mt * ((g.N + wide / 2 - 1) / (wide / 2)) <= 148;
-  bool vec = g.K % 4 == 0 && g.ldx % 4 == 0 && ((uintptr_t)g.x & 15u) == 0 && ((uintptr_t)g.gain & (4 * sizeof(T) - 1)) == 0;
-  for (int j = 0; j < 3; ++j) vec = vec && ((uintptr_t)g.w[j] & (4 * sizeof(T) - 1)) == 0;
-  const int cols = narrow ? wide / 2 : wide, bn = narrow ? 16 : 32;
-  const size_t smem = (size_t)(RG_M + bn) * RG_LD * sizeof(float);
-  const dim3 grid((g.N + cols - 1) / cols, mt);
+template <typename T, typename Tile>
+int gemm_rows_tile(const RowsGemm &g, bool vec, cudaStream_t stream) {
+  const int cols = g.epilogue == RG_SWIGLU ? Tile::BN / 2 : Tile::BN;
+  const int n_tiles = (g.N + cols - 1) / cols, layers = (n_tiles + 65534) / 65535;
+  const dim3 grid((g.M + Tile::BM - 1) / Tile::BM, (n_tiles + layers - 1) / layers, layers);
   auto launch = [&](auto kernel) -> int {
-    const int rc = smem > 40 * 1024 ? allow_smem(kernel, smem) : SJD_OK;   // (the size follows from the kernel's tile)
+    const int rc = Tile::kSmem > 40 * 1024 ? allow_smem(kernel, Tile::kSmem) : SJD_OK;
     if (rc != SJD_OK) return rc;
-    SJD_CUDA(launch_kernel(kernel, grid, dim3(256), smem, stream, g));
+    SJD_CUDA(launch_kernel(kernel, grid, dim3(256), Tile::kSmem, stream, g));
     SJD_CHECK_LAUNCH();
     return SJD_OK;
   };
-  if (narrow) return vec ? launch(gemm_rows_kernel<T, 2, true>) : launch(gemm_rows_kernel<T, 2, false>);
-  return vec ? launch(gemm_rows_kernel<T, 4, true>) : launch(gemm_rows_kernel<T, 4, false>);
+  return vec ? launch(gemm_rows_kernel<T, Tile, true>) : launch(gemm_rows_kernel<T, Tile, false>);
+}
+
+template <typename T>
+int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
+  auto tiles = [&](int rows, int cols) { return (long)((g.M + rows - 1) / rows) * ((g.N + cols - 1) / cols); };
+  const int glu = g.epilogue == RG_SWIGLU ? 2 : 1;   // weight rows of an output column
+  bool vec = g.K % 4 == 0 && g.ldx % 4 == 0 && ((uintptr_t)g.x & 15u) == 0 && ((uintptr_t)g.gain & (4 * sizeof(T) - 1)) == 0;
+  for (int j = 0; j < 3; ++j) vec = vec && ((uintptr_t)g.w[j] & (4 * sizeof(T) - 1)) == 0;
+  // us, smallest / middle / largest tile.  The smallest while its grid is one wave (fp32 64 x 256 x 683: 8.3 / 14.5 / 18.5), the
+  // middle one up to two (64 x 1024 x 2816: 25 / 23 / 35; 64 x 4096 x 4096, more than that: 123 / 103 / 85; a step of four layers
+  // of d 1024 and 128 rows 957 us, 1007 if the line is at one wave).  The largest is not for rows that would fill half of it (16 x
+  // 12288 x 4096: 108 / 82 / 125).
+  constexpr int kSms = 148;
+  if (tiles(RowsNarrow::BM, RowsNarrow::BN / glu) <= kSms) return gemm_rows_tile<T, RowsNarrow>(g, vec, stream);
+  if (g.M <= RowsFew::BM || tiles(RowsFew::BM, RowsFew::BN / glu) <= 2 * kSms) return gemm_rows_tile<T, RowsFew>(g, vec, stream);
+  return gemm_rows_tile<T, RowsMany>(g, vec, stream);
 }
 
 // ------------------------------------------------------------------------------------ embedding

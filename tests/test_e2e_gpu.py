@@ -462,7 +462,9 @@ def test_sweep_points_two_layers(batch, window, prompt_len, init, steps):
 
 @pytest.mark.parametrize("name,over,batch,window", [
     ("tiny", dict(n_heads=3, n_kv_heads=3, head_dim=62, d_model=250, vocab=1021), 1, 5),   # rows off 16 bytes, widths off the tiles
-    ("tiny", {}, 5, 31),                                                                    # 155 rows: four weight rows per lane
+    ("tiny", {}, 5, 31),                                                                    # 155 rows: 16 x 32 and 32 x 32 tiles
+    ("tiny", dict(ffn_hidden=1503, vocab=2050), 9, 31),                                     # 279 rows, the last tiles partly outside
+    ("small-bf16", dict(ffn_hidden=1003, d_model=500, vocab=1501), 6, 33),                  # bf16, 198 rows, groups and single entries
     ("small-bf16", dict(ffn_hidden=1003, vocab=1001), 2, 7),                                # bf16, some matrices unaligned
 ])
 def test_generic_projections(name, over, batch, window):
