@@ -17,9 +17,9 @@
 //     one grid.  With more than one K split every CTA writes an fp32 partial plane; the consumer
 //     kernel (residual + RMSNorm, RoPE + cache append, SwiGLU, or a plain sum) adds the planes in
 //     split order: deterministic, no atomics, no serial reduction tail inside the GEMM.
-//   * Warp 0 issues TMA loads (128B-swizzled 128x64 W tiles with an evict-first L2 policy, plus the
-//     activation tiles) into a ring of shared-memory stages guarded by mbarriers; warp 1 issues the
-//     MMAs into a TMEM accumulator and commits to the stage's "empty" barrier; warps 2-5 drain the
+//   * Warp 0 issues TMA loads of 128B-swizzled 128x64 W tiles (evict-first L2 policy) into a ring of shared-memory stages
+//     guarded by mbarriers, warp 6 those of the activation tiles into a shorter ring of their own; warp 1 issues the
+//     MMAs into a TMEM accumulator and commits to the stages' "empty" barriers; warps 2-5 drain the
 //     accumulator with tcgen05.ld and store.
 //   * Every wait is bounded: after ~2 s a role records an error in the status word and leaves; the
 //     CTA still frees its TMEM.
@@ -38,14 +38,14 @@ constexpr int TILE_N = 128;   // weight rows per tile (MMA M)
 constexpr int TILE_K = 64;    // bf16 elements per k-block = one 128-byte swizzle atom
 constexpr int UMMA_K = 16;
 constexpr int W_TILE_BYTES = TILE_N * TILE_K * 2;
-constexpr int kThreads = 192;
+constexpr int kThreads = 224;   // weight producer, issuer, four epilogue warps, activation producer
 constexpr int kMaxStages = 8;
 // tunables (defaults chosen by measurement on B200)
 #ifndef SJD_GEMM_SMEM_BUDGET
-#define SJD_GEMM_SMEM_BUDGET (100 * 1024)   // ring bytes per CTA when two CTAs share an SM
+#define SJD_GEMM_SMEM_BUDGET (104 * 1024)   // ring bytes per CTA when two CTAs share an SM, see ring_stages
 #endif
 #ifndef SJD_GEMM_DEEP_RING
-#define SJD_GEMM_DEEP_RING 1                // double the ring when the grid has at most one CTA per SM
+#define SJD_GEMM_DEEP_RING (200 * 1024)     // and when the grid has at most one CTA per SM
 #endif
 #ifndef SJD_GEMM_L2_PROMO
 #define SJD_GEMM_L2_PROMO CU_TENSOR_MAP_L2_PROMOTION_L2_256B
@@ -56,7 +56,11 @@ constexpr int kMaxStages = 8;
 #ifndef SJD_GEMM_CTAS_PER_SM
 #define SJD_GEMM_CTAS_PER_SM 2
 #endif
-constexpr int kSmemBudget = SJD_GEMM_SMEM_BUDGET;
+// CTA t starts t * kTileSkew k-blocks into its range of K.  In step, all of a launch's CTAs ask L2 for the same few lines of the
+// activations at the same time (gate|up, 172 CTAs: 34.2 us, with skew 32.5; logits 91 and 86.4; us of a step of 16 layers, 7B,
+// 32 rows: skew 0 / 4 / 8 / 12: 1655 / 1617 / 1616 / 1614, also skewed where K is split 1600 against 1605).
+constexpr int kTileSkew = 8;
+constexpr int kSmemBudget = SJD_GEMM_SMEM_BUDGET, kDeepRing = SJD_GEMM_DEEP_RING;
 constexpr unsigned long long kWaitNs = 2000000000ull;
 
 struct GemmParams {
@@ -70,7 +74,7 @@ struct GemmParams {
   int k_blocks, splits;   // K / 64, K splits (gridDim.y)
   int tile_end[3];        // matrix j owns tiles [tile_end[j-1], tile_end[j])
   int col_off[3];         // first output column of matrix j
-  int stages;
+  int stages, x_stages;
   int store_bf16;
   int *status;            // device status word (non-zero = a bounded wait ran out)
   const float *ss_part;   // optional [M][n_part] partial sums of squares: rows are scaled by
@@ -131,6 +135,11 @@ __device__ __forceinline__ bool elect_one() {
   return r != 0;
 }
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity)); }
+// both barriers: their first tests do not wait for one another
+__device__ __forceinline__ bool warp_wait_both(uint64_t *a, uint32_t pa, uint64_t *b, uint32_t pb) {
+  const bool ra = mbar_try_wait(a, pa), rb = mbar_try_wait(b, pb);
+  return __all_sync(0xffffffffu, ra && rb) || (warp_wait(a, pa) && warp_wait(b, pb));
+}
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar,
                                             uint64_t policy) {
@@ -226,28 +235,36 @@ __device__ __forceinline__ void store_column(O *out, size_t ld, float *v, const 
   }
 }
 
+constexpr int kTcBarriers = 3 * kMaxStages + 1;
+// behind the rings of a CTA
+struct TcShared {
+  uint64_t full[kMaxStages], x_full[kMaxStages];   // (one array of kTcBarriers to set up)
+  uint64_t done[kMaxStages];                       // k-block it has been multiplied: number it % kMaxStages
+  uint64_t acc_full;
+  uint32_t tmem_base;
+  float scale[TILE_N];   // per-row output scales (epilogue)
+};
+
 // ---------------------------------------------------------------------------------- kernel
 // GU: the gate|up launch that applies SwiGLU in its epilogue
 template <bool GU>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant__ CUtensorMap w_map1,
                const __grid_constant__ CUtensorMap w_map2, const __grid_constant__ CUtensorMap x_map, const GemmParams p) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t bar_full[kMaxStages], bar_empty[kMaxStages], bar_acc_full;
-  __shared__ uint32_t s_tmem_base;
-  __shared__ float s_scale[TILE_N];   // per-row output scales of this CTA's token slab (epilogue)
-
-  pdl_trigger();   // the next kernel in the stream may be scheduled as soon as every CTA got here
-  SJD_TL(TL_GEMM, 0, threadIdx.x == 0);
+  extern __shared__ __align__(1024) uint8_t smem[];   // no static shared memory: it starts on 1024 bytes
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tile = blockIdx.x, split = blockIdx.y;
   constexpr int m_base = 0;   // one slab: more rows run on CTA pairs
   const int NN = 2 * p.Mp;                           // MMA N
   const int x_tile_bytes = NN * TILE_K * 2;
-  const int stage_bytes = W_TILE_BYTES + x_tile_bytes;
+  uint8_t *smem_x = smem + p.stages * W_TILE_BYTES;
+  TcShared &sh = *reinterpret_cast<TcShared *>(smem_x + p.x_stages * x_tile_bytes);
+  float *s_scale = sh.scale;
+
+  pdl_trigger();   // the next kernel in the stream may be scheduled as soon as every CTA got here
+  SJD_TL(TL_GEMM, 0, threadIdx.x == 0);
   const int R = p.tile_rows;
-  const uint32_t stage_tx = (uint32_t)((GU ? 2 : 1) * R * TILE_K * 2 + x_tile_bytes);   // bytes the copies of a stage deliver
-  uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const uint32_t w_tx = (uint32_t)((GU ? 2 : 1) * R * TILE_K * 2);   // bytes the copies of a weight stage deliver
 
   // which weight matrix this tile belongs to
   const int mat = GU ? 0 : (tile < p.tile_end[0] ? 0 : (tile < p.tile_end[1] ? 1 : 2));
@@ -262,18 +279,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   while ((int)tmem_cols < NN) tmem_cols <<= 1;
 
   if (tid == 0) {
+    if (smem_u32(smem) & 1023u) atomicExch(p.status, 5);   // (the swizzled tiles have to start on 1024 bytes)
     tma_prefetch_desc(w_map);
     tma_prefetch_desc(&x_map);
-    for (int s = 0; s < p.stages; ++s) {
-      mbar_init(&bar_full[s], 1);
-      mbar_init(&bar_empty[s], 1);
-    }
-    mbar_init(&bar_acc_full, 1);
+  }
+  if (tid < kTcBarriers) {
+    mbar_init(&sh.full[tid], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)),
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)),
                  "r"(tmem_cols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -281,82 +297,75 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = s_tmem_base;
+  const uint32_t tmem_base = sh.tmem_base;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
+  if (warp == 0 || warp == 6) {
+    // ------------------------------------------------------------------ TMA producers: weights (0), activations (6)
+    // The weights do not depend on the preceding kernel: they are streamed from the start, the activations that it produced are
+    // waited for.
+    const bool is_w = warp == 0;
+    const int ring = is_w ? p.stages : p.x_stages;
+    uint64_t *full = is_w ? sh.full : sh.x_full;
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-    auto load_w = [&](int kcol, int s) {
-      uint8_t *dst = smem + s * stage_bytes;
-      mbar_expect_tx(&bar_full[s], stage_tx);
-      if (GU) {
-        tma_load_2d(dst, &w_map0, kcol, tile * R, &bar_full[s], policy);
-        tma_load_2d(dst + W_TILE_BYTES / 2, &w_map1, kcol, tile * R, &bar_full[s], policy);
-      } else {
-        tma_load_2d(dst, w_map, kcol, tile_in_mat * R, &bar_full[s], policy);
-      }
-    };
-    auto load_x = [&](int kcol, int s) {
-      uint8_t *dst = smem + s * stage_bytes + W_TILE_BYTES;
-      tma_load_2d_nohint(dst, &x_map, kcol, m_base, &bar_full[s]);
-      tma_load_2d_nohint(dst + x_tile_bytes / 2, &x_map, kcol, p.x_lo_row + m_base, &bar_full[s]);
-    };
-    // The weights do not depend on the preceding kernel: fill the ring with W tiles right away,
-    // then wait for the predecessor before fetching the activation tiles it produced.
-    const int pre = n_kb < p.stages ? n_kb : p.stages;
-    for (int i = 0; i < pre; ++i) {
-      if (elect_one()) load_w((kb_begin + i) * TILE_K, i);
-      __syncwarp();
-    }
-    SJD_TL(TL_GEMM, 3, lane == 0);
-    pdl_wait();
-    SJD_TL(TL_GEMM, 1, lane == 0);
-    for (int i = 0; i < pre; ++i) {
-      if (elect_one()) load_x((kb_begin + i) * TILE_K, i);
-      __syncwarp();
-    }
-    int s = pre == p.stages ? 0 : pre;
-    uint32_t ph = pre == p.stages ? 1u : 0u;
+    if (!is_w) pdl_wait();
+    SJD_TL(TL_GEMM, 1, !is_w && lane == 0);
+    const int first = (tile * kTileSkew) % n_kb;
+    int s = 0, it = 0;
     bool ok = true;
-    int it = pre;
     for (; it < n_kb; ++it) {
-      if (!warp_wait(&bar_empty[s], ph ^ 1u)) { ok = false; break; }
+      const int of = it - ring;   // the k-block whose stage this is
+      if (of >= 0 && !warp_wait(&sh.done[of % kMaxStages], (uint32_t)(of / kMaxStages) & 1u)) { ok = false; break; }
       if (elect_one()) {
-        load_w((kb_begin + it) * TILE_K, s);
-        load_x((kb_begin + it) * TILE_K, s);
+        const int kcol = (kb_begin + (it + first < n_kb ? it + first : it + first - n_kb)) * TILE_K;
+        if (is_w) {
+          uint8_t *dst = smem + s * W_TILE_BYTES;
+          mbar_expect_tx(&full[s], w_tx);
+          if (GU) {
+            tma_load_2d(dst, &w_map0, kcol, tile * R, &full[s], policy);
+            tma_load_2d(dst + W_TILE_BYTES / 2, &w_map1, kcol, tile * R, &full[s], policy);
+          } else {
+            tma_load_2d(dst, w_map, kcol, tile_in_mat * R, &full[s], policy);
+          }
+        } else {
+          uint8_t *dst = smem_x + s * x_tile_bytes;
+          mbar_expect_tx(&full[s], (uint32_t)x_tile_bytes);
+          tma_load_2d_nohint(dst, &x_map, kcol, m_base, &full[s]);
+          tma_load_2d_nohint(dst + x_tile_bytes / 2, &x_map, kcol, p.x_lo_row + m_base, &full[s]);
+        }
       }
       __syncwarp();
-      if (++s == p.stages) { s = 0; ph ^= 1u; }
+      if (++s == ring) s = 0;
     }
     if (!ok) {
       if (lane == 0) atomicExch(p.status, 1);
       // leave no copy in flight: wait (bounded) for the stages armed most recently
-      const int armed = it < p.stages ? it : p.stages;
-      for (int j = it - armed; j < it; ++j) mbar_wait(&bar_full[j % p.stages], (uint32_t)((j / p.stages) & 1));
+      const int armed = it < ring ? it : ring;
+      for (int j = it - armed; j < it; ++j) mbar_wait(&full[j % ring], (uint32_t)((j / ring) & 1));
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t idesc = umma_idesc_bf16(NN);
     const uint64_t desc0 = umma_desc_sw128(0);
-    int s = 0;
-    uint32_t ph = 0;
+    int s = 0, sx = 0;
+    uint32_t ph = 0, phx = 0;
     bool ok = true;
     for (int it = 0; it < n_kb; ++it) {
-      if (!warp_wait(&bar_full[s], ph)) { ok = false; break; }
+      if (!warp_wait_both(&sh.full[s], ph, &sh.x_full[sx], phx)) { ok = false; break; }
       tc_fence_after();
       if (elect_one()) {
-        const uint32_t at = smem_u32(smem + s * stage_bytes);
-        const uint64_t a = desc0 | (uint64_t)(at >> 4), b = desc0 | (uint64_t)((at + W_TILE_BYTES) >> 4);
+        const uint64_t a = desc0 | (uint64_t)(smem_u32(smem + s * W_TILE_BYTES) >> 4);
+        const uint64_t b = desc0 | (uint64_t)(smem_u32(smem_x + sx * x_tile_bytes) >> 4);
 #pragma unroll
         for (int k = 0; k < TILE_K / UMMA_K; ++k) umma_bf16(tmem_base, a + k * 2, b + k * 2, idesc, !(it == 0 && k == 0));
-        umma_commit(&bar_empty[s]);   // frees the stage once these MMAs have read it
+        umma_commit(&sh.done[it % kMaxStages]);   // frees both stages once these MMAs have read them
       }
       __syncwarp();
       if (++s == p.stages) { s = 0; ph ^= 1u; }
+      if (++sx == p.x_stages) { sx = 0; phx ^= 1u; }
     }
     if (ok) {
-      if (elect_one()) umma_commit(&bar_acc_full);
+      if (elect_one()) umma_commit(&sh.acc_full);
     } else if (lane == 0) {
       atomicExch(p.status, 2);
     }
@@ -365,7 +374,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
     // ------------------------------------------------------------------ epilogue warps (2..5)
     const int quarter = warp & 3;                 // TMEM lane quarter this warp may read
     const int row = quarter * 32 + lane;          // weight row inside the tile
-    const bool ok = epilogue_all(mbar_wait(&bar_acc_full, 0));
+    const bool ok = epilogue_all(mbar_wait(&sh.acc_full, 0));
     if (ok) {
       tc_fence_after();
       pdl_wait();   // the planes may still be read, and the row scales written, by the preceding kernel
@@ -933,13 +942,30 @@ static int allow_gemm_smem() {
   SJD_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return SJD_ERR_UNSUPPORTED;
   if (done.load() >> dev & 1) return SJD_OK;
-  constexpr size_t kMost = 2 * kSmemBudget + 2048;   // stages * stage_bytes + 1024 is at most that
+  constexpr size_t kMost = (kDeepRing > kSmemBudget ? kDeepRing : kSmemBudget) + sizeof(TcShared);
   int rc = allow_smem(gemm_tc_kernel<false>, kMost);
   if (rc == SJD_OK) rc = allow_smem(gemm_tc_kernel<true>, kMost);
   if (rc == SJD_OK) rc = allow_smem(gemm_pair_kernel<false>, kPairSmem);
   if (rc == SJD_OK) rc = allow_smem(gemm_pair_kernel<true>, kPairSmem);
   if (rc == SJD_OK) done.fetch_or(1ull << dev);
   return rc;
+}
+
+// Stages of the two rings of a gemm_tc_kernel CTA.  Weights come from HBM and want as many bytes in flight as there is room for;
+// activations come from L2, but under the stream of weights that still takes two to three k-blocks.  Two CTAs of an SM have to
+// leave a few KB: without them no CTA of the next kernel can wait beside them, and its launch and the weights that it
+// prefetches come late.  us of a step of 16 layers, stages of weights + activations: 7B, 32 rows: 6 + 2 (no
+// room left) 1755, 5 + 2 1696, 4 + 3 1663, 5 + 3 1646, 4 + 4 1670; 64 rows: 3 + 3 1946, 4 + 2 1905, 4 + 3 (no room left) 1937.
+// At most one CTA per SM (small models, short K): both rings hold all or much of K.
+void ring_stages(bool deep, int x_bytes, int *stages, int *x_stages) {
+  if (deep) {
+    const int n = kDeepRing / (W_TILE_BYTES + x_bytes);
+    *stages = *x_stages = n > kMaxStages ? kMaxStages : n;
+    return;
+  }
+  *x_stages = x_bytes <= W_TILE_BYTES / 2 ? 3 : 2;
+  const int n = (kSmemBudget - *x_stages * x_bytes) / W_TILE_BYTES;
+  *stages = n > kMaxStages ? kMaxStages : n;
 }
 
 static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles, cudaStream_t stream) {
@@ -1026,16 +1052,11 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   const int rc = allow_gemm_smem();
   if (rc != SJD_OK) return rc;
   if (gemm_tc_pairs(pl)) return launch_gemm_pair(g, p, tiles, stream);
-  const int stage_bytes = W_TILE_BYTES + 2 * p.Mp * TILE_K * 2;
+  const int x_bytes = 2 * p.Mp * TILE_K * 2;
   const int ctas = tiles;
-  // one CTA per SM or fewer: give each the deeper ring
-  const int budget =
-      (SJD_GEMM_DEEP_RING && g.n_sms > 0 && ctas * g.splits <= g.n_sms) ? 2 * kSmemBudget : kSmemBudget;
-  int stages = budget / stage_bytes;
-  stages = stages > kMaxStages ? kMaxStages : stages;
-  if (stages < 2) return SJD_ERR_UNSUPPORTED;
-  p.stages = stages;
-  const size_t smem = (size_t)stages * stage_bytes + 1024;
+  const bool deep = g.n_sms > 0 && ctas * g.splits <= g.n_sms;
+  ring_stages(deep, x_bytes, &p.stages, &p.x_stages);
+  const size_t smem = (size_t)p.stages * W_TILE_BYTES + (size_t)p.x_stages * x_bytes + sizeof(TcShared);
   const CUtensorMap &w0 = reinterpret_cast<const CUtensorMap &>(*g.w_map[0]);
   const CUtensorMap &w1 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 1 ? 1 : 0]);
   const CUtensorMap &w2 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 2 ? 2 : 0]);
