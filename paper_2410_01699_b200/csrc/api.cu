@@ -197,7 +197,7 @@ int attn_splits(int n_heads, int batch) { return sjd::attention_splits(n_heads, 
 }  // namespace
 
 extern "C" size_t sjd_attention_workspace_bytes(int batch, int window, int n_heads, int head_dim) {
-  if (batch < 1 || window < 1 || n_heads < 1 || !attention_mma_supported(head_dim, window)) return 0;
+  if (batch < 1 || window < 1 || n_heads < 1 || !attention_tc_supported(head_dim, window)) return 0;
   return 256 + (size_t)batch * window * n_heads * attn_splits(n_heads, batch) * (head_dim + 2) * 4;
 }
 
@@ -207,7 +207,7 @@ extern "C" int sjd_attention(int batch, int window, int n_heads, int n_kv_heads,
   if (batch < 1 || window < 1 || n_heads < 1 || n_kv_heads < 1 || max_seq < 1 || !q || !kv_cache || !in_pos || !out || !ws)
     return SJD_ERR_BAD_ARG;
   if (n_heads % n_kv_heads != 0) return SJD_ERR_BAD_ARG;
-  if (!attention_mma_supported(head_dim, window)) return SJD_ERR_UNSUPPORTED;
+  if (!attention_tc_supported(head_dim, window)) return SJD_ERR_UNSUPPORTED;
   if (((uintptr_t)ws & 255u) != 0) return SJD_ERR_BAD_ARG;
   if (ws_bytes < sjd_attention_workspace_bytes(batch, window, n_heads, head_dim)) return SJD_ERR_CAPACITY;
   int dev = 0, cc_major = 0;
@@ -217,15 +217,14 @@ extern "C" int sjd_attention(int batch, int window, int n_heads, int n_kv_heads,
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   int *status = (int *)ws;
   float *partial = (float *)((char *)ws + 256);
-  SJD_CUDA(cudaMemsetAsync(status, 0, 256, stream));
   TensorMap kv_map;
   int rc = make_kv_tensor_map(&kv_map, kv_cache, (long)batch * 2 * n_kv_heads, max_seq, head_dim);
   if (rc != SJD_OK) return rc;
   const int splits = attn_splits(n_heads, batch);
   const int M = batch * window;
   const KvLayout contiguous = {const_cast<void *>(kv_cache), n_kv_heads, max_seq, head_dim, nullptr, 0, 0, 1};
-  rc = launch_attention_mma(kv_map, 0, contiguous, q, in_pos, partial, out, HiLoOut{nullptr, 0}, status, M,
-                            RowSegs{window, nullptr}, n_heads, n_kv_heads, head_dim, splits, stream);
+  rc = launch_attention_tc(kv_map, 0, contiguous, q, in_pos, partial, out, HiLoOut{nullptr, 0}, status, M,
+                            RowSegs{window, nullptr}, n_heads, n_kv_heads, head_dim, splits, true, stream);
   if (rc != SJD_OK || splits == 1) return rc;
   return launch_attention_combine(partial, in_pos, out, M, n_heads, head_dim, splits, stream, HiLoOut{nullptr, 0});
 }

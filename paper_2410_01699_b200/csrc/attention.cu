@@ -139,103 +139,84 @@ __global__ void __launch_bounds__(NWARPS * 32) attention_partial_kernel(
     __syncthreads();
   }
 
-  // partial record per (row, head, split): [m, l, o[hd]]
+  // partial records: o [row][head][split][hd], then (m, l) [row][head][split]
+  float *ml = partial + (size_t)gridDim.y * W * n_heads * splits * hd;
 #pragma unroll
   for (int i = 0; i < MAXQ; ++i) {
     const int qi = warp + i * NWARPS;
     if (qi >= W) continue;
-    float *dst = partial + (((size_t)(m0 + qi) * n_heads + h) * splits + s) * (hd + 2);
-    if (lane == 0) {
-      dst[0] = m_run[i];
-      dst[1] = l_run[i];
-    }
+    const size_t rec = ((size_t)(m0 + qi) * n_heads + h) * splits + s;
+    if (lane == 0) *reinterpret_cast<float2 *>(ml + rec * 2) = make_float2(m_run[i], l_run[i]);
 #pragma unroll
     for (int j = 0; j < MAXD; ++j) {
       const int d = lane + 32 * j;
-      if (d < hd) dst[2 + d] = o[i][j];
+      if (d < hd) partial[rec * hd + d] = o[i][j];
     }
   }
 }
 
-__global__ void attention_combine_kernel(const float *__restrict__ partial, const int32_t *__restrict__ in_pos,
-                                         float *__restrict__ out, int n_heads, int hd, int splits, HiLoOut hilo) {
+// Merge of the key ranges: a warp per (row, head), whose loads are all in flight at once (those of the records do not wait for the
+// references): the launch is a link of the chain of a step and costs a round trip or two, not its work.  (A block per (row, head) whose
+// threads each read every reference took three round trips with more than eight ranges: 5.8 us of a layer of the 7B step.)
+constexpr int kCombineWarps = 4;
+constexpr int kCombineSplits = 16;
+
+__global__ void __launch_bounds__(kCombineWarps * 32) attention_combine_kernel(const float *__restrict__ partial,
+                                                                               const int32_t *__restrict__ in_pos,
+                                                                               float *__restrict__ out, int M, int n_heads, int hd,
+                                                                               int splits, HiLoOut hilo) {
   pdl_trigger();
   SJD_TL(TL_COMBINE, 0, threadIdx.x == 0);
   pdl_wait();
   SJD_TL(TL_COMBINE, 1, threadIdx.x == 0);
-  const int m = blockIdx.x, h = blockIdx.y;
-  const float *src = partial + ((size_t)m * n_heads + h) * splits * (hd + 2);
-  const size_t base = ((size_t)m * n_heads + h) * hd;
-  auto put = [&](int d, float v) {
-    if (out) out[base + d] = v;
+  const int lane = threadIdx.x & 31, mh = blockIdx.x * kCombineWarps + (threadIdx.x >> 5);
+  if (mh >= M * n_heads) return;
+  const float *src = partial + (size_t)mh * splits * hd + 2 * lane;
+  const float *ml = partial + (size_t)M * n_heads * splits * hd + (size_t)mh * splits * 2;
+  const int pos = in_pos[mh / n_heads];
+  const float2 r = lane < splits ? *reinterpret_cast<const float2 *>(ml + 2 * lane) : make_float2(-INFINITY, 0.0f);
+  const bool on0 = 2 * lane < hd, on1 = 2 * lane + 64 < hd;   // (hd is even)
+  float2 v0[kCombineSplits], v1[kCombineSplits];
+#pragma unroll
+  for (int s = 0; s < kCombineSplits; ++s) {
+    v0[s] = v1[s] = make_float2(0.0f, 0.0f);
+    if (s < splits && on0) v0[s] = *reinterpret_cast<const float2 *>(src + (size_t)s * hd);
+    if (s < splits && on1) v1[s] = *reinterpret_cast<const float2 *>(src + (size_t)s * hd + 64);
+  }
+  const float g = warp_max(r.x);
+  const float wgt = r.x > -INFINITY ? expf(r.x - g) : 0.0f;
+  const float denom = warp_sum(r.y * wgt);
+  float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
+#pragma unroll
+  for (int s = 0; s < kCombineSplits; ++s) {
+    if (s >= splits) break;
+    const float w = __shfl_sync(0xffffffffu, wgt, s);
+    if (w > 0.0f) {   // (the record of an empty range is not written)
+      a0.x += v0[s].x * w;
+      a0.y += v0[s].y * w;
+      a1.x += v1[s].x * w;
+      a1.y += v1[s].y * w;
+    }
+  }
+  const bool live = pos >= 0 && denom > 0.0f;
+  auto put = [&](int d, float2 a) {
+    const float x = live ? a.x / denom : 0.0f, y = live ? a.y / denom : 0.0f;
+    const size_t idx = (size_t)mh * hd + d;
+    if (out && ((uintptr_t)out & 7u) == 0) {
+      *reinterpret_cast<float2 *>(out + idx) = make_float2(x, y);
+    } else if (out) {   // (a caller's buffer may start on any float)
+      out[idx] = x;
+      out[idx + 1] = y;
+    }
     if (hilo.base) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      hilo.base[base + d] = hi;
-      hilo.base[hilo.lo_offset + base + d] = __float2bfloat16_rn(v - __bfloat162float(hi));
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+      const float2 f = __bfloat1622float2(h);
+      *reinterpret_cast<__nv_bfloat162 *>(hilo.base + idx) = h;
+      *reinterpret_cast<__nv_bfloat162 *>(hilo.base + hilo.lo_offset + idx) = __floats2bfloat162_rn(x - f.x, y - f.y);
     }
   };
-  constexpr int NS = 8;
-  if (splits <= NS && hd <= (int)blockDim.x) {
-    // Few key ranges (the usual case): every thread fetches the row's position, all record heads and its own
-    // entry of every record at once, so the kernel costs one memory round trip instead of three in a row.
-    // Same arithmetic, in the same order, as the general path below.
-    const int d = threadIdx.x;
-    const int pos = in_pos[m];
-    float mm[NS], ll[NS], vv[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const bool on = s < splits;
-      mm[s] = on ? src[(size_t)s * (hd + 2)] : -INFINITY;
-      ll[s] = on ? src[(size_t)s * (hd + 2) + 1] : 0.0f;
-      vv[s] = on && d < hd ? src[(size_t)s * (hd + 2) + 2 + d] : 0.0f;
-    }
-    if (d >= hd) return;
-    float v = 0.0f;
-    if (pos >= 0) {
-      float gmax = -INFINITY;
-#pragma unroll
-      for (int s = 0; s < NS; ++s) gmax = fmaxf(gmax, mm[s]);
-      float denom = 0.0f, acc = 0.0f;
-#pragma unroll
-      for (int s = 0; s < NS; ++s)
-        if (s < splits && mm[s] > -INFINITY) denom += ll[s] * expf(mm[s] - gmax);
-#pragma unroll
-      for (int s = 0; s < NS; ++s)
-        if (s < splits) acc += vv[s] * (mm[s] > -INFINITY ? expf(mm[s] - gmax) : 0.0f);
-      v = denom > 0.0f ? acc / denom : 0.0f;
-    }
-    put(d, v);
-    return;
-  }
-  if (in_pos[m] < 0) {
-    for (int d = threadIdx.x; d < hd; d += blockDim.x) {
-      put(d, 0.0f);
-    }
-    return;
-  }
-  // heads of the records once (one thread per key range), then the weights from shared memory: the
-  // loads over the records below do not wait on one another
-  __shared__ float s_m[64], s_l[64], s_w[64];
-  const int ns = splits < 64 ? splits : 64;
-  if ((int)threadIdx.x < ns) {
-    s_m[threadIdx.x] = src[(size_t)threadIdx.x * (hd + 2)];
-    s_l[threadIdx.x] = src[(size_t)threadIdx.x * (hd + 2) + 1];
-  }
-  __syncthreads();
-  float gmax = -INFINITY;
-  for (int s = 0; s < ns; ++s) gmax = fmaxf(gmax, s_m[s]);
-  float denom = 0.0f;
-  for (int s = 0; s < ns; ++s)
-    if (s_m[s] > -INFINITY) denom += s_l[s] * expf(s_m[s] - gmax);
-  if ((int)threadIdx.x < ns) s_w[threadIdx.x] = s_m[threadIdx.x] > -INFINITY ? expf(s_m[threadIdx.x] - gmax) : 0.0f;
-  __syncthreads();
-  for (int d = threadIdx.x; d < hd; d += blockDim.x) {
-    float acc = 0.0f;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) acc += src[(size_t)s * (hd + 2) + 2 + d] * s_w[s];
-    const float v = denom > 0.0f ? acc / denom : 0.0f;
-    put(d, v);
-  }
+  if (on0) put(2 * lane, a0);
+  if (on1) put(2 * lane + 64, a1);
 }
 
 template <typename T>
@@ -258,8 +239,9 @@ int attention_t(const float *q, KvLayout kv, const int32_t *in_pos, float *out, 
 
 int launch_attention_combine(const float *partial, const int32_t *in_pos, float *out, int M, int n_heads, int head_dim,
                              int splits, cudaStream_t stream, HiLoOut hilo) {
-  SJD_CUDA(launch_kernel(attention_combine_kernel, dim3(M, n_heads), dim3(128), 0, stream, partial, in_pos, out, n_heads,
-                         head_dim, splits, hilo));
+  if (splits > kCombineSplits || head_dim > 128) return SJD_ERR_UNSUPPORTED;
+  SJD_CUDA(launch_kernel(attention_combine_kernel, dim3((M * n_heads + kCombineWarps - 1) / kCombineWarps), dim3(kCombineWarps * 32), 0,
+                         stream, partial, in_pos, out, M, n_heads, head_dim, splits, hilo));
   SJD_CHECK_LAUNCH();
   return SJD_OK;
 }

@@ -380,20 +380,20 @@ int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const
 int launch_qkv_finish(PlaneSet ps, RowScale rs, const int32_t *in_pos, const float2 *rope_table, float *q,
                       KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream);
 // Window-causal attention: query row m (position in_pos[m] of its segment's sequence) attends cache rows
-// 0 .. in_pos[m].  q, out: fp32 [M][H*hd]; cache of `dtype`.  partial: fp32 scratch [M][H][splits][hd + 2].
+// 0 .. in_pos[m].  q, out: fp32 [M][H*hd]; cache of `dtype`.  partial: fp32 scratch, M * H * splits * (hd + 2) entries.
 int launch_attention(int dtype, const float *q, KvLayout kv, const int32_t *in_pos, float *out, float *partial,
                      int M, RowSegs segs, int n_heads, int splits, cudaStream_t stream,
                      HiLoOut hilo = HiLoOut{nullptr, 0});
-// merge of the split-KV partials only (used after launch_attention_mma); out may be null when only the hi/lo planes are wanted
+// merge of the split-KV partials only (used after launch_attention_tc); out may be null when only the hi/lo planes are wanted
 int launch_attention_combine(const float *partial, const int32_t *in_pos, float *out, int M, int n_heads, int head_dim,
                              int splits, cudaStream_t stream, HiLoOut hilo);
-// tensor-core split-KV attention for bf16 caches (attention_mma.cu)
+// tensor-core split-KV attention for bf16 caches (attention_tc.cu)
 int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim);
-bool attention_mma_supported(int head_dim, int rows_per_seq);
+bool attention_tc_supported(int head_dim, int rows_per_seq);
 // plane0: first plane of this layer in the contiguous map [planes][max_seq][hd]; with kv.page_table set the map is
 // the pool's [planes][KV_PAGE][hd] and the plane of a tile comes from the page table.
-int launch_attention_mma(const TensorMap &kv_map, int plane0, KvLayout kv, const float *q, const int32_t *in_pos, float *partial,
+int launch_attention_tc(const TensorMap &kv_map, int plane0, KvLayout kv, const float *q, const int32_t *in_pos, float *partial,
                          float *out, HiLoOut hilo, int *status, int M, RowSegs segs, int n_heads, int n_kv_heads,
-                         int head_dim, int splits, cudaStream_t stream);
+                         int head_dim, int splits, bool clear_status, cudaStream_t stream);
 
 }  // namespace sjd

@@ -146,7 +146,7 @@ Layout make_layout(const sjd_model_cfg &c) {
   for (size_t b = 1; b * 16 <= Mp + 64 || b <= (size_t)c.max_batch; ++b) {   // b segments of a step or of a pre-fill pass
     const int splits = attention_splits(c.n_heads, (int)b);
     // with one key range the tensor-core attention writes its output itself: only the generic kernel needs records then
-    const bool direct = splits == 1 && tc && attention_mma_supported(c.head_dim, 64);
+    const bool direct = splits == 1 && tc && attention_tc_supported(c.head_dim, 64);
     const size_t cap = direct ? Mg : Mp, rows = b * 64 < cap ? b * 64 : cap;
     const size_t need = rows * c.n_heads * splits * (c.head_dim + 2);
     part = need > part ? need : part;
@@ -352,7 +352,7 @@ struct sjd_ctx {
   // (one that could not be encoded) the generic attention has to have room for the rows.
   bool tc_pass(int M) const {
     return use_tc && all_tc && M <= kMaxTcRows &&
-           (kv_map_valid || !attention_mma_supported(cfg.head_dim, 64) || (size_t)M <= lay.generic_rows);
+           (kv_map_valid || !attention_tc_supported(cfg.head_dim, 64) || (size_t)M <= lay.generic_rows);
   }
   int rows_alloc() const { return ((int)lay.pass_rows + 15) / 16 * 16; }
 
@@ -548,10 +548,10 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
     const KvLayout kv = c->kv_layer(l);
     SJD_TR(TC_OTHER, launch_qkv_finish(ps, rs, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
     if (!logits_out && l == g.n_layers - 1) break;
-    if (c->kv_map_valid && attention_mma_supported(g.head_dim, segs.rows)) {
-      SJD_TR(TC_ATTENTION, launch_attention_mma(c->kv_map, l * g.max_batch * 2 * g.n_kv_heads, kv, q, st.in_pos, partial, nullptr,
+    if (c->kv_map_valid && attention_tc_supported(g.head_dim, segs.rows)) {
+      SJD_TR(TC_ATTENTION, launch_attention_tc(c->kv_map, l * g.max_batch * 2 * g.n_kv_heads, kv, q, st.in_pos, partial, nullptr,
                                                 hl_attn, status, M, segs, g.n_heads, g.n_kv_heads, g.head_dim,
-                                                att_splits, stream));
+                                                att_splits, false, stream));
       if (att_splits > 1)
         SJD_TR(TC_ATTENTION,
                launch_attention_combine(partial, st.in_pos, nullptr, M, g.n_heads, g.head_dim, att_splits, stream, hl_attn));
@@ -761,7 +761,7 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
     const long planes = paged ? (long)(cfg->kv_pages + 1) * L * 2 * cfg->n_kv_heads
                               : (long)L * cfg->max_batch * 2 * cfg->n_kv_heads;
     const long plane_rows = paged ? KV_PAGE : cfg->max_seq;
-    if (attention_mma_supported(cfg->head_dim, cfg->max_window) &&
+    if (attention_tc_supported(cfg->head_dim, cfg->max_window) &&
         make_kv_tensor_map(&c->kv_map, c->ws + lay.kv, planes, plane_rows, cfg->head_dim) == SJD_OK &&
         cudaMemset(c->ws + lay.kv, 0, (size_t)planes * plane_rows * cfg->head_dim * 2) == cudaSuccess)
       c->kv_map_valid = true;
@@ -1002,7 +1002,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   const bool tc = c->tc_pass(M) && c->xmaps.count((M + 15) / 16 * 16) != 0;
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
-      (tc && c->kv_map_valid && attention_mma_supported(c->cfg.head_dim, c->window)) ? 1 : 0;
+      (tc && c->kv_map_valid && attention_tc_supported(c->cfg.head_dim, c->window)) ? 1 : 0;
   info->step_graph = c->graphs_enabled ? 1 : 0;
   info->rows_per_step = M;
   return SJD_OK;

@@ -250,8 +250,10 @@ int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
 template <typename T>
 __global__ void embed_kernel(const T *__restrict__ emb, const int32_t *__restrict__ tok, float *__restrict__ x, int d,
                              int vocab) {
-  pdl_trigger();
   pdl_wait();
+  // First kernel of a pass, and the only one that lets the next one start after its own wait: whatever was written before the pass
+  // (positions, the cache of earlier steps) is there for every later kernel of the pass, also before that kernel's wait.
+  pdl_trigger();
   const int m = blockIdx.x;
   int t = tok[m];
   t = min(max(t, 0), vocab - 1);
