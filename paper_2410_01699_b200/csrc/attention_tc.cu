@@ -338,9 +338,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
       // Q, pre-scaled by log2(e) / sqrt(HD), as K-major planes: rows 0.. hi, rows WP.. lo
       uint8_t *Qs = attn_smem + st * Q_BYTES;
       const float sc = 1.4426950408889634f * rsqrtf((float)HD);
-#pragma unroll 4
-      for (int i = ts; i < WP * (HD / 8); i += 128) {
-        const int r = i / (HD / 8), c = i % (HD / 8);
+#pragma unroll   // all loads in flight at once
+      for (int j0 = 0; j0 < WP * (HD / 8) / 128; ++j0) {
+        const int i = ts + j0 * 128, r = i / (HD / 8), c = i % (HD / 8);
         float2 v[4] = {};
         if (sh.pos[st][r] >= 0) {   // (the caller's rows start on 8 bytes)
           const float2 *src = reinterpret_cast<const float2 *>(p.q + ((size_t)(me.m0 + r) * p.n_heads + me.h) * HD + c * 8);
@@ -484,71 +484,86 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
       if (lane == 0) mbar_arrive(&sh.p_full[st]);
     }
     SJD_TL(TL_ATTN, 2, threadIdx.x == 0);
-    // ---- the sums over the keys, then the output rows
+    // ---- the sums over the keys, while the last tile is multiplied; then the output rows
+    stream_sync(st);
+#pragma unroll
+    for (int g = 0; g < WP / 32; ++g) {
+      float v[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = l_acc[g * 32 + i];
+      sh.red[st][w][g * 32 + lane] = lanes_combine(v, [](float a, float b) { return a + b; });
+    }
     if (ok && n > 0) ok = mbar_wait(&sh.pv_done[st], (uint32_t)((n - 1) & 1));
     if (!stream_any(st, !ok)) {
       tc_fence_after();
-#pragma unroll
-      for (int g = 0; g < WP / 32; ++g) {
-        float v[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = l_acc[g * 32 + i];
-        sh.red[st][w][g * 32 + lane] = lanes_combine(v, [](float a, float b) { return a + b; });
-      }
-      stream_sync(st);
       const bool direct = p.splits == 1;
-      const size_t rec0 = ((size_t)me.m0 * p.n_heads + me.h) * p.splits + me.split;   // record of query 0; the next one H * splits further
+      const size_t rec_step = (size_t)p.n_heads * p.splits;   // from a query's record to the next one's
+      const size_t rec0 = (size_t)me.m0 * rec_step + (size_t)me.h * p.splits + me.split;
       float l = 0.0f;
       if (ts < W) {
         l = sh.pos[st][ts] >= 0 ? (sh.red[st][0][ts] + sh.red[st][1][ts]) + (sh.red[st][2][ts] + sh.red[st][3][ts]) : 0.0f;
         if (!direct)   // (reference in natural log units)
-          *reinterpret_cast<float2 *>(ml + (rec0 + (size_t)ts * p.n_heads * p.splits) * 2) =
-              make_float2(l > 0.0f ? my_ref * 0.6931471805599453f : -INFINITY, l);
+          *reinterpret_cast<float2 *>(ml + (rec0 + ts * rec_step) * 2) = make_float2(l > 0.0f ? my_ref * 0.6931471805599453f : -INFINITY, l);
       }
       if (direct) {
-        stream_sync(st);
-        if (ts < WP) sh.red[st][0][ts] = l > 0.0f ? 1.0f / l : 0.0f;   // inactive rows: zeros
+        if (ts < WP) sh.red[st][0][ts] = l > 0.0f ? 1.0f / l : 0.0f;   // inactive rows: zeros  (each thread has read its column only)
         stream_sync(st);
       }
-      if (n > 0 || direct) {
-        const int dim = w * 32 + lane;
+      const int dim = w * 32 + lane;
+      if ((n > 0 || direct) && w * 32 < HD) {
+        const size_t step = direct ? (size_t)p.n_heads * HD : rec_step * HD;
+        const size_t at0 = direct ? ((size_t)me.m0 * p.n_heads + me.h) * HD + dim : rec0 * HD + dim;
 #pragma unroll 1
         for (int c = 0; c < NC; ++c) {
           if (c * 16 >= W) break;
           uint32_t hi[16], lo[16];
-          float ov[16];
+          float v[16];
           if (n > 0) {
             tmem_ld16_issue(t_o + c * 16, hi);
             tmem_ld16_issue(t_o + WP + c * 16, lo);
             tmem_ld_wait();
           }
 #pragma unroll
-          for (int i = 0; i < 16; ++i) ov[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+          for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
           if (NO == 2 && n > 1) {
             tmem_ld16_issue(t_o + 2 * WP + c * 16, hi);
             tmem_ld16_issue(t_o + 3 * WP + c * 16, lo);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) ov[i] += __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+            for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
           }
-          if (dim >= HD) continue;
+          const size_t at = at0 + (size_t)(c * 16) * step;
+          const int left = W - c * 16;
+          auto each = [&](auto store) {   // (no tests per row but in a ragged chunk)
+            if (left >= 16) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int r = c * 16 + i;
-            if (r >= W) break;
-            float v = ov[i];
-            if (direct) {
-              const float inv = sh.red[st][0][r];
-              v = inv > 0.0f ? v * inv : 0.0f;
-              const size_t idx = ((size_t)(me.m0 + r) * p.n_heads + me.h) * HD + dim;
-              if constexpr (OUT) p.out[idx] = v;
-              if (p.hilo.base) {
-                const __nv_bfloat16 vh = __float2bfloat16_rn(v);
-                p.hilo.base[idx] = vh;
-                p.hilo.base[p.hilo.lo_offset + idx] = __float2bfloat16_rn(v - __bfloat162float(vh));
-              }
+              for (int i = 0; i < 16; ++i) store(i);
             } else {
-              p.partial[(rec0 + (size_t)r * p.n_heads * p.splits) * HD + dim] = v;
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                if (i < left) store(i);
+            }
+          };
+          if (!direct) {
+            float *dst = p.partial + at;
+            each([&](int i) { dst[i * step] = v[i]; });
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float inv = sh.red[st][0][c * 16 + i];
+              v[i] = inv > 0.0f ? v[i] * inv : 0.0f;
+            }
+            if constexpr (OUT) {
+              float *dst = p.out + at;
+              each([&](int i) { dst[i * step] = v[i]; });
+            }
+            if (p.hilo.base) {
+              __nv_bfloat16 *dst = p.hilo.base + at, *dst_lo = dst + p.hilo.lo_offset;
+              each([&](int i) {
+                const __nv_bfloat16 vh = __float2bfloat16_rn(v[i]);
+                dst[i * step] = vh;
+                dst_lo[i * step] = __float2bfloat16_rn(v[i] - __bfloat162float(vh));
+              });
             }
           }
         }
