@@ -263,8 +263,7 @@ struct alignas(64) TensorMap {   // an encoded TMA descriptor (same size and ali
 // bf16 row-major [rows][cols] matrix cut into boxes of box_rows x 64 columns, 128-byte swizzle
 int make_tensor_map_bf16(TensorMap *out, const void *base, long rows, long cols, int box_rows);
 bool gemm_tc_supported(int M, int N, int K);
-// Shape of a launch of M rows: token slabs and rows per slab (a multiple of 16: the box height of the
-// activation tensor map).
+// Shape of a launch of M rows: token slabs and rows per slab (the box height of the activation tensor map).
 struct GemmTcPlan {
   int n_slabs, slab_rows;
 };

@@ -159,9 +159,11 @@ Layout make_layout(const sjd_model_cfg &c) {
     const size_t cols[3] = {nq + 2 * nk, (size_t)c.d_model, (size_t)c.d_model};
     size_t need = 0;
     for (int i = 0; i < 3 && tc; ++i) {
-      for (size_t rows = 16; rows < Mp + 16 && rows <= kMaxTcRows; rows += 16) {   // splits shrink as the token slabs grow
-        const size_t m = rows < Mp ? rows : Mp;
-        const size_t n = (size_t)gemm_tc_splits_max(gemm_tc_plan((int)m), tiles[i] > 0 ? tiles[i] : 1, kbs[i]) * m * cols[i];
+      const size_t most = Mp < (size_t)kMaxTcRows ? Mp : (size_t)kMaxTcRows;
+      for (size_t m = 1; m <= most; ++m) {   // splits depend on the token slabs alone: the most rows of each layout
+        const GemmTcPlan here = gemm_tc_plan((int)m), next = gemm_tc_plan((int)m + 1);
+        if (m < most && here.n_slabs == next.n_slabs && here.slab_rows == next.slab_rows) continue;
+        const size_t n = (size_t)gemm_tc_splits_max(here, tiles[i] > 0 ? tiles[i] : 1, kbs[i]) * m * cols[i];
         need = n > need ? n : need;
       }
     }
@@ -345,7 +347,7 @@ struct sjd_ctx {
   int n_ctas = 0;
   std::vector<LayerMaps> wmaps;
   WMap wmap_head;
-  std::map<int, XMaps> xmaps;   // keyed by padded row count
+  std::map<int, XMaps> xmaps;   // keyed by the rows of a token slab
   TensorMap kv_map;             // whole KV cache as [planes][max_seq][head_dim]
   bool kv_map_valid = false;
   // a pass of M rows may take the tensor-core pipeline (given its activation descriptors).  Without the cache's descriptor
@@ -590,7 +592,7 @@ int forward_tc(sjd_ctx *c, const XMaps &xm, int n_segs, RowSegs segs, void *logi
 int forward(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cudaStream_t stream) {
   const int M = n_segs * segs.rows;
   if (c->tc_pass(M)) {
-    auto it = c->xmaps.find((M + 15) / 16 * 16);
+    auto it = c->xmaps.find(gemm_tc_plan(M).slab_rows);
     if (it != c->xmaps.end()) {
       // every kernel of this pipeline waits for its predecessor itself: launch them overlapped
       g_pdl = !c->tracer.on;
@@ -776,19 +778,18 @@ extern "C" int sjd_init(sjd_ctx **out, const sjd_model_cfg *cfg, const sjd_weigh
 }
 
 namespace {
-// activation descriptors for passes of `rows` rows (once per padded row count and context); false: no such pass
+// activation descriptors for passes of `rows` rows (once per height of a token slab and context); false: no such pass
 bool add_x_maps(sjd_ctx *c, int rows) {
-  const int Mp = (rows + 15) / 16 * 16;
+  const int box = gemm_tc_plan(rows).slab_rows;
   if (!c->tc_pass(rows)) return false;
-  if (c->xmaps.count(Mp)) return true;
+  if (c->xmaps.count(box)) return true;
   const int Ma = c->rows_alloc();
   const int nq = c->cfg.n_heads * c->cfg.head_dim;
   XMaps xm;
-  const int box = gemm_tc_plan(rows).slab_rows;
   const bool ok = make_tensor_map_bf16(&xm.h, c->ws + c->lay.xs_h, 2L * Ma, c->cfg.d_model, box) == SJD_OK &&
                   make_tensor_map_bf16(&xm.attn, c->ws + c->lay.xs_attn, 2L * Ma, nq, box) == SJD_OK &&
                   make_tensor_map_bf16(&xm.act, c->ws + c->lay.xs_act, 2L * Ma, c->cfg.ffn_hidden, box) == SJD_OK;
-  if (ok) c->xmaps[Mp] = xm;
+  if (ok) c->xmaps[box] = xm;
   return ok;
 }
 }  // namespace
@@ -999,7 +1000,7 @@ extern "C" int sjd_get_info(sjd_ctx *c, sjd_info *info) {
   if (!c || !info) return SJD_ERR_BAD_ARG;
   if (!c->prefilled) return SJD_ERR_STATE;
   const int M = c->batch * c->window;
-  const bool tc = c->tc_pass(M) && c->xmaps.count((M + 15) / 16 * 16) != 0;
+  const bool tc = c->tc_pass(M) && c->xmaps.count(gemm_tc_plan(M).slab_rows) != 0;
   info->tensor_core_projections = tc ? 1 : 0;
   info->tensor_core_attention =
       (tc && c->kv_map_valid && attention_tc_supported(c->cfg.head_dim, c->window)) ? 1 : 0;

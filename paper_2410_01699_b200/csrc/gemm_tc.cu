@@ -610,7 +610,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
       }
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * NN;
-      const int mat = mat_of(t.tile), m_left = p.M - m_base;
+      const int mat = mat_of(t.tile), m_left = min(p.M - m_base, p.Mp);   // (the last 16 tokens of a slab may be eight)
       const size_t piece = (size_t)2 * p.Mp * TILE_N;
       float *share = q.scratch + (size_t)(t.shared < 0 ? 0 : t.shared) * q.parts * piece + (size_t)rank * p.Mp * TILE_N + row;
       bool finish = true, gather = false;   // this CTA does the unit's epilogue; from the parts' sums
@@ -622,7 +622,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
           tmem_ld16_issue(t_addr + p.Mp + m0, lo);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) dst[(size_t)(m0 + i) * TILE_N] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+          for (int i = 0; i < 16; ++i)
+            if (i < 8 || m0 + 8 < p.Mp) dst[(size_t)(m0 + i) * TILE_N] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
         }
         __threadfence();
         pair_epilogue_all(true);
@@ -642,7 +643,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
 #pragma unroll
           for (int k = 0; k < kShareParts; ++k)
 #pragma unroll
-            for (int i = 0; i < 16; ++i) w[k][i] = k < q.parts ? __ldcg(share + k * piece + (size_t)(m0 + i) * TILE_N) : 0.0f;
+            for (int i = 0; i < 16; ++i) w[k][i] = k < q.parts && (i < 8 || m0 + 8 < p.Mp) ? __ldcg(share + k * piece + (size_t)(m0 + i) * TILE_N) : 0.0f;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             v[i] = w[0][i];
@@ -778,12 +779,13 @@ int make_tensor_map_bf16(TensorMap *out, const void *base, long rows, long cols,
 bool gemm_tc_supported(int M, int N, int K) { return M >= 1 && M <= 1024 && N % TILE_N == 0 && K % TILE_K == 0; }
 
 // How M token rows are laid over the MMA N dimension (at most 256 columns per accumulator, two per token
-// row: hi and lo plane): slabs of at most 128 rows.
+// row: hi and lo plane): slabs of at most 128 rows, in steps of 16 for one CTA per tile and of 8 for CTA pairs, whose CTAs hold a
+// plane each (the tensor pipe is their bound: 200 rows are two slabs of 104 and not of 112).
 GemmTcPlan gemm_tc_plan(int M) {
   GemmTcPlan pl;
   pl.n_slabs = (M + 127) / 128;
-  const int per = (M + pl.n_slabs - 1) / pl.n_slabs;
-  pl.slab_rows = (per + 15) / 16 * 16;
+  const int per = (M + pl.n_slabs - 1) / pl.n_slabs, step = M > 64 ? 8 : 16;
+  pl.slab_rows = (per + step - 1) / step * step;
   return pl;
 }
 

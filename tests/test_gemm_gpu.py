@@ -46,6 +46,9 @@ def _tolerance(x, w, k):
     (65, 128, 64),            # CTA pairs: one tile (the second CTA has none), one k-block
     (130, 384, 1088),         # three tiles (an odd pair), two slabs of 80 rows, K over several splits
     (257, 19200, 256),        # more units than pairs, three slabs, few k-blocks per unit
+    (72, 384, 1088),          # slabs whose rows are not a multiple of 16: one of 72,
+    (200, 1024, 512),         # two of 104,
+    (258, 256, 320),          # three of 88 (the last holds 82)
 ])
 def test_gemm_matches_fp64_product(m, n, k):
     x, w, ref = _case(m, n, k, seed=m + n + k)
