@@ -237,25 +237,6 @@ int launch_retain_rows(const VerifyParams &p, int dtype, cudaStream_t stream);
 size_t verify_scratch_bytes(int batch, int window);
 int check_sample_cfg(const sjd_sample_cfg *s, int vocab);
 
-// ---- model forward (model_kernels.cu, attention.cu); `dtype` selects float / bf16 storage
-enum RowsEpilogue { RG_STORE = 0, RG_ADD = 1, RG_LOGITS = 2, RG_SWIGLU = 3 };
-// One launch of the generic projections: out[m][n] (epilogue) = s(m) * sum_k x[m][k] * gain[k] * W[n][k], fp32 sums.  The
-// rows of up to three matrices of `dtype` (n[j] rows each, N in all) follow one another; gain (of `dtype`) null: s = gain = 1,
-// else s(m) = 1 / sqrt(mean(x[m]^2) + eps).  RG_ADD: out += product; RG_LOGITS: out is of `dtype`; RG_SWIGLU: w[0] gate,
-// w[1] up, N features, out = silu(gate) * up.
-struct RowsGemm {
-  const float *x;
-  int ldx;
-  const void *w[3];
-  int n[3];
-  const void *gain;
-  float eps;
-  void *out;
-  int ldc;
-  int M, N, K;
-  int epilogue;
-};
-int launch_gemm_rows(int dtype, const RowsGemm &g, cudaStream_t stream);
 // ---- tensor-core weight-streaming GEMM (gemm_tc.cu), bf16 weights
 struct alignas(64) TensorMap {   // an encoded TMA descriptor (same size and alignment as the driver's)
   unsigned char bytes[128];
@@ -368,6 +349,31 @@ __device__ __forceinline__ size_t kv_row_offset(const KvLayout &kv, int b, int w
   return (((((size_t)page * kv.n_layers + kv.layer) * 2 + which) * kv.n_kv_heads + kh) * KV_PAGE + pos % KV_PAGE) *
          kv.head_dim;
 }
+// ---- model forward (model_kernels.cu, attention.cu); `dtype` selects float / bf16 storage
+enum RowsEpilogue { RG_STORE = 0, RG_ADD = 1, RG_LOGITS = 2, RG_SWIGLU = 3, RG_QKV = 4 };
+// One launch of the generic projections: out[m][n] (epilogue) = s(m) * sum_k x[m][k] * gain[k] * W[n][k], fp32 sums.  The
+// rows of up to three matrices of `dtype` (n[j] rows each, N in all) follow one another; gain (of `dtype`) null: s = gain = 1,
+// else s(m) = 1 / sqrt(mean(x[m]^2) + eps).  RG_ADD: out += product; RG_LOGITS: out is of `dtype`; RG_SWIGLU: w[0] gate,
+// w[1] up, N features, out = silu(gate) * up.  RG_QKV: w the query, key and value matrices, N half of their rows (pairs j,
+// j + head_dim / 2 of a head); q and k are rotated by the row's position, q goes to out [M][H*hd], k and v to the cache row.
+struct RowsGemm {
+  const float *x;
+  int ldx;
+  const void *w[3];
+  int n[3];
+  const void *gain;
+  float eps;
+  void *out;
+  int ldc;
+  int M, N, K;
+  int epilogue;
+  const int32_t *in_pos;   // RG_QKV only, as of launch_rope_append
+  const float2 *rope;
+  KvLayout kv;
+  RowSegs segs;
+  int n_heads;
+};
+int launch_gemm_rows(int dtype, const RowsGemm &g, cudaStream_t stream);
 // QK-norm variant: every head of q and of k is RMS-normalised over its head_dim entries (gains of `dtype`,
 // length head_dim) before the rotary step; null gains: the plain model.
 struct QkNorm {

@@ -427,8 +427,9 @@ int forward_generic(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cuda
   int rc;
   Tracer &tr = c->tracer;
   auto gemm = [&](const float *a, int lda, const void *gain, const void *w0, int n0, const void *w1, int n1, const void *w2, int n2,
-                  void *out, int ldc, int k_in, int epilogue) -> int {
+                  void *out, int ldc, int k_in, int epilogue, const KvLayout *kv = nullptr) -> int {
     RowsGemm r;
+    memset(&r, 0, sizeof(r));
     r.x = a;
     r.ldx = lda;
     r.w[0] = w0; r.w[1] = w1; r.w[2] = w2;
@@ -438,9 +439,16 @@ int forward_generic(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cuda
     r.out = out;
     r.ldc = ldc;
     r.M = M;
-    r.N = epilogue == RG_SWIGLU ? n0 : n0 + n1 + n2;
+    r.N = epilogue == RG_SWIGLU ? n0 : epilogue == RG_QKV ? (n0 + n1 + n2) / 2 : n0 + n1 + n2;
     r.K = k_in;
     r.epilogue = epilogue;
+    if (kv) {
+      r.in_pos = st.in_pos;
+      r.rope = rope;
+      r.kv = *kv;
+      r.segs = segs;
+      r.n_heads = g.n_heads;
+    }
     if (tr.on) tr.gemm_weight_bytes += (double)(n0 + n1 + n2) * (double)k_in * (double)esize(dt);
     tr.begin(TC_GEMM, stream);
     const int rcg = launch_gemm_rows(dt, r, stream);
@@ -450,9 +458,13 @@ int forward_generic(sjd_ctx *c, int n_segs, RowSegs segs, void *logits_out, cuda
   const int lda = act_stride(g);
   SJD_TR(TC_OTHER, launch_embed(dt, c->tok_emb, st.in_tok, x, M, d, g.vocab, stream));
   for (int l = 0; l < g.n_layers; ++l) {
-    SJD_TRY(gemm(x, d, c->attn_norm[l], c->wq[l], nq, c->wk[l], nk, c->wv[l], nk, qkv, nqkv, d, RG_STORE));
     const KvLayout kv = c->kv_layer(l);
-    SJD_TR(TC_OTHER, launch_rope_append(dt, qkv, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
+    if (c->q_norm[l]) {   // QK-norm takes the whole head before the rotary step
+      SJD_TRY(gemm(x, d, c->attn_norm[l], c->wq[l], nq, c->wk[l], nk, c->wv[l], nk, qkv, nqkv, d, RG_STORE));
+      SJD_TR(TC_OTHER, launch_rope_append(dt, qkv, st.in_pos, rope, q, kv, M, segs, g.n_heads, c->qk_norm(l), stream));
+    } else {
+      SJD_TRY(gemm(x, d, c->attn_norm[l], c->wq[l], nq, c->wk[l], nk, c->wv[l], nk, q, nq, d, RG_QKV, &kv));
+    }
     if (!logits_out && l == g.n_layers - 1) break;
     SJD_TR(TC_ATTENTION, launch_attention(dt, q, kv, st.in_pos, attn, partial, M, segs, g.n_heads, splits, stream));
     SJD_TRY(gemm(attn, nq, nullptr, c->wo[l], d, nullptr, 0, nullptr, 0, x, d, nq, RG_ADD));

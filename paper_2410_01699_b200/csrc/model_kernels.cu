@@ -57,7 +57,7 @@ __device__ __forceinline__ void store_hilo(const HiLoOut &o, size_t idx, float v
 // 32, one dependent load after the other; 16 launches and the verification in 107 us now).  Hence: the eight warps of a CTA
 // split every chunk of KC columns between them, so that a whole chunk is one round trip to memory, and the next chunk is
 // on its way while this one is multiplied.  The RMS normalisation before a projection (its row scale commutes with the
-// product), the residual add and SwiGLU are part of the launch.  Any M, N, K; the sums have one fixed order.
+// product), the residual add, SwiGLU and the rotary step with its cache append are part of the launch.  Any M, N, K; the sums have one fixed order.
 // A tile: 4 * MI rows x 8 * NJ weight rows; BLOCKS: CTAs that an SM has registers for.  (LD: + 4, rows eight apart meet in
 // different banks.)
 template <int MI_, int NJ_, int KC_, int BLOCKS_>
@@ -85,14 +85,22 @@ __global__ void __launch_bounds__(256, Tile::BLOCKS) gemm_rows_kernel(const Rows
   pdl_trigger();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.x * RG_M, t0 = blockIdx.y + blockIdx.z * gridDim.y;   // (blocks that share weight rows run side by side)
-  const bool glu = g.epilogue == RG_SWIGLU;
+  const bool qkv = g.epilogue == RG_QKV, glu = g.epilogue == RG_SWIGLU || qkv;   // an output column is made of two weight rows
+  const int half = g.kv.head_dim >> 1;
   const T *gain = reinterpret_cast<const T *>(g.gain);
-  // weight row r of this tile: under SwiGLU the first half of the rows are gate features, the second the same up features
+  // weight row r of this tile: under SwiGLU the first half of the rows are gate features, the second the same up features; of
+  // rotated pairs the first half of the rows holds the first entries, the second the others
   auto wrow = [&](int r) -> const T * {
     int n, j = 0;
     if (glu) {
       j = r >= BN / 2;
       n = t0 * (BN / 2) + r - j * (BN / 2);
+      if (qkv) {
+        if (n >= g.N) return nullptr;
+        n = n / half * (2 * half) + n % half + j * half;
+        j = 0;
+        while (j < 2 && n >= g.n[j]) n -= g.n[j++];
+      }
     } else {
       n = t0 * BN + r;
       while (j < 2 && n >= g.n[j]) n -= g.n[j++];
@@ -204,6 +212,30 @@ __global__ void __launch_bounds__(256, Tile::BLOCKS) gemm_rows_kernel(const Rows
       scale = rsqrtf(t / (float)g.K + g.eps);
     }
     float v = total(r, c) * scale;
+    if (qkv) {
+      const float u = total(r, c + BN / 2) * scale;
+      const int pos = g.in_pos[m];
+      if (pos < 0) continue;
+      const int head = n / half, j = n % half, kh = head - g.n_heads, nkv = g.kv.n_kv_heads;
+      const bool is_v = kh >= nkv;
+      float x1 = v, x2 = u;
+      if (!is_v) {
+        const float2 cs = g.rope[(size_t)pos * half + j];
+        x1 = v * cs.x - u * cs.y;
+        x2 = u * cs.x + v * cs.y;
+      }
+      if (kh < 0) {
+        float *dst = reinterpret_cast<float *>(g.out) + (size_t)m * g.ldc + head * 2 * half + j;
+        dst[0] = x1;
+        dst[half] = x2;
+      } else {
+        T *dst = reinterpret_cast<T *>(g.kv.base) +
+                 kv_row_offset(g.kv, seg_sequence(g.segs, m / g.segs.rows), is_v ? 1 : 0, kh - (is_v ? nkv : 0), pos) + j;
+        dst[0] = from_f<T>(x1);
+        dst[half] = from_f<T>(x2);
+      }
+      continue;
+    }
     if (glu) {
       const float u = total(r, c + BN / 2) * scale;
       v = v / (1.0f + expf(-v)) * u;
@@ -217,7 +249,7 @@ __global__ void __launch_bounds__(256, Tile::BLOCKS) gemm_rows_kernel(const Rows
 
 template <typename T, typename Tile>
 int gemm_rows_tile(const RowsGemm &g, bool vec, cudaStream_t stream) {
-  const int cols = g.epilogue == RG_SWIGLU ? Tile::BN / 2 : Tile::BN;
+  const int cols = g.epilogue == RG_SWIGLU || g.epilogue == RG_QKV ? Tile::BN / 2 : Tile::BN;
   const int n_tiles = (g.N + cols - 1) / cols, layers = (n_tiles + 65534) / 65535;
   const dim3 grid((g.M + Tile::BM - 1) / Tile::BM, (n_tiles + layers - 1) / layers, layers);
   auto launch = [&](auto kernel) -> int {
@@ -233,7 +265,7 @@ int gemm_rows_tile(const RowsGemm &g, bool vec, cudaStream_t stream) {
 template <typename T>
 int gemm_rows_t(const RowsGemm &g, cudaStream_t stream) {
   auto tiles = [&](int rows, int cols) { return (long)((g.M + rows - 1) / rows) * ((g.N + cols - 1) / cols); };
-  const int glu = g.epilogue == RG_SWIGLU ? 2 : 1;   // weight rows of an output column
+  const int glu = g.epilogue == RG_SWIGLU || g.epilogue == RG_QKV ? 2 : 1;   // weight rows of an output column
   bool vec = g.K % 4 == 0 && g.ldx % 4 == 0 && ((uintptr_t)g.x & 15u) == 0 && ((uintptr_t)g.gain & (4 * sizeof(T) - 1)) == 0;
   for (int j = 0; j < 3; ++j) vec = vec && ((uintptr_t)g.w[j] & (4 * sizeof(T) - 1)) == 0;
   // us, smallest / middle / largest tile.  The smallest while its grid is one wave (fp32 64 x 256 x 683: 8.3 / 14.5 / 18.5), the
