@@ -15,6 +15,9 @@
 //
 // Bound: the bytes of K and V (a tile of 64 KB takes the tensor pipe 500 to 1000 cycles, an SM's share of HBM about 2800).
 // One CTA per SM with all of its shared memory: 96 to 160 KB of tiles in flight.
+// (us a call, 32 heads of 128, mma.sync with a CTA per stream and tiles of 64 keys -> now: 8 x 32 rows x 4009 keys 123 -> 101 (K and V
+// at 5.2 TB/s, launch included; 88 back to back), 8 x 64 rows 202 -> 119, 5 x 32 x 3032 94 -> 62, 1 x 32 x 2232 with the merge
+// 31 -> 23.  Windows of up to 32 rows take 64 columns, longer ones 128: with 128 the ring holds three tiles and not five.)
 // Partials (reference, sum, unnormalised output) go to the merge kernel of attention.cu.  Every barrier wait is bounded.
 #include <type_traits>
 
