@@ -109,11 +109,9 @@ __global__ void __launch_bounds__(NWARPS * 32) attention_partial_kernel(
       const float sv = visible ? sc[i] * scale : -INFINITY;
       const float tmax = warp_max(sv);
       const float m_new = fmaxf(m_run[i], tmax);
-      float pexp = 0.0f, alpha = 1.0f;
-      if (m_new > -INFINITY) {
-        pexp = visible ? expf(sv - m_new) : 0.0f;
-        alpha = m_run[i] > -INFINITY ? expf(m_run[i] - m_new) : 0.0f;
-      }
+      // (no finite score so far: zeros, or the NaN that a maximum does not show)
+      const float pexp = visible ? expf(sv - (m_new > -INFINITY ? m_new : 0.0f)) : 0.0f;
+      const float alpha = m_run[i] > -INFINITY ? expf(m_run[i] - m_new) : 1.0f;
       const float psum = warp_sum(pexp);
       l_run[i] = l_run[i] * alpha + psum;
       m_run[i] = m_new;
@@ -198,7 +196,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attention_combine_kernel(c
       a1.y += v1[s].y * w;
     }
   }
-  const bool live = pos >= 0 && denom > 0.0f;
+  const bool live = pos >= 0 && denom != 0.0f;   // (a range with a NaN among its scores has a NaN for its sum: the row becomes NaN)
   auto put = [&](int d, float2 a) {
     const float x = live ? a.x / denom : 0.0f, y = live ? a.y / denom : 0.0f;
     const size_t idx = (size_t)mh * hd + d;

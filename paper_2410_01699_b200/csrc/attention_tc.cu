@@ -509,7 +509,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
           *reinterpret_cast<float2 *>(ml + (rec0 + ts * rec_step) * 2) = make_float2(l > 0.0f ? my_ref * 0.6931471805599453f : -INFINITY, l);
       }
       if (direct) {
-        if (ts < WP) sh.red[st][0][ts] = l > 0.0f ? 1.0f / l : 0.0f;   // inactive rows: zeros  (each thread has read its column only)
+        // inactive rows: zeros; the NaN of a score that is not finite stays  (each thread has read its column only)
+        if (ts < WP) sh.red[st][0][ts] = l == 0.0f ? 0.0f : 1.0f / l;
         stream_sync(st);
       }
       const int dim = w * 32 + lane;
@@ -554,7 +555,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const float inv = sh.red[st][0][c * 16 + i];
-              v[i] = inv > 0.0f ? v[i] * inv : 0.0f;
+              v[i] = inv == 0.0f ? 0.0f : v[i] * inv;
             }
             if constexpr (OUT) {
               float *dst = p.out + at;

@@ -91,3 +91,37 @@ def test_attention_tiles_and_growing_scores(batch, window, keys, heads, kv_heads
     tol = 2e-4 + 4 * 2.0 ** -17 * bound * kv[some][:, 1].abs().max().item()
     err = np.abs(out.cpu()[rows].double().numpy() - ref).max()
     assert err <= tol, f"max |err| {err:.3e} (bound {tol:.3e})"
+
+
+@pytest.mark.parametrize("batch,window,keys,heads,kv_heads,hd", [
+    (20, 40, 300, 8, 4, 128),    # one key range: the kernel writes the rows itself
+    (20, 24, 300, 8, 8, 64),
+    (2, 20, 600, 4, 2, 128),     # several key ranges and the merge; the bad key is in the first, the window in the last
+    (1, 64, 150, 2, 1, 64),      # more ranges than tiles
+])
+def test_attention_shows_scores_that_are_not_numbers(batch, window, keys, heads, kv_heads, hd):
+    """A NaN in a key reaches every row that sees it and no other, one in a query its own row."""
+    g = torch.Generator().manual_seed(keys + window)
+    n, group = keys - window, heads // kv_heads
+    q = torch.randn(batch * window, heads, hd, generator=g)
+    kv = torch.randn(batch, 2, kv_heads, keys, hd, generator=g).to(torch.bfloat16)
+    pos = (n + torch.arange(window, dtype=torch.int32)).repeat(batch)
+    pos[:2] = -1
+    clean, _ = B.sjd_attention(q.cuda(), kv.cuda(), pos.cuda(), window, kv_heads)
+    b = batch - 1
+    for key in (70, n + window // 2):
+        bad = kv.clone()
+        bad[b, 0, kv_heads - 1, key, 3] = float("nan")
+        out, status = B.sjd_attention(q.cuda(), bad.cuda(), pos.cuda(), window, kv_heads)
+        sees = torch.zeros(batch * window, heads, dtype=torch.bool)
+        sees[b * window:, heads - group:] = (pos[b * window:] >= key)[:, None]
+        assert int(status.item()) == 0 and sees.any()
+        assert torch.all(out.cpu()[sees].isnan())
+        assert torch.equal(out.cpu()[~sees], clean.cpu()[~sees])
+    q[window // 2, 0, 5] = float("nan")
+    out, status = B.sjd_attention(q.cuda(), kv.cuda(), pos.cuda(), window, kv_heads)
+    hit = torch.zeros(batch * window, heads, dtype=torch.bool)
+    hit[window // 2, 0] = True
+    assert int(status.item()) == 0
+    assert torch.all(out.cpu()[hit].isnan())
+    assert torch.equal(out.cpu()[~hit], clean.cpu()[~hit])

@@ -552,6 +552,28 @@ def test_api_errors_and_state():
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize("name,over", [("tiny", {}), ("small-bf16", {}), ("small-bf16", dict(ffn_hidden=1400))])
+def test_bad_prompt_token_raises_the_flag(name, over):
+    """A prompt token whose embedding is not a number makes every key it leaves in the cache one: the iterations of its sequence
+    say so, those of the other sequence do not.  (Both pipelines, several key ranges: the long prompt's keys are in all of them.)"""
+    wl = WORKLOADS[name].with_(**over)
+    weights = make_weights(wl)
+    weights["tok_emb"][7] = float("nan")
+    prompt = torch.randint(8, wl.vocab, (2, 300), generator=torch.Generator().manual_seed(3), dtype=torch.int32)
+    prompt[0, 40] = 7
+    ctx = B.Context(B.make_model_cfg(wl, max_batch=2, max_seq=400, max_window=wl.window), B.weights_to_device(weights))
+    ctx.prefill(prompt.cuda(), B.make_sample_cfg(top_k=50, window=wl.window, n_generate=40, seed=1))
+    out = B.StepOut(2, wl.window)
+    ctx.get_window(out)
+    assert not (out.host()["draft"] == 7).any()   # (no draft of this seed is the bad token)
+    ctx.step(out)
+    flags = out.host()["flags"]
+    assert flags[0] & B.SJD_FLAG_NONFINITE and not flags[1] & B.SJD_FLAG_NONFINITE
+    logits = ctx.peek_logits()
+    assert logits[0].isnan().all() and not logits[1].isnan().any()
+    assert ctx.device_status() == B.SJD_OK
+
+
 @pytest.mark.parametrize("refused", [
     dict(batch=1, seed=5, n_generate=250),   # five pages needed, four there
     dict(batch=2, seed=2, n_generate=120),   # six pages for a larger batch
