@@ -93,6 +93,22 @@ def test_attention_tiles_and_growing_scores(batch, window, keys, heads, kv_heads
     assert err <= tol, f"max |err| {err:.3e} (bound {tol:.3e})"
 
 
+@pytest.mark.parametrize("window,heads,hd", [(5, 4, 64), (32, 2, 128), (48, 4, 64), (64, 2, 128)])
+def test_attention_takes_queries_that_start_on_eight_bytes(window, heads, hd):
+    """They are loaded in pairs instead of in fours: the same values, so the same output."""
+    g = torch.Generator().manual_seed(window)
+    q = torch.randn(2 * window, heads, hd, generator=g).cuda()
+    kv = torch.randn(2, 2, heads, 200, hd, generator=g).to(torch.bfloat16).cuda()
+    pos = (200 - window + torch.arange(window, dtype=torch.int32)).repeat(2).cuda()
+    pos[-2:] = -1
+    shifted = torch.full((q.numel() + 2,), float("nan"), device="cuda")[2:].view(q.shape)
+    shifted.copy_(q)
+    assert q.data_ptr() % 16 == 0 and shifted.data_ptr() % 16 == 8
+    want, _ = B.sjd_attention(q, kv, pos, window, heads)
+    got, status = B.sjd_attention(shifted, kv, pos, window, heads)
+    assert int(status.item()) == 0 and torch.equal(got, want)
+
+
 @pytest.mark.parametrize("batch,window,keys,heads,kv_heads,hd", [
     (20, 40, 300, 8, 4, 128),    # one key range: the kernel writes the rows itself
     (20, 24, 300, 8, 8, 64),
