@@ -19,7 +19,7 @@
 //     split order: deterministic, no atomics, no serial reduction tail inside the GEMM.
 //   * Warp 0 issues TMA loads of 128B-swizzled 128x64 W tiles (evict-first L2 policy) into a ring of shared-memory stages
 //     guarded by mbarriers, warp 6 those of the activation tiles into a shorter ring of their own; warp 1 issues the
-//     MMAs into a TMEM accumulator and commits to the stages' "empty" barriers; warps 2-5 drain the
+//     MMAs into a TMEM accumulator and commits to the k-block's "done" barrier, which frees both stages; warps 2-5 drain the
 //     accumulator with tcgen05.ld and store.
 //   * Every wait is bounded: after ~2 s a role records an error in the status word and leaves; the
 //     CTA still frees its TMEM.
@@ -849,16 +849,19 @@ static int allow_gemm_smem() {
 // leave a few KB: without them no CTA of the next kernel can wait beside them, and its launch and the weights that it
 // prefetches come late.  us of a step of 16 layers, stages of weights + activations: 7B, 32 rows: 6 + 2 (no
 // room left) 1755, 5 + 2 1696, 4 + 3 1663, 5 + 3 1646, 4 + 4 1670; 64 rows: 3 + 3 1946, 4 + 2 1905, 4 + 3 (no room left) 1937.
+// 48 rows, two layers and the logits: 7B 5 + 2 344, 4 + 3 338; 8B 570 and 559.  Where K is split a CTA has 8 to 24 k-blocks, and the
+// room is worth more than the fifth stage (7B, 32 rows, two layers and the logits 311, with 4 + 3 there 307; sjd_gemm
+// 32 x 4096 x 4096 12.2 and 11.7, one ring for both operands 11.6).
 // At most one CTA per SM (small models, short K): both rings hold all or much of K.
-void ring_stages(bool deep, int x_bytes, int *stages, int *x_stages) {
+void ring_stages(bool deep, bool split, int x_bytes, int *stages, int *x_stages) {
   if (deep) {
     const int n = kDeepRing / (W_TILE_BYTES + x_bytes);
     *stages = *x_stages = n > kMaxStages ? kMaxStages : n;
     return;
   }
-  *x_stages = x_bytes <= W_TILE_BYTES / 2 ? 3 : 2;
-  const int n = (kSmemBudget - *x_stages * x_bytes) / W_TILE_BYTES;
-  *stages = n > kMaxStages ? kMaxStages : n;
+  *x_stages = x_bytes <= W_TILE_BYTES * 3 / 4 ? 3 : 2;
+  const int n = (kSmemBudget - *x_stages * x_bytes) / W_TILE_BYTES, most = split ? 4 : kMaxStages;
+  *stages = n > most ? most : n;
 }
 
 static int launch_gemm_pair(const GemmTcCall &g, const GemmParams &p, int tiles, cudaStream_t stream) {
@@ -948,7 +951,7 @@ int launch_gemm_tc(const GemmTcCall &g, cudaStream_t stream) {
   const int x_bytes = 2 * p.Mp * TILE_K * 2;
   const int ctas = tiles;
   const bool deep = g.n_sms > 0 && ctas * g.splits <= g.n_sms;
-  ring_stages(deep, x_bytes, &p.stages, &p.x_stages);
+  ring_stages(deep, g.splits > 1, x_bytes, &p.stages, &p.x_stages);
   const size_t smem = (size_t)p.stages * W_TILE_BYTES + (size_t)p.x_stages * x_bytes + sizeof(TcShared);
   const CUtensorMap &w0 = reinterpret_cast<const CUtensorMap &>(*g.w_map[0]);
   const CUtensorMap &w1 = reinterpret_cast<const CUtensorMap &>(*g.w_map[g.n_mats > 1 ? 1 : 0]);

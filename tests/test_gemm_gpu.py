@@ -34,6 +34,8 @@ def _tolerance(x, w, k):
     (17, 384, 512),       # ragged row count (padded to 32 columns of the MMA)
     (1, 128, 128),        # single row
     (64, 2048, 1024),     # W = 64
+    (48, 4096, 4096),     # W = 48: three activation stages beside four of weights, K split
+    (33, 19200, 640),     # the same with whole K, two CTAs on some SMs
     (128, 512, 256),      # widest supported window batch
     (32, 65536, 512),     # 512 tiles (vocabulary-sized N)
     (112, 768, 1024),     # 112 rows in one slab: accumulators of 224 columns
