@@ -314,7 +314,8 @@ int sjd_gemm(int M, int N, int K, const float *x, const void *w, float *out, int
  * tensor-core split-KV kernel sjd_step uses for bf16 caches: query row m = b * window + k, at absolute
  * position in_pos[m] (-1: inactive row, output zeros), attends cache rows 0 .. in_pos[m] of sequence b:
  *     out[m][h] = softmax(q[m][h] . K[b][h / (H/KVh)][0..pos]^T / sqrt(head_dim)) V[b][...][0..pos]
- * q, out: device fp32 [batch*window][n_heads*head_dim]; kv_cache: device bf16
+ * q, out: device fp32 [batch*window][n_heads*head_dim], q starting on a multiple of 8 bytes (of 16: a little
+ * faster; BAD_ARG on any other address); kv_cache: device bf16
  * [batch][K|V][n_kv_heads][max_seq][head_dim], finite everywhere (rows beyond the positions are read
  * and masked); in_pos: device int32 [batch*window].  Covered: head_dim 64 or 128, window <= 64,
  * compute capability >= 9; anything else returns SJD_ERR_UNSUPPORTED.  ws: device scratch of

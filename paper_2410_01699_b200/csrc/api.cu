@@ -208,7 +208,7 @@ extern "C" int sjd_attention(int batch, int window, int n_heads, int n_kv_heads,
     return SJD_ERR_BAD_ARG;
   if (n_heads % n_kv_heads != 0) return SJD_ERR_BAD_ARG;
   if (!attention_tc_supported(head_dim, window)) return SJD_ERR_UNSUPPORTED;
-  if (((uintptr_t)ws & 255u) != 0) return SJD_ERR_BAD_ARG;
+  if (((uintptr_t)ws & 255u) != 0 || ((uintptr_t)q & 7u) != 0) return SJD_ERR_BAD_ARG;   // (q is loaded in pairs of floats)
   if (ws_bytes < sjd_attention_workspace_bytes(batch, window, n_heads, head_dim)) return SJD_ERR_CAPACITY;
   int dev = 0, cc_major = 0;
   SJD_CUDA(cudaGetDevice(&dev));

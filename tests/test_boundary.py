@@ -75,6 +75,10 @@ def test_calls_reject_bad_arguments_without_a_device():
     assert lib.sjd_verify(1, 65, 16, 0, one, one, one, None, None, C.byref(s), 0, C.byref(out), one, 1 << 20, None) == B.SJD_ERR_CAPACITY
     assert lib.sjd_verify(1, 4, 16, 0, one, one, one, None, None, C.byref(s), 0, C.byref(out), one, 8, None) == B.SJD_ERR_CAPACITY
     assert lib.sjd_verify(1, 4, 16, 0, None, one, one, None, None, C.byref(s), 0, C.byref(out), one, 1 << 20, None) == B.SJD_ERR_BAD_ARG
+    # queries are loaded in pairs of floats: any other address is refused before the device is asked for
+    def attention(q):
+        return lib.sjd_attention(1, 4, 2, 2, 64, 32, C.c_void_p(q), one, one, one, one, 1 << 20, None)
+    assert attention(256 + 4) == B.SJD_ERR_BAD_ARG and attention(256 + 2) == B.SJD_ERR_BAD_ARG
     ctx = C.c_void_p()
     cfg = B.make_model_cfg(WORKLOADS["tiny"], 1, 64, 8)
     assert lib.sjd_init(C.byref(ctx), C.byref(cfg), None, one, 1 << 30) == B.SJD_ERR_BAD_ARG
