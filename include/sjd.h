@@ -318,7 +318,7 @@ int sjd_gemm(int M, int N, int K, const float *x, const void *w, float *out, int
  * faster; BAD_ARG on any other address); kv_cache: device bf16
  * [batch][K|V][n_kv_heads][max_seq][head_dim], finite everywhere (rows beyond the positions are read
  * and masked); in_pos: device int32 [batch*window].  Covered: head_dim 64 or 128, window <= 64,
- * compute capability >= 9; anything else returns SJD_ERR_UNSUPPORTED.  ws: device scratch of
+ * compute capability 10.x; anything else returns SJD_ERR_UNSUPPORTED.  ws: device scratch of
  * sjd_attention_workspace_bytes(...), 256-byte aligned; its first int32 is non-zero after the stream
  * has drained if a bounded device-side wait ran out.
  * Errors: BAD_ARG, UNSUPPORTED, CAPACITY, CUDA.

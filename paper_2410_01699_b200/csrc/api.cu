@@ -213,7 +213,7 @@ extern "C" int sjd_attention(int batch, int window, int n_heads, int n_kv_heads,
   int dev = 0, cc_major = 0;
   SJD_CUDA(cudaGetDevice(&dev));
   SJD_CUDA(cudaDeviceGetAttribute(&cc_major, cudaDevAttrComputeCapabilityMajor, dev));
-  if (cc_major < 9) return SJD_ERR_UNSUPPORTED;
+  if (cc_major != 10) return SJD_ERR_UNSUPPORTED;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   int *status = (int *)ws;
   float *partial = (float *)((char *)ws + 256);
