@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
     if (!waited) pdl_wait();
     if (!ok && lane == 0) atomicExch(p.status, 4);
     // leave no copy in flight, whatever the other roles do
-    for (int j = it > p.slots ? it - p.slots : 0; j < it; ++j) mbar_wait(&sh.full[j % p.slots], (uint32_t)((j / p.slots) & 1));
+    for (int j = it > p.slots ? it - p.slots : 0; j < it; ++j) warp_wait(&sh.full[j % p.slots], (uint32_t)((j / p.slots) & 1));
   } else if (warp == 9) {
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t idesc = umma_idesc_bf16(2 * WP);
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
     const int first = sh.first[st];
     for (int t = 0; t < n; ++t) {
       const int key0 = me.k_begin + t * KT, key = key0 + ts;
-      ok = mbar_wait(&sh.s_full[st], (uint32_t)(t & 1));   // (a wait that ran out is noticed at the vote below)
+      ok = warp_wait(&sh.s_full[st], (uint32_t)(t & 1));   // (a wait that ran out is noticed at the vote below)
       tc_fence_after();
       float sv[WP];
 #pragma unroll
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
         }
       }
       // the tile before is multiplied: P may be written, O^T is at rest
-      if (t > 0) ok = mbar_wait(&sh.pv_done[st], (uint32_t)((t - 1) & 1)) && ok;
+      if (t > 0) ok = warp_wait(&sh.pv_done[st], (uint32_t)((t - 1) & 1)) && ok;
       float over = 0.0f;
       if (t > 0) {
 #pragma unroll
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
       for (int i = 0; i < 32; ++i) v[i] = l_acc[g * 32 + i];
       sh.red[st][w][g * 32 + lane] = lanes_combine(v, [](float a, float b) { return a + b; });
     }
-    if (ok && n > 0) ok = mbar_wait(&sh.pv_done[st], (uint32_t)((n - 1) & 1));
+    if (ok && n > 0) ok = warp_wait(&sh.pv_done[st], (uint32_t)((n - 1) & 1));
     if (!stream_any(st, !ok)) {
       tc_fence_after();
       const bool direct = p.splits == 1;

@@ -232,7 +232,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
       if (lane == 0) atomicExch(p.status, 1);
       // leave no copy in flight: wait (bounded) for the stages armed most recently
       const int armed = it < ring ? it : ring;
-      for (int j = it - armed; j < it; ++j) mbar_wait(&full[j % ring], (uint32_t)((j / ring) & 1));
+      for (int j = it - armed; j < it; ++j) warp_wait(&full[j % ring], (uint32_t)((j / ring) & 1));
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -265,7 +265,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
     // ------------------------------------------------------------------ epilogue warps (2..5)
     const int quarter = warp & 3;                 // TMEM lane quarter this warp may read
     const int row = quarter * 32 + lane;          // weight row inside the tile
-    const bool ok = epilogue_all(mbar_wait(&sh.acc_full, 0));
+    const bool ok = epilogue_all(warp_wait(&sh.acc_full, 0));
     if (ok) {
       tc_fence_after();
       pdl_wait();   // the planes may still be read, and the row scales written, by the preceding kernel
@@ -604,7 +604,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
         }
         pair_epilogue_all(true);
       }
-      if (!pair_epilogue_all(mbar_wait(&acc_full[buf], (n >> 1) & 1))) {
+      if (!pair_epilogue_all(warp_wait(&acc_full[buf], (n >> 1) & 1))) {
         if (tid == 64) atomicExch(p.status, 3);
         break;
       }

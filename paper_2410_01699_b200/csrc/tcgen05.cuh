@@ -34,7 +34,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait: false if the barrier did not flip within kWaitNs.
+// Bounded wait: false if the barrier did not flip within kWaitNs.  A thread's own: its lanes may leave the loop in different rounds, and what
+// follows is tcgen05.ld, a named barrier or an election, which want the warp together.  Roles wait with warp_wait.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_ns();

@@ -99,6 +99,14 @@ def test_every_entry_point_of_the_tensor_core_kernels_asks_for_the_same_device()
     assert re.findall(r"compute\s[\s*]*capability\s([^;]*?);", header) == ["10.x", "10.x"]
 
 
+def test_tensor_core_roles_wait_as_a_warp():
+    """The lanes of a warp may leave a polling loop in different rounds; the tcgen05 loads and named barriers that follow the waits are
+    defined for a converged warp.  So no kernel calls the wait of a single thread."""
+    csrc = os.path.join(ROOT, "paper_2410_01699_b200", "csrc")
+    calls = {f: len(re.findall(r"\bmbar_wait\(", open(os.path.join(csrc, f)).read())) for f in ("attention_tc.cu", "gemm_tc.cu", "tcgen05.cuh")}
+    assert calls == {"attention_tc.cu": 0, "gemm_tc.cu": 0, "tcgen05.cuh": 2}   # its definition and warp_wait
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libsjd.so")
