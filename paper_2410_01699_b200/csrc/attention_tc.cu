@@ -151,7 +151,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int W = p.rows_per_seq;
   const int n_streams = p.n_heads * p.n_segs * p.splits;
-  if (p.clear_status && blockIdx.x == 0 && tid == 0) *p.status = 0;   // (the first error is 2 s away)
+  // The swizzled tiles have to start on 1024 bytes (the same for every CTA of a launch); any other error is 2 s away.
+  const bool skewed = (smem_u32(attn_smem) & 1023u) != 0;
+  if (tid == 0 && (skewed || (p.clear_status && blockIdx.x == 0))) *p.status = skewed ? 5 : 0;
   if (PACKED) pdl_wait();   // (a window's positions, and its keys before it, are older than the step: see embed_kernel)
 
   auto stream_of = [&](int st) {

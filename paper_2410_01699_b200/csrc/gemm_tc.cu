@@ -170,7 +170,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
   while ((int)tmem_cols < NN) tmem_cols <<= 1;
 
   if (tid == 0) {
-    if (smem_u32(smem) & 1023u) atomicExch(p.status, 5);   // (the swizzled tiles have to start on 1024 bytes)
     tma_prefetch_desc(w_map);
     tma_prefetch_desc(&x_map);
   }
@@ -200,6 +199,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     if (!is_w) pdl_wait();
+    // (the swizzled tiles have to start on 1024 bytes; not before the wait: sjd_gemm's split kernel clears the word)
+    if (!is_w && lane == 0 && (smem_u32(smem) & 1023u) != 0) atomicExch(p.status, 5);
     SJD_TL(TL_GEMM, 1, !is_w && lane == 0);
     const int first = (tile * kTileSkew) % n_kb;
     int s = 0, it = 0;
