@@ -14,10 +14,12 @@
 // lanes; the sums of the probabilities stay in registers until the end.
 //
 // Bound: the bytes of K and V (a tile of 64 KB takes the tensor pipe 500 to 1000 cycles, an SM's share of HBM about 2800).
-// One CTA per SM with all of its shared memory: 96 to 160 KB of tiles in flight.
+// One CTA per SM, with all of its shared memory (head_dim 64 and up to 32 columns: 147 KB, the six tiles of the longest ring): 96 to
+// 160 KB of tiles in flight.
 // (us a call, 32 heads of 128, mma.sync with a CTA per stream and tiles of 64 keys -> now: 8 x 32 rows x 4009 keys 123 -> 101 (K and V
 // at 5.2 TB/s, launch included; 88 back to back), 8 x 64 rows 202 -> 119, 5 x 32 x 3032 94 -> 62, 1 x 32 x 2232 with the merge
-// 31 -> 23.  Windows of up to 32 rows take 64 columns, longer ones 128: with 128 the ring holds three tiles and not five.)
+// 31 -> 23.  Windows of up to 32 rows take 64 columns, longer ones 128: with 128 the ring holds three tiles and not five, and a thread
+// has twice the columns.  Over few keys that thread is the bound: 10 x 48 rows x 64 keys, two rounds of the grid, 20 -> 22.)
 // Partials (reference, sum, unnormalised output) go to the merge kernel of attention.cu.  Every barrier wait is bounded.
 #include <type_traits>
 
@@ -89,14 +91,6 @@ __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-// two floats -> packed bf16 hi pair and bf16 lo pair (lo = value - hi, rounded)
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t &hi, uint32_t &lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  const uint32_t w = *reinterpret_cast<const uint32_t *>(&h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(a - __uint_as_float(w << 16), b - __uint_as_float(w & 0xFFFF0000u));
-  hi = w;
-  lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 // value i of 32, combined over the lanes of the warp, in lane i (31 exchanges)
 template <typename F>
@@ -624,22 +618,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_tc_kernel(const __g
   }
 }
 
-typedef CUresult (*EncodeTiledFn3)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 }  // namespace
 
 // bf16 cache [planes][max_seq][head_dim] as boxes of 64 keys x 64 dims, 128-byte swizzle
 int make_kv_tensor_map(TensorMap *out, const void *base, long planes, long max_seq, int head_dim) {
-  static EncodeTiledFn3 fn = nullptr;
-  if (!fn) {
-    void *sym = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn3>(sym);
-  }
+  EncodeTiledFn fn = encode_fn();
   if (!fn) return SJD_ERR_UNSUPPORTED;
   if (((uintptr_t)base & 15u) != 0 || (head_dim != 64 && head_dim != 128)) return SJD_ERR_UNSUPPORTED;
   cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)max_seq, (cuuint64_t)planes};

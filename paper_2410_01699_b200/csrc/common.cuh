@@ -349,6 +349,14 @@ __device__ __forceinline__ size_t kv_row_offset(const KvLayout &kv, int b, int w
   return (((((size_t)page * kv.n_layers + kv.layer) * 2 + which) * kv.n_kv_heads + kh) * KV_PAGE + pos % KV_PAGE) *
          kv.head_dim;
 }
+// two floats -> packed bf16 hi pair and bf16 lo pair (lo = value - hi, rounded)
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t &hi, uint32_t &lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  const uint32_t w = *reinterpret_cast<const uint32_t *>(&h);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(a - __uint_as_float(w << 16), b - __uint_as_float(w & 0xFFFF0000u));
+  hi = w;
+  lo = *reinterpret_cast<const uint32_t *>(&l);
+}
 // ---- model forward (model_kernels.cu, attention.cu); `dtype` selects float / bf16 storage
 enum RowsEpilogue { RG_STORE = 0, RG_ADD = 1, RG_LOGITS = 2, RG_SWIGLU = 3, RG_QKV = 4 };
 // One launch of the generic projections: out[m][n] (epilogue) = s(m) * sum_k x[m][k] * gain[k] * W[n][k], fp32 sums.  The
@@ -375,7 +383,7 @@ struct RowsGemm {
 };
 int launch_gemm_rows(int dtype, const RowsGemm &g, cudaStream_t stream);
 // QK-norm variant: every head of q and of k is RMS-normalised over its head_dim entries (gains of `dtype`,
-// length head_dim) before the rotary step; null gains: the plain model.
+// length head_dim) before the rotary step; null gains (launch_qkv_finish only): the plain model.
 struct QkNorm {
   const void *q_gain, *k_gain;
   float eps;

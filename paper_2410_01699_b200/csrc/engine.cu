@@ -13,8 +13,8 @@
 #include "common.cuh"
 
 namespace sjd {
-// Key-range splits of the attention grid: heads * batch * splits CTAs, two of which fit one SM (their
-// K/V rings take ~99 KB each), so the grid is sized to fill one wave of 2 * 148 slots and no more.
+// Key ranges per (head, sequence): a stream of the attention is one of heads * batch * splits, a CTA works on two, an SM holds one
+// CTA, so the grid is sized to fill one wave of 2 * 148 streams and no more.
 #ifndef SJD_ATTN_SLOTS
 #define SJD_ATTN_SLOTS (2 * 148)
 #endif

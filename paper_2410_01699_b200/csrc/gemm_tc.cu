@@ -58,7 +58,8 @@ constexpr int kMaxStages = 8;
 #endif
 // CTA t starts t * kTileSkew k-blocks into its range of K.  In step, all of a launch's CTAs ask L2 for the same few lines of the
 // activations at the same time (gate|up, 172 CTAs: 34.2 us, with skew 32.5; logits 91 and 86.4; us of a step of 16 layers, 7B,
-// 32 rows: skew 0 / 4 / 8 / 12: 1655 / 1617 / 1616 / 1614, also skewed where K is split 1600 against 1605).
+// 32 rows: skew 0 / 4 / 8 / 12: 1655 / 1617 / 1616 / 1614, also skewed where K is split 1600 against 1605; two layers and the logits,
+// 0 and 8: 7B 48 rows 350 and 344, 64 rows 364 and 356, 8B 64 rows 600 and 592).  Of eight k-blocks (the O projection) all start at the first.
 constexpr int kTileSkew = 8;
 constexpr int kSmemBudget = SJD_GEMM_SMEM_BUDGET, kDeepRing = SJD_GEMM_DEEP_RING;
 
@@ -67,7 +68,7 @@ struct GemmParams {
   size_t plane_stride;    // elements between planes
   int ldc;
   int M;                  // valid token rows
-  int Mp;                 // token rows of one slab, a multiple of 16 (MMA N = 2 * Mp: hi and lo plane)
+  int Mp;                 // token rows of one slab, a multiple of 16, on CTA pairs of 8 (MMA N = 2 * Mp: hi and lo plane)
   int n_slabs;            // token slabs (CTA pairs only: more than one)
   int x_lo_row;           // row of the lo plane inside the activation tensor map
   int k_blocks, splits;   // K / 64, K splits (gridDim.y)
@@ -721,22 +722,6 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_consta
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
-}
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void *sym = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(sym);
-  }
-  return fn;
 }
 
 // plain sum of split planes (sjd_gemm): out[m][n] (+)= sum_s P[s][m][n]; V: entries per thread (4 when out is 16-byte aligned)

@@ -283,8 +283,9 @@ template <typename T>
 __global__ void embed_kernel(const T *__restrict__ emb, const int32_t *__restrict__ tok, float *__restrict__ x, int d,
                              int vocab) {
   pdl_wait();
-  // First kernel of a pass, and the only one that lets the next one start after its own wait: whatever was written before the pass
-  // (positions, the cache of earlier steps) is there for every later kernel of the pass, also before that kernel's wait.
+  // First kernel of a pass, and in a step the only one that lets the next one start after its own wait (the attention of a pre-fill pass
+  // does so too): whatever was written before the pass (positions, the cache of earlier steps) is there for every later kernel of the
+  // pass, also before that kernel's wait.
   pdl_trigger();
   const int m = blockIdx.x;
   int t = tok[m];
@@ -294,6 +295,7 @@ __global__ void embed_kernel(const T *__restrict__ emb, const int32_t *__restric
 }
 
 // ------------------------------------------------------------------------------------ RoPE + KV append
+// of models with QK-norm; without it both are part of the query-key-value launch (RG_QKV).
 template <typename T>
 __global__ void rope_append_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ in_pos,
                                    const float2 *__restrict__ rope, float *__restrict__ q, KvLayout kv, RowSegs segs,
@@ -313,16 +315,13 @@ __global__ void rope_append_kernel(const float *__restrict__ qkv, const int32_t 
   for (int i = threadIdx.x; i < (n_heads + nkv) * half; i += blockDim.x) {
     const int head = i / half, j = i % half;
     const float2 c = cs[j];
-    float g1 = 1.0f, g2 = 1.0f;
-    if (qkn.q_gain) {   // QK-norm: this head's RMS over its hd entries (every thread of the head sums them itself)
-      const float *hv = row + (head < n_heads ? head * hd : nq + (head - n_heads) * hd);
-      float ss = 0.0f;
-      for (int t = 0; t < hd; ++t) ss += hv[t] * hv[t];
-      const float rinv = rsqrtf(ss / (float)hd + qkn.eps);
-      const T *gain = reinterpret_cast<const T *>(head < n_heads ? qkn.q_gain : qkn.k_gain);
-      g1 = rinv * to_f<T>(gain[j]);
-      g2 = rinv * to_f<T>(gain[j + half]);
-    }
+    // this head's RMS over its hd entries (every thread of the head sums them itself)
+    const float *hv = row + (head < n_heads ? head * hd : nq + (head - n_heads) * hd);
+    float ss = 0.0f;
+    for (int t = 0; t < hd; ++t) ss += hv[t] * hv[t];
+    const float rinv = rsqrtf(ss / (float)hd + qkn.eps);
+    const T *gain = reinterpret_cast<const T *>(head < n_heads ? qkn.q_gain : qkn.k_gain);
+    const float g1 = rinv * to_f<T>(gain[j]), g2 = rinv * to_f<T>(gain[j + half]);
     if (head < n_heads) {
       const float x1 = g1 * row[head * hd + j], x2 = g2 * row[head * hd + j + half];
       q[(size_t)m * nq + head * hd + j] = x1 * c.x - x2 * c.y;
@@ -365,6 +364,7 @@ int launch_embed(int dtype, const void *tok_emb, const int32_t *tok, float *x, i
 
 int launch_rope_append(int dtype, const float *qkv, const int32_t *in_pos, const float2 *rope_table, float *q,
                        KvLayout kv, int M, RowSegs segs, int n_heads, QkNorm qkn, cudaStream_t stream) {
+  if (!qkn.q_gain || !qkn.k_gain) return SJD_ERR_BAD_ARG;
   SJD_DISPATCH(dtype, SJD_CUDA(launch_kernel(rope_append_kernel<T>, dim3(M), dim3(256), 0, stream, qkv, in_pos, rope_table, q, kv,
                                              segs, n_heads, qkn)));
   SJD_CHECK_LAUNCH();

@@ -446,7 +446,7 @@ def test_large_shapes_reduced_depth(name, layers, steps):
 
 @pytest.mark.parametrize("batch,window,prompt_len,init,steps", [
     (4, 8, 64, INIT_COPY_ABOVE, 3),    # small window, spatial initialisation (grid stride 49), 32 rows per pass
-    (2, 64, 64, INIT_RANDOM, 2),       # widest window: 128 rows per pass, attention with four row bands per CTA
+    (2, 64, 64, INIT_RANDOM, 2),       # widest window: 128 rows per pass, attention in 128 columns with a ring of three tiles
     (8, 32, 64, INIT_RANDOM, 2),       # 256 rows per pass: two token slabs per weight tile at the 7B widths
     (3, 24, 64, INIT_RANDOM, 2),       # 72 rows: a slab that is not a multiple of 16, shared units among its tiles
     (1, 32, 700, INIT_COPY_ABOVE, 2),  # long prefix: several key tiles per split-KV range, pre-fill in 22 chunks

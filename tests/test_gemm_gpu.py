@@ -40,13 +40,13 @@ def _tolerance(x, w, k):
     (32, 65536, 512),     # 512 tiles (vocabulary-sized N)
     (112, 768, 1024),     # 112 rows in one slab: accumulators of 224 columns
     (128, 22016, 4096),   # four images x W = 32 on the gate|up projection: 172 tiles on 148 SMs
-    (129, 256, 512),      # first row count cut into token slabs: two of 80 rows (the second holds 49)
+    (129, 256, 512),      # first row count cut into token slabs: two of 72 rows (the second holds 57)
     (256, 1024, 1024),    # two full slabs of 128 rows
-    (300, 384, 640),      # three ragged slabs of 112 rows (the last holds 76)
+    (300, 384, 640),      # three ragged slabs of 104 rows (the last holds 92)
     (512, 4096, 4096),    # 8 images x W = 64 on the attention output projection: 4 slabs x 32 tiles x K splits
     (1024, 256, 256),     # most rows covered: eight slabs
     (65, 128, 64),            # CTA pairs: one tile (the second CTA has none), one k-block
-    (130, 384, 1088),         # three tiles (an odd pair), two slabs of 80 rows, K over several splits
+    (130, 384, 1088),         # three tiles (an odd pair), two slabs of 72 rows, K over several splits
     (257, 19200, 256),        # more units than pairs, three slabs, few k-blocks per unit
     (72, 384, 1088),          # slabs whose rows are not a multiple of 16: one of 72,
     (200, 1024, 512),         # two of 104,
