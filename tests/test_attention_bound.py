@@ -1,4 +1,4 @@
-"""The error bound of the attention kernel's tile test, on the CPU: it has room for hi and lo planes of both operands and none for
+"""The error bound of the attention kernel's test by entries, on the CPU: it has room for hi and lo planes of both operands and none for
 a kernel that lost one of them."""
 import pytest
 

@@ -60,6 +60,39 @@ def test_attention_rejects_uncovered_shapes():
     assert B.lib().sjd_attention_workspace_bytes(1, 65, 8, 128) == 0
 
 
+@pytest.mark.parametrize("batch,window,keys,heads,kv_heads,hd,grow", [
+    (1, 32, 128, 2, 2, 128, 0.0),     # a tile of 128 keys, full
+    (2, 17, 129, 2, 1, 128, 0.0),     # one key more
+    (1, 16, 65, 4, 4, 64, 0.0),       # one key in the second box of a tile
+    (1, 33, 64, 2, 2, 64, 0.0),       # first window of 64 columns; a tile with one box
+    (51, 3, 140, 3, 3, 64, 0.0),      # an odd number of (head, sequence) pairs with one key range each
+    (20, 64, 400, 8, 2, 128, 1.0),    # scores grow along the keys past every reference: output rescaled, 64 columns, one range
+    (10, 32, 700, 32, 32, 128, 1.0),  # the same with 32 columns, two output accumulators
+    (1, 20, 900, 2, 2, 64, 1.0),      # and over several key ranges
+])
+def test_attention_tiles_and_growing_scores(batch, window, keys, heads, kv_heads, hd, grow):
+    g = torch.Generator().manual_seed(keys + window)
+    n = keys - window
+    q = torch.randn(batch * window, heads, hd, generator=g)
+    kv = torch.randn(batch, 2, kv_heads, keys + 1, hd, generator=g)
+    if grow:   # key j adds grow * j / 2 to every score: sum(q * u) / sqrt(hd) = 1 for u along q's common direction
+        q += 4.0
+        kv[:, 0] += (grow * 0.125 / hd ** 0.5) * torch.arange(keys + 1)[:, None]
+    kv = kv.to(torch.bfloat16)
+    pos = (n + torch.arange(window, dtype=torch.int32)).repeat(batch)
+    out, status = B.sjd_attention(q.cuda(), kv.cuda(), pos.cuda(), window, kv_heads)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    rows = torch.cat([torch.arange(window), torch.arange((batch - 1) * window, batch * window)]).unique()   # first and last sequence
+    some = sorted({0, batch - 1})
+    ref = _reference(q[rows], kv[some], pos[rows], window, kv_heads)
+    # as above, and a score's own error: q is off by 2^-17 of each entry, and 4 * |score error| * max|v| bounds the output's
+    bound = (q[rows].abs().amax(0).amax(0).double() @ kv[some][:, 0].double().abs().amax((0, 1)).T / hd ** 0.5).max().item()
+    tol = 2e-4 + 4 * 2.0 ** -17 * bound * kv[some][:, 1].abs().max().item()
+    err = np.abs(out.cpu()[rows].double().numpy() - ref).max()
+    assert err <= tol, f"max |err| {err:.3e} (bound {tol:.3e})"
+
+
 # batch, window, keys, heads, kv_heads, head_dim, ramp: scores grow by a quarter per key over `ramp` keys and start again
 TILE_CASES = [
     (1, 32, 128, 2, 2, 128, 0),       # a tile of 128 keys, full
@@ -122,7 +155,7 @@ def definition_and_bound(q, kv, pos, window, seqs, q_lo=None, p_lo=None):
 
 
 @pytest.mark.parametrize("case", TILE_CASES)
-def test_attention_tiles_and_growing_scores(case):
+def test_attention_entries_within_their_own_bounds(case):
     """(tests/test_attention_bound.py: the bound notices a lost plane of Q or of the probabilities in every one of these.)"""
     batch, window, kv_heads = case[0], case[1], case[4]
     q, kv, pos = tile_case(*case)
