@@ -17,8 +17,8 @@
 // One CTA per SM, with all of its shared memory (head_dim 64 and up to 32 columns: 147 KB, the six tiles of the longest ring): 96 to
 // 160 KB of tiles in flight.
 // (us a call, 32 heads of 128, mma.sync with a CTA per stream and tiles of 64 keys -> now: 8 x 32 rows x 4009 keys 123 -> 101 (K and V
-// at 5.2 TB/s, launch included; 88 back to back), 8 x 64 rows 202 -> 119, 5 x 32 x 3032 94 -> 62, 1 x 32 x 2232 with the merge
-// 31 -> 23.  Windows of up to 32 rows take 64 columns, longer ones 128: with 128 the ring holds three tiles and not five, and a thread
+// at 5.2 TB/s, launch included; 82 in a graph, 6.4 TB/s), 8 x 64 rows 202 -> 119 (95 in a graph), 5 x 32 x 3032 94 -> 62, 1 x 32 x 2232
+// with the merge 31 -> 23 (13 in a graph).  Windows of up to 32 rows take 64 columns, longer ones 128: with 128 the ring holds three tiles and not five, and a thread
 // has twice the columns.  Over few keys that thread is the bound: 10 x 48 rows x 64 keys, two rounds of the grid, 20 -> 22.)
 // Partials (reference, sum, unnormalised output) go to the merge kernel of attention.cu.  Every barrier wait is bounded.
 #include <type_traits>
